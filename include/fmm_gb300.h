@@ -64,7 +64,7 @@ typedef enum {
 } fmm_status;
 
 typedef enum {
-    FMM_FP64 = 0,       /* every step in FP64                                         */
+    FMM_FP64 = 0,       /* every step in FP64, or with at least FP64's accuracy       */
     FMM_FP32 = 1,       /* mixed: FP32 pair and contraction arithmetic, FP64 elsewhere */
     FMM_3XTF32 = 2      /* mixed: split-precision contraction, FP32 pair arithmetic   */
 } fmm_precision;
@@ -125,9 +125,9 @@ fmm_status fmm_set_sources(fmm_tree *t, const double *positions, const double *m
  * its limit p + s_lo <= 12 refer to s_lo.  Every other rule is that of
  * fmm_set_sources; fmm_update_moments takes rows of the same width.  The FP64
  * form only: FMM_EORDER on an FMM_FP32 / FMM_3XTF32 handle with s_hi > s_lo,
- * and unless 0 <= s_lo <= s_hi <= 2.  The symmetric P2P (p2p_variant 2, the
- * FP64 default) takes mixed systems, each shell's reverse term with its own
- * parity; variants 0 and 1 both run the two-targets-per-thread kernel.
+ * and unless 0 <= s_lo <= s_hi <= 2.  The symmetric P2P (p2p_variant 2)
+ * takes mixed systems, each shell's reverse term with its own parity; variants
+ * 0 and 1 both run the fixed-point kernel.
  */
 fmm_status fmm_set_sources_mixed(fmm_tree *t, const double *positions, const double *moments,
                                  int64_t n, int s_lo, int s_hi);
@@ -411,8 +411,9 @@ fmm_status fmm_evaluate_graph(fmm_tree *t, int p, double theta, int want_potenti
  * Autotuner: times the handle's kernel variants on its own tree and lists
  * (reps evaluates each, after one warm-up, CUDA events on the handle's
  * stream) and keeps the fastest for later evaluates.  Candidates:
- *   FMM_FP64    P2P with one or two targets per thread (p2p_variant 0, 1),
- *               or each mirrored leaf pair once for both directions (2)
+ *   FMM_FP64    P2P one way in FP64 arithmetic (p2p_variant 0), one way in
+ *               64-bit fixed-point arithmetic (1), or in FP64 with each mirrored
+ *               leaf pair once for both directions (2)
  *   FMM_3XTF32  the tensor-core M2L with 8, 16 or 32 key rows per chunk, or
  *               the tiled SIMT FP32 M2L (m2l_tensor 0); then, with the fastest
  *               of those, the P2P tile of the other shape (p2p_targets 1 or 2)
@@ -424,16 +425,16 @@ fmm_status fmm_evaluate_graph(fmm_tree *t, int p, double theta, int want_potenti
  * the target leaf in double-float arithmetic, which holds the near field's
  * rounding at the FP64 form's level; their symmetric kernel (2, selectable
  * with fmm_set_tuning) evaluates every pair in FP32 and is not a candidate.
- * Defaults before tuning: p2p_variant 2 (FP64) or 1 (FP32 forms), the
- * tensor-core M2L (FMM_3XTF32), the tiled SIMT M2L (FMM_FP32), 16 rows per
- * chunk, harmonic M2L.
+ * Defaults before tuning: p2p_variant 1, the tensor-core M2L (FMM_3XTF32), the
+ * tiled SIMT M2L (FMM_FP32), 16 rows per chunk, harmonic M2L.
  * The variants compute the same sums in another order: results agree to the
  * form's rounding, not bitwise.  Synchronises the stream.  out may be NULL.
  */
 typedef struct {
-    int p2p_variant;        /* P2P: 0 one target per thread, 1 two, 2 each       */
+    int p2p_variant;        /* P2P: 0 FP64 arithmetic, 1 64-bit fixed-point      */
+                            /* arithmetic with FP64's accuracy, 2 FP64 and each  */
                             /* mirrored leaf pair once for both directions (the  */
-                            /* FP32 forms: 0 and 1 are their two-target kernel)  */
+                            /* FP32 forms: 0 and 1 are their one-way kernel)     */
     int m2l_tensor;         /* FMM_3XTF32: 1 tensor-core M2L, 0 SIMT FP32 M2L   */
     int tc_chunk_rows;      /* key rows summed per chunk of the tensor-core M2L  */
     int candidates;         /* variants timed                                    */

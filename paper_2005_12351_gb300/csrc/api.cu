@@ -216,9 +216,9 @@ fmm_status fmm_create_tree(fmm_tree **out, int device, void *cuda_stream, int ma
     t->stream = (cudaStream_t)cuda_stream;
     t->max_leaf = max_leaf;
     t->prec = prec;
-    // the symmetric near field pays off where pairs are FP64; the FP32 forms'
-    // pairs are cheap next to its warp sums, so they start one-way
-    t->p2p_variant = prec == FMM_FP64 ? 2 : 1;
+    // one way in every form: the FP64 form's fixed-point pairs and the FP32 forms'
+    // pairs are cheap next to the symmetric kernels' warp sums and reverse rows
+    t->p2p_variant = 1;
     t->budget = mem_budget_bytes;
     if (const char *env = getenv("FMM_FAIL_ALLOC")) t->fail_alloc_at = std::max(0ll, atoll(env));
     std::memset(t->phase_ms, 0, sizeof(t->phase_ms));

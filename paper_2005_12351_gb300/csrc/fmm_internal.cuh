@@ -297,10 +297,10 @@ struct fmm_tree {
     DevBuf b_sym_mir, b_sym_cnt, b_sym_base, b_sym_scan, b_sym_tot, b_sym_rev, b_sym_fwd;
 
     // tuning (fmm_autotune, fmm_set_tuning; defaults otherwise): FP64 P2P kernel
-    // (0 one target per thread, 1 two, 2 each leaf pair once for both
-    // directions), FMM_3XTF32 M2L on the SIMT FP32 kernel instead of the
+    // (0 FP64 arithmetic, 1 fixed-point arithmetic, 2 FP64 and each leaf pair once
+    // for both directions), FMM_3XTF32 M2L on the SIMT FP32 kernel instead of the
     // tensor cores, rows per chunk of the tensor-core M2L (tc_G above)
-    int p2p_variant = 2;
+    int p2p_variant = 1;
     int p2p_tt = 2;                        // FP32 forms' one-way P2P: targets per thread (1 or 2)
     bool m2l_simt = false;
     bool m2l_tiled = true;                 // SIMT FP32 M2L over the plan's tiles (else per target cell)
@@ -419,6 +419,8 @@ fmm_status evaluate_body(fmm_tree *t, int p, int want_phi, int want_field, doubl
 void drop_graph(fmm_tree *t);
 // p2p.cu
 fmm_status run_p2p(fmm_tree *t, int want_phi, int want_field, double *phi_out, double *E_out);
+// p2p_fx.cu: the one-way near field in fixed-point arithmetic (p2p_variant 1)
+void launch_p2p_fx(fmm_tree *t, int want_phi, int want_field, double *phi, double *E);
 // the symmetric P2P's plan (mirror entries, reverse-row offsets; one host sync
 // when built) and its buffers for NC output components (rows of NC doubles, or
 // of NC floats in the FP32 forms); FMM_EBUDGET over the handle's budget

@@ -220,114 +220,6 @@ k_p2p(const int32_t *leaves, const int32_t *begin, const int32_t *end, const int
     }
 }
 
-// Variant with two targets per thread: each staged source is read once from
-// shared memory for two pair evaluations.  A chunk of up to 2*128 targets is
-// split into halves of h = ceil(cnt/2); thread (ti, copy) owns targets ti and
-// ti + h (the second one only if it exists).
-// SHI > S: every particle carries the orders S..SHI (mixed systems), the pair
-// terms summed shell by shell; fewer sources staged per round when the rows
-// are wide.
-template <int S, bool PHI, bool FIELD, int SHI = S>
-__global__ void __launch_bounds__(kP2PThreads)
-k_p2p_x2(const int32_t *leaves, const int32_t *begin, const int32_t *end, const int32_t *off,
-         const int32_t *src, const double *px, const double *py, const double *pz,
-         const double *Sm, const double *phi_far, const double *E_far, const int32_t *perm,
-         double *phi_out, double *E_out)
-{
-    constexpr int nS = Orders<S, SHI>::n;
-    constexpr bool kS3 = S == 1 && SHI == 1;           // 3 S staged for the dipole field
-    constexpr int kP2PChunk = nS > 6 ? 256 : fmm::kP2PChunk;
-    __shared__ double sx[kP2PChunk], sy[kP2PChunk], sz[kP2PChunk];
-    __shared__ double sS[kP2PChunk * nS], sS3[kS3 ? kP2PChunk * 3 : 1];
-    __shared__ double red[8][kP2PThreads];
-    __shared__ int gbeg[kP2PGroups], gpre[kP2PGroups + 1];
-    __shared__ int s_next_q, s_next_j, s_ngroups;
-    const int c = leaves[blockIdx.x];
-    const int b = begin[c], e = end[c], nt = e - b;
-    const int q0 = off[c], q1 = off[c + 1];
-    const int tid = threadIdx.x;
-    for (int t0 = 0; t0 < nt; t0 += 2 * kP2PThreads) {
-        const int cnt = min(2 * kP2PThreads, nt - t0);
-        const int h = (cnt + 1) / 2;
-        const int k = max(1, kP2PThreads / h);
-        const int ti = tid % h, sp = tid / h;
-        const bool act = sp < k;
-        const bool two = act && (ti + h < cnt);
-        const int i = b + t0 + ti, i2 = i + h;
-        const double xi = act ? px[i] : 0.0, yi = act ? py[i] : 0.0, zi = act ? pz[i] : 0.0;
-        const double xj = two ? px[i2] : 0.0, yj = two ? py[i2] : 0.0, zj = two ? pz[i2] : 0.0;
-        double f = 0.0, e0 = 0.0, e1 = 0.0, e2 = 0.0;
-        double g = 0.0, g0 = 0.0, g1 = 0.0, g2 = 0.0;
-        int q = q0, j_in = 0;
-        while (q < q1) {
-            __syncthreads();
-            if (tid < 32)
-                stage_groups(tid, q, q1, j_in, kP2PChunk, src, begin, end, gbeg, gpre, &s_ngroups,
-                             &s_next_q, &s_next_j);
-            __syncthreads();
-            const int ng = s_ngroups, used = gpre[ng];
-            for (int d = tid; d < used; d += kP2PThreads) {
-                int lo = 0, hi = ng - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (gpre[mid] <= d) lo = mid; else hi = mid - 1;
-                }
-                const int j = gbeg[lo] + (d - gpre[lo]);
-                sx[d] = px[j]; sy[d] = py[j]; sz[d] = pz[j];
-#pragma unroll
-                for (int a = 0; a < nS; ++a) {
-                    const double v = Sm[(int64_t)j * nS + a];
-                    sS[d * nS + a] = v;
-                    if (kS3) sS3[d * 3 + a] = 3.0 * v;
-                }
-            }
-            __syncthreads();
-            if (act) {
-                for (int j = sp; j < used; j += k) {
-                    const double ax = sx[j], ay = sy[j], az = sz[j];
-                    const double *Sj = sS + j * nS, *S3 = kS3 ? sS3 + j * 3 : sS;
-                    if constexpr (SHI == S) {
-                        pair_p2p<S, PHI, FIELD>(xi - ax, yi - ay, zi - az, Sj, S3, f, e0, e1, e2);
-                        if (two) pair_p2p<S, PHI, FIELD>(xj - ax, yj - ay, zj - az, Sj, S3, g, g0, g1, g2);
-                    } else {
-                        pair_orders<S, SHI, PHI, FIELD>(xi - ax, yi - ay, zi - az, Sj, f, e0, e1, e2);
-                        if (two) pair_orders<S, SHI, PHI, FIELD>(xj - ax, yj - ay, zj - az, Sj, g, g0, g1, g2);
-                    }
-                }
-            }
-            q = s_next_q;
-            j_in = s_next_j;
-        }
-        __syncthreads();
-        red[0][tid] = f; red[1][tid] = e0; red[2][tid] = e1; red[3][tid] = e2;
-        red[4][tid] = g; red[5][tid] = g0; red[6][tid] = g1; red[7][tid] = g2;
-        __syncthreads();
-        if (tid < h) {
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                if (half == 1 && tid + h >= cnt) break;
-                const int r = 4 * half;
-                double F = red[r][tid], A = red[r + 1][tid], B = red[r + 2][tid], C = red[r + 3][tid];
-                for (int u = 1; u < k; ++u) {
-                    F += red[r][u * h + tid];
-                    A += red[r + 1][u * h + tid];
-                    B += red[r + 2][u * h + tid];
-                    C += red[r + 3][u * h + tid];
-                }
-                const int ii = b + t0 + tid + half * h;
-                const int64_t o = perm[ii];
-                if (PHI) phi_out[o] = phi_far[ii] + F;
-                if (FIELD) {
-                    E_out[3 * o] = E_far[3 * (int64_t)ii] + A;
-                    E_out[3 * o + 1] = E_far[3 * (int64_t)ii + 1] + B;
-                    E_out[3 * o + 2] = E_far[3 * (int64_t)ii + 2] + C;
-                }
-            }
-        }
-        __syncthreads();
-    }
-}
-
 // ------------------------------------------------------------ symmetric P2P
 // Newton's third law in the near field.  The lists hold a leaf pair in both
 // rows, (A, B) and (B, A), whenever the traversal reaches both orders (on the
@@ -787,7 +679,7 @@ void launch_sym_s(fmm_tree *t, int want_phi, int want_field, double *phi, double
     else run(k_p2p_sym<S, false, true, SHI>, k_p2p_sym_gather<false, true>);
 }
 
-template <int S, int SHI = S>
+template <int S>
 void launch_p2p_s(fmm_tree *t, int want_phi, int want_field, double *phi, double *E)
 {
     auto args = [&](auto kern) {
@@ -799,12 +691,6 @@ void launch_p2p_s(fmm_tree *t, int want_phi, int want_field, double *phi, double
             (const double *)t->b_phi.ptr, (const double *)t->b_E.ptr,
             (const int32_t *)t->b_perm.ptr, phi, E);
     };
-    if (t->p2p_variant >= 1 || SHI != S) {         // mixed orders: this kernel only
-        if (want_phi && want_field) args(k_p2p_x2<S, true, true, SHI>);
-        else if (want_phi) args(k_p2p_x2<S, true, false, SHI>);
-        else args(k_p2p_x2<S, false, true, SHI>);
-        return;
-    }
     if (want_phi && want_field) args(k_p2p<S, true, true>);
     else if (want_phi) args(k_p2p<S, true, false>);
     else args(k_p2p<S, false, true>);
@@ -877,15 +763,10 @@ fmm_status run_p2p(fmm_tree *t, int want_phi, int want_field, double *phi_out, d
             return cuda_check(t, cudaGetLastError(), "symmetric p2p kernels");
         }
         if (ps != FMM_OK && ps != FMM_EBUDGET) return ps;
-        t->err.clear();               // over the budget or the row index: two targets per thread
+        t->err.clear();               // over the budget or the row index: the one-way kernel
     }
-    if (t->s_hi != t->s) {                            // mixed orders: two targets per thread
-        switch (so) {
-        case 1: launch_p2p_s<0, 1>(t, want_phi, want_field, phi_out, E_out); break;
-        case 2: launch_p2p_s<0, 2>(t, want_phi, want_field, phi_out, E_out); break;
-        default: launch_p2p_s<1, 2>(t, want_phi, want_field, phi_out, E_out); break;
-        }
-        ++t->launches;
+    if (t->p2p_variant >= 1 || t->s_hi != t->s) {
+        launch_p2p_fx(t, want_phi, want_field, phi_out, E_out);
         return cuda_check(t, cudaGetLastError(), "p2p kernel");
     }
     switch (t->s) {
