@@ -32,6 +32,7 @@ constexpr int kErrHashFull = 4;
 constexpr int kErrTcTimeout = 8;       // a tensor-core M2L wait gave up (word 1 of b_err)
 constexpr int kErrSortWait = 16;       // a look-back wait of the radix sort gave up
 constexpr int kErrLongRow = 32;        // a row of an interaction list too long for the row sort
+constexpr int kErrTieRun = 64;         // a run of equal leading key bits too long for the tie sort
 
 inline int ntot(int p) { return p < 0 ? 0 : (p + 1) * (p + 2) * (p + 3) / 6; }
 inline int nshell(int k) { return (k + 1) * (k + 2) / 2; }
@@ -228,6 +229,7 @@ struct fmm_tree {
     bool have_lists = false;
     int64_t n_m2l = 0, n_p2p = 0, n_p2p_inter = 0, n_doff = 0;
     size_t m2l_cap_hint = 0;
+    bool sort_full = false;                // an earlier set had a long run of equal leading key bits
     int max_gap = 0;                       // largest level gap of an M2L pair
     // D tables / operator tables
     int d_p = -1;                          // p the D table was built for
@@ -353,6 +355,11 @@ size_t radix_hist_bytes(int64_t n);
 void radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys2, uint32_t *vals2, int64_t n,
                       int end_bit, uint32_t *hist, int *err, cudaStream_t st, int64_t *launches,
                       bool counted = false);
+// The passes p0 .. 7 of that sort alone, on counted keys (bits 8 p0 and up of
+// 64; k_keys' counts): the result ends in (keys, vals) after an even number of
+// passes, in (keys2, vals2) after an odd one.
+void radix_sort_top(uint64_t *keys, uint32_t *vals, uint64_t *keys2, uint32_t *vals2, int64_t n, int p0,
+                    uint32_t *hist, int *err, cudaStream_t st, int64_t *launches);
 
 // Per-device set-up of the sort (its kernels loaded, the scatter's shared-
 // memory limit raised); radix_sort_pairs calls it, and callers that must not
@@ -364,10 +371,17 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom);
 fmm_status build_lists(fmm_tree *t, double theta);
 // loads the Morton-order kernels on the current device (no launch)
 void morton_order_prepare();
+// Morton order of one point set, on scratch of the caller's: *err (device) is
+// zeroed here; synchronises st once (twice where a long run of equal leading
+// key bits sends the keys through every pass).  FMM_EINVAL for a non-finite
+// position, FMM_ETIMEOUT if a bounded wait of the sort gave up (still exact).
 fmm_status morton_order_raw(cudaStream_t st, const double *pos, int64_t n, uint64_t *keys,
                             uint32_t *idx, uint64_t *keys2, uint32_t *idx2, uint32_t *hist,
-                            unsigned long long *box_scratch, double *box_out, int *err,
-                            int64_t *launches);
+                            unsigned long long *box_scratch, double *box_out, int *err);
+// noalloc.cu: the Morton order on the library's fixed scratch array when n fits
+// it and no other thread is using it; *used says whether that was so
+fmm_status morton_order_scratch(cudaStream_t st, const double *pos, int64_t n, uint64_t *keys, uint32_t *idx,
+                                bool wait, bool *used);
 
 // operators.cu
 fmm_status upload_tables(fmm_tree *t, int s, int p, int n_lo, DevTables *dt, const int32_t **lut);

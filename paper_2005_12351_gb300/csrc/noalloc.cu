@@ -32,6 +32,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 void *g_addr[kMaxDevices] = {nullptr};
+std::mutex g_use[kMaxDevices];             // the scratch array of a device is in use
 
 // Device address of the scratch array on the current device, looked up once
 // per device with that device current.
@@ -58,43 +59,49 @@ fmm_status scratch_address(unsigned char **out)
 
 }  // namespace
 
+namespace fmm {
+
+// The call holds the array's mutex until its work on the GPU has ended, so
+// that callers of different threads and streams never share it at once.
+fmm_status morton_order_scratch(cudaStream_t st, const double *pos, int64_t n, uint64_t *keys, uint32_t *idx,
+                                bool wait, bool *used)
+{
+    *used = false;
+    int dev = -1;
+    if (n > kMaxPoints || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
+        cudaGetLastError();
+        return FMM_ECUDA;
+    }
+    std::unique_lock<std::mutex> lk(g_use[dev], std::defer_lock);
+    if (wait) lk.lock();
+    else if (!lk.try_lock()) return FMM_OK;
+    unsigned char *base = nullptr;
+    const fmm_status s = scratch_address(&base);
+    if (s != FMM_OK) return s;
+    *used = true;
+    return morton_order_raw(st, pos, n, keys, idx, (uint64_t *)(base + kOffKeys2), (uint32_t *)(base + kOffIdx2),
+                            (uint32_t *)(base + kOffHist), (unsigned long long *)(base + kOffBox),
+                            (double *)(base + kOffBox) + 8, (int *)(base + kOffErr));
+}
+
+}  // namespace fmm
+
 extern "C" fmm_status fmm_morton_order_noalloc(void *cuda_stream, const double *positions,
                                                int64_t n, uint64_t *keys_out, int32_t *perm_out)
 {
     if (n < 0) return FMM_EINVAL;
     if (n > kMaxPoints) return FMM_EBUDGET;       // larger than the fixed scratch array
-    unsigned char *base = nullptr;
     if (n == 0) {
         // the per-device set-up alone: load the kernels and this file's module
         // (which holds the scratch array), look up its address, raise the
         // sort's shared-memory limit -- everything a later call would
         // otherwise do on its first use
+        unsigned char *base = nullptr;
         fmm::morton_order_prepare();
         return scratch_address(&base);
     }
     if (!positions || !keys_out || !perm_out) return FMM_EINVAL;
-    fmm_status st = scratch_address(&base);
-    if (st != FMM_OK) return st;
-    cudaStream_t s = (cudaStream_t)cuda_stream;
-    int *err = (int *)(base + kOffErr);
-    // only the error word must start at zero; the sort clears its own
-    // counters, and every other region is fully written before it is read
-    if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) {
-        cudaGetLastError();
-        return FMM_ECUDA;
-    }
-    int64_t launches = 0;
-    fmm::morton_order_raw(s, positions, n, keys_out, (uint32_t *)perm_out,
-                          (uint64_t *)(base + kOffKeys2), (uint32_t *)(base + kOffIdx2),
-                          (uint32_t *)(base + kOffHist), (unsigned long long *)(base + kOffBox), (double *)(base + kOffBox) + 8,
-                          err, &launches);
-    int herr = 0;
-    cudaError_t e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return FMM_ECUDA;
-    }
-    if (herr & fmm::kErrNonFinite) return FMM_EINVAL;
-    return (herr & fmm::kErrSortWait) ? FMM_ETIMEOUT : FMM_OK;
+    bool used = false;
+    return fmm::morton_order_scratch((cudaStream_t)cuda_stream, positions, n, keys_out, (uint32_t *)perm_out, true,
+                                     &used);
 }

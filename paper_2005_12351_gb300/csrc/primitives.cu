@@ -314,6 +314,32 @@ void radix_sort_prepare()
     }
 }
 
+// passes p0 .. passes - 1; q counts the passes run, status area 0 is zero
+static void scatter_passes(uint64_t *&ka, uint32_t *&va, uint64_t *&kb, uint32_t *&vb, int64_t n, int p0, int passes,
+                           uint32_t *hist, int *err, cudaStream_t st, int64_t *launches)
+{
+    const int64_t ntiles = (n + kSortTile - 1) / kSortTile;
+    // hist: digit counts [passes][256], tile counters [16], two status areas [ntiles][256]
+    uint32_t *ghist = hist, *ctr = hist + kRadixMaxPasses * 256;
+    uint64_t *status[2] = {(uint64_t *)(hist + kRadixHead), (uint64_t *)(hist + kRadixHead) + ntiles * 256};
+    int max_polls = kOsWait;
+    if (const char *env = getenv("FMM_SORT_POLLS")) max_polls = std::max(0, atoi(env));
+    for (int p = p0, q = 0; p < passes; ++p, ++q) {
+        k_os_scatter<<<(unsigned)ntiles, kSortThreads, kOsSmem, st>>>(
+            ka, va, kb, vb, n, p, passes, ghist, ctr, status[q & 1], status[(q + 1) & 1], err, max_polls);
+        ++*launches;
+        std::swap(ka, kb);
+        std::swap(va, vb);
+    }
+}
+
+void radix_sort_top(uint64_t *keys, uint32_t *vals, uint64_t *keys2, uint32_t *vals2, int64_t n, int p0,
+                    uint32_t *hist, int *err, cudaStream_t st, int64_t *launches)
+{
+    radix_sort_prepare();
+    scatter_passes(keys, vals, keys2, vals2, n, p0, kRadixMaxPasses, hist, err, st, launches);
+}
+
 void radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys2, uint32_t *vals2, int64_t n,
                       int end_bit, uint32_t *hist, int *err, cudaStream_t st, int64_t *launches,
                       bool counted)
@@ -321,28 +347,17 @@ void radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys2, uint32_t 
     if (n <= 1) return;
     const int passes = std::min((end_bit + 7) / 8, kRadixMaxPasses);
     const int64_t ntiles = (n + kSortTile - 1) / kSortTile;
-    // hist: digit counts [passes][256], tile counters [16], two status areas [ntiles][256]
-    uint32_t *ghist = hist, *ctr = hist + kRadixMaxPasses * 256;
-    uint64_t *status[2] = {(uint64_t *)(hist + kRadixHead), (uint64_t *)(hist + kRadixHead) + ntiles * 256};
     radix_sort_prepare();
-    int max_polls = kOsWait;
-    if (const char *env = getenv("FMM_SORT_POLLS")) max_polls = std::max(0, atoi(env));
     if (!counted) {
         cudaMemsetAsync(hist, 0, 4 * (size_t)kRadixHead, st);
         const unsigned hgrid = (unsigned)std::min<int64_t>((n + kSortThreads - 1) / kSortThreads,
                                                            4 * (int64_t)sm_count());
-        k_os_hist<<<hgrid, kSortThreads, 0, st>>>(keys, n, passes, ghist, status[0], ntiles);
+        k_os_hist<<<hgrid, kSortThreads, 0, st>>>(keys, n, passes, hist, (uint64_t *)(hist + kRadixHead), ntiles);
         ++*launches;
     }
     uint64_t *ka = keys, *kb = keys2;
     uint32_t *va = vals, *vb = vals2;
-    for (int p = 0; p < passes; ++p) {
-        k_os_scatter<<<(unsigned)ntiles, kSortThreads, kOsSmem, st>>>(
-            ka, va, kb, vb, n, p, passes, ghist, ctr, status[p & 1], status[(p + 1) & 1], err, max_polls);
-        ++*launches;
-        std::swap(ka, kb);
-        std::swap(va, vb);
-    }
+    scatter_passes(ka, va, kb, vb, n, 0, passes, hist, err, st, launches);
     if (passes & 1) {
         cudaMemcpyAsync(keys, ka, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, st);
         cudaMemcpyAsync(vals, va, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st);

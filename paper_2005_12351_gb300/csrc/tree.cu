@@ -32,11 +32,13 @@ __device__ __forceinline__ double from_ordered_bits(unsigned long long b)
     return __longlong_as_double((long long)b);
 }
 
-__global__ void k_box_init(unsigned long long *box)
+// the running box and the head words of the sort's scratch, one block
+__global__ void k_sort_init(unsigned long long *box, uint32_t *hist)
 {
-    int i = threadIdx.x;
+    const int i = threadIdx.x;
     if (i < 3) box[i] = ~0ull;            // running minimum
     else if (i < 6) box[i] = 0ull;        // running maximum
+    for (int w = i; w < kRadixHead; w += blockDim.x) hist[w] = 0u;
 }
 
 __global__ void k_bbox(const double *pos, int64_t n, unsigned long long *box, int *err)
@@ -81,8 +83,8 @@ __global__ void k_bbox(const double *pos, int64_t n, unsigned long long *box, in
     if (bad) atomicOr(err, kErrNonFinite);
 }
 
-// box_out = (lo_x, lo_y, lo_z, side)
-__global__ void k_box_final(const unsigned long long *box, double *box_out)
+// (lo_x, lo_y, lo_z, side) of the ordered bits of the minima and maxima
+__device__ __forceinline__ void box_final(const unsigned long long *box, double *out)
 {
     double lo[3], ext = 0.0;
     for (int d = 0; d < 3; ++d) {
@@ -96,7 +98,7 @@ __global__ void k_box_final(const unsigned long long *box, double *box_out)
         double m = frexp(ext, &e2);        // ext = m 2^e2, m in [0.5, 1)
         side = ldexp(1.0, m == 0.5 ? e2 - 1 : e2);
     }
-    box_out[0] = lo[0]; box_out[1] = lo[1]; box_out[2] = lo[2]; box_out[3] = side;
+    out[0] = lo[0]; out[1] = lo[1]; out[2] = lo[2]; out[3] = side;
 }
 
 __device__ __forceinline__ uint64_t spread3(uint64_t x)
@@ -126,20 +128,23 @@ __device__ __forceinline__ uint64_t grid_coord(double d, int k)
     return sh <= -64 ? 0 : ((m >> -sh) > top ? top : (m >> -sh));
 }
 
-// The keys, and for the radix sort that follows the counts of every 8-bit
-// digit of them (per block in shared memory, then one atomic per digit and
-// block) and the zeroed status words of its first pass.
+// The keys, and for the radix sort that follows the counts of the 8-bit digits
+// p0 .. 7 of them (per block in shared memory, then one atomic per digit and
+// block) and the zeroed status words of its first pass.  Every block forms the
+// box from its six words (the first one stores it), which saves a launch.
 __global__ void __launch_bounds__(256)
-k_keys(const double *pos, int64_t n, const double *box, uint64_t *keys, uint32_t *idx,
-       uint32_t *ghist, uint64_t *status0, int64_t nstatus)
+k_keys(const double *pos, int64_t n, const unsigned long long *raw_box, double *box_out, uint64_t *keys,
+       uint32_t *idx, int p0, uint32_t *ghist, uint64_t *status0, int64_t nstatus)
 {
     __shared__ uint32_t h[kRadixMaxPasses][256];
-#pragma unroll
-    for (int p = 0; p < kRadixMaxPasses; ++p) h[p][threadIdx.x] = 0;
+    __shared__ double box[4];
+    for (int p = p0; p < kRadixMaxPasses; ++p) h[p][threadIdx.x] = 0;
     for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < nstatus;
          w += (int64_t)gridDim.x * blockDim.x)
         status0[w] = 0ull;
+    if (threadIdx.x == 0) box_final(raw_box, box);
     __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x < 4) box_out[threadIdx.x] = box[threadIdx.x];
     const int k = kLevels - ilogb(box[3]);          // scale = 2^kLevels / side = 2^k
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -149,16 +154,68 @@ k_keys(const double *pos, int64_t n, const double *box, uint64_t *keys, uint32_t
         const uint64_t key = spread3(q[0]) << 2 | spread3(q[1]) << 1 | spread3(q[2]);
         keys[i] = key;
         idx[i] = (uint32_t)i;
-#pragma unroll
-        for (int p = 0; p < kRadixMaxPasses; ++p) atomicAdd(&h[p][(unsigned)(key >> (8 * p)) & 255u], 1u);
+        for (int p = p0; p < kRadixMaxPasses; ++p) atomicAdd(&h[p][(unsigned)(key >> (8 * p)) & 255u], 1u);
     }
     __syncthreads();
-#pragma unroll
-    for (int p = 0; p < kRadixMaxPasses; ++p)
+    for (int p = p0; p < kRadixMaxPasses; ++p)
         if (h[p][threadIdx.x]) atomicAdd(&ghist[p * 256 + threadIdx.x], h[p][threadIdx.x]);
 }
 
-// ---- systems (a forest of independent octrees, one root per system)
+// The first radix pass of a set of n Morton keys.  Sorting by the leading bits
+// alone leaves runs of equal leading bits, which k_tie_sort puts in order; at
+// these depths (23 bits up to 2^14 points, 31 up to 2^22, 39 up to 2^30) a
+// uniform set has hardly any and the core of a Plummer sphere of scale radius
+// a twentieth of the box some four points to a run.  Each pass saved is a
+// launch and 24 bytes a key: 8 -> 4 passes and the tie sort, 0.230 -> 0.130 ms
+// at 1M points, 0.072 -> 0.037 ms at 2,000.
+inline int first_pass(int64_t n) { return n <= (1 << 14) ? 5 : (n <= (1 << 22) ? 4 : (n <= (1 << 30) ? 3 : 2)); }
+
+// Keys in order of their bits from `shift` up -> keys in order, stable: within
+// a run of equal leading bits an element goes behind the smaller keys and the
+// equal ones before it.  A run of more than kTieRun keys stays as it is (each
+// of its elements sees at least kTieRun neighbours, so they agree) and sets
+// kErrTieRun: the caller sorts by all bits instead.  GATHER: the particle
+// arrays in the new order too.
+constexpr int kTieRun = 256;
+
+template <bool GATHER>
+__global__ void __launch_bounds__(256)
+k_tie_sort(const uint64_t *keys, const uint32_t *idx, int64_t n, int shift, uint64_t *okeys, uint32_t *oidx, int *err,
+           const double *pos, const double *mom, int nS, double *px, double *py, double *pz, double *S,
+           int32_t *perm_out)
+{
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const uint64_t key = keys[i], top = key >> shift;
+    const uint32_t id = idx[i];
+    int left = 0, right = 0, move = 0;
+    for (; left < kTieRun && i - left - 1 >= 0; ++left) {
+        const uint64_t o = keys[i - left - 1];
+        if (o >> shift != top) break;
+        move -= o > key;
+    }
+    for (; right < kTieRun && i + right + 1 < n; ++right) {
+        const uint64_t o = keys[i + right + 1];
+        if (o >> shift != top) break;
+        move += o < key;
+    }
+    if (left + right + 1 > kTieRun) {
+        move = 0;
+        if ((*(volatile int *)err & kErrTieRun) == 0) atomicOr(err, kErrTieRun);
+    }
+    const int64_t k = i + move;
+    okeys[k] = key;
+    oidx[k] = id;
+    if (GATHER) {
+        const int64_t o = id;
+        px[k] = pos[3 * o];
+        py[k] = pos[3 * o + 1];
+        pz[k] = pos[3 * o + 2];
+        for (int a = 0; a < nS; ++a) S[k * nS + a] = mom[o * nS + a];
+        perm_out[k] = (int32_t)o;
+    }
+}
+
 __global__ void k_sys_of(const int64_t *off, int nsys, int64_t n, int32_t *sys_of)
 {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -329,7 +386,7 @@ __device__ __forceinline__ int digit_at(uint64_t key, int level)
 // batch.  A level that would pass the cell capacity sets ctl[kCtlOverflow]
 // instead; every later kernel then does nothing and the host rebuilds with
 // more room.
-constexpr int kCtlOverflow = 0, kCtlLevel = 1, kCtlWords = 32;
+constexpr int kCtlOverflow = 0, kCtlLevel = 1, kCtlTie = 31, kCtlWords = 32;
 constexpr int kLevelBatch = 8;                  // levels launched per host round trip
 constexpr int kLevelScanPer = 16;               // child counts per thread of the one-block scan
 
@@ -523,10 +580,13 @@ k_level_write(CellArrays c, const unsigned *ctl, int level, const int32_t *cb, c
     }
 }
 
-__global__ void k_level_init(unsigned *ctl, int nsys)
+// Where the tie sort left a run unsorted there are no cells to build (the host
+// sorts again).
+__global__ void k_level_init(unsigned *ctl, int nsys, const int *err)
 {
     const int i = threadIdx.x;
-    if (i < kCtlWords) ctl[i] = i == kCtlLevel + 1 ? (unsigned)nsys : 0u;
+    const bool tie = (*err & kErrTieRun) != 0;
+    if (i < kCtlWords) ctl[i] = i == kCtlLevel + 1 ? (tie ? 0u : (unsigned)nsys) : (i == kCtlTie ? (unsigned)tie : 0u);
 }
 
 // Besides the geometry, each cell gets the packed record the traversal reads
@@ -1065,27 +1125,26 @@ void record(fmm_tree *t, int i)
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// keys of one system, with the digit counts of their radix sort (hist: the
-// sort's scratch, its head zeroed here)
-static void morton_keys(cudaStream_t st, const double *pos, int64_t n, uint64_t *keys,
-                        uint32_t *idx, unsigned long long *box_scratch, double *box_out, int *err,
-                        uint32_t *hist, int64_t *launches)
+// keys of one system, with the counts of their digits p0 .. 7 (hist: the sort's
+// scratch, its head zeroed here)
+static void morton_keys(cudaStream_t st, const double *pos, int64_t n, int p0, uint64_t *keys, uint32_t *idx,
+                        unsigned long long *box_scratch, double *box_out, int *err, uint32_t *hist,
+                        int64_t *launches)
 {
-    k_box_init<<<1, 32, 0, st>>>(box_scratch);
-    k_bbox<<<(unsigned)std::min<int64_t>(grid(n, 256), 4 * (int64_t)sm_count()), 256, 0, st>>>(pos, n, box_scratch, err);
-    k_box_final<<<1, 1, 0, st>>>(box_scratch, box_out);
-    cudaMemsetAsync(hist, 0, 4 * (size_t)kRadixHead, st);
+    const unsigned g = (unsigned)std::min<int64_t>(grid(n, 256), 4 * (int64_t)sm_count());
+    k_sort_init<<<1, 256, 0, st>>>(box_scratch, hist);
+    k_bbox<<<g, 256, 0, st>>>(pos, n, box_scratch, err);
     const int64_t ntiles = (n + kRadixTile - 1) / kRadixTile;
-    k_keys<<<(unsigned)std::min<int64_t>(grid(n, 256), 4 * (int64_t)sm_count()), 256, 0, st>>>(
-        pos, n, box_out, keys, idx, hist, (uint64_t *)(hist + kRadixHead), ntiles * 256);
-    *launches += 4;
+    k_keys<<<g, 256, 0, st>>>(pos, n, box_scratch, box_out, keys, idx, p0, hist, (uint64_t *)(hist + kRadixHead),
+                              ntiles * 256);
+    *launches += 3;
 }
 
 void morton_order_prepare()
 {
     cudaFuncAttributes fa;
-    const void *kerns[] = {(const void *)k_box_init, (const void *)k_bbox, (const void *)k_box_final,
-                           (const void *)k_keys};
+    const void *kerns[] = {(const void *)k_sort_init, (const void *)k_bbox, (const void *)k_keys,
+                           (const void *)k_tie_sort<false>};
     for (const void *k : kerns)
         if (cudaFuncGetAttributes(&fa, k) != cudaSuccess) cudaGetLastError();
     radix_sort_prepare();
@@ -1093,12 +1152,37 @@ void morton_order_prepare()
 
 fmm_status morton_order_raw(cudaStream_t st, const double *pos, int64_t n, uint64_t *keys,
                             uint32_t *idx, uint64_t *keys2, uint32_t *idx2, uint32_t *hist,
-                            unsigned long long *box_scratch, double *box_out, int *err,
-                            int64_t *launches)
+                            unsigned long long *box_scratch, double *box_out, int *err)
 {
-    morton_keys(st, pos, n, keys, idx, box_scratch, box_out, err, hist, launches);
-    radix_sort_pairs(keys, idx, keys2, idx2, n, 3 * kLevels, hist, err, st, launches, true);
-    return FMM_OK;
+    int64_t launches = 0;
+    int herr = 0;
+    const int p0 = first_pass(n);
+    // the passes end in (keys2, idx2), the tie sort in (keys, idx)
+    const bool even = (kRadixMaxPasses - p0) % 2 == 0;
+    uint64_t *ka = even ? keys2 : keys, *kb = even ? keys : keys2;
+    uint32_t *va = even ? idx2 : idx, *vb = even ? idx : idx2;
+    if (cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess) {
+        cudaGetLastError();
+        return FMM_ECUDA;
+    }
+    morton_keys(st, pos, n, p0, ka, va, box_scratch, box_out, err, hist, &launches);
+    radix_sort_top(ka, va, kb, vb, n, p0, hist, err, st, &launches);
+    k_tie_sort<false><<<grid(n, 256), 256, 0, st>>>(keys2, idx2, n, 8 * p0, keys, idx, err, nullptr, nullptr, 0,
+                                                     nullptr, nullptr, nullptr, nullptr, nullptr);
+    cudaError_t e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess && (herr & kErrTieRun)) {
+        // every pass, over the keys as they stand (each key still carries its index)
+        radix_sort_pairs(keys, idx, keys2, idx2, n, 3 * kLevels, hist, err, st, &launches);
+        e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return FMM_ECUDA;
+    }
+    if (herr & kErrNonFinite) return FMM_EINVAL;
+    return (herr & kErrSortWait) ? FMM_ETIMEOUT : FMM_OK;
 }
 
 fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
@@ -1135,9 +1219,33 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
     cudaMemsetAsync(t->b_err.ptr, 0, sizeof(int), st);
     FMM_TRY(cuda_check(t, cudaMemcpyAsync(off, t->sys_off.data(), 8 * (size_t)(nsys + 1),
                                           cudaMemcpyHostToDevice, st), "system offsets"));
+    // one system: by the leading key bits and the tie sort, by all bits where an
+    // earlier set of this handle (or, below, this one) had a long run of ties
+    auto sort_one = [&](bool full) {
+        uint64_t *keys2 = (uint64_t *)t->b_keys2.ptr;
+        uint32_t *idx2 = (uint32_t *)t->b_idx2.ptr, *hist = (uint32_t *)t->b_hist.ptr;
+        int *err = (int *)t->b_err.ptr;
+        double *px = (double *)t->b_px.ptr, *py = (double *)t->b_py.ptr, *pz = (double *)t->b_pz.ptr,
+               *S = (double *)t->b_S.ptr;
+        int32_t *perm = (int32_t *)t->b_perm.ptr;
+        const int p0 = full ? 0 : first_pass(n);
+        const bool swap = !full && (kRadixMaxPasses - p0) % 2 == 0;      // the passes end in (keys2, idx2)
+        uint64_t *ka = swap ? keys2 : keys, *kb = swap ? keys : keys2;
+        uint32_t *va = swap ? idx2 : idx, *vb = swap ? idx : idx2;
+        morton_keys(st, pos, n, p0, ka, va, sbox_raw, sbox, err, hist, &t->launches);
+        record(t, 1);
+        radix_sort_top(ka, va, kb, vb, n, p0, hist, err, st, &t->launches);
+        if (full)
+            k_gather<<<grid(n, 256), 256, 0, st>>>(pos, mom, t->nS, idx, n, px, py, pz, S, perm);
+        else
+            k_tie_sort<true><<<grid(n, 256), 256, 0, st>>>(keys2, idx2, n, 8 * p0, keys, idx, err, pos, mom, t->nS,
+                                                            px, py, pz, S, perm);
+        ++t->launches;
+        record(t, 2);
+    };
+    bool full = t->sort_full;
     if (nsys == 1) {
-        morton_keys(st, pos, n, keys, idx, sbox_raw, sbox, (int *)t->b_err.ptr, (uint32_t *)t->b_hist.ptr,
-                    &t->launches);
+        sort_one(full);
     } else {
         // particle -> system (kept in b_idx2 until the sort needs it)
         FMM_TRY(ensure(t, t->b_lval2, 4 * n));
@@ -1148,12 +1256,9 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
         k_box_final_seg<<<grid(nsys, 128), 128, 0, st>>>(sbox_raw, nsys, sbox);
         k_keys_seg<<<grid(n, 256), 256, 0, st>>>(pos, n, sys_of, sbox, keys, idx);
         t->launches += 5;
-    }
-    record(t, 1);
-    radix_sort_pairs(keys, idx, (uint64_t *)t->b_keys2.ptr, (uint32_t *)t->b_idx2.ptr, n,
-                     3 * kLevels, (uint32_t *)t->b_hist.ptr, (int *)t->b_err.ptr, st, &t->launches,
-                     nsys == 1);                   // one system: k_keys counted the digits
-    if (nsys > 1) {
+        record(t, 1);
+        radix_sort_pairs(keys, idx, (uint64_t *)t->b_keys2.ptr, (uint32_t *)t->b_idx2.ptr, n,
+                         3 * kLevels, (uint32_t *)t->b_hist.ptr, (int *)t->b_err.ptr, st, &t->launches);
         // stable second pass by system: order = (system, key, original index)
         FMM_TRY(ensure(t, t->b_lkeys, 8 * n));
         FMM_TRY(ensure(t, t->b_lkeys2, 8 * n));
@@ -1165,13 +1270,12 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
         radix_sort_pairs(skeys, idx, (uint64_t *)t->b_keys2.ptr, (uint32_t *)t->b_idx2.ptr, n,
                          sbits, (uint32_t *)t->b_hist.ptr, (int *)t->b_err.ptr, st, &t->launches);
         k_regather_keys<<<grid(n, 256), 256, 0, st>>>(key_of, idx, n, keys);
-        t->launches += 2;
+        k_gather<<<grid(n, 256), 256, 0, st>>>(pos, mom, t->nS, idx, n, (double *)t->b_px.ptr,
+                                               (double *)t->b_py.ptr, (double *)t->b_pz.ptr,
+                                               (double *)t->b_S.ptr, (int32_t *)t->b_perm.ptr);
+        t->launches += 3;
+        record(t, 2);
     }
-    k_gather<<<grid(n, 256), 256, 0, st>>>(pos, mom, t->nS, idx, n, (double *)t->b_px.ptr,
-                                           (double *)t->b_py.ptr, (double *)t->b_pz.ptr,
-                                           (double *)t->b_S.ptr, (int32_t *)t->b_perm.ptr);
-    ++t->launches;
-    record(t, 2);
 
     // ---- cells, level by level on the device (level 0 holds one root per system);
     // the host reads the level counts once per batch of levels
@@ -1193,10 +1297,10 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
         uint32_t *cnt = (uint32_t *)t->b_flags.ptr, *off8 = (uint32_t *)t->b_scan.ptr;
         int32_t *cbeg = (int32_t *)t->b_front.ptr, *cend = cbeg + 8 * cap;
         k_roots<<<grid(nsys, 128), 128, 0, st>>>(c, off, nsys);
-        k_level_init<<<1, kCtlWords, 0, st>>>(ctl, nsys);
+        k_level_init<<<1, kCtlWords, 0, st>>>(ctl, nsys, (const int *)t->b_err.ptr);
         t->launches += 2;
         int level = 0;
-        bool overflow = false;
+        bool overflow = false, tie = false;
         for (;;) {
             const int end = std::min(level + kLevelBatch, kLevels + 1);
             for (; level < end; ++level) {
@@ -1212,8 +1316,18 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
                 overflow = true;
                 break;
             }
+            if (hc[kCtlTie]) {               // a long run of ties: by all bits, and from now on
+                tie = true;
+                break;
+            }
             // done once a level came out empty (or the deepest level was processed)
             if (hc[kCtlLevel + level + 1] == hc[kCtlLevel + level] || level > kLevels) break;
+        }
+        if (tie) {
+            full = true;
+            cudaMemsetAsync(t->b_err.ptr, 0, sizeof(int), st);
+            sort_one(full);
+            continue;
         }
         if (!overflow) {
             // levels 0 .. nlev - 1 hold cells
@@ -1249,6 +1363,7 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
                                           cudaMemcpyDeviceToHost, st), "box"));
     record(t, 3);
     FMM_TRY(read_err(t));
+    t->sort_full = nsys == 1 && full;
     t->nleaves = nleaves;
     t->lo[0] = t->sys_box[0]; t->lo[1] = t->sys_box[1]; t->lo[2] = t->sys_box[2];
     t->side = t->sys_box[3];
