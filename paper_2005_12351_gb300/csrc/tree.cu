@@ -14,6 +14,7 @@
 // (the target on a tie); a self pair opens into all ordered child pairs.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 
 #include "fmm_internal.cuh"
 
@@ -359,15 +360,6 @@ struct CellArrays {
     int32_t *level, *parent, *child, *nchild, *begin, *end, *cx, *cy, *cz, *sys;
 };
 
-__global__ void k_roots(CellArrays c, const int64_t *off, int nsys)
-{
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nsys) return;
-    c.level[s] = 0; c.parent[s] = -1; c.begin[s] = (int32_t)off[s]; c.end[s] = (int32_t)off[s + 1];
-    c.cx[s] = c.cy[s] = c.cz[s] = 0;
-    c.sys[s] = s;
-}
-
 __global__ void k_root_pairs(int2 *front, int nsys, unsigned *nf0)
 {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -380,22 +372,28 @@ __device__ __forceinline__ int digit_at(uint64_t key, int level)
     return (int)((key >> (3 * (kLevels - level))) & 7ull);
 }
 
-// ---- cells, level by level without host round trips: the range of a level's
-// cells lives in device words (ctl[kCtlLevel + l] = first cell of level l), so
-// the host launches the levels back to back and reads the counts once per
-// batch.  A level that would pass the cell capacity sets ctl[kCtlOverflow]
-// instead; every later kernel then does nothing and the host rebuilds with
-// more room.
-constexpr int kCtlOverflow = 0, kCtlLevel = 1, kCtlTie = 31, kCtlWords = 32;
-constexpr int kLevelBatch = 8;                  // levels launched per host round trip
-constexpr int kLevelScanPer = 16;               // child counts per thread of the one-block scan
+// ---- cells, all levels in one launch by one thread-block cluster.
+// A level's cells need the level above and a scan of its child counts: three
+// small launches a level, or one cluster barrier and a few block barriers.  A
+// cluster of eight blocks is co-scheduled, so its barriers need no host and no
+// bounded waits; eight SMs are enough for the work (a binary search per cell
+// and octant), which is a chain of memory latencies whatever the width.
+// Cells phase, before (26 launches, two host syncs) and now: 0.165 -> 0.054 ms at 2,000 points,
+// 0.22 -> 0.12 ms at 1M, 0.43 -> 0.34 ms at 4M.
+//
+// ctl: [0] overflow (more cells than cap), [1 + l] first cell of level l, then
+// the leaf count, the error word, the tie flag (a run the tie sort left: no
+// cells, the host sorts again), and the first system's box as four doubles.
+constexpr int kCtlOverflow = 0, kCtlLevel = 1, kCtlLeaves = 26, kCtlErr = 27, kCtlTie = 28, kCtlBox = 32,
+              kCtlHost = 40, kCtlTot = 40, kCtlWords = 40 + 4 * 16;   // words [0, kCtlHost) go to the host
+constexpr int kCellBlocks = 8, kCellThreads = 1024;
 
-// child ranges of every (cell of this level, octant), and each cell's child
-// count.  When the level has at most as many cells as the grid has warps
-// (the shallow levels, whose cells hold many particles) a warp takes a cell:
-// its seven groups of four lanes each find one octant boundary by a 5-way
-// search (four probes a step); otherwise a thread takes a (cell, octant) and
-// binary-searches both ends of its range.
+__device__ __forceinline__ void cluster_sync_all()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// first index in [L, R) whose octant at this level is >= o
 __device__ __forceinline__ int first_digit_ge(const uint64_t *keys, int L, int R, int level, int o)
 {
     while (L < R) {
@@ -405,217 +403,215 @@ __device__ __forceinline__ int first_digit_ge(const uint64_t *keys, int L, int R
     return L;
 }
 
-__global__ void __launch_bounds__(256)
-k_level_ranges(CellArrays c, const unsigned *ctl, int level, int ncrit, const uint64_t *keys,
-               int32_t *cb, int32_t *ce, uint32_t *cnt)
+// The same by the four lanes of a group (g = lane / 4), four probes a step.
+__device__ __forceinline__ int first_digit_ge4(const uint64_t *keys, int L, int R, int level, int o, int lane)
 {
-    if (ctl[kCtlOverflow]) return;
-    const int lb = (int)ctl[kCtlLevel + level];
-    const int ncl = (int)ctl[kCtlLevel + level + 1] - lb;
-    const int64_t n8 = 8 * (int64_t)ncl;
-    const unsigned lane = threadIdx.x & 31;
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    if (ncl <= nwarps) {
-        const int64_t wi = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-        if (wi >= ncl) return;
-        const int cell = lb + (int)wi;
-        const int b = c.begin[cell], e = c.end[cell];
-        if (!(e - b > ncrit && level < kLevels)) {
-            if (lane < 8) { cb[8 * wi + lane] = b; ce[8 * wi + lane] = b; }
-            if (lane == 0) cnt[wi] = 0u;
-            return;
-        }
-        const int g = (int)lane >> 2, q = (int)lane & 3;       // group g finds boundary g + 1
-        int bnd = b;
-        if (g < 7) {
-            const unsigned gm = 0xfu << (4 * g);
-            int L = b, R = e;
-            while (R - L > 4) {
-                const int len = R - L;
-                const bool lt = digit_at(keys[L + (int)(((int64_t)(q + 1) * len) / 5)], level + 1) < g + 1;
-                const int k = __popc(__ballot_sync(gm, lt) & gm);
-                const int nL = k > 0 ? L + (int)(((int64_t)k * len) / 5) + 1 : L;
-                const int nR = k < 4 ? L + (int)(((int64_t)(k + 1) * len) / 5) : R;
-                L = nL;
-                R = nR;
-            }
-            const bool lt = q < R - L && digit_at(keys[L + q], level + 1) < g + 1;
-            bnd = L + __popc(__ballot_sync(gm, lt) & gm);
-        }
-        const int o = (int)(lane & 7);
-        const int bl = __shfl_sync(0xffffffffu, bnd, (4 * (o - 1)) & 31);
-        const int bh = __shfl_sync(0xffffffffu, bnd, (4 * o) & 31);
-        const int lo_i = o == 0 ? b : bl, hi_i = o == 7 ? e : bh;
-        const unsigned m = __ballot_sync(0xffffffffu, lane < 8 && hi_i > lo_i);
-        if (lane < 8) { cb[8 * wi + lane] = lo_i; ce[8 * wi + lane] = hi_i; }
-        if (lane == 0) cnt[wi] = __popc(m);
-        return;
+    const int q = lane & 3;
+    const unsigned gm = 0xfu << (lane & ~3);
+    while (R - L > 4) {
+        const int len = R - L;
+        const bool lt = digit_at(keys[L + (int)(((int64_t)(q + 1) * len) / 5)], level) < o;
+        const int k = __popc(__ballot_sync(gm, lt) & gm);
+        const int nL = k > 0 ? L + (int)(((int64_t)k * len) / 5) + 1 : L;
+        const int nR = k < 4 ? L + (int)(((int64_t)(k + 1) * len) / 5) : R;
+        L = nL;
+        R = nR;
     }
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n8; base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t = base + threadIdx.x;
-        bool flag = false;
-        if (t < n8) {
-            const int cell = lb + (int)(t >> 3), o = (int)(t & 7);
-            const int b = c.begin[cell], e = c.end[cell];
-            int lo_i = b, hi_i = b;
-            if (e - b > ncrit && level < kLevels) {
-                // first index in [b, e) whose child digit is >= o (resp. >= o + 1)
-                lo_i = first_digit_ge(keys, b, e, level + 1, o);
-                hi_i = first_digit_ge(keys, lo_i, e, level + 1, o + 1);
-                flag = hi_i > lo_i;
-            }
-            cb[t] = lo_i;
-            ce[t] = hi_i;
-        }
-        // a cell's 8 octants are 8 aligned lanes of one warp
-        const unsigned m = __ballot_sync(0xffffffffu, flag);
-        if (t < n8 && (t & 7) == 0) cnt[t >> 3] = __popc((m >> (lane & ~7u)) & 0xffu);
-    }
+    const bool lt = q < R - L && digit_at(keys[L + q], level) < o;
+    return L + __popc(__ballot_sync(gm, lt) & gm);
 }
 
-// one block: the first-child offset of every cell of this level (an exclusive
-// scan of the child counts) and the next level's range, or the overflow flag
-__global__ void __launch_bounds__(1024)
-k_level_scan(unsigned *ctl, int level, const uint32_t *cnt, uint32_t *off, int64_t cap)
+// Exclusive prefix of v over the block's threads; *total = the block's sum.
+__device__ __forceinline__ unsigned cells_scan(unsigned v, unsigned *wsum, unsigned *total)
 {
-    __shared__ uint32_t wsum[32];
-    __shared__ uint32_t carry;
-    if (ctl[kCtlOverflow]) return;
-    const int lb = (int)ctl[kCtlLevel + level], le = (int)ctl[kCtlLevel + level + 1];
-    const int ncl = le - lb;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (threadIdx.x == 0) carry = 0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[warp] = x;
     __syncthreads();
-    for (int base = 0; base < ncl; base += kLevelScanPer * (int)blockDim.x) {
-        const int i0 = base + kLevelScanPer * (int)threadIdx.x;
-        uint32_t v[kLevelScanPer], sum = 0;
-        if (i0 + kLevelScanPer <= ncl) {             // whole: 16-byte loads (i0 is a multiple of 16)
+    const unsigned w = wsum[lane];                 // kCellThreads / 32 = 32 warps
+    unsigned s = w;
 #pragma unroll
-            for (int k = 0; k < kLevelScanPer; k += 4) {
-                const uint4 q = *(const uint4 *)(cnt + i0 + k);
-                v[k] = q.x; v[k + 1] = q.y; v[k + 2] = q.z; v[k + 3] = q.w;
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < kLevelScanPer; ++k) v[k] = i0 + k < ncl ? cnt[i0 + k] : 0u;
-        }
-#pragma unroll
-        for (int k = 0; k < kLevelScanPer; ++k) sum += v[k];
-        uint32_t x = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) wsum[warp] = x;
-        __syncthreads();
-        if (warp == 0) {
-            uint32_t w = lane < nw ? wsum[lane] : 0u;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
-                if (lane >= o) w += y;
-            }
-            wsum[lane] = w;
-        }
-        __syncthreads();
-        uint32_t ex = carry + (warp ? wsum[warp - 1] : 0u) + x - sum;
-        uint32_t o[kLevelScanPer];
-#pragma unroll
-        for (int k = 0; k < kLevelScanPer; ++k) {
-            o[k] = ex;
-            ex += v[k];
-        }
-        if (i0 + kLevelScanPer <= ncl) {
-#pragma unroll
-            for (int k = 0; k < kLevelScanPer; k += 4)
-                *(uint4 *)(off + i0 + k) = make_uint4(o[k], o[k + 1], o[k + 2], o[k + 3]);
-        } else {
-#pragma unroll
-            for (int k = 0; k < kLevelScanPer; ++k)
-                if (i0 + k < ncl) off[i0 + k] = o[k];
-        }
-        const uint32_t tot = wsum[nw - 1];
-        __syncthreads();
-        if (threadIdx.x == 0) carry += tot;
-        __syncthreads();
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += y;
     }
-    if (threadIdx.x == 0) {
-        if ((int64_t)le + carry > cap) ctl[kCtlOverflow] = 1u;
-        else ctl[kCtlLevel + level + 2] = (unsigned)le + carry;
-    }
+    *total = __shfl_sync(0xffffffffu, s, 31);
+    const unsigned before = __shfl_sync(0xffffffffu, s - w, warp);
+    __syncthreads();                               // wsum is free again
+    return before + x - v;
 }
 
-// the children of this level's cells, in (parent, octant) order
-__global__ void __launch_bounds__(256)
-k_level_write(CellArrays c, const unsigned *ctl, int level, const int32_t *cb, const int32_t *ce,
-              const uint32_t *off)
+// Each block takes a contiguous part of the level's cells.  It lists the cells
+// to split (a thread per cell), finds their octants' first particles (eight
+// lanes per cell, or a warp with four lanes to a search while there are few)
+// and counts their children; the blocks' totals meet over the cluster barrier;
+// then the children are written, and each cell's rank among the leaves or
+// among the cells with children.  c.nchild holds a split cell's children
+// before it until its children are written.
+__global__ void __cluster_dims__(kCellBlocks, 1, 1) __launch_bounds__(kCellThreads)
+k_cells(CellArrays c, const int64_t *off, int nsys, const double *box, const int *err, int ncrit,
+        const uint64_t *keys, int64_t cap, int32_t *cb, int32_t *ce, uint32_t *list, uint32_t *rank,
+        unsigned *ctl)
 {
-    if (ctl[kCtlOverflow]) return;
-    const int lb = (int)ctl[kCtlLevel + level], le = (int)ctl[kCtlLevel + level + 1];
-    const int64_t n8 = 8 * (int64_t)(le - lb);
-    const unsigned lane = threadIdx.x & 31;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n8; base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t = base + threadIdx.x;
-        const bool valid = t < n8;
-        const bool flag = valid && ce[t] > cb[t];
-        const unsigned grp = (__ballot_sync(0xffffffffu, flag) >> (lane & ~7u)) & 0xffu;
-        if (!valid) continue;
-        const int i = (int)(t >> 3), o = (int)(t & 7), cell = lb + i;
-        if (o == 0) {
-            const int nch = __popc(grp);
-            c.nchild[cell] = nch;
-            c.child[cell] = nch ? le + (int)off[i] : -1;
+    __shared__ unsigned s_w[kCellThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = kCellThreads / 32;
+    const int blk = blockIdx.x;
+    const unsigned e = *(volatile const int *)err;
+    const bool tie = (e & kErrTieRun) != 0;
+    for (int s = blk * kCellThreads + tid; s < nsys; s += kCellBlocks * kCellThreads) {
+        c.level[s] = 0; c.parent[s] = -1; c.begin[s] = (int32_t)off[s]; c.end[s] = (int32_t)off[s + 1];
+        c.cx[s] = c.cy[s] = c.cz[s] = 0;
+        c.sys[s] = s;
+    }
+    cluster_sync_all();
+    int lb = 0, le = tie ? 0 : nsys;
+    unsigned leaves = 0, inner = 0;            // before this level
+    bool over = (int64_t)le > cap;
+    int level = 0;
+    for (; level <= kLevels && le > lb && !over; ++level) {
+        const int ncl = le - lb;
+        const int chunk = (ncl + kCellBlocks - 1) / kCellBlocks;
+        const int i0 = min(ncl, blk * chunk), i1 = min(ncl, i0 + chunk);
+        uint32_t *mylist = list + i0;
+        // the cells to split
+        unsigned np = 0;
+        for (int base = i0; base < i1; base += kCellThreads) {
+            const int i = base + tid;
+            const bool split = i < i1 && level < kLevels &&
+                               __ldcg(c.end + lb + i) - __ldcg(c.begin + lb + i) > ncrit;
+            unsigned tot;
+            const unsigned k = np + cells_scan(split, s_w, &tot);
+            if (i < i1) rank[lb + i] = k;                      // cells to split before it
+            if (split) mylist[k] = (uint32_t)(lb + i);
+            np += tot;
         }
-        if (!flag) continue;
-        const int ch = le + (int)off[i] + __popc(grp & ((1u << o) - 1u));
-        c.level[ch] = level + 1;
-        c.parent[ch] = cell;
-        c.begin[ch] = cb[t];
-        c.end[ch] = ce[t];
-        c.cx[ch] = 2 * c.cx[cell] + ((o >> 2) & 1);
-        c.cy[ch] = 2 * c.cy[cell] + ((o >> 1) & 1);
-        c.cz[ch] = 2 * c.cz[cell] + (o & 1);
-        c.sys[ch] = c.sys[cell];
+        __syncthreads();
+        // their octants
+        const bool wide = np <= (unsigned)nw;                  // a warp per cell
+        const int per = wide ? nw : kCellThreads / 8;
+        unsigned nch = 0;
+        for (unsigned base = 0; base < np; base += per) {
+            const unsigned k = base + (wide ? warp : tid >> 3);
+            const int o = lane & 7;
+            int lo_i = 0, hi_i = 0, cell = 0;
+            if (k < np) {                                      // uniform in a warp (8 lanes) that shares a cell
+                cell = (int)mylist[k];
+                const int b = __ldcg(c.begin + cell), en = __ldcg(c.end + cell);
+                if (wide) {
+                    const int g = lane >> 2;                   // the first particle of octant g
+                    const int bnd = g ? first_digit_ge4(keys, b, en, level + 1, g, lane) : b;
+                    lo_i = __shfl_sync(0xffffffffu, bnd, 4 * o);
+                    hi_i = __shfl_sync(0xffffffffu, bnd, (4 * o + 4) & 31);
+                } else {
+                    lo_i = o ? first_digit_ge(keys, b, en, level + 1, o) : b;
+                    hi_i = __shfl_down_sync(0xffu << (lane & ~7), lo_i, 1, 8);
+                }
+                if (o == 7) hi_i = en;
+            }
+            const bool flag = hi_i > lo_i && (!wide || lane < 8);
+            const unsigned m = (__ballot_sync(0xffffffffu, flag) >> (lane & ~7)) & 0xffu;
+            const bool first = k < np && o == 0 && (!wide || lane == 0);
+            unsigned tot;
+            const unsigned before = nch + cells_scan(first ? __popc(m) : 0u, s_w, &tot);
+            if (k < np && (!wide || lane < 8)) {
+                const int64_t at = 8 * ((int64_t)i0 + k) + o;
+                cb[at] = lo_i;
+                ce[at] = hi_i;
+            }
+            if (first) c.nchild[cell] = (int)before;
+            nch += tot;
+        }
+        unsigned *tot = ctl + kCtlTot + (level & 1) * 2 * kCellBlocks;
+        if (tid == 0) { __stcg(tot + 2 * blk, nch); __stcg(tot + 2 * blk + 1, np); }
+        cluster_sync_all();
+        unsigned c0 = 0, p0 = 0, ca = 0, pa = 0;
+        for (int k = 0; k < kCellBlocks; ++k) {
+            const unsigned x = __ldcg(tot + 2 * k), y = __ldcg(tot + 2 * k + 1);
+            if (k < blk) { c0 += x; p0 += y; }
+            ca += x;
+            pa += y;
+        }
+        over = (int64_t)le + ca > cap;
+        if (!over) {
+            for (unsigned t = tid; t < 8 * np; t += kCellThreads) {      // eight lanes per split cell
+                const unsigned k = t >> 3;
+                const int o = (int)(t & 7), cell = (int)mylist[k];
+                const int64_t at = 8 * ((int64_t)i0 + k) + o;
+                const int beg = cb[at], en = ce[at];
+                const unsigned gm = 0xffu << (lane & ~7);
+                const unsigned m = (__ballot_sync(gm, en > beg) >> (lane & ~7)) & 0xffu;
+                const int ch0 = le + (int)(c0 + (unsigned)c.nchild[cell]);
+                __syncwarp(gm);                                // every lane has read the count before the cell
+                if (o == 0) {
+                    c.nchild[cell] = __popc(m);
+                    c.child[cell] = ch0;
+                    rank[cell] = inner + p0 + k;
+                }
+                if (en > beg) {
+                    const int ch = ch0 + __popc(m & ((1u << o) - 1u));
+                    c.level[ch] = level + 1;
+                    c.parent[ch] = cell;
+                    c.begin[ch] = beg;
+                    c.end[ch] = en;
+                    c.cx[ch] = 2 * __ldcg(c.cx + cell) + ((o >> 2) & 1);
+                    c.cy[ch] = 2 * __ldcg(c.cy + cell) + ((o >> 1) & 1);
+                    c.cz[ch] = 2 * __ldcg(c.cz + cell) + (o & 1);
+                    c.sys[ch] = __ldcg(c.sys + cell);
+                }
+            }
+            for (int i = i0 + tid; i < i1; i += kCellThreads) {
+                const int cell = lb + i;
+                if (level < kLevels && __ldcg(c.end + cell) - __ldcg(c.begin + cell) > ncrit) continue;
+                c.nchild[cell] = 0;
+                c.child[cell] = -1;
+                rank[cell] = leaves + (unsigned)i - (p0 + rank[cell]);
+            }
+        }
+        if (blk == 0 && tid == 0) ctl[kCtlLevel + level] = (unsigned)lb;
+        leaves += (unsigned)ncl - pa;
+        inner += pa;
+        lb = le;
+        le += (int)ca;
+        cluster_sync_all();
+    }
+    if (blk == 0) {
+        for (int l = level + tid; l <= kLevels + 2; l += kCellThreads) ctl[kCtlLevel + l] = (unsigned)lb;
+        if (tid == 0) {
+            ctl[kCtlOverflow] = over;
+            ctl[kCtlLeaves] = leaves;
+            ctl[kCtlErr] = e;
+            ctl[kCtlTie] = tie;
+        }
+        if (tid < 4) ((double *)(ctl + kCtlBox))[tid] = box[tid];
     }
 }
 
-// Where the tie sort left a run unsorted there are no cells to build (the host
-// sorts again).
-__global__ void k_level_init(unsigned *ctl, int nsys, const int *err)
-{
-    const int i = threadIdx.x;
-    const bool tie = (*err & kErrTieRun) != 0;
-    if (i < kCtlWords) ctl[i] = i == kCtlLevel + 1 ? (tie ? 0u : (unsigned)nsys) : (i == kCtlTie ? (unsigned)tie : 0u);
-}
-
-// Besides the geometry, each cell gets the packed record the traversal reads
-// with one 16-byte load: {cx | level << 21, cy | nchild << 21, cz, child}.
-__global__ void k_cell_geometry(CellArrays c, int64_t ncells, const double *box, double *centre,
-                                double *half, uint32_t *leaf_flag, int4 *tcell)
+// Besides the geometry, each cell gets its place among the leaves or the cells
+// with children (rank: k_cells) and the packed record the traversal reads with
+// one 16-byte load: {cx | level << 21, cy | nchild << 21, cz, child}.
+__global__ void k_cell_geometry(CellArrays c, int64_t ncells, int64_t nleaves, const uint32_t *rank,
+                                const double *box, int nsys, double *centre, double *half, int32_t *leaves,
+                                int *eside, int4 *tcell)
 {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= ncells) return;
+    if (i < nsys) eside[i] = ilogb(box[4 * i + 3]);        // the first cells are the roots
     const double *bx = box + 4 * c.sys[i];
     const double h = ldexp(bx[3], -(c.level[i] + 1));
     half[i] = h;
     centre[3 * i] = __dadd_rn(bx[0], __dmul_rn((double)(2 * c.cx[i] + 1), h));
     centre[3 * i + 1] = __dadd_rn(bx[1], __dmul_rn((double)(2 * c.cy[i] + 1), h));
     centre[3 * i + 2] = __dadd_rn(bx[2], __dmul_rn((double)(2 * c.cz[i] + 1), h));
-    leaf_flag[i] = c.nchild[i] == 0;
-    tcell[i] = make_int4(c.cx[i] | c.level[i] << kLevels, c.cy[i] | c.nchild[i] << kLevels, c.cz[i],
-                         c.child[i]);
-}
-
-// leaves[0, nleaves): the leaves in index order; leaves[nleaves, ncells): the
-// cells with children in index (so breadth-first) order, for the downward pass
-__global__ void k_compact_leaves(const uint32_t *flag, const uint32_t *pos, int64_t ncells,
-                                 int32_t *leaves)
-{
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= ncells) return;
-    if (flag[i]) leaves[pos[i]] = (int32_t)i;
-    else leaves[pos[ncells] + (i - pos[i])] = (int32_t)i;
+    // leaves[0, nleaves): the leaves in index order; leaves[nleaves, ncells): the
+    // cells with children in index (so breadth-first) order, for the downward pass
+    const int nch = c.nchild[i];
+    leaves[nch ? nleaves + rank[i] : rank[i]] = (int32_t)i;
+    tcell[i] = make_int4(c.cx[i] | c.level[i] << kLevels, c.cy[i] | nch << kLevels, c.cz[i], c.child[i]);
 }
 
 // ----------------------------------------------------------- traversal
@@ -1102,12 +1098,8 @@ fmm_status grow_keep(fmm_tree *t, DevBuf &b, size_t bytes, size_t keep_bytes)
     return FMM_OK;
 }
 
-fmm_status read_err(fmm_tree *t)
+fmm_status check_err(fmm_tree *t, int e)
 {
-    int e = 0;
-    FMM_TRY(cuda_check(t, cudaMemcpyAsync(&e, t->b_err.ptr, sizeof(int), cudaMemcpyDeviceToHost,
-                                          t->stream), "read error word"));
-    FMM_TRY(cuda_check(t, cudaStreamSynchronize(t->stream), "sync"));
     if (e & kErrNonFinite) { t->err = "non-finite particle position"; return FMM_EINVAL; }
     if (e & kErrKeyRange) {
         t->err = "an accepted M2L offset exceeds 2^16 finer half-cells (theta too small for the tree)";
@@ -1277,103 +1269,65 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
         record(t, 2);
     }
 
-    // ---- cells, level by level on the device (level 0 holds one root per system);
-    // the host reads the level counts once per batch of levels
+    // ---- cells: one launch, one host sync (again with more room where they overflow)
     FMM_TRY(ensure(t, t->b_ctl, 4 * kCtlWords));
     unsigned *ctl = (unsigned *)t->b_ctl.ptr;
     DevBuf *cb[10] = {&t->b_level, &t->b_parent, &t->b_child, &t->b_nchild, &t->b_begin,
                       &t->b_end, &t->b_cx, &t->b_cy, &t->b_cz, &t->b_sys};
     int64_t cap = std::max<int64_t>(t->b_level.bytes / 4,
                                     std::max<int64_t>(1024, 5 * (n / std::max(1, t->max_leaf)) + 64 + 2 * nsys));
-    const unsigned lgrid = (unsigned)(8 * sm_count());
-    std::vector<unsigned> hc(kCtlWords);
-    int nlev = 0;
+    unsigned hc[kCtlHost];
+    t->sys_box.assign(4 * (size_t)nsys, 0.0);
     for (;;) {
         for (DevBuf *b : cb) FMM_TRY(ensure(t, *b, 4 * cap));
         FMM_TRY(ensure(t, t->b_flags, 4 * cap));
         FMM_TRY(ensure(t, t->b_scan, 4 * cap));
         FMM_TRY(ensure(t, t->b_front, 8 * 8 * cap));      // child begin/end of every octant
-        CellArrays c = cells_of(t);
-        uint32_t *cnt = (uint32_t *)t->b_flags.ptr, *off8 = (uint32_t *)t->b_scan.ptr;
         int32_t *cbeg = (int32_t *)t->b_front.ptr, *cend = cbeg + 8 * cap;
-        k_roots<<<grid(nsys, 128), 128, 0, st>>>(c, off, nsys);
-        k_level_init<<<1, kCtlWords, 0, st>>>(ctl, nsys, (const int *)t->b_err.ptr);
-        t->launches += 2;
-        int level = 0;
-        bool overflow = false, tie = false;
-        for (;;) {
-            const int end = std::min(level + kLevelBatch, kLevels + 1);
-            for (; level < end; ++level) {
-                k_level_ranges<<<lgrid, 256, 0, st>>>(c, ctl, level, t->max_leaf, keys, cbeg, cend, cnt);
-                k_level_scan<<<1, 1024, 0, st>>>(ctl, level, cnt, off8, cap);
-                k_level_write<<<lgrid, 256, 0, st>>>(c, ctl, level, cbeg, cend, off8);
-                t->launches += 3;
-            }
-            FMM_TRY(cuda_check(t, cudaMemcpyAsync(hc.data(), ctl, 4 * kCtlWords, cudaMemcpyDeviceToHost, st),
-                               "level counts"));
-            FMM_TRY(cuda_check(t, cudaStreamSynchronize(st), "sync"));
-            if (hc[kCtlOverflow]) {
-                overflow = true;
-                break;
-            }
-            if (hc[kCtlTie]) {               // a long run of ties: by all bits, and from now on
-                tie = true;
-                break;
-            }
-            // done once a level came out empty (or the deepest level was processed)
-            if (hc[kCtlLevel + level + 1] == hc[kCtlLevel + level] || level > kLevels) break;
-        }
-        if (tie) {
+        k_cells<<<kCellBlocks, kCellThreads, 0, st>>>(cells_of(t), off, nsys, sbox, (const int *)t->b_err.ptr,
+                                                      t->max_leaf, keys, cap, cbeg, cend, (uint32_t *)t->b_scan.ptr,
+                                                      (uint32_t *)t->b_flags.ptr, ctl);
+        ++t->launches;
+        FMM_TRY(cuda_check(t, cudaGetLastError(), "cells"));
+        FMM_TRY(cuda_check(t, cudaMemcpyAsync(hc, ctl, sizeof(hc), cudaMemcpyDeviceToHost, st), "level counts"));
+        if (nsys > 1)
+            FMM_TRY(cuda_check(t, cudaMemcpyAsync(t->sys_box.data(), sbox, 32 * (size_t)nsys,
+                                                  cudaMemcpyDeviceToHost, st), "box"));
+        FMM_TRY(cuda_check(t, cudaStreamSynchronize(st), "sync"));
+        if (hc[kCtlTie]) {                  // a long run of ties: by all bits
             full = true;
             cudaMemsetAsync(t->b_err.ptr, 0, sizeof(int), st);
             sort_one(full);
             continue;
         }
-        if (!overflow) {
-            // levels 0 .. nlev - 1 hold cells
-            nlev = 1;
-            while (nlev <= kLevels && hc[kCtlLevel + nlev + 1] > hc[kCtlLevel + nlev]) ++nlev;
-            break;
-        }
+        if (!hc[kCtlOverflow]) break;
         cap *= 2;
     }
-    t->level_begin.assign(hc.begin() + kCtlLevel, hc.begin() + kCtlLevel + nlev + 1);
+    FMM_TRY(check_err(t, (int)hc[kCtlErr]));
+    t->sort_full = nsys == 1 && full;
+    if (nsys == 1) std::memcpy(t->sys_box.data(), hc + kCtlBox, 32);
+    // levels 0 .. nlev - 1 hold cells
+    int nlev = 1;
+    while (nlev <= kLevels && hc[kCtlLevel + nlev + 1] > hc[kCtlLevel + nlev]) ++nlev;
+    t->level_begin.assign(hc + kCtlLevel, hc + kCtlLevel + nlev + 1);
     t->ncells = t->level_begin.back();
     t->nlevels = nlev;
-    CellArrays c = cells_of(t);
+    t->nleaves = hc[kCtlLeaves];
+    t->lo[0] = t->sys_box[0]; t->lo[1] = t->sys_box[1]; t->lo[2] = t->sys_box[2];
+    t->side = t->sys_box[3];
     const int64_t nc = t->ncells;
     FMM_TRY(ensure(t, t->b_centre, 8 * 3 * nc));
     FMM_TRY(ensure(t, t->b_half, 8 * nc));
-    FMM_TRY(ensure(t, t->b_flags, 4 * (nc + 1)));
-    FMM_TRY(ensure(t, t->b_scan, 4 * (nc + 1)));
-    uint32_t *flags = (uint32_t *)t->b_flags.ptr, *posc = (uint32_t *)t->b_scan.ptr;
-    cudaMemsetAsync(flags + nc, 0, 4, st);
     FMM_TRY(ensure(t, t->b_tcell, 16 * nc));
-    k_cell_geometry<<<grid(nc, 256), 256, 0, st>>>(c, nc, sbox, (double *)t->b_centre.ptr,
-                                                    (double *)t->b_half.ptr, flags, (int4 *)t->b_tcell.ptr);
-    exclusive_scan_u32(flags, posc, nc + 1, (uint32_t *)t->b_scan_tmp.ptr, st, &t->launches);
-    uint32_t nleaves = 0;
-    FMM_TRY(cuda_check(t, cudaMemcpyAsync(&nleaves, posc + nc, 4, cudaMemcpyDeviceToHost, st),
-                       "leaf count"));
     FMM_TRY(ensure(t, t->b_leaves, 4 * (size_t)nc));
-    k_compact_leaves<<<grid(nc, 256), 256, 0, st>>>(flags, posc, nc, (int32_t *)t->b_leaves.ptr);
-    t->launches += 2;
-    t->sys_box.assign(4 * (size_t)nsys, 0.0);
-    FMM_TRY(cuda_check(t, cudaMemcpyAsync(t->sys_box.data(), sbox, 32 * (size_t)nsys,
-                                          cudaMemcpyDeviceToHost, st), "box"));
-    record(t, 3);
-    FMM_TRY(read_err(t));
-    t->sort_full = nsys == 1 && full;
-    t->nleaves = nleaves;
-    t->lo[0] = t->sys_box[0]; t->lo[1] = t->sys_box[1]; t->lo[2] = t->sys_box[2];
-    t->side = t->sys_box[3];
-    std::vector<int> es((size_t)nsys);
-    for (int s = 0; s < nsys; ++s) es[s] = std::ilogb(t->sys_box[4 * s + 3]);
     FMM_TRY(ensure(t, t->b_syseside, 4 * (size_t)nsys));
-    FMM_TRY(cuda_check(t, cudaMemcpyAsync(t->b_syseside.ptr, es.data(), 4 * (size_t)nsys,
-                                          cudaMemcpyHostToDevice, st), "system sides"));
-    FMM_TRY(cuda_check(t, cudaStreamSynchronize(st), "sync"));
-    return FMM_OK;
+    k_cell_geometry<<<grid(nc, 256), 256, 0, st>>>(cells_of(t), nc, t->nleaves, (const uint32_t *)t->b_flags.ptr, sbox,
+                                                    nsys, (double *)t->b_centre.ptr, (double *)t->b_half.ptr,
+                                                    (int32_t *)t->b_leaves.ptr, (int *)t->b_syseside.ptr,
+                                                    (int4 *)t->b_tcell.ptr);
+    ++t->launches;
+    record(t, 3);
+    return cuda_check(t, cudaGetLastError(), "cell geometry");
 }
 
 fmm_status build_lists(fmm_tree *t, double theta)
