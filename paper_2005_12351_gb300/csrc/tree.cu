@@ -360,11 +360,13 @@ struct CellArrays {
     int32_t *level, *parent, *child, *nchild, *begin, *end, *cx, *cy, *cz, *sys;
 };
 
-__global__ void k_root_pairs(int2 *front, int nsys, unsigned *nf0)
+// the traversal's start: counters and row counts zero, one (root, root) pair per system
+__global__ void k_list_init(unsigned *cnt, int ncnt, unsigned *rows, int64_t nrows, int2 *front, int nsys, int nf0)
 {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < nsys) front[s] = make_int2(s, s);
-    if (s == 0) *nf0 = (unsigned)nsys;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    for (int64_t i = i0; i < ncnt; i += stride) cnt[i] = i == nf0 ? (unsigned)nsys : 0u;
+    for (int64_t i = i0; i < nrows; i += stride) rows[i] = 0u;
+    for (int64_t i = i0; i < nsys; i += stride) front[i] = make_int2((int)i, (int)i);
 }
 
 __device__ __forceinline__ int digit_at(uint64_t key, int level)
@@ -805,13 +807,51 @@ k_traverse_round(const int4 *__restrict__ tc, int round, double theta2, const in
 
 // ------------------------------------------------- lists laid out by target
 // A pair goes to its row at the position the traversal gave it.
-__global__ void k_list_scatter(const int2 *pairs, const uint32_t *slot, int64_t np,
-                               const uint32_t *off, int32_t *src)
+struct ListArgs {
+    const int2 *pairs;
+    const uint32_t *slot;
+    int64_t np;
+    const uint32_t *off;
+    int32_t *src;
+};
+__global__ void k_list_scatter(const ListArgs m, const ListArgs p)
 {
     int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= np) return;
-    const int2 p = pairs[k];
-    src[off[p.x] + slot[k]] = p.y;
+    const bool second = k >= m.np;
+    const ListArgs &l = second ? p : m;
+    if (second) k -= m.np;
+    if (k >= l.np) return;
+    const int2 q = l.pairs[k];
+    l.src[l.off[q.x] + l.slot[k]] = q.y;
+}
+
+// The exclusive scans of both lists' row counts, a block each (rows and off:
+// two arrays of n words one after the other).  One launch for up to kScanRows
+// cells; larger trees take the general scan, three launches a list.
+constexpr int kScanRows = 1 << 16;
+__global__ void __launch_bounds__(1024)
+k_scan_rows(const unsigned *rows, int n, uint32_t *off_a, uint32_t *off_b)
+{
+    __shared__ unsigned s_w[32];
+    const unsigned *in = rows + (int64_t)blockIdx.x * n;
+    uint32_t *out = blockIdx.x ? off_b : off_a;
+    unsigned carry = 0;
+    for (int base = 0; base < n; base += 4096) {
+        const int i = base + 4 * (int)threadIdx.x;
+        unsigned v[4], sum = 0, tot;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[k] = i + k < n ? in[i + k] : 0u;
+            sum += v[k];
+        }
+        unsigned x = carry + cells_scan(sum, s_w, &tot);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (i + k < n) out[i + k] = x;
+            x += v[k];
+        }
+        carry += tot;
+    }
 }
 
 // Rows of a list sorted by source, in place, so that every build gives the
@@ -837,11 +877,10 @@ __device__ __forceinline__ void bitonic_smem(uint32_t *v, int n, int tid, int nt
 }
 
 template <bool COUNT>
-__global__ void __launch_bounds__(256)
-k_row_sort(const uint32_t *off, int32_t *src, int64_t nrows, const int32_t *cbeg, const int32_t *cend,
-           unsigned long long *inter, uint32_t *long_rows, unsigned *n_long, int warp_max)
+__device__ __forceinline__ void
+row_sort(uint32_t (*buf)[kRowWarpMax], const uint32_t *off, int32_t *src, int64_t nrows, const int32_t *cbeg,
+         const int32_t *cend, unsigned long long *inter, uint32_t *long_rows, unsigned *n_long, int warp_max)
 {
-    __shared__ uint32_t buf[8][kRowWarpMax];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t nwarps = (int64_t)gridDim.x * 8;
     unsigned long long acc = 0;
@@ -888,15 +927,31 @@ k_row_sort(const uint32_t *off, int32_t *src, int64_t nrows, const int32_t *cbeg
     }
 }
 
+// both lists in one launch: blockIdx.y 0 the M2L rows, 1 the P2P rows
+__global__ void __launch_bounds__(256)
+k_row_sort(const uint32_t *m2l_off, int32_t *m2l_src, const uint32_t *p2p_off, int32_t *p2p_src, int64_t nrows,
+           const int32_t *cbeg, const int32_t *cend, unsigned long long *inter, uint32_t *long_rows,
+           unsigned *n_long, int warp_max)
+{
+    __shared__ uint32_t buf[8][kRowWarpMax];
+    if (blockIdx.y == 0)
+        row_sort<false>(buf, m2l_off, m2l_src, nrows, cbeg, cend, nullptr, long_rows, n_long, warp_max);
+    else
+        row_sort<true>(buf, p2p_off, p2p_src, nrows, cbeg, cend, inter, long_rows + nrows + 1, n_long + 1, warp_max);
+}
+
 // The queued long rows, one block each; a row longer than block_max (at most
 // kRowBlockMax) sets kErrLongRow in *err and is left for the host, which
 // then sorts the whole list by (target, source) with the radix sort.
 __global__ void __launch_bounds__(1024)
-k_row_sort_long(const uint32_t *off, int32_t *src, const uint32_t *long_rows, const unsigned *n_long,
-                int *err, int block_max)
+k_row_sort_long(const uint32_t *m2l_off, int32_t *m2l_src, const uint32_t *p2p_off, int32_t *p2p_src,
+                int64_t nrows, const uint32_t *long_rows, const unsigned *n_long, int *err, int block_max)
 {
     __shared__ uint32_t v[kRowBlockMax];
-    const unsigned nl = *n_long;
+    const uint32_t *off = blockIdx.y ? p2p_off : m2l_off;
+    int32_t *src = blockIdx.y ? p2p_src : m2l_src;
+    if (blockIdx.y) long_rows += nrows + 1;
+    const unsigned nl = n_long[blockIdx.y];
     for (unsigned q = blockIdx.x; q < nl; q += gridDim.x) {
         const uint32_t r = long_rows[q], b0 = off[r], L = off[r + 1] - b0;
         if (L > (uint32_t)block_max) {
@@ -968,12 +1023,17 @@ __device__ __forceinline__ uint64_t hash64(uint64_t x)
     return x;
 }
 
+// Probes before the table counts as full: a table under half full needs fewer
+// than a hundred, and walking all of a full one for every pair would take seconds.
+constexpr int kMaxProbes = 256;
+
 // Offset keys of the M2L pairs, one warp per target row (CSR order): the
 // key of a pair is its level gap, which side is finer and the centre offset
 // in finer half-cells; equal keys share one derivative row.
 __global__ void k_offset_keys(CellArrays c, const int32_t *off, const int32_t *src, int64_t nrows,
                               unsigned long long *table, uint32_t hmask, uint32_t *slot_of,
-                              int *err, unsigned *max_gap)
+                              uint64_t *new_key, uint32_t *new_slot, unsigned *n_new, int *err,
+                              unsigned *max_gap)
 {
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -1000,11 +1060,16 @@ __global__ void k_offset_keys(CellArrays c, const int32_t *off, const int32_t *s
             if (bad) { atomicOr(err, kErrKeyRange); slot_of[k] = 0; continue; }
             uint32_t h = (uint32_t)hash64(key) & hmask;
             bool placed = false;
-            for (uint32_t probe = 0; probe <= hmask; ++probe) {
+            for (int probe = 0; probe < kMaxProbes; ++probe) {
                 unsigned long long cur = table[h];
                 if (cur == key) { placed = true; break; }
                 if (cur == ~0ull) {
                     unsigned long long prev = atomicCAS(&table[h], ~0ull, (unsigned long long)key);
+                    if (prev == ~0ull) {                     // a key seen first here joins the list
+                        const unsigned k = atomicAdd(n_new, 1u);
+                        new_key[k] = key;
+                        new_slot[k] = h;
+                    }
                     if (prev == ~0ull || prev == key) { placed = true; break; }
                 }
                 h = (h + 1) & hmask;
@@ -1018,56 +1083,44 @@ __global__ void k_offset_keys(CellArrays c, const int32_t *off, const int32_t *s
     }
 }
 
-__global__ void k_slot_flags(const unsigned long long *table, uint32_t H, uint32_t *flag)
+// Which colliding key wins a hash slot depends on timing, so neither the slots
+// nor the list's order are reproducible: the distinct keys are sorted by value
+// and a pair's D row is the rank of its key.
+// A key's rank is the number of smaller keys among the n distinct ones: a warp
+// per key up to kRankSmall keys (the radix sort beyond).  keys_out[rank] = key,
+// rank_of[slot of the key in the table] = rank.
+constexpr unsigned kRankSmall = 4096;
+__global__ void __launch_bounds__(256)
+k_rank_keys(const uint64_t *key, const uint32_t *slot, const unsigned *n_keys, uint64_t *keys_out, uint32_t *rank_of)
 {
-    uint32_t h = blockIdx.x * blockDim.x + threadIdx.x;
-    if (h < H) flag[h] = table[h] != ~0ull;
-}
-
-__global__ void k_slot_compact(const unsigned long long *table, uint32_t H, const uint32_t *dense,
-                               uint64_t *dkeys)
-{
-    uint32_t h = blockIdx.x * blockDim.x + threadIdx.x;
-    if (h < H && table[h] != ~0ull) dkeys[dense[h]] = table[h];
-}
-
-// Which colliding key wins a hash slot depends on timing, so slot order is
-// not reproducible: the distinct keys are sorted by value and a pair's D row
-// is the rank of its key (rank_of[dense index]).
-__global__ void k_slot_to_dense(int32_t *didx, int64_t np, const uint32_t *dense, const uint32_t *rank_of)
-{
-    int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k < np) didx[k] = (int32_t)rank_of[dense[(uint32_t)didx[k]]];
-}
-
-__global__ void k_iota(uint32_t *v, int64_t n)
-{
-    int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k < n) v[k] = (uint32_t)k;
-}
-
-// Distinct keys (n <= kRankSmall) sorted in place in one block: a key's rank
-// is the number of smaller keys.  The result equals the radix sort's.
-constexpr int kRankSmall = 4096;
-
-__global__ void __launch_bounds__(1024) k_rank_small(uint64_t *keys, int n, uint32_t *rank_of)
-{
-    extern __shared__ uint64_t sk[];
-    for (int i = threadIdx.x; i < n; i += blockDim.x) sk[i] = keys[i];
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const uint64_t v = sk[i];
-        int r = 0;
-        for (int j = 0; j < n; ++j) r += sk[j] < v;
-        rank_of[i] = (uint32_t)r;
-        keys[r] = v;                 // every read is from shared memory
+    const unsigned n = *n_keys;
+    if (n > kRankSmall) return;
+    const unsigned lane = threadIdx.x & 31, nw = gridDim.x * (blockDim.x >> 5);
+    for (unsigned i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nw) {
+        const uint64_t v = key[i];
+        unsigned r = 0;
+        for (unsigned j = lane; j < n; j += 32) r += key[j] < v;
+        r = __reduce_add_sync(0xffffffffu, r);
+        if (lane == 0) {
+            keys_out[r] = v;
+            rank_of[slot[i]] = r;
+        }
     }
 }
 
-__global__ void k_rank_of(const uint32_t *old_of_rank, int64_t n, uint32_t *rank_of)
+// the sorted list's ranks (more than kRankSmall keys)
+__global__ void k_rank_sorted(const uint32_t *slot, int64_t n, uint32_t *rank_of)
 {
-    int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (r < n) rank_of[old_of_rank[r]] = (uint32_t)r;
+    const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (r < n) rank_of[slot[r]] = (uint32_t)r;
+}
+
+// table slots -> ranks, once rank_of is known (max_keys: up to how many keys it is)
+__global__ void k_slot_to_rank(int32_t *didx, int64_t np, const uint32_t *rank_of, const unsigned *n_keys,
+                               unsigned max_keys)
+{
+    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (*n_keys <= max_keys && k < np) didx[k] = (int32_t)rank_of[didx[k]];
 }
 
 inline unsigned grid(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
@@ -1369,10 +1422,8 @@ fmm_status build_lists(fmm_tree *t, double theta)
         p2p_cap = t->b_p2p_raw.bytes / 8;
         front_cap = std::min(t->b_front.bytes, t->b_front2.bytes) / 8;
         int2 *fr[2] = {(int2 *)t->b_front.ptr, (int2 *)t->b_front2.ptr};
-        FMM_TRY(cuda_check(t, cudaMemsetAsync(cnt, 0, 4 * (kTravFront + kTravMaxRounds + 1), st),
-                           "counters"));
-        FMM_TRY(cuda_check(t, cudaMemsetAsync(rows, 0, 8 * (size_t)(nc + 1), st), "row counts"));
-        k_root_pairs<<<grid(nsys, 128), 128, 0, st>>>(fr[0], nsys, cnt + kTravFront);
+        k_list_init<<<(unsigned)std::min<int64_t>(grid(std::max<int64_t>(2 * (nc + 1), nsys), 256), 2 * (int64_t)sm_count()),
+                      256, 0, st>>>(cnt, kTravFront + kTravMaxRounds + 1, rows, 2 * (nc + 1), fr[0], nsys, kTravFront);
         ++t->launches;
         int r = 0;
         bool retry = false;
@@ -1423,9 +1474,27 @@ fmm_status build_lists(fmm_tree *t, double theta)
     FMM_TRY(ensure(t, t->b_p2p_src, 4 * std::max<int64_t>(np2p, 1)));
     FMM_TRY(ensure(t, t->b_p2p_off, 4 * (nc + 1)));
     FMM_TRY(ensure(t, t->b_long, 8 * (size_t)(nc + 1)));
+    // counter words (zero since k_list_init): 4, 5 long rows of each list, 6 their
+    // flag, 8-9 P2P interactions, 10 errors of the offset hash, 12 largest level
+    // gap, 13 distinct offsets, 14 sort status; one copy brings them to the host
     int *sort_err = (int *)(cnt + 14), *long_err = (int *)(cnt + 6);
-    unsigned *n_long = cnt + 4;                          // queued long rows: M2L, P2P
+    unsigned *n_long = cnt + 4;
     unsigned long long *inter_d = (unsigned long long *)(cnt + 8);
+    struct Words {
+        unsigned pad0[4], n_long[2];
+        int le;
+        unsigned pad1;
+        unsigned long long inter;
+        int he;
+        unsigned pad2, gmax, nd;
+        int serr;
+        unsigned pad3;
+    } hw;
+    static_assert(sizeof(Words) == 64, "counter words 0 .. 15");
+    auto read_words = [&]() -> fmm_status {
+        FMM_TRY(cuda_check(t, cudaMemcpyAsync(&hw, cnt, sizeof(hw), cudaMemcpyDeviceToHost, st), "list counters"));
+        return cuda_check(t, cudaStreamSynchronize(st), "sync");
+    };
     int32_t *m2l_off = (int32_t *)t->b_m2l_off.ptr, *p2p_off = (int32_t *)t->b_p2p_off.ptr;
     int32_t *m2l_src = (int32_t *)t->b_m2l_src.ptr, *p2p_src = (int32_t *)t->b_p2p_src.ptr;
     int cbits = 1;
@@ -1434,30 +1503,28 @@ fmm_status build_lists(fmm_tree *t, double theta)
     int row_lim = kRowBlockMax;
     if (const char *env = getenv("FMM_ROW_SORT_LIMIT")) row_lim = std::min(std::max(2, atoi(env)), kRowBlockMax);
     auto layout_rows = [&]() {
-        cudaMemsetAsync(cnt + 4, 0, 4 * 6, st);          // words 4 .. 9: long rows, flag, P2P count
-        exclusive_scan_u32(rows, (uint32_t *)m2l_off, nc + 1, (uint32_t *)t->b_scan_tmp.ptr, st, &t->launches);
-        exclusive_scan_u32(rows + nc + 1, (uint32_t *)p2p_off, nc + 1, (uint32_t *)t->b_scan_tmp.ptr, st,
-                           &t->launches);
+        if (nc + 1 <= kScanRows) {
+            k_scan_rows<<<2, 1024, 0, st>>>(rows, (int)(nc + 1), (uint32_t *)m2l_off, (uint32_t *)p2p_off);
+            ++t->launches;
+        } else {
+            exclusive_scan_u32(rows, (uint32_t *)m2l_off, nc + 1, (uint32_t *)t->b_scan_tmp.ptr, st, &t->launches);
+            exclusive_scan_u32(rows + nc + 1, (uint32_t *)p2p_off, nc + 1, (uint32_t *)t->b_scan_tmp.ptr, st,
+                               &t->launches);
+        }
+        const ListArgs lm = {(const int2 *)t->b_m2l_raw.ptr, (const uint32_t *)t->b_m2l_slot.ptr, nm2l,
+                             (const uint32_t *)m2l_off, m2l_src};
+        const ListArgs lp = {(const int2 *)t->b_p2p_raw.ptr, (const uint32_t *)t->b_p2p_slot.ptr, np2p,
+                             (const uint32_t *)p2p_off, p2p_src};
+        if (nm2l + np2p > 0) k_list_scatter<<<grid(nm2l + np2p, 256), 256, 0, st>>>(lm, lp);
         uint32_t *lq = (uint32_t *)t->b_long.ptr;
         const unsigned rgrid = (unsigned)std::min<int64_t>((nc + 7) / 8, 6 * (int64_t)sm_count());
-        if (nm2l > 0)
-            k_list_scatter<<<grid(nm2l, 256), 256, 0, st>>>((const int2 *)t->b_m2l_raw.ptr,
-                                                            (const uint32_t *)t->b_m2l_slot.ptr, nm2l,
-                                                            (const uint32_t *)m2l_off, m2l_src);
-        if (np2p > 0)
-            k_list_scatter<<<grid(np2p, 256), 256, 0, st>>>((const int2 *)t->b_p2p_raw.ptr,
-                                                            (const uint32_t *)t->b_p2p_slot.ptr, np2p,
-                                                            (const uint32_t *)p2p_off, p2p_src);
-        k_row_sort<false><<<rgrid, 256, 0, st>>>((const uint32_t *)m2l_off, m2l_src, nc, c.begin, c.end,
-                                                  nullptr, lq, n_long, std::min(row_lim, kRowWarpMax));
-        k_row_sort<true><<<rgrid, 256, 0, st>>>((const uint32_t *)p2p_off, p2p_src, nc, c.begin, c.end,
-                                                 inter_d, lq + nc + 1, n_long + 1,
-                                                 std::min(row_lim, kRowWarpMax));
-        k_row_sort_long<<<(unsigned)sm_count(), 1024, 0, st>>>((const uint32_t *)m2l_off, m2l_src, lq,
-                                                                n_long, long_err, row_lim);
-        k_row_sort_long<<<(unsigned)sm_count(), 1024, 0, st>>>((const uint32_t *)p2p_off, p2p_src,
-                                                                lq + nc + 1, n_long + 1, long_err, row_lim);
-        t->launches += 6;
+        k_row_sort<<<dim3(rgrid, 2), 256, 0, st>>>((const uint32_t *)m2l_off, m2l_src, (const uint32_t *)p2p_off,
+                                                    p2p_src, nc, c.begin, c.end, inter_d, lq, n_long,
+                                                    std::min(row_lim, kRowWarpMax));
+        k_row_sort_long<<<dim3((unsigned)sm_count(), 2), 1024, 0, st>>>((const uint32_t *)m2l_off, m2l_src,
+                                                                         (const uint32_t *)p2p_off, p2p_src, nc, lq,
+                                                                         n_long, long_err, row_lim);
+        t->launches += 3;
     };
     auto layout_radix = [&]() -> fmm_status {
         const int64_t nmax = std::max<int64_t>({nm2l, np2p, 1});
@@ -1487,95 +1554,75 @@ fmm_status build_lists(fmm_tree *t, double theta)
         ++t->launches;
         return FMM_OK;
     };
-    cudaMemsetAsync(sort_err, 0, 4, st);
     layout_rows();
 
-    // ---- distinct M2L offsets (rows of the derivative table).  One host sync
-    // reads everything at once: the hash status, the long-row flag, the
-    // distinct count, the largest level gap and the P2P interaction count;
-    // a full hash table or a long row (rare) redoes the part concerned.
+    // ---- distinct M2L offsets (rows of the derivative table), numbered by value.
+    // The ranks and the pairs' rows are formed before the host knows the count;
+    // one host sync then reads everything at once: the hash status, the long-row
+    // flag, the distinct count, the largest level gap and the P2P interaction
+    // count.  A full hash table, a long row or more than kRankSmall offsets
+    // (rare) redo the part concerned.  The table starts at 64k slots whatever the
+    // list's length: even deep adaptive trees have a few thousand offsets.
     int64_t ndoff = 0;
-    int serr = 0, le = 0;
-    unsigned long long inter = 0;
-    bool dsort = false;                    // the distinct keys went through the radix sort
     if (nm2l > 0) {
         uint32_t H = 1u << 16;
-        while (H < 4 * (uint32_t)std::min<int64_t>(nm2l, 1 << 22) && H < (1u << 20)) H <<= 1;
-        uint32_t nd = 0;
-        for (;;) {
+        for (bool again = false;; again = true) {
             FMM_TRY(ensure(t, t->b_hash, 8 * (size_t)H));
-            FMM_TRY(ensure(t, t->b_flags, 4 * ((size_t)H + 1)));
-            FMM_TRY(ensure(t, t->b_scan, 4 * ((size_t)H + 1)));
-            FMM_TRY(ensure(t, t->b_scan_tmp, scan_scratch_bytes((int64_t)H + 1)));
+            FMM_TRY(ensure(t, t->b_dsort, 12 * (size_t)H));       // the list: keys, then slots
+            FMM_TRY(ensure(t, t->b_scan, 4 * (size_t)H));         // slot -> rank
+            FMM_TRY(ensure(t, t->b_dkeys, 8 * (size_t)kRankSmall));
+            uint64_t *lkey = (uint64_t *)t->b_dsort.ptr;
+            uint32_t *lslot = (uint32_t *)(lkey + H), *rank_of = (uint32_t *)t->b_scan.ptr;
             cudaMemsetAsync(t->b_hash.ptr, 0xff, 8 * (size_t)H, st);
-            cudaMemsetAsync(t->b_err.ptr, 0, sizeof(int), st);
-            cudaMemsetAsync(cnt + 12, 0, 4, st);
+            if (again) cudaMemsetAsync(cnt + 10, 0, 4 * 4, st);   // errors, gap, count
             k_offset_keys<<<(unsigned)std::min<int64_t>((nc + 7) / 8, 8 * (int64_t)sm_count()), 256, 0, st>>>(
                 c, m2l_off, m2l_src, nc, (unsigned long long *)t->b_hash.ptr, H - 1,
-                (uint32_t *)t->b_m2l_didx.ptr, (int *)t->b_err.ptr, cnt + 12);
-            uint32_t *flag = (uint32_t *)t->b_flags.ptr, *dense = (uint32_t *)t->b_scan.ptr;
-            cudaMemsetAsync(flag + H, 0, 4, st);
-            k_slot_flags<<<grid(H, 256), 256, 0, st>>>((unsigned long long *)t->b_hash.ptr, H, flag);
-            exclusive_scan_u32(flag, dense, (int64_t)H + 1, (uint32_t *)t->b_scan_tmp.ptr, st, &t->launches);
-            t->launches += 2;
-            int e = 0;
-            unsigned gmax = 0;
-            FMM_TRY(cuda_check(t, cudaMemcpyAsync(&e, t->b_err.ptr, 4, cudaMemcpyDeviceToHost, st), "err"));
-            FMM_TRY(cuda_check(t, cudaMemcpyAsync(&le, long_err, 4, cudaMemcpyDeviceToHost, st), "rows"));
-            FMM_TRY(cuda_check(t, cudaMemcpyAsync(&gmax, cnt + 12, 4, cudaMemcpyDeviceToHost, st), "gap"));
-            FMM_TRY(cuda_check(t, cudaMemcpyAsync(&nd, dense + H, 4, cudaMemcpyDeviceToHost, st), "ndoff"));
-            FMM_TRY(cuda_check(t, cudaMemcpyAsync(&inter, inter_d, 8, cudaMemcpyDeviceToHost, st), "p2p count"));
-            FMM_TRY(cuda_check(t, cudaMemcpyAsync(&serr, sort_err, 4, cudaMemcpyDeviceToHost, st), "sort status"));
-            FMM_TRY(cuda_check(t, cudaStreamSynchronize(st), "sync"));
-            if (le) {
+                (uint32_t *)t->b_m2l_didx.ptr, lkey, lslot, cnt + 13, (int *)(cnt + 10), cnt + 12);
+            k_rank_keys<<<(unsigned)sm_count(), 256, 0, st>>>(lkey, lslot, cnt + 13, (uint64_t *)t->b_dkeys.ptr,
+                                                              rank_of);
+            k_slot_to_rank<<<grid(nm2l, 256), 256, 0, st>>>((int32_t *)t->b_m2l_didx.ptr, nm2l, rank_of, cnt + 13,
+                                                            kRankSmall);
+            t->launches += 3;
+            FMM_TRY(read_words());
+            if (hw.le) {
                 FMM_TRY(layout_radix());
-                le = 0;
+                hw.le = 0;
                 continue;
             }
-            if (e & kErrKeyRange) {
+            if (hw.he & kErrKeyRange) {
                 t->err = "an accepted M2L offset exceeds 2^16 finer half-cells (theta too small for the tree)";
                 return FMM_EINVAL;
             }
-            if (!(e & kErrHashFull)) {
-                t->max_gap = (int)gmax;
-                break;
-            }
+            if (!(hw.he & kErrHashFull)) break;
             H <<= 1;
         }
-        uint32_t *dense = (uint32_t *)t->b_scan.ptr;
-        ndoff = nd;
-        FMM_TRY(ensure(t, t->b_dkeys, 8 * std::max<int64_t>(ndoff, 1)));
-        k_slot_compact<<<grid(H, 256), 256, 0, st>>>((unsigned long long *)t->b_hash.ptr, H, dense,
-                                                       (uint64_t *)t->b_dkeys.ptr);
-        // canonical numbering: keys by value (57-bit keys: gap, side, offsets)
-        const int64_t nd1 = std::max<int64_t>(ndoff, 1);
-        FMM_TRY(ensure(t, t->b_dsort, 20 * (size_t)nd1));
-        FMM_TRY(ensure(t, t->b_dsort_h, radix_hist_bytes(nd1)));
-        uint64_t *keys2 = (uint64_t *)t->b_dsort.ptr;
-        uint32_t *vals = (uint32_t *)(keys2 + nd1), *vals2 = vals + nd1, *rank_of = vals2 + nd1;
-        if (ndoff <= kRankSmall) {
-            k_rank_small<<<1, 1024, 8 * (size_t)ndoff, st>>>((uint64_t *)t->b_dkeys.ptr, (int)ndoff, rank_of);
-            t->launches += 2;
-        } else {
-            k_iota<<<grid(ndoff, 256), 256, 0, st>>>(vals, ndoff);
-            radix_sort_pairs((uint64_t *)t->b_dkeys.ptr, vals, keys2, vals2, ndoff, 57,
+        t->max_gap = (int)hw.gmax;
+        ndoff = hw.nd;
+        if (ndoff > (int64_t)kRankSmall) {
+            uint64_t *lkey = (uint64_t *)t->b_dsort.ptr;
+            uint32_t *lslot = (uint32_t *)(lkey + H), *rank_of = (uint32_t *)t->b_scan.ptr;
+            FMM_TRY(ensure(t, t->b_dkeys, 8 * (size_t)ndoff));
+            FMM_TRY(ensure(t, t->b_lkeys2, 8 * (size_t)ndoff));
+            FMM_TRY(ensure(t, t->b_lval2, 4 * (size_t)ndoff));
+            FMM_TRY(ensure(t, t->b_dsort_h, radix_hist_bytes(ndoff)));
+            radix_sort_pairs(lkey, lslot, (uint64_t *)t->b_lkeys2.ptr, (uint32_t *)t->b_lval2.ptr, ndoff, 57,
                              (uint32_t *)t->b_dsort_h.ptr, sort_err, st, &t->launches);
-            k_rank_of<<<grid(ndoff, 256), 256, 0, st>>>(vals, ndoff, rank_of);
-            t->launches += 3;
-            dsort = true;
+            k_rank_sorted<<<grid(ndoff, 256), 256, 0, st>>>(lslot, ndoff, rank_of);
+            k_slot_to_rank<<<grid(nm2l, 256), 256, 0, st>>>((int32_t *)t->b_m2l_didx.ptr, nm2l, rank_of, cnt + 13, ~0u);
+            t->launches += 2;
+            FMM_TRY(cuda_check(t, cudaMemcpyAsync(t->b_dkeys.ptr, lkey, 8 * (size_t)ndoff, cudaMemcpyDeviceToDevice, st),
+                               "offset keys"));
+            FMM_TRY(read_words());                                // the sort's status
         }
-        k_slot_to_dense<<<grid(nm2l, 256), 256, 0, st>>>((int32_t *)t->b_m2l_didx.ptr, nm2l, dense, rank_of);
+    } else {
+        FMM_TRY(read_words());
+        while (hw.le) {                     // a long P2P row with no M2L list to catch it earlier
+            FMM_TRY(layout_radix());
+            FMM_TRY(read_words());
+        }
     }
-    // the sort status once more when a radix sort ran after the read above; the
-    // long-row flag and the P2P count when there was no M2L list to read them with
-    while (nm2l == 0 || dsort) {
-        FMM_TRY(cuda_check(t, cudaMemcpyAsync(&serr, sort_err, 4, cudaMemcpyDeviceToHost, st), "sort status"));
-        FMM_TRY(cuda_check(t, cudaMemcpyAsync(&le, long_err, 4, cudaMemcpyDeviceToHost, st), "rows"));
-        FMM_TRY(cuda_check(t, cudaMemcpyAsync(&inter, inter_d, 8, cudaMemcpyDeviceToHost, st), "p2p count"));
-        FMM_TRY(cuda_check(t, cudaStreamSynchronize(st), "sync"));
-        if (!le) break;
-        FMM_TRY(layout_radix());        // a long P2P row with no M2L list to catch it earlier
-    }
+    const int serr = hw.serr;
+    const unsigned long long inter = hw.inter;
     if (serr & kErrSortWait) {
         t->err = "a bounded wait of the radix sort gave up";
         return FMM_ETIMEOUT;
