@@ -119,6 +119,19 @@ struct T32Layout {
     std::vector<int> col_n, mb, boff, el_src;
 };
 
+// Layout of the fixed-point FP64 M2L (m2l_fx.cu): the kept locals as columns in
+// groups of 4, group g's image elements [first[g], first[g + 1]) at 4 m + j for
+// the multipoles m that reach its lowest order (rounded up to even).  el: D
+// entry | |n + m| << 9 | (|m| - s) << 13 | (a_m + b_n + 64) << 17, -1 for zero;
+// am: a_m 256 + |m| - s; col: n | |n| << 9 | b_n << 13.  owner: the warp that
+// sums a group, at most cap groups to each of the four.
+constexpr int kFxMaxGroups = 16;
+struct FxLayout {
+    int s = -1, p = -1, h = -1, n_lo = -1, nM = 0, nq = 0, ncol = 0, groups = 0, E = 0, cap = 0;
+    int bits = 0, products = 0;   // fraction bits of a multipole, terms (n, m) of a pair
+    std::vector<int> el, first, am, col, owner;
+};
+
 // threads of the M2L blocks (the per-thread term lists are built for it)
 constexpr int kM2LThreadsShared = 128;
 
@@ -288,6 +301,12 @@ struct fmm_tree {
     fmm::T32Layout m32_lay;
     int m32_img_p = -1;
     DevBuf b_m32_el, b_m32_img;
+    // fixed-point FP64 M2L on the same plan: layout, operator images and their
+    // exponents, exponents of the cells and targets, the targets' sums
+    fmm::FxLayout fx_lay;
+    int fx_img_p = -1;
+    DevBuf b_fx_el, b_fx_img, b_fx_ekey, b_fx_em, b_fx_et, b_fx_acc;
+    bool soft_alloc = false;               // a failing allocation is FMM_EBUDGET, the handle keeps its state
 
     // symmetric FP64 P2P (p2p_variant 2), derived from the lists: per list
     // entry its mirror entry (-1: none) and, for an entry (A, B) with B > A,
@@ -424,6 +443,13 @@ void launch_tc_reduce(fmm_tree *t, int Np, int ncol, const int32_t *col_n, int n
 bool m32_usable(fmm_tree *t, int s, int p, int harmonic, int n_lo);
 fmm_status m32_prepare(fmm_tree *t, int p);
 fmm_status run_m2l32_tile(fmm_tree *t, int p, const float *M, int ldM, const DevTables &tb, float *L);
+// m2l_fx.cu: the FP64 form's M2L in fixed point over the plan.  Usable on lists
+// long enough to pay for the plan, on handles without a memory budget (fills
+// t->fx_lay); prepare builds the plan, images and buffers
+bool fx_usable(fmm_tree *t, int s, int p, int harmonic, int n_lo);
+fmm_status fx_prepare(fmm_tree *t, int p);
+fmm_status run_fx_exps(fmm_tree *t, const double *M, const DevTables &tb);
+fmm_status run_m2l_fx(fmm_tree *t, const DevTables &tb, double *L);
 // api.cu: the handle's side stream and join events, created on first use
 fmm_status side_stream(fmm_tree *t);
 // api.cu: the compute of an evaluate whose lists are current (no host sync)

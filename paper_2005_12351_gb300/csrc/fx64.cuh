@@ -30,6 +30,14 @@ __device__ __forceinline__ s64 madw(int a, int b, s64 c)
     asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
     return d;
 }
+// the same as a product and an addition, which the compiler fuses: a chain of
+// these into one sum costs 4.6 clocks each, of madw 5.4 (a move beside it)
+__device__ __forceinline__ s64 madp(int a, int b, s64 c)
+{
+    s64 d;
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
+    return d + c;
+}
 __device__ __forceinline__ u64 madu(uint32_t a, uint32_t b, u64 c)
 {
     u64 d;

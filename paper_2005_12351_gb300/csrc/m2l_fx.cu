@@ -1,0 +1,596 @@
+// m2l_fx.cu -- the FP64 form's M2L in 64-bit fixed point over the target tiles
+// of the plan (m2l_tc.cu).
+//
+// The per-cell FP64 kernel (k_m2l) is bound by the FP64 pipe: one warp
+// instruction per 64 clocks and scheduler, 812 multiply-adds a pair at p = 6,
+// 5.0 of its 5.6 ms at 1M dipoles.  Three 32 x 32 + 64 bit integer
+// multiply-adds (5.6 clocks each) carry the same product to 57 bits, provided
+// both factors have a common scale per sum.  The plan gives it: the 128
+// targets of a tile share the operator of a row's key, so the operator is
+// scaled once per key, a multipole once per cell, and the sums of a target in
+// a unit that holds all of its list.
+//
+// Scaling (powers of two throughout, so exact).  With h_t, h_s the half sides,
+//   M'_m = M_m h_s^(s-|m|) 2^(a_m),   a_m = round(log2 m!) - (|m| - s),
+//   T'_nm = D_{n+m} (level factors) 2^(-a_m - b_n),   b_n = round(log2 n!),
+//   L_n = h_t^(-|n|-1-s) 2^(b_n) sum_pairs sum_m T'_nm M'_m.
+// a_m and b_n level the magnitudes over the orders: for particles spread over
+// a cell, or bunched in its corner, 1 <= p <= 12, max |M'| times the largest
+// row sum of |T'| is 1.2 to 7 times the sum of the absolute values of the
+// terms of a first-order component, so that 57 bits of the product of those
+// bounds are more than the 53 of each FP64 rounding.
+//   per cell  e_s:  |M'| < 2^e_s;  M' = (Mh 2^26 + Ml) 2^(e_s - B), B = 57 (56 for nM > 126)
+//   per key   e_k:  sum_m |T'_nm| < 2^e_k for every n; T' likewise at 2^(e_k - 57)
+//   per target e_t: sum over its list of 2^(e_s + e_k) <= 2^e_t
+// A row's sum A1 + A0 / 2^26, A1 = sum Th Mh, A0 = sum (Th Ml + Tl Mh), stays
+// below 2^(B + 5) (the row sums of T' bound it) and A0 below 2^63 (nM 2^(B - 1)
+// and 2^56); it is shifted right by e_t - e_s - e_k into a 64-bit sum that
+// cannot pass 2^(B + 5) either.
+// Integer sums do not depend on their order: the chunks add theirs with
+// 64-bit reductions to one array, and a target's result does not depend on
+// the other targets of its tile.
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+
+#include "fmm_internal.cuh"
+#include "fx64.cuh"
+#include "umma.cuh"
+
+namespace fmm {
+
+using namespace umma;
+using namespace fx;
+
+namespace {
+
+constexpr int kFxThreads = 128;
+// rows of a block: a part of a chunk (1M dipoles, p = 6: 1.84 ms with 8 rows,
+// 1.86 with 16, 1.91 with 32; 200k: 0.25, 0.275, 0.33: the last blocks' wait)
+constexpr int kFxRows = 8;
+constexpr int kFxMaxNM = 253;        // A0 stays below 2^63
+constexpr int kFxSmemMax = 216 * 1024;
+constexpr int kFxPad = 33;           // 16-byte pieces per line of 32 targets: staging by rows without conflicts
+constexpr int kZeroExp = -(1 << 20); // exponent of an all-zero row
+constexpr int kBadExp = 1 << 24;     // a row that holds an infinity or a NaN
+
+// What turns a target's sums into its row of L
+struct FxOut {
+    const int32_t *tile_tgt, *col, *level, *sys, *rn;    // rn: full index of each stored component
+    const int *e_side;
+    double *L;
+    int s, ncol, nL, nLh, unit;
+};
+
+struct FxArgs {
+    const int32_t *chunk_rb, *chunk_re, *row_key, *slot;
+    const uint32_t *tile_chunk;          // [tiles + 1] first chunk of each tile
+    const int4 *M;                       // [cells][nq]: two limb pairs (h, l, h, l) each
+    const int *eM, *ekey, *etgt;
+    const int2 *img;                     // [keys][E] limb pairs
+    u64 *acc;                            // [tile][4][ncolp][32]
+    unsigned *arrive;                    // [tile][4] blocks done, from 0
+    FxOut out;
+    int parts, tiles, nq, E, ncolp;      // parts: blocks of kFxRows rows a chunk can take
+    // the column groups (4 columns each) dealt to the four warps: image offset
+    // (elements), pairs of multipoles, first column
+    int ng[4];
+    int g_off[4][kFxMaxGroups], g_mq[4][kFxMaxGroups], g_col[4][kFxMaxGroups];
+};
+
+struct Sum {
+    s64 a1, a0;
+};
+
+__device__ __forceinline__ void mac(Sum &s, int th, int tl, int mh, int ml)
+{
+    s.a1 = madp(th, mh, s.a1);
+    s.a0 = madp(th, ml, s.a0);
+    s.a0 = madp(tl, mh, s.a0);
+}
+
+// The sums of 32 targets back to FP64 rows, by the block that arrives last: a
+// column's sums read side by side and turned in shared memory.
+__device__ __noinline__ void fx_finish(const FxArgs &a, int slot0, s64 *fs)
+{
+    __shared__ int s_pos[kMaxTot];                   // full index -> column
+    const FxOut &o = a.out;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int k = threadIdx.x; k < o.nL; k += kFxThreads) s_pos[k] = -1;
+    const u64 *acc = a.acc + (size_t)slot0 * a.ncolp;
+    for (int k = threadIdx.x; k < a.ncolp * 32; k += kFxThreads)
+        fs[(k >> 5) * kFxPad + (k & 31)] = (s64)__ldcg(acc + k);
+    __syncthreads();
+    for (int k = threadIdx.x; k < o.ncol; k += kFxThreads) s_pos[o.col[k] & 511] = k;
+    __syncthreads();
+    for (int t = w; t < 32; t += 4) {
+        const int c = o.tile_tgt[slot0 + t];
+        if (c < 0) continue;
+        const int et = a.etgt[slot0 + t], hl = o.e_side[o.sys[c]] - o.level[c] - 1;
+        for (int r = lane; r < o.nLh; r += 32) {
+            const int k = s_pos[o.rn[r]];
+            double v = 0.0;
+            if (k >= 0) {
+                const int cv = o.col[k], nn = (cv >> 9) & 15, bn = cv >> 13;
+                v = ldexp((double)fs[k * kFxPad + t], et - o.unit + bn - (nn + 1 + o.s) * hl);
+                if (et >= kBadExp / 2) v = __longlong_as_double(0x7ff8000000000000ll);
+            }
+            o.L[(size_t)c * o.nLh + r] = v;
+        }
+    }
+}
+
+// One block per (part of a chunk, 32 targets of the tile): lane = target, the
+// four warps share the staged multipoles and divide the columns.  Shared
+// memory: [nq][33] 16-byte multipole pieces and E limb pairs of the operator of
+// one row; the other blocks of the SM compute while one waits for its row.  Bound
+// by the integer pipes, 3 multiply-adds a product: M2L phase (this kernel; the
+// per-cell k_m2l before) 5.59 -> 1.69 ms at 1M dipoles, p = 6 (32 targets 87 %
+// full); 3.30 -> 1.54 ms at 262k Plummer, p = 8 (47 % full); 0.57 -> 0.23 ms at
+// 200k charges and dipoles, p = 6; 125k dipoles, p = 6: 0.68 -> 0.28 ms.  (Two stages with the next
+// row's copies in flight halve the blocks an SM holds: 1M dipoles, p = 6, 1.96
+// instead of 1.86 ms; 262k Plummer, p = 8, 1.99 instead of 1.67.)
+template <int NG>
+__global__ void __launch_bounds__(kFxThreads) k_m2l_fx(const __grid_constant__ FxArgs a)
+{
+    extern __shared__ int4 sm4[];
+    __shared__ int s_src[kFxRows][32], s_sh[kFxRows][32], s_key[kFxRows], s_act[kFxRows], s_tile, s_last;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int qt = blockIdx.x & 3, chunk = (blockIdx.x >> 2) / a.parts, part = (blockIdx.x >> 2) - chunk * a.parts;
+    const int rb = a.chunk_rb[chunk] + part * kFxRows, n = min(a.chunk_re[chunk] - rb, kFxRows);
+    for (int i = tid; i < a.tiles; i += kFxThreads)
+        if ((int)a.tile_chunk[i] <= chunk && chunk < (int)a.tile_chunk[i + 1]) s_tile = i;
+    __syncthreads();
+    const int slot0 = s_tile * 128 + 32 * qt, et = a.etgt[slot0 + lane];
+    int any = 0;
+    for (int r = w; r < n; r += 4) {
+        const int src = a.slot[(size_t)(rb + r) * 128 + 32 * qt + lane], key = a.row_key[rb + r];
+        s_src[r][lane] = src;
+        // 0..62: a pair 2^62 below its target's unit adds nothing
+        s_sh[r][lane] = src >= 0 ? min(max(et - a.eM[src] - a.ekey[key], 0), 62) : 0;
+        const int act = __any_sync(0xffffffffu, src >= 0);
+        any |= act;
+        if (lane == 0) {
+            s_key[r] = key;
+            s_act[r] = act;
+        }
+    }
+    any = __syncthreads_or(any);
+    int4 *Ts = sm4 + a.nq * kFxPad;
+    auto stage = [&](int r) {
+        for (int k = tid, t = tid / a.nq, q = tid - t * a.nq; k < 32 * a.nq; k += kFxThreads) {
+            const int src = s_src[r][t];
+            cp_async16(smem_u32(sm4 + q * kFxPad + t), a.M + (size_t)max(src, 0) * a.nq + q, src < 0 ? 0 : 16);
+            q += kFxThreads;
+            while (q >= a.nq) {
+                q -= a.nq;
+                ++t;
+            }
+        }
+        const int4 *ti = (const int4 *)(a.img + (size_t)s_key[r] * a.E);
+        for (int e = tid; e < (a.E >> 1); e += kFxThreads) cp_async16(smem_u32(Ts + e), ti + e, 16);
+        cp_async_commit();
+    };
+    s64 P[NG][4];
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) P[g][c] = 0;
+    const int ng = any ? a.ng[w] : 0;
+    for (int r = 0; r < n; ++r) {
+        if (!s_act[r]) continue;                     // no pair of these 32 targets
+        stage(r);
+        cp_async_wait<0>();
+        __syncthreads();
+        const int4 *Ms = sm4 + lane;
+        const int sh = s_sh[r][lane];
+        const s64 half = (1ll << sh) >> 1;
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+            if (g < ng) {
+                const int4 *T4 = Ts + (a.g_off[w][g] >> 1);
+                const int mq = a.g_mq[w][g];
+                Sum s[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) s[c] = {half, 1ll << 25};    // both shifts round
+#pragma unroll 4
+                for (int q = 0; q < mq; ++q) {
+                    const int4 m = Ms[q * kFxPad];
+                    const int4 t0 = T4[4 * q], t1 = T4[4 * q + 1], t2 = T4[4 * q + 2], t3 = T4[4 * q + 3];
+                    mac(s[0], t0.x, t0.y, m.x, m.y);
+                    mac(s[1], t0.z, t0.w, m.x, m.y);
+                    mac(s[2], t1.x, t1.y, m.x, m.y);
+                    mac(s[3], t1.z, t1.w, m.x, m.y);
+                    mac(s[0], t2.x, t2.y, m.z, m.w);
+                    mac(s[1], t2.z, t2.w, m.z, m.w);
+                    mac(s[2], t3.x, t3.y, m.z, m.w);
+                    mac(s[3], t3.z, t3.w, m.z, m.w);
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) P[g][c] += (s[c].a1 + (s[c].a0 >> 26)) >> sh;
+            }
+        }
+        __syncthreads();                             // before the next row is staged
+    }
+    u64 *acc = a.acc + (size_t)slot0 * a.ncolp + lane;
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+        if (g < ng)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) atomicAdd(acc + (size_t)(a.g_col[w][g] + c) * 32, (u64)P[g][c]);
+    __threadfence();                                 // the sums are added before the block counts as done
+    __syncthreads();
+    if (tid == 0) {
+        const unsigned blocks = (a.tile_chunk[s_tile + 1] - a.tile_chunk[s_tile]) * a.parts;
+        s_last = atomicAdd(a.arrive + s_tile * 4 + qt, 1u) + 1u == blocks;
+        __threadfence();
+    }
+    __syncthreads();
+    if (s_last) fx_finish(a, slot0, (s64 *)sm4);
+}
+
+// The cells' multipoles as limbs, then the exponents of the plan's targets, in
+// one cooperative launch (every block is resident, so the barrier between the
+// two ends; it is bounded all the same).  One warp per cell: the row folded as
+// in k_fold_m, its exponent, the limbs.  One warp per target: e_t from its list.
+__global__ void __launch_bounds__(128)
+k_fx_exps(const double *M, int64_t nc, DevTables tb, const int32_t *am, const int32_t *level, const int32_t *sys,
+          const int *e_side, int nq, int bits, int2 *Mx, int *eM, int slots, const int32_t *tile_tgt,
+          const int32_t *off, const int32_t *src, const int32_t *didx, const int *ekey, int *etgt, unsigned *bar)
+{
+    extern __shared__ double fsm[];
+    __shared__ int s_ok;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double *v = fsm + w * tb.nM;
+    for (int64_t c = blockIdx.x * 4ll + w; c < nc; c += gridDim.x * 4ll) {
+        for (int m = lane; m < tb.nM; m += 32) v[m] = M[c * tb.nM + m];
+        __syncwarp();
+        for (int l = 0; l < tb.h_fold_lev; ++l) {
+            for (int q = tb.h_fold_off[l] + lane; q < tb.h_fold_off[l + 1]; q += 32) {
+                const int i = tb.h_fold[3 * q], a = tb.h_fold[3 * q + 1], b = tb.h_fold[3 * q + 2];
+                double x = v[i];
+                if (a >= 0) x -= v[a];
+                if (b >= 0) x -= v[b];
+                v[i] = x;
+            }
+            __syncwarp();
+        }
+        const int hl = e_side[sys[c]] - level[c] - 1;        // log2 of the half side
+        int e = kZeroExp;
+        for (int r = lane; r < tb.nMh; r += 32) {
+            const int k = am[r], wr = (k >> 8) - (k & 255) * hl;
+            const u64 b = (u64)__double_as_longlong(v[tb.h_rm[r]]) & 0x7fffffffffffffffull;
+            if (b >= 0x7ff0000000000000ull) e = kBadExp;
+            // a value within 2^-29 of the next power of two would round to it: Mh < 2^31
+            else if (b) e = max(e, (int)((b + (1ull << 23)) >> 52) - 1022 + wr);
+        }
+        e = __reduce_max_sync(0xffffffffu, e);
+        if (lane == 0) eM[c] = e;
+        for (int r = lane; r < 2 * nq; r += 32) {
+            s64 x = 0;
+            if (r < tb.nMh && e != kBadExp) {
+                const int k = am[r], wr = (k >> 8) - (k & 255) * hl;
+                x = fix64(v[tb.h_rm[r]], wr + bits - e);
+            }
+            const int h = (int)((x + (1ll << 25)) >> 26);
+            Mx[c * 2 * nq + r] = make_int2(h, (int)(x - ((s64)h << 26)));
+        }
+        __syncwarp();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1u);
+        const volatile unsigned *b = bar;
+        const long long t0 = clock64();
+        while (*b < gridDim.x && clock64() - t0 < (1ll << 31)) __nanosleep(32);
+        s_ok = *b >= gridDim.x;
+        __threadfence();
+    }
+    __syncthreads();
+    for (int q = blockIdx.x * 4 + w; q < slots; q += gridDim.x * 4) {
+        const int c = tile_tgt[q];
+        int e = kZeroExp;
+        if (c >= 0 && s_ok) {
+            const int b = off[c], en = off[c + 1];
+            for (int k = b + lane; k < en; k += 32) e = max(e, __ldcg(eM + src[k]) + ekey[didx[k]]);
+            e = __reduce_max_sync(0xffffffffu, e);
+            float f = 0.0f;
+            for (int k = b + lane; k < en; k += 32)
+                f += exp2f((float)max(__ldcg(eM + src[k]) + ekey[didx[k]] - e, -100));
+            for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+            e += ilogbf(f * 1.01f) + 1;
+        }
+        if (lane == 0) etgt[q] = s_ok ? e : kBadExp;          // a wait that gave up shows as NaN
+    }
+}
+
+// Operator images, a block per key (17 us at 346 keys, p = 6): T'_nm of every element, the key's exponent
+// from the largest row sum, the limbs.
+__device__ __forceinline__ double fx_element(int el, const double *D, int esc, int dl)
+{
+    if (el < 0) return 0.0;
+    const int k = el & 511, nm = (el >> 9) & 15, msh = (el >> 13) & 15, sh = (el >> 17) - 64;
+    return ldexp(D[k], (nm + 1) * esc + dl * msh - sh);
+}
+
+__global__ void __launch_bounds__(128)
+k_fx_images(const uint64_t *dkeys, const double *D, int nD, int E, int ngroups, const int32_t *g_first,
+            const int32_t *el, int2 *img, int *ekey)
+{
+    __shared__ double s_max[4];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t r = blockIdx.x;
+    const uint64_t key = dkeys[r];
+    const int gap = (int)((key >> 52) & 31), tfiner = (int)((key >> 51) & 1);
+    const int esc = tfiner ? 0 : gap, dl = tfiner ? gap : -gap;
+    const double *Dr = D + r * nD;
+    double big = 0.0;
+    for (int g = w; g < ngroups; g += 4) {
+        double v = 0.0;                              // lanes of equal (lane & 3) share a column
+        for (int e = g_first[g] + lane; e < g_first[g + 1]; e += 32) v += fabs(fx_element(el[e], Dr, esc, dl));
+        v += __shfl_xor_sync(0xffffffffu, v, 4);
+        v += __shfl_xor_sync(0xffffffffu, v, 8);
+        v += __shfl_xor_sync(0xffffffffu, v, 16);
+        big = fmax(big, v);
+    }
+    big = fmax(big, __shfl_xor_sync(0xffffffffu, big, 1));
+    big = fmax(big, __shfl_xor_sync(0xffffffffu, big, 2));
+    if (lane == 0) s_max[w] = big;
+    __syncthreads();
+    big = fmax(fmax(s_max[0], s_max[1]), fmax(s_max[2], s_max[3]));
+    // row sums below 2^ek less a margin for their own rounding: Th < 2^31
+    const int ek = big > 0.0 ? ilogb(big * 1.004) + 1 : 0;
+    if (threadIdx.x == 0) ekey[r] = ek;
+    for (int e = threadIdx.x; e < E; e += blockDim.x) {
+        const s64 x = __double2ll_rn(ldexp(fx_element(el[e], Dr, esc, dl), 57 - ek));
+        const int h = (int)((x + (1ll << 25)) >> 26);
+        img[r * E + e] = make_int2(h, (int)(x - ((s64)h << 26)));
+    }
+}
+
+int log2_factorial(const MultiIndex &I, int k)
+{
+    double v = 1.0;
+    for (int q : {I.nx[k], I.ny[k], I.nz[k]})
+        for (int j = 2; j <= q; ++j) v *= j;
+    return (int)std::lround(std::log2(v));
+}
+
+void build_layout_fx(FxLayout &Ly, int s, int p, int h, int n_lo)
+{
+    const MultiIndex &I = multi_index();
+    auto shell = [&](int k) { return I.nx[k] + I.ny[k] + I.nz[k]; };
+    std::vector<int> ms, ns;
+    for (int k = ntot(s - 1); k < ntot(p + s); ++k)
+        if (!h || I.nz[k] <= 1) ms.push_back(k);
+    for (int n = 0; n < ntot(p); ++n)
+        if (shell(n) >= n_lo && (!h || I.nz[n] <= 1)) ns.push_back(n);
+    Ly.s = s;
+    Ly.p = p;
+    Ly.h = h;
+    Ly.n_lo = n_lo;
+    Ly.nM = (int)ms.size();
+    Ly.nq = (Ly.nM + 1) / 2;
+    Ly.bits = Ly.nM <= 126 ? 57 : 56;
+    Ly.ncol = (int)ns.size();
+    Ly.groups = (Ly.ncol + 3) / 4;
+    auto a_of = [&](int gm) { return log2_factorial(I, gm) - (shell(gm) - s); };
+    Ly.am.clear();
+    for (int gm : ms) Ly.am.push_back(a_of(gm) * 256 + (shell(gm) - s));
+    Ly.col.clear();
+    for (int n : ns) Ly.col.push_back(n | shell(n) << 9 | log2_factorial(I, n) << 13);
+    Ly.first.assign(1, 0);
+    Ly.el.clear();
+    Ly.products = 0;
+    for (int g = 0; g < Ly.groups; ++g) {
+        const int reach = p + s - shell(ns[4 * g]);      // graded: the group's lowest order comes first
+        int cnt = 0;
+        while (cnt < Ly.nM && shell(ms[cnt]) <= reach) ++cnt;
+        cnt = (cnt + 1) & ~1;
+        for (int m = 0; m < cnt; ++m)
+            for (int j = 0; j < 4; ++j) {
+                const int c = 4 * g + j;
+                int v = -1;
+                if (c < Ly.ncol && m < Ly.nM) {
+                    const int n = ns[c], gm = ms[m], tot = shell(n) + shell(gm);
+                    if (tot <= p + s) {
+                        const int d = I(I.nx[n] + I.nx[gm], I.ny[n] + I.ny[gm], I.nz[n] + I.nz[gm]);
+                        const int sh = a_of(gm) + log2_factorial(I, n);
+                        // the shift may be negative: kept in the upper bits with the sign
+                        // bit clear (offset by 64)
+                        ++Ly.products;
+                        v = d | tot << 9 | (shell(gm) - s) << 13 | (sh + 64) << 17;
+                    }
+                }
+                Ly.el.push_back(v);
+            }
+        Ly.first.push_back((int)Ly.el.size());
+    }
+    Ly.E = (int)Ly.el.size();
+    // columns to warps: the longest group to the least loaded warp, at most cap
+    // groups to a warp; the smallest cap within a tenth of the best balance
+    Ly.cap = 0;
+    int best = 0;
+    for (int cap : {16, 12, 8, 6, 4}) {
+        if (4 * cap < Ly.groups) break;
+        int load[4] = {0, 0, 0, 0}, cnt[4] = {0, 0, 0, 0};
+        std::vector<int> owner(Ly.groups);
+        for (int g = 0; g < Ly.groups; ++g) {            // lengths fall with g
+            int w = -1;
+            for (int k = 0; k < 4; ++k)
+                if (cnt[k] < cap && (w < 0 || load[k] < load[w])) w = k;
+            owner[g] = w;
+            load[w] += Ly.first[g + 1] - Ly.first[g];
+            ++cnt[w];
+        }
+        const int span = std::max(std::max(load[0], load[1]), std::max(load[2], load[3]));
+        if (!Ly.cap) best = span;
+        if (!Ly.cap || 10 * span <= 11 * best) {
+            Ly.cap = cap;
+            Ly.owner = owner;
+        }
+    }
+}
+
+inline size_t fx_smem(const FxLayout &Ly) { return 16 * (size_t)Ly.nq * kFxPad + 8 * (size_t)Ly.E; }
+
+inline unsigned gridn(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
+
+}  // namespace
+
+// The line between this form and the per-cell k_m2l: the list's products a
+// system.  The plan costs 40 to 100 us on new lists, and small or strongly
+// graded sets fill the 32 lanes badly.  Evaluates with new lists, per cell ->
+// here: 1 6 (source order, p) uniform, 419k pairs (3.4e8 products) 2.00 -> 1.60
+// ms; 1 6 Plummer, 174k pairs (1.4e8) 1.82 -> 1.84; 2 8 Plummer, 78k pairs
+// (2.0e8) 2.22 -> 2.33 and 172k pairs (4.3e8) 3.10 -> 2.86; 0 3 uniform, 419k
+// pairs (0.4e8) no difference.  Handles with a memory budget keep the per-cell
+// kernel, so that a served request's bits do not depend on its slot's memory.
+constexpr double kFxMinWork = 2.0e8;
+
+bool fx_usable(fmm_tree *t, int s, int p, int harmonic, int n_lo)
+{
+    if (!t->m2l_tiled || t->budget) return false;
+    FxLayout &Ly = t->fx_lay;
+    const int h = harmonic ? 1 : 0;
+    if (Ly.s != s || Ly.p != p || Ly.h != h || Ly.n_lo != n_lo) {
+        build_layout_fx(Ly, s, p, h, n_lo);
+        t->fx_img_p = -1;                     // images and maps of the old layout
+    }
+    const double nsys = (double)std::max<int64_t>(1, (int64_t)t->sys_off.size() - 1);
+    return (double)t->n_m2l * Ly.products >= kFxMinWork * nsys && Ly.cap > 0 && Ly.nM <= kFxMaxNM &&
+           fx_smem(Ly) <= (size_t)kFxSmemMax;
+}
+
+fmm_status fx_prepare(fmm_tree *t, int p)
+{
+    cudaStream_t st = t->stream;
+    const FxLayout &Ly = t->fx_lay;
+    if (!t->tc_plan) FMM_TRY(tc_build_plan(t));
+    if (t->tc_chunks == 0) return FMM_OK;
+    const size_t slots = (size_t)t->tc_tiles * 128;
+    if (t->fx_img_p != p) {
+        const size_t n1 = (size_t)Ly.E, n2 = Ly.first.size(), n3 = Ly.am.size(), n4 = Ly.col.size();
+        FMM_TRY(ensure(t, t->b_fx_el, 4 * (n1 + n2 + n3 + n4)));
+        int32_t *d = (int32_t *)t->b_fx_el.ptr;
+        auto up = [&](const std::vector<int> &v) {
+            const cudaError_t e = cudaMemcpyAsync(d, v.data(), 4 * v.size(), cudaMemcpyHostToDevice, st);
+            d += v.size();
+            return cuda_check(t, e, "upload");
+        };
+        FMM_TRY(up(Ly.el));
+        FMM_TRY(up(Ly.first));
+        FMM_TRY(up(Ly.am));
+        FMM_TRY(up(Ly.col));
+        FMM_TRY(ensure(t, t->b_fx_img, 8 * (size_t)t->n_doff * Ly.E));
+        FMM_TRY(ensure(t, t->b_fx_ekey, 4 * (size_t)t->n_doff));
+        d = (int32_t *)t->b_fx_el.ptr;
+        k_fx_images<<<(unsigned)t->n_doff, 128, 0, st>>>(
+            (const uint64_t *)t->b_dkeys.ptr, (const double *)t->b_D.ptr, ntot(p + t->s), Ly.E, Ly.groups, d + n1, d,
+            (int2 *)t->b_fx_img.ptr, (int *)t->b_fx_ekey.ptr);
+        ++t->launches;
+        t->fx_img_p = p;
+    }
+    FMM_TRY(ensure(t, t->b_fx_em, 4 * (size_t)t->ncells));
+    FMM_TRY(ensure(t, t->b_fx_et, 4 * slots));
+    // the sums, the blocks done per 32 targets, the barrier
+    FMM_TRY(ensure(t, t->b_fx_acc, 32 * slots * Ly.groups + slots / 8 + 16));
+    // the limbs take the place of the folded multipoles
+    return ensure(t, t->b_Mh, 16 * (size_t)t->ncells * Ly.nq);
+}
+
+fmm_status run_fx_exps(fmm_tree *t, const double *M, const DevTables &tb)
+{
+    cudaStream_t st = t->stream;
+    const FxLayout &Ly = t->fx_lay;
+    if (Ly.nM != tb.nMh || (Ly.h == 1) != (tb.harmonic == 1)) {
+        t->err = "fixed-point M2L: layout and tables disagree";
+        return FMM_EINVAL;                   // not reachable: both follow the handle's flag
+    }
+    if (t->tc_chunks == 0) return FMM_OK;
+    int slots = (int)t->tc_tiles * 128, per_sm = 0;
+    const size_t acc = 32 * (size_t)slots * Ly.groups, smem = 32 * (size_t)tb.nM;
+    FMM_TRY(cuda_check(t, cudaMemsetAsync(t->b_fx_acc.ptr, 0, acc + slots / 8 + 16, st), "memset"));
+    FMM_TRY(cuda_check(t, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fx_exps, 128, smem), "occupancy"));
+    const int64_t grid = std::min<int64_t>((std::max<int64_t>(t->ncells, slots) + 3) / 4,
+                                           (int64_t)std::max(per_sm, 1) * sm_count());
+    int64_t nc = t->ncells;
+    DevTables tv = tb;
+    const int32_t *am = (const int32_t *)t->b_fx_el.ptr + Ly.E + Ly.first.size();
+    const int32_t *level = (const int32_t *)t->b_level.ptr, *sys = (const int32_t *)t->b_sys.ptr;
+    const int *es = t->sys_eside_dev();
+    int nq = Ly.nq, bits = Ly.bits;
+    int2 *Mx = (int2 *)t->b_Mh.ptr;
+    int *eM = (int *)t->b_fx_em.ptr, *et = (int *)t->b_fx_et.ptr;
+    const int32_t *tgt = (const int32_t *)t->b_tc_tgt.ptr, *off = (const int32_t *)t->b_m2l_off.ptr,
+                  *src = (const int32_t *)t->b_m2l_src.ptr, *didx = (const int32_t *)t->b_m2l_didx.ptr;
+    const int *ekey = (const int *)t->b_fx_ekey.ptr;
+    unsigned *bar = (unsigned *)((char *)t->b_fx_acc.ptr + acc + slots / 8);
+    void *args[] = {&M, &nc, &tv, &am, &level, &sys, &es, &nq, &bits, &Mx, &eM, &slots, &tgt, &off, &src, &didx,
+                    &ekey, &et, &bar};
+    ++t->launches;
+    return cuda_check(t, cudaLaunchCooperativeKernel((const void *)k_fx_exps, dim3((unsigned)grid), dim3(128), args,
+                                                     smem, st), "fixed-point multipoles");
+}
+
+fmm_status run_m2l_fx(fmm_tree *t, const DevTables &tb, double *L)
+{
+    cudaStream_t st = t->stream;
+    const FxLayout &Ly = t->fx_lay;
+    if (t->tc_chunks == 0) return FMM_OK;
+    const int slots = (int)t->tc_tiles * 128, ncolp = 4 * Ly.groups;
+    FxArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.chunk_rb = (const int32_t *)t->b_tc_crb.ptr;
+    a.chunk_re = (const int32_t *)t->b_tc_cre.ptr;
+    a.row_key = (const int32_t *)t->b_tc_rowkey.ptr;
+    a.slot = (const int32_t *)t->b_tc_slot.ptr;
+    a.tile_chunk = (const uint32_t *)t->b_tc_coff.ptr;
+    a.M = (const int4 *)t->b_Mh.ptr;
+    a.eM = (const int *)t->b_fx_em.ptr;
+    a.ekey = (const int *)t->b_fx_ekey.ptr;
+    a.etgt = (const int *)t->b_fx_et.ptr;
+    a.img = (const int2 *)t->b_fx_img.ptr;
+    a.acc = (u64 *)t->b_fx_acc.ptr;
+    a.arrive = (unsigned *)(a.acc + (size_t)slots * ncolp);
+    a.out.tile_tgt = (const int32_t *)t->b_tc_tgt.ptr;
+    a.out.col = (const int32_t *)t->b_fx_el.ptr + Ly.E + Ly.first.size() + Ly.am.size();
+    a.out.level = (const int32_t *)t->b_level.ptr;
+    a.out.sys = (const int32_t *)t->b_sys.ptr;
+    a.out.rn = tb.h_rn;
+    a.out.e_side = t->sys_eside_dev();
+    a.out.L = L;
+    a.out.s = t->s;
+    a.out.ncol = Ly.ncol;
+    a.out.nL = tb.nL;
+    a.out.nLh = tb.nLh;
+    a.out.unit = Ly.bits + 5;
+    a.tiles = (int)t->tc_tiles;
+    a.parts = (t->tc_G + kFxRows - 1) / kFxRows;
+    a.nq = Ly.nq;
+    a.E = Ly.E;
+    a.ncolp = ncolp;
+    for (int g = 0; g < Ly.groups; ++g) {
+        const int w = Ly.owner[g], k = a.ng[w]++;
+        a.g_off[w][k] = Ly.first[g];
+        a.g_mq[w][k] = (Ly.first[g + 1] - Ly.first[g]) / 8;
+        a.g_col[w][k] = 4 * g;
+    }
+    const size_t smem = std::max(fx_smem(Ly), 32 * (size_t)Ly.groups * kFxPad);   // the last block's turn
+    auto go = [&](auto kern) {
+        allow_max_dynamic_smem(kern);
+        kern<<<(unsigned)(4 * t->tc_chunks * a.parts), kFxThreads, smem, st>>>(a);
+    };
+    switch (Ly.cap) {
+    case 4: go(k_m2l_fx<4>); break;
+    case 6: go(k_m2l_fx<6>); break;
+    case 8: go(k_m2l_fx<8>); break;
+    case 12: go(k_m2l_fx<12>); break;
+    default: go(k_m2l_fx<16>); break;
+    }
+    ++t->launches;
+    return cuda_check(t, cudaGetLastError(), "fixed-point M2L");
+}
+
+}  // namespace fmm

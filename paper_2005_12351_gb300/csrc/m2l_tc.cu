@@ -939,11 +939,13 @@ void tc_release(fmm_tree *t)
     for (DevBuf *b : {&t->b_tc_keys, &t->b_tc_keys2, &t->b_tc_vals, &t->b_tc_vals2, &t->b_tc_hist,
                       &t->b_tc_scan, &t->b_tc_tgt, &t->b_tc_bits, &t->b_tc_wpre, &t->b_tc_rowkey,
                       &t->b_tc_crb, &t->b_tc_cre, &t->b_tc_slot, &t->b_tc_el, &t->b_tc_img, &t->b_tc_part,
-                      &t->b_m32_el, &t->b_m32_img})
+                      &t->b_m32_el, &t->b_m32_img, &t->b_fx_el, &t->b_fx_img, &t->b_fx_ekey, &t->b_fx_em, &t->b_fx_et,
+                      &t->b_fx_acc})
         release(t, *b);
     t->tc_plan = false;
     t->tc_img_p = -1;
     t->m32_img_p = -1;
+    t->fx_img_p = -1;
     t->tc_T = t->tc_tiles = t->tc_rows = t->tc_chunks = 0;
 }
 

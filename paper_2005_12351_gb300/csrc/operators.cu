@@ -772,6 +772,7 @@ fmm_status build_dtables(fmm_tree *t, int p, const DevTables &tb, const int32_t 
         t->d32_p = -1;
         t->tc_img_p = -1;
         t->m32_img_p = -1;
+        t->fx_img_p = -1;
     }
     return FMM_OK;
 }
@@ -825,6 +826,20 @@ fmm_status run_expansions(fmm_tree *t, int p, int want_phi, int want_field)
     FMM_TRY(ensure(t, t->b_L, 8 * (size_t)nc * tb.nLh));
     FMM_TRY(ensure(t, t->b_phi, 8 * (size_t)n));
     FMM_TRY(ensure(t, t->b_E, 24 * (size_t)n));
+    // The M2L: in fixed point over the tiles of a plan (m2l_fx.cu) where the
+    // lists are long enough, else one block per target cell.  A plan that has to
+    // be built (new lists or p: two host syncs) is built on the handle's side
+    // stream while the upward pass runs; not while the stream is being captured
+    // (the graph's evaluate follows an ordinary one, which built it).
+    bool fx = t->n_m2l > 0 && fx_usable(t, s, p, tb.harmonic, tb.n_lo);
+    const bool stale = fx && (!t->tc_plan || t->fx_img_p != p);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (stale) FMM_TRY(cuda_check(t, cudaStreamIsCapturing(st, &cap), "capture status"));
+    const bool side = stale && cap == cudaStreamCaptureStatusNone;
+    if (side) {
+        FMM_TRY(side_stream(t));
+        FMM_TRY(cuda_check(t, cudaEventRecord(t->ev_lists, st), "event"));
+    }
     FMM_TRY(run_upward(t, tb, true));
     double *M = (double *)t->b_M.ptr, *L = (double *)t->b_L.ptr;
     const int32_t *leaves = (const int32_t *)t->b_leaves.ptr;
@@ -832,17 +847,42 @@ fmm_status run_expansions(fmm_tree *t, int p, int want_phi, int want_field)
     const double *centre = (const double *)t->b_centre.ptr;
     const double *px = (const double *)t->b_px.ptr, *py = (const double *)t->b_py.ptr,
                  *pz = (const double *)t->b_pz.ptr;
-    // M2L over the stored lists (harmonic: on the folded multipoles)
     cudaMemsetAsync(L, 0, 8 * (size_t)nc * tb.nLh, st);
+    if (fx) {
+        if (side) {
+            cudaStreamWaitEvent(t->side_st, t->ev_lists, 0);
+            t->stream = t->side_st;
+        }
+        t->soft_alloc = true;                 // no memory for the plan: the per-cell kernel needs none
+        const fmm_status ps = fx_prepare(t, p);
+        t->soft_alloc = false;
+        t->stream = st;
+        if (side) {
+            cudaEventRecord(t->ev_plan, t->side_st);
+            cudaStreamWaitEvent(st, t->ev_plan, 0);
+        }
+        if (ps == FMM_EBUDGET) {
+            tc_release(t);
+            t->err.clear();
+            fx = false;
+        } else {
+            FMM_TRY(ps);
+        }
+    }
+    // M2L over the stored lists (harmonic: on the folded multipoles)
     const double *Ms = M;
-    if (t->n_m2l > 0 && tb.harmonic) {
+    if (fx) {
+        FMM_TRY(run_fx_exps(t, M, tb));
+    } else if (t->n_m2l > 0 && tb.harmonic) {
         FMM_TRY(ensure(t, t->b_Mh, 8 * (size_t)nc * tb.nMh));
         launch_fold_m(st, M, tb.nM, nc, tb, (double *)t->b_Mh.ptr, tb.nMh);
         ++t->launches;
         Ms = (const double *)t->b_Mh.ptr;
     }
     record(t, 8);
-    if (t->n_m2l > 0) {
+    if (fx) {
+        FMM_TRY(run_m2l_fx(t, tb, L));
+    } else if (t->n_m2l > 0) {
         const int ldM = tb.nMh | 1, ldD = tb.nD | 1;
         size_t fixed = 8 * (size_t)tb.m2l_slots * kM2LThreads + 4 * (size_t)tb.m2l_T * kM2LThreads;
         size_t smem = fixed + 8 * (size_t)kM2LBatch * (ldM + ldD);
