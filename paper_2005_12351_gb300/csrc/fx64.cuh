@@ -30,8 +30,10 @@ __device__ __forceinline__ s64 madw(int a, int b, s64 c)
     asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
     return d;
 }
-// the same as a product and an addition, which the compiler fuses: a chain of
-// these into one sum costs 4.6 clocks each, of madw 5.4 (a move beside it)
+// The same as a product and an addition, which the compiler fuses: a chain of
+// them into one sum costs 4.6 clocks each where madw, whose sum it moves first,
+// costs 5.4.  Where several results meet in later additions it reorders those
+// and the form with the addend is the faster one (mulhi, the sums of p2p_fx.cu).
 __device__ __forceinline__ s64 madp(int a, int b, s64 c)
 {
     s64 d;
@@ -41,8 +43,8 @@ __device__ __forceinline__ s64 madp(int a, int b, s64 c)
 __device__ __forceinline__ u64 madu(uint32_t a, uint32_t b, u64 c)
 {
     u64 d;
-    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
-    return d;
+    asm("mul.wide.u32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
+    return d + c;
 }
 
 // shifts whose amount may pass the width (the result is then 0)
@@ -95,17 +97,17 @@ __device__ __forceinline__ s64 mulhi(I2 a, I2 b, s64 add = 0)
 // a b / 2^62, rounded: two more bits where the product is known to stay below 2^62
 __device__ __forceinline__ s64 mulhi_62(I2 a, I2 b)
 {
-    const s64 c = madw(a.h, b.l, madw(a.l, b.h, kHalfUlp / 4));
-    return (madw(a.h, b.h, 0) << 2) + (c >> 30);
+    const s64 c = madp(a.h, b.l, madp(a.l, b.h, kHalfUlp / 4));
+    return (madp(a.h, b.h, 0) << 2) + (c >> 30);
 }
 // add + (a0 b0 + a1 b1 + a2 b2) / 2^64, rounded; the halves' cross products must
 // sum below 2^63
 __device__ __forceinline__ s64 dot3hi(I2 a0, I2 b0, I2 a1, I2 b1, I2 a2, I2 b2, s64 add = 0)
 {
-    s64 c = madw(a0.h, b0.l, madw(a0.l, b0.h, kHalfUlp));
-    c = madw(a1.h, b1.l, madw(a1.l, b1.h, c));
-    c = madw(a2.h, b2.l, madw(a2.l, b2.h, c));
-    return madw(a2.h, b2.h, madw(a1.h, b1.h, madw(a0.h, b0.h, add + (s64)hi32(c))));
+    s64 c = madp(a0.h, b0.l, madp(a0.l, b0.h, kHalfUlp));
+    c = madp(a1.h, b1.l, madp(a1.l, b1.h, c));
+    c = madp(a2.h, b2.l, madp(a2.l, b2.h, c));
+    return madp(a2.h, b2.h, madp(a1.h, b1.h, madp(a0.h, b0.h, add + (s64)hi32(c))));
 }
 // add + a b / 2^64 modulo 2^64, for 0 <= a, b < 2^63 (error below two units, downward)
 __device__ __forceinline__ u64 mulhi_u(u64 a, u64 b, u64 add = 0)

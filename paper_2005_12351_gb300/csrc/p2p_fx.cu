@@ -5,12 +5,12 @@
 // shared), and GB300 issues one FP64 warp instruction per 64 clocks and
 // scheduler: 1,100 clocks or more per warp step.  The same dipole terms in
 // 64-bit fixed point (fx64.cuh) take about 60 integer multiply-adds and 130
-// other instructions, some 400 clocks.  Inside one leaf's near field every
+// other instructions, some 390 clocks.  Inside one leaf's near field every
 // quantity has a known range, so fixed point carries 55 to 60 significant bits
 // per factor: a pair term's error is at or below an FP64 evaluation's (about
 // ten roundings of 2^-53), and the sums over pairs are exact integers.
 // Measured, one million dipoles, field, 946 M interactions: 36.3 ms with the
-// symmetric FP64 kernel -> 11.1 ms; error against long double at or below the
+// symmetric FP64 kernel -> 11.0 ms; error against long double at or below the
 // FP64 kernels' (a set of 700: 1e-16 to 4e-16 against 2e-16 to 1e-15).
 // Bound: the integer multiply pipe (67 % busy) and the ALU (57 %) together; 16
 // or 32 warps per SM run alike.  Measured and not better: cross products by
@@ -165,14 +165,14 @@ __device__ __forceinline__ FxGeo fx_geo(s64 dx, s64 dy, s64 dz)
     g.x = bal(shl_any(dx, g.sh));
     g.y = bal(shl_any(dy, g.sh));
     g.z = bal(shl_any(dz, g.sh));
-    const s64 c = madw(g.z.h, g.z.l, madw(g.y.h, g.y.l, madw(g.x.h, g.x.l, kHalfUlp / 2)));
-    const u64 r2 = (u64)madw(g.z.h, g.z.h, madw(g.y.h, g.y.h, madw(g.x.h, g.x.h, c >> 31)));   // |R|^2 2^60
+    const s64 c = madp(g.z.h, g.z.l, madp(g.y.h, g.y.l, madp(g.x.h, g.x.l, kHalfUlp / 2)));
+    const u64 r2 = (u64)madp(g.z.h, g.z.h, madp(g.y.h, g.y.h, madp(g.x.h, g.x.h, c >> 31)));   // |R|^2 2^60
     const s64 en = (s64)mulhi_u(r2, madu(n0, n0, 0), -(1ull << 56));            // -e 2^56, |e| < 2^-19
     const int es = (int)(en >> 6);
-    const int e2 = hi32(madw(es, es, 0)) >> 12;                          // e^2 2^56
+    const int e2 = hi32(madp(es, es, 0)) >> 12;                          // e^2 2^56
     const s64 h = ((s64)(e2 - (e2 >> 2)) - en) << 7;                     // (e/2 + 3/8 e^2) 2^64
     const u64 u = madu(n0, (uint32_t)h, 0);
-    g.y1 = (u64)madw((int)n0, hi32(h), (s64)(((u64)n0 << 32) | (u >> 32)));
+    g.y1 = (u64)madp((int)n0, hi32(h), (s64)(((u64)n0 << 32) | (u >> 32)));
     g.y2 = mulhi_u(g.y1, g.y1);
     g.y3 = mulhi_u(g.y2, g.y1);
     return g;
@@ -214,7 +214,7 @@ __device__ __forceinline__ void fx_pair(const FxGeo &g, const int *r, bool dead,
         if (FIELD) {
             const I2 v1 = bal_biased(mulhi(bal_biased(srb), bal((s64)g.y2), kBias));   // (M.R) y^2 2^55
             // -3 (M.R) y^2 2^58: the factor -24
-            const s64 vb = madw(v1.l, -24, kBias);
+            const s64 vb = madp(v1.l, -24, kBias);
             const I2 v = {hi32(vb) + v1.h * -24, lo32(vb) ^ (int)0x80000000};
             const Fx4 f = fx_factor(g.y3, se);
             // (M - 3 (M.R) y^2 R) 2^56
