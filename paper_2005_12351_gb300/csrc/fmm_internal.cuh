@@ -62,6 +62,8 @@ struct OpTables {
     std::vector<int> l2l_off, l2l_k, l2l_q;
     // L2P gradient: for |k| <= p-1, L index of k + e_d (3 per k)
     std::vector<int> l2p_grad;
+    // and the k in the order of L2P's loops: |k| <= p, then |k| <= p - 1
+    std::vector<int> l2p_ord;
     // M2L: per-thread term lists (slot-major) and the partial-sum reduction map
     int m2l_threads = 0, m2l_T = 0, m2l_slots = 0;
     std::vector<uint32_t> m2l_desc;      // [T x threads]
@@ -141,7 +143,8 @@ struct DevTables {
     const int *p2m_terms;
     const int *m2m_off, *m2m_k, *m2m_q;
     const int *l2l_off, *l2l_k, *l2l_q;
-    const int *l2p_grad;
+    const int *l2p_grad, *l2p_ord;
+    const int *inv_fact;                 // 1/k! of every k, a double as two words
     const int *m2l_red_off, *m2l_red_src;
     const uint32_t *m2l_desc;
     int m2l_T, m2l_slots;
