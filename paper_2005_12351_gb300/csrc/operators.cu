@@ -376,9 +376,8 @@ __device__ __forceinline__ double inv_factorial(const DevTables &tb, int k)
 // once); the multipole m is then the sum over a of the terms m - a.  Per
 // particle 84 monomials (p = 6) of two products and nS sums of three
 // multiply-adds each, where the FP64 form issued 570 operations: upward pass
-// (with M2M) 1.69 -> 0.81 ms at 1M dipoles, p = 6; 0.50 -> 0.26 ms at 200k charges
-// and dipoles, p = 6; 2.22 -> 0.79 ms at 96 quadrupole systems,
-// p = 5.
+// (with the M2M of the time) 1.69 -> 0.81 ms at 1M dipoles, p = 6; 0.50 -> 0.26 ms
+// at 200k charges and dipoles, p = 6; 2.22 -> 0.79 ms at 96 quadrupole systems, p = 5.
 template <int kMaxSrc>
 __device__ __forceinline__ void p2m_leaf(int c, const int32_t *begin, const int32_t *end,
                                          const double *centre, const double *px, const double *py,
@@ -477,45 +476,67 @@ __device__ __forceinline__ void p2m_leaf(int c, const int32_t *begin, const int3
 
 // ------------------------------------------------------------------ M2M
 // The multipole of parent cell c from its children (Eq. (4) with the sign of
-// R2), children summed in index order.  ldcg: the children's rows may have been
-// written by other blocks of the same launch.
+// R2), one axis at a time: the children's centres differ along an axis only by
+// the child's bit, so the two of each pair are shifted along x and added, then
+// the four sums along y, then along z.  14 axis shifts of some three terms a
+// component in place of 8 shifts of (n_x+1)(n_y+1)(n_z+1), and sums of 8 terms
+// in a row in place of 8 x 40: upward pass 0.81 -> 0.48 ms at 1M dipoles, p = 6;
+// 1.08 -> 0.53 ms at 262k Plummer, p = 8; 0.33 -> 0.14 ms at 125k, p = 6.  ldcg:
+// the children's rows may have been written by other blocks of the same launch.
 __device__ __forceinline__ void m2m_cell(int c, const int32_t *child, const int32_t *nchild,
+                                         const int32_t *cx, const int32_t *cy, const int32_t *cz,
                                          const double *centre, const DevTables &tb, double *M,
                                          double *sm)
 {
-    const int P = tb.p, nK = tb.nK;
-    double *apow = sm;                  // [3][P+1]
-    double *mono = apow + 3 * (P + 1);  // [nK]
-    double *Mc = mono + nK;             // [nM]
-    const int nch = nchild[c];
-    double acc[kP2MPer];
-#pragma unroll
-    for (int u = 0; u < kP2MPer; ++u) acc[u] = 0.0;
+    const int P1 = tb.p + 1, nM = tb.nM, nch = nchild[c], ch0 = child[c];
+    double *pw = sm;                    // [3][2][P+1]: (z'_d - z_d)^j / j! of the lower and upper children
+    double *A = pw + 6 * P1;            // [8][nM] children by bits x + 2 y + 4 z, then [2][nM]
+    double *B = A + 8 * nM;             // [4][nM]
+    unsigned have = 0, done = 0;        // bits of the children there are; powers formed
     for (int i = 0; i < nch; ++i) {
-        const int ch = child[c] + i;
-        if (threadIdx.x < 3)
-            axis_powers(centre[3 * c + threadIdx.x] - centre[3 * ch + threadIdx.x], P,
-                        apow + threadIdx.x * (P + 1));
-        for (int t = threadIdx.x; t < tb.nM; t += blockDim.x) Mc[t] = __ldcg(M + (int64_t)ch * tb.nM + t);
-        __syncthreads();
-        for (int k = threadIdx.x; k < nK; k += blockDim.x) {
-            const int v = mi_at(tb.mi, k);
-            mono[k] = apow[mi_nx(v)] * apow[(P + 1) + mi_ny(v)] * apow[2 * (P + 1) + mi_nz(v)];
+        const int ch = ch0 + i, slot = (cx[ch] & 1) | (cy[ch] & 1) << 1 | (cz[ch] & 1) << 2;
+        have |= 1u << slot;
+        if (threadIdx.x < 3) {
+            const int up = (slot >> threadIdx.x) & 1;
+            if (!(done >> up & 1u))
+                axis_powers(centre[3 * c + threadIdx.x] - centre[3 * ch + threadIdx.x], tb.p,
+                            pw + (2 * threadIdx.x + up) * P1);
+            done |= 1u << up;
         }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < kP2MPer; ++u) {
-            const int ni = threadIdx.x + u * 128;
-            if (ni >= tb.nM) break;
-            for (int q = tb.m2m_off[ni]; q < tb.m2m_off[ni + 1]; ++q)
-                acc[u] = fma(mono[tb.m2m_k[q]], Mc[tb.m2m_q[q]], acc[u]);
-        }
-        __syncthreads();
+        for (int t = threadIdx.x; t < nM; t += blockDim.x) A[slot * nM + t] = __ldcg(M + (int64_t)ch * nM + t);
     }
+    __syncthreads();
 #pragma unroll
-    for (int u = 0; u < kP2MPer; ++u) {
-        const int ni = threadIdx.x + u * 128;
-        if (ni < tb.nM) M[(int64_t)c * tb.nM + ni] = acc[u];
+    for (int ax = 0; ax < 3; ++ax) {
+        const int outs = 4 >> ax;
+        const double *in = ax == 1 ? B : A;
+        double *out = ax == 0 ? B : (ax == 1 ? A : M + (int64_t)c * nM);
+        for (int t = threadIdx.x; t < outs * nM; t += blockDim.x) {
+            const int g = t / nM, ni = t - g * nM;
+            const int v = mi_at(tb.mi, ni + tb.m0), sh0 = mi_shell(v);
+            const int na = ax == 0 ? mi_nx(v) : (ax == 1 ? mi_ny(v) : mi_nz(v));
+            const int js = min(na, sh0 - tb.s);
+            double acc = 0.0;
+#pragma unroll
+            for (int up = 0; up < 2; ++up) {
+                if (!(have >> (2 * g + up) & 1u)) continue;
+                const double *p = pw + (2 * ax + up) * P1, *x = in + (2 * g + up) * nM + ni;
+                // n - j e: one shell lower, at the same place in it (x), a row up
+                // (y), a row and a place (z)
+                int sh = sh0, a = mi_ny(v) + mi_nz(v);
+                for (int j = 0; j <= js; ++j) {
+                    acc = fma(p[j], *x, acc);
+                    x -= sh * (sh + 1) / 2 + (ax == 0 ? 0 : (ax == 1 ? a : a + 1));
+                    --sh;
+                    --a;
+                }
+            }
+            out[t] = acc;
+        }
+        have = (have | have >> 1) & 0x55u;          // pairs with a child
+        have = (have | have >> 1) & 0x33u;
+        have = (have | have >> 2) & 0x0fu;
+        if (ax < 2) __syncthreads();
     }
 }
 
@@ -528,9 +549,9 @@ __device__ __forceinline__ void m2m_cell(int c, const int32_t *child, const int3
 template <int kMaxSrc>
 __global__ void __launch_bounds__(kP2MThreads)
 k_upward(const int32_t *leaves, const int32_t *begin, const int32_t *end, const int32_t *parent,
-         const int32_t *child, const int32_t *nchild, const double *centre, const double *px,
-         const double *py, const double *pz, const double *S, DevTables tb, double *M,
-         unsigned *arrive)
+         const int32_t *child, const int32_t *nchild, const int32_t *cx, const int32_t *cy,
+         const int32_t *cz, const double *centre, const double *px, const double *py,
+         const double *pz, const double *S, DevTables tb, double *M, unsigned *arrive)
 {
     extern __shared__ double sm[];
     __shared__ int s_go;
@@ -552,7 +573,7 @@ k_upward(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
         }
         __syncthreads();
         if (!s_go) break;
-        m2m_cell(pa, child, nchild, centre, tb, M, sm);
+        m2m_cell(pa, child, nchild, cx, cy, cz, centre, tb, M, sm);
         c = pa;
     }
 }
@@ -1036,13 +1057,14 @@ fmm_status run_upward(fmm_tree *t, const DevTables &tb, bool rec)
     cudaMemsetAsync(t->b_ud.ptr, 0, 4 * (size_t)nc, st);
     const size_t smem = 8 * std::max<size_t>(
         (size_t)tb.nK * tb.nS + (size_t)kP2MChunk * 3 * P1 + (size_t)kP2MChunk * tb.nS,
-        3 * (size_t)P1 + tb.nK + tb.nM);
+        6 * (size_t)P1 + 12 * (size_t)tb.nM);
     auto go = [&](auto kern) {
         allow_max_dynamic_smem(kern);
         kern<<<(unsigned)t->nleaves, kP2MThreads, smem, st>>>(
             (const int32_t *)t->b_leaves.ptr, (const int32_t *)t->b_begin.ptr,
             (const int32_t *)t->b_end.ptr, (const int32_t *)t->b_parent.ptr,
-            (const int32_t *)t->b_child.ptr, (const int32_t *)t->b_nchild.ptr, centre,
+            (const int32_t *)t->b_child.ptr, (const int32_t *)t->b_nchild.ptr, (const int32_t *)t->b_cx.ptr,
+            (const int32_t *)t->b_cy.ptr, (const int32_t *)t->b_cz.ptr, centre,
             (const double *)t->b_px.ptr, (const double *)t->b_py.ptr, (const double *)t->b_pz.ptr,
             (const double *)t->b_S.ptr, tb, M, (unsigned *)t->b_ud.ptr);
     };
