@@ -54,10 +54,8 @@ struct OpTables {
     int nS = 0, nM = 0, nL = 0, nD = 0, m0 = 0;
     // P2M: for each m (0..nM), up to nS terms (a, mono index of m - a); -1 = none
     std::vector<int> p2m_terms;          // [nM x nS] mono index or -1
-    // monomial recurrences: mono[k] = mono[par[k]] * d[axis[k]] / k_axis
-    std::vector<int> mono_par, mono_axis, mono_pow;   // [ntot(P)]
-    // M2M: CSR over outputs n (M storage), terms (mono k, M index q)
-    std::vector<int> m2m_off, m2m_k, m2m_q;
+    // M2M (FP32 forms): CSR over outputs n (M storage), terms mono k | M index q << 16
+    std::vector<int> m2m_off, m2m_kq;
     // L2L: CSR over outputs n (L storage), terms (mono k, L index n+k)
     std::vector<int> l2l_off, l2l_k, l2l_q;
     // L2P gradient: for |k| <= p-1, L index of k + e_d (3 per k)
@@ -141,7 +139,7 @@ constexpr int kM2LThreadsShared = 128;
 struct DevTables {
     int s, p, n_lo, nS, nM, nL, nD, m0, nK, nG;
     const int *p2m_terms;
-    const int *m2m_off, *m2m_k, *m2m_q;
+    const int *m2m_off, *m2m_kq;
     const int *l2l_off, *l2l_k, *l2l_q;
     const int *l2p_grad, *l2p_ord;
     const int *inv_fact;                 // 1/k! of every k, a double as two words

@@ -55,19 +55,17 @@ void build_tables(OpTables &T, int s, int s_hi, int p, int n_lo, int m2l_threads
             if (kx >= 0 && ky >= 0 && kz >= 0) T.p2m_terms[(size_t)mi * T.nS + ai] = I(kx, ky, kz);
         }
     }
-    T.mono_par.assign(nK, 0); T.mono_axis.assign(nK, 0); T.mono_pow.assign(nK, 0);
 
-    T.m2m_off.assign(1, 0); T.m2m_k.clear(); T.m2m_q.clear();
+    T.m2m_off.assign(1, 0); T.m2m_kq.clear();
     for (int ni = 0; ni < T.nM; ++ni) {
         const int n = ni + T.m0;
         for (int qi = 0; qi < T.nM; ++qi) {
             const int q = qi + T.m0;
             int kx = I.nx[n] - I.nx[q], ky = I.ny[n] - I.ny[q], kz = I.nz[n] - I.nz[q];
             if (kx < 0 || ky < 0 || kz < 0) continue;
-            T.m2m_k.push_back(I(kx, ky, kz));
-            T.m2m_q.push_back(qi);
+            T.m2m_kq.push_back(I(kx, ky, kz) | qi << 16);
         }
-        T.m2m_off.push_back((int)T.m2m_k.size());
+        T.m2m_off.push_back((int)T.m2m_kq.size());
     }
     T.l2l_off.assign(1, 0); T.l2l_k.clear(); T.l2l_q.clear();
     for (int n = 0; n < T.nL; ++n) {
@@ -899,7 +897,7 @@ k_downward(int64_t nc, const int32_t *parent, const double *centre, DevTables tb
 
 inline unsigned grid(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
-// Table buffer layout (int32): lut | p2m | m2m_off | m2m_k | m2m_q | l2l_off |
+// Table buffer layout (int32): lut | p2m | m2m_off | m2m_kq | l2l_off |
 // l2l_k | l2l_q | l2p_grad | red_off | red_src
 fmm_status upload_tables(fmm_tree *t, int s, int p, int n_lo, DevTables *dt, const int32_t **lut)
 {
@@ -921,7 +919,7 @@ fmm_status upload_tables(fmm_tree *t, int s, int p, int n_lo, DevTables *dt, con
     }
     OpTables &T = t->tab;
     std::vector<int32_t> buf;
-    size_t o_lut, o_p2m, o_m2m_off, o_m2m_k, o_m2m_q, o_l2l_off, o_l2l_k, o_l2l_q, o_grad, o_roff, o_rsrc;
+    size_t o_lut, o_p2m, o_m2m_off, o_m2m_kq, o_l2l_off, o_l2l_k, o_l2l_q, o_grad, o_roff, o_rsrc;
     auto put = [&](const std::vector<int> &v) {
         size_t o = buf.size();
         buf.insert(buf.end(), v.begin(), v.end());
@@ -939,8 +937,8 @@ fmm_status upload_tables(fmm_tree *t, int s, int p, int n_lo, DevTables *dt, con
         for (int i = 0; i < (int)lutv.size(); ++i) lutv[i] = ((const int16_t *)I.lut)[i];
         o_lut = put(lutv);
     }
-    o_p2m = put(T.p2m_terms); o_m2m_off = put(T.m2m_off); o_m2m_k = put(T.m2m_k);
-    o_m2m_q = put(T.m2m_q); o_l2l_off = put(T.l2l_off); o_l2l_k = put(T.l2l_k);
+    o_p2m = put(T.p2m_terms); o_m2m_off = put(T.m2m_off); o_m2m_kq = put(T.m2m_kq);
+    o_l2l_off = put(T.l2l_off); o_l2l_k = put(T.l2l_k);
     o_l2l_q = put(T.l2l_q); o_grad = put(T.l2p_grad); o_roff = put(T.m2l_red_off);
     const size_t o_ord = put(T.l2p_ord);
     size_t o_if;
@@ -981,8 +979,8 @@ fmm_status upload_tables(fmm_tree *t, int s, int p, int n_lo, DevTables *dt, con
     const int32_t *B = (const int32_t *)t->b_tab_i32.ptr;
     dt->s = s; dt->p = p; dt->n_lo = n_lo; dt->nS = T.nS; dt->nM = T.nM; dt->nL = T.nL;
     dt->nD = T.nD; dt->m0 = T.m0; dt->nK = ntot(p); dt->nG = ntot(p - 1);
-    dt->p2m_terms = B + o_p2m; dt->m2m_off = B + o_m2m_off; dt->m2m_k = B + o_m2m_k;
-    dt->m2m_q = B + o_m2m_q; dt->l2l_off = B + o_l2l_off; dt->l2l_k = B + o_l2l_k;
+    dt->p2m_terms = B + o_p2m; dt->m2m_off = B + o_m2m_off; dt->m2m_kq = B + o_m2m_kq;
+    dt->l2l_off = B + o_l2l_off; dt->l2l_k = B + o_l2l_k;
     dt->l2l_q = B + o_l2l_q; dt->l2p_grad = B + o_grad; dt->l2p_ord = B + o_ord; dt->inv_fact = B + o_if; dt->m2l_red_off = B + o_roff;
     dt->m2l_red_src = B + o_rsrc;
     dt->m2l_desc = (const uint32_t *)t->b_tab_u32.ptr;
