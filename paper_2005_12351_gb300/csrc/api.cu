@@ -71,8 +71,14 @@ static void forget_state(fmm_tree *t)
 
 fmm_status side_stream(fmm_tree *t)
 {
-    if (!t->side_st)
-        FMM_TRY(cuda_check(t, cudaStreamCreateWithFlags(&t->side_st, cudaStreamNonBlocking), "stream"));
+    if (!t->side_st) {
+        // the highest priority: its small kernels take the blocks' places that the
+        // upward pass's fall free, instead of waiting for all of them to start (1M
+        // dipoles FP32: M2L's wait for the plan 0.08 ms less)
+        int least = 0, greatest = 0;
+        FMM_TRY(cuda_check(t, cudaDeviceGetStreamPriorityRange(&least, &greatest), "priorities"));
+        FMM_TRY(cuda_check(t, cudaStreamCreateWithPriority(&t->side_st, cudaStreamNonBlocking, greatest), "stream"));
+    }
     if (!t->ev_lists)
         FMM_TRY(cuda_check(t, cudaEventCreateWithFlags(&t->ev_lists, cudaEventDisableTiming), "event"));
     if (!t->ev_plan)
