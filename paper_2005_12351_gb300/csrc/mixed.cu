@@ -40,13 +40,13 @@ __host__ __device__ __forceinline__ int row4(int n) { return (n + 3) & ~3; }
 
 
 // per-axis scaled powers w^q / q!, q <= P
-__device__ __forceinline__ void axis_powers32(float w, int P, float *out)
+__device__ __forceinline__ void axis_powers32(float w, int P, float *out, int stride = 1)
 {
     float v = 1.0f;
     out[0] = 1.0f;
     for (int q = 1; q <= P; ++q) {
         v = v * w * x_invint[q];
-        out[q] = v;
+        out[q * stride] = v;
     }
 }
 
@@ -96,50 +96,64 @@ __device__ __forceinline__ void two_sum_lo(float a, float b, float c, float &s, 
 // ------------------------------------------------------------------ P2M
 constexpr int kChunk = 32;
 constexpr int kPer = 4;                   // up to 4 * 128 = 512 components per thread block
-constexpr int kMaxSrc = 6;
+
+constexpr int kCh4 = kChunk + 4;          // row stride of the staged values: 16-byte reads of rows without conflicts
 
 // One block per leaf; each thread owns up to kPer components, with the
-// monomial index of each of a component's source terms taken per chunk
-// (absent terms hit a zero slot).  FP32 sums over groups of 8 particles,
-// double-float across groups.
+// monomial row of each of a component's source terms taken per chunk (absent
+// terms hit a row of zeros).  FP32 sums over groups of 8 particles in particle
+// order, double-float across groups.  Powers, monomials and moments lie in
+// rows of particles, so a 16-byte read serves four of them; the rows are
+// padded to a multiple of four with zero moments, which leave a sum as it is.
+// With a read per particle and value the upward pass took 2.40 instead of 2.15
+// ms at 4M Plummer, p = 8, and 0.44 instead of 0.39 ms at 1M, p = 6.  Not
+// better: chunks of 16 particles, 10 or 12 blocks an SM (spills), a persistent
+// grid (1.1 ms at 1M).
+template <int NS>
 __device__ __forceinline__ void p2m32_leaf(int c, const int32_t *begin, const int32_t *end,
                                            const double *half, const float4 *o, const float *S32,
                                            const DevTables &tb, float *M, float *sf)
 {
-    const int P = tb.p, P1 = tb.p + 1, nK = tb.nK, nK1 = tb.nK + 1, nS = tb.nS;
-    float *apow = sf;                              // [chunk][3][P1]
-    float *mono = apow + kChunk * 3 * P1;          // [chunk][nK + 1], last = 0
-    float *Ssm = mono + kChunk * nK1;              // [chunk][8], padded with zeros
-    Ssm = (float *)(((uintptr_t)Ssm + 15) & ~(uintptr_t)15);
+    const int P = tb.p, P1 = tb.p + 1, nK = tb.nK;
+    sf = (float *)(((uintptr_t)sf + 15) & ~(uintptr_t)15);
+    float *apow = sf;                              // [3][P1][kCh4]
+    float *mono = apow + 3 * P1 * kCh4;            // [nK + 1][kCh4], last row = 0
+    float *Ssm = mono + (nK + 1) * kCh4;           // [NS][kCh4]
     const int b = begin[c], e = end[c];
     // h is a power of two: 1/h from its exponent (exact, as the FP64 quotient
     // rounded to float would be), no FP64 division in every thread
     const float inv_h = ldexpf(1.0f, -ilogb(half[c]));
-    const int nS32 = nS == 6 ? 7 : nS;
+    constexpr int nS32 = NS == 6 ? 7 : NS;
     df32 acc[kPer];                                // double-float: no FP64 in the pass
 #pragma unroll
     for (int u = 0; u < kPer; ++u) acc[u] = {0.0f, 0.0f};
+    for (int t = threadIdx.x; t < kCh4; t += blockDim.x) mono[nK * kCh4 + t] = 0.0f;
     for (int j0 = b; j0 < e; j0 += kChunk) {
-        const int nj = min(kChunk, e - j0);
-        for (int t = threadIdx.x; t < 3 * nj; t += blockDim.x) {
-            const int j = t / 3, ax = t % 3;
-            const float4 v = o[j0 + j];
-            const float d = ax == 0 ? v.x : (ax == 1 ? v.y : v.z);
-            axis_powers32(-d * inv_h, P, apow + (j * 3 + ax) * P1);
+        const int nj = min(kChunk, e - j0), n4 = (nj + 3) & ~3;
+        for (int t = threadIdx.x; t < 3 * kChunk; t += blockDim.x) {
+            const int j = t & (kChunk - 1), ax = t / kChunk;
+            if (j < n4) {
+                const float4 v = j < nj ? o[j0 + j] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                const float d = ax == 0 ? v.x : (ax == 1 ? v.y : v.z);
+                axis_powers32(-d * inv_h, P, apow + ax * P1 * kCh4 + j, kCh4);
+            }
         }
-        for (int t = threadIdx.x; t < nj * 8; t += blockDim.x)
-            Ssm[t] = (t & 7) < nS ? S32[(int64_t)(j0 + (t >> 3)) * nS32 + (t & 7)] : 0.0f;
+        for (int t = threadIdx.x; t < NS * kChunk; t += blockDim.x) {
+            const int j = t & (kChunk - 1), a = t / kChunk;
+            Ssm[a * kCh4 + j] = j < nj ? S32[(int64_t)(j0 + j) * nS32 + a] : 0.0f;
+        }
         __syncthreads();
         // each thread its monomials k (exponents decoded once) for every particle
-        for (int k = threadIdx.x; k < nK1; k += blockDim.x) {
-            int ox = 0, oy = 0, oz = 0;
-            if (k < nK) {
-                const int v = mi_at(tb.mi, k);
-                ox = mi_nx(v); oy = P1 + mi_ny(v); oz = 2 * P1 + mi_nz(v);
-            }
-            for (int j = 0; j < nj; ++j) {
-                const float *a = apow + j * 3 * P1;
-                mono[j * nK1 + k] = k < nK ? a[ox] * a[oy] * a[oz] : 0.0f;
+        for (int k = threadIdx.x; k < nK; k += blockDim.x) {
+            const int v = mi_at(tb.mi, k);
+            const float4 *x = (const float4 *)(apow + mi_nx(v) * kCh4);
+            const float4 *y = (const float4 *)(apow + (P1 + mi_ny(v)) * kCh4);
+            const float4 *z = (const float4 *)(apow + (2 * P1 + mi_nz(v)) * kCh4);
+            float4 *m = (float4 *)(mono + k * kCh4);
+#pragma unroll 2
+            for (int q = 0; q < n4 / 4; ++q) {
+                const float4 a = x[q], bb = y[q], cc = z[q];
+                m[q] = make_float4(a.x * bb.x * cc.x, a.y * bb.y * cc.y, a.z * bb.z * cc.z, a.w * bb.w * cc.w);
             }
         }
         __syncthreads();
@@ -147,28 +161,31 @@ __device__ __forceinline__ void p2m32_leaf(int c, const int32_t *begin, const in
         for (int u = 0; u < kPer; ++u) {
             const int mi = threadIdx.x + u * 128;
             if (mi >= tb.nM) break;
-            // the monomial index of each source term of component mi (absent: the zero slot)
-            int kt[kMaxSrc];
+            // the monomial row of each source term of component mi (absent: the zeros)
+            const float4 *mk[NS];
 #pragma unroll
-            for (int a = 0; a < kMaxSrc; ++a) {
-                const int k = a < nS ? tb.p2m_terms[mi * nS + a] : -1;
-                kt[a] = k >= 0 ? k : nK;
+            for (int a = 0; a < NS; ++a) {
+                const int k = tb.p2m_terms[mi * NS + a];
+                mk[a] = (const float4 *)(mono + (k >= 0 ? k : nK) * kCh4);
             }
-            for (int j8 = 0; j8 < nj; j8 += 8) {
+            for (int q8 = 0; q8 < n4 / 4; q8 += 2) {
                 float sum = 0.0f;
-                const int je = min(j8 + 8, nj);
-                for (int j = j8; j < je; ++j) {
-                    const float *mj = mono + j * nK1;
-                    const float4 s0 = *(const float4 *)(Ssm + 8 * j);
-                    sum = fmaf(mj[kt[0]], s0.x, sum);
-                    if (nS > 1) sum = fmaf(mj[kt[1]], s0.y, sum);
-                    if (nS > 2) sum = fmaf(mj[kt[2]], s0.z, sum);
-                    if (nS > 3) sum = fmaf(mj[kt[3]], s0.w, sum);
-                    if (nS > 4) {
-                        const float2 s1 = *(const float2 *)(Ssm + 8 * j + 4);
-                        sum = fmaf(mj[kt[4]], s1.x, sum);
-                        if (nS > 5) sum = fmaf(mj[kt[5]], s1.y, sum);
+                const int qe = min(q8 + 2, n4 / 4);
+                for (int q = q8; q < qe; ++q) {
+                    float4 m[NS], w[NS];
+#pragma unroll
+                    for (int a = 0; a < NS; ++a) {
+                        m[a] = mk[a][q];
+                        w[a] = ((const float4 *)(Ssm + a * kCh4))[q];
                     }
+#pragma unroll
+                    for (int a = 0; a < NS; ++a) sum = fmaf(m[a].x, w[a].x, sum);
+#pragma unroll
+                    for (int a = 0; a < NS; ++a) sum = fmaf(m[a].y, w[a].y, sum);
+#pragma unroll
+                    for (int a = 0; a < NS; ++a) sum = fmaf(m[a].z, w[a].z, sum);
+#pragma unroll
+                    for (int a = 0; a < NS; ++a) sum = fmaf(m[a].w, w[a].w, sum);
                 }
                 acc[u] = df_addf(acc[u], sum);
             }
@@ -256,6 +273,7 @@ __device__ __forceinline__ void m2m32_cell(int c, const int32_t *child, const in
 // of leaf b's particles (prep32_leaf), its P2M, then the block whose child
 // arrives last at a parent forms the parent's multipole, up to the root (the
 // FP64 form's k_upward, same counters and ordering).
+template <int NS>
 __global__ void __launch_bounds__(128, 8)
 k_upward32(const int32_t *leaves, const int32_t *begin, const int32_t *end, const int32_t *parent,
            const int32_t *child, const int32_t *nchild, const int32_t *cx, const int32_t *cy,
@@ -268,7 +286,7 @@ k_upward32(const int32_t *leaves, const int32_t *begin, const int32_t *end, cons
     int c = leaves[blockIdx.x];
     prep32_leaf(c, begin, end, centre, px, py, pz, S, nS_in, n, o, o + n, S32);
     __syncthreads();
-    p2m32_leaf(c, begin, end, half, o, S32, tb, M, sf);
+    p2m32_leaf<NS>(c, begin, end, half, o, S32, tb, M, sf);
     for (;;) {
         const int pa = parent[c];
         if (pa < 0) break;
@@ -1616,15 +1634,19 @@ fmm_status run_mixed(fmm_tree *t, int p, int want_phi, int want_field, double *p
     {
         // prep, P2M and M2M in one launch; the arrival counters start (and end) at zero
         cudaMemsetAsync(t->b_ud.ptr, 0, 4 * (size_t)nc, st);
-        size_t smem = 4 * std::max<size_t>((size_t)kChunk * 3 * P1 + (size_t)kChunk * (tb.nK + 1) +
-                                               (size_t)kChunk * 8 + 4,
+        size_t smem = 4 * std::max<size_t>((size_t)kCh4 * (3 * P1 + tb.nK + 1 + tb.nS) + 4,
                                            2 * (size_t)tb.nK + 8 * (size_t)tb.nM + 4);
-        allow_max_dynamic_smem(k_upward32);
-        k_upward32<<<(unsigned)t->nleaves, 128, smem, st>>>(
-            leaves, begin, end, (const int32_t *)t->b_parent.ptr, (const int32_t *)t->b_child.ptr,
-            (const int32_t *)t->b_nchild.ptr, cx, cy, cz, half, (const double *)t->b_centre.ptr,
-            (const double *)t->b_px.ptr, (const double *)t->b_py.ptr, (const double *)t->b_pz.ptr,
-            (const double *)t->b_S.ptr, t->nS, n, o, S32, tb, M, (unsigned *)t->b_ud.ptr);
+        auto up = [&](auto kern) {
+            allow_max_dynamic_smem(kern);
+            kern<<<(unsigned)t->nleaves, 128, smem, st>>>(
+                leaves, begin, end, (const int32_t *)t->b_parent.ptr, (const int32_t *)t->b_child.ptr,
+                (const int32_t *)t->b_nchild.ptr, cx, cy, cz, half, (const double *)t->b_centre.ptr,
+                (const double *)t->b_px.ptr, (const double *)t->b_py.ptr, (const double *)t->b_pz.ptr,
+                (const double *)t->b_S.ptr, t->nS, n, o, S32, tb, M, (unsigned *)t->b_ud.ptr);
+        };
+        if (s == 0) up(k_upward32<1>);
+        else if (s == 1) up(k_upward32<3>);
+        else up(k_upward32<6>);
     }
     t->launches += 1;
     record(t, 7);
