@@ -33,7 +33,7 @@ __device__ __forceinline__ s64 madw(int a, int b, s64 c)
 // The same as a product and an addition, which the compiler fuses: a chain of
 // them into one sum costs 4.6 clocks each where madw, whose sum it moves first,
 // costs 5.4.  Where several results meet in later additions it reorders those
-// and the form with the addend is the faster one (mulhi, the sums of p2p_fx.cu).
+// and the form with the addend can be the faster one (the sums of p2p_fx.cu).
 __device__ __forceinline__ s64 madp(int a, int b, s64 c)
 {
     s64 d;
@@ -91,8 +91,8 @@ __device__ __forceinline__ I2 bal_biased(s64 vb) { return {hi32(vb), lo32(vb) ^ 
 // add + a b / 2^64, rounded (error below one unit); |a|, |b| < 2^62.6
 __device__ __forceinline__ s64 mulhi(I2 a, I2 b, s64 add = 0)
 {
-    const s64 c = madw(a.h, b.l, madw(a.l, b.h, kHalfUlp));
-    return madw(a.h, b.h, add + (s64)hi32(c));
+    const s64 c = madp(a.h, b.l, madp(a.l, b.h, kHalfUlp));
+    return madp(a.h, b.h, add + (s64)hi32(c));
 }
 // a b / 2^62, rounded: two more bits where the product is known to stay below 2^62
 __device__ __forceinline__ s64 mulhi_62(I2 a, I2 b)

@@ -10,12 +10,16 @@
 // per factor: a pair term's error is at or below an FP64 evaluation's (about
 // ten roundings of 2^-53), and the sums over pairs are exact integers.
 // Measured, one million dipoles, field, 946 M interactions: 36.3 ms with the
-// symmetric FP64 kernel -> 11.0 ms; error against long double at or below the
+// symmetric FP64 kernel -> 10.3 ms; error against long double at or below the
 // FP64 kernels' (a set of 700: 1e-16 to 4e-16 against 2e-16 to 1e-15).
-// Bound: the integer multiply pipe (67 % busy) and the ALU (57 %) together; 16
-// or 32 warps per SM run alike.  Measured and not better: cross products by
-// IMAD.HI, 96-bit sums by shifts and carries (4 %), the cross products' upper
-// half added by a multiply-add, 64 to 104 registers for more warps.
+// Bound: the integer multiply pipe and the ALU together; 16 or 32 warps per SM
+// run alike.  Measured and not better: cross products by IMAD.HI, sums by
+// shifts and carries in place of the two multiply-adds by a power of two, the
+// cross products' upper half added by a multiply-add, 64 to 104 registers for
+// more warps.  The sums as the factor's four limbs times the term's two (seven
+// multiply-adds a component, nothing rounded) took 11.0 ms; 262k Plummer
+// dipoles 6.9 instead of 6.0, 200k charges and dipoles 5.9 instead of 5.1,
+// 96 quadrupole systems 32.0 instead of 29.1.
 //
 //   R    separation, source minus target: exact differences of coordinates
 //        rounded to 2^-58 of the coarser leaf's half side, shifted left by sh
@@ -23,12 +27,12 @@
 //   y    1/|R|: FP32 hardware seed y0 (21 bits kept), e = 1 - |R|^2 y0^2, one
 //        third-order step y = y0 (1 + e/2 + 3/8 e^2) (error 5/16 e^3 < 2^-60)
 //   M    a source's moments times a power of two of its own
-//   sums four 28-bit limbs of the factor y^k, shifted right to a scale common
-//        to the target leaf, times the two limbs of the bracketed term, added
-//        into four 64-bit sums with no rounding.  The scale leaves room for the
-//        row's largest moments at the closest fixed-point separation, so a
-//        target with only far neighbours starts up to 28 bits lower; the 112
-//        bits hold 60 significant ones even then
+//   sums the term as one 59-bit integer (rounded at 2^-52 of the moment over the
+//        normalised distance's power, which is at least 1), times a power of two
+//        into 28-bit limbs of four 64-bit sums.  The scale leaves room for the
+//        row's largest moments at the closest fixed-point separation; a term
+//        keeps all its bits down to 2^-56 of the largest possible, and some down
+//        to 2^-84
 //
 // Pairs closer than 2^-7 of the coordinate range (a sixteenth of a half side;
 // a few in a million of a uniform set's) and coincident points take the FP64
@@ -68,42 +72,46 @@ struct FxRec {
     static constexpr int ch = nw <= 6 ? 256 : 128;         // sources staged per round
 };
 
-// exponent adjustments of the shells' terms against the sums' unit
-__host__ __device__ constexpr int fx_off_e(int s) { return s == 2 ? -6 : 0; }
-__host__ __device__ constexpr int fx_off_p(int s) { return s == 0 ? 4 : (s == 2 ? -2 : 0); }
-constexpr int kUnitE = 137, kUnitP = 138;  // a sum's unit is 2^(base - this)
+// A term T Y (T the bracket, Y the power of y) enters as t = T Y / 2^K, |t| <
+// 2^59, times 2^(56 - shift).  The shells' terms stand at different powers of
+// two; these adjust their shifts to the sums' common unit, 2^(base - kUnit).
+__host__ __device__ constexpr int fx_off_e(int s) { return s == 2 ? -4 : 0; }
+__host__ __device__ constexpr int fx_off_p(int s) { return s == 0 ? 2 : (s == 2 ? -2 : 0); }
+constexpr int kUnitE = 108, kUnitP = 111;
 
 // the shift amount that stands for "contributes nothing"
 constexpr int kFar = 160;
 
-// A factor Y (below 2^61) shifted right by s: Y 2^(51 - s) in limbs of 28 bits.
-struct Fx4 {
-    int a3, a2, a1, a0;
-};
-__device__ __forceinline__ Fx4 fx_factor(u64 Y, int s)
+// the two forms of a multiply-add (fx64.cuh): the quadrupoles' sums run faster
+// fused, the others' with the addend in the instruction
+template <bool Q>
+__device__ __forceinline__ s64 mac(int a, int b, s64 c)
 {
-    Fx4 f;
-    const uint32_t us = (uint32_t)s, lo = (uint32_t)Y;
-    f.a3 = (int)shr32((uint32_t)(Y >> 32), us + 1u);
-    f.a2 = (int)((uint32_t)shr64(Y, us + 5u) & kM28);
-    // bits s - 23 .. s + 4 and s - 51 .. s - 24 of Y: one of the two shifts has passed its width
-    f.a1 = (int)(((uint32_t)shr64(Y, us - 23u) | shl32(lo, 23u - us)) & kM28);
-    f.a0 = (int)(((uint32_t)shr64(Y, us - 51u) | shl32(lo, 51u - us)) & kM28);
-    return f;
+    return Q ? madp(a, b, c) : madw(a, b, c);
 }
-// T = i1 2^28 + i0 times the factor into the four sums (units 2^28 apart); the
-// product of the two lowest limbs, 2^-84 of the largest term, is left out
-__device__ __forceinline__ void fx_mac(int i1, int i0, Fx4 f, s64 *P)
+// N terms of one shift s: t 2^(56 - s) in limbs of 28 bits.  Nearly every pair
+// has s <= 28 and takes two multiply-adds by 2^(28 - s); beyond, a limb (two)
+// further down; past 84 nothing.
+template <int N, bool Q>
+__device__ __forceinline__ void fx_add(const s64 (&t)[N], int s, s64 (*P)[4])
 {
-    P[0] = madw(i0, f.a1, madw(i1, f.a0, P[0]));
-    P[1] = madw(i0, f.a2, madw(i1, f.a1, P[1]));
-    P[2] = madw(i0, f.a3, madw(i1, f.a2, P[2]));
-    P[3] = madw(i1, f.a3, P[3]);
-}
-template <int DROP>
-__device__ __forceinline__ void fx_add(s64 T, Fx4 f, s64 *P)
-{
-    fx_mac((int)(T >> (28 + DROP)), (int)((uint32_t)(T >> DROP) & kM28), f, P);
+    int h[N], l[N];
+    const int m = (int)shl32(1u, (uint32_t)(28 - s));
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+        h[c] = (int)(t[c] >> 28);
+        l[c] = (int)((uint32_t)t[c] & kM28);
+        P[c][2] = mac<Q>(h[c], m, P[c][2]);
+        P[c][1] = mac<Q>(l[c], m, P[c][1]);
+    }
+    if (s > 28 && s <= 84) {
+        const int m1 = (int)shl32(1u, (uint32_t)(56 - s)), m0 = s > 56 ? (int)shl32(1u, (uint32_t)(84 - s)) : 0;
+#pragma unroll
+        for (int c = 0; c < N; ++c) {
+            P[c][1] = mac<Q>(h[c], m1, P[c][1]);
+            P[c][0] = mac<Q>(h[c], m0, mac<Q>(l[c], m1, P[c][0]));
+        }
+    }
 }
 // carries: afterwards the lower three sums are in [0, 2^28)
 __device__ __forceinline__ void fx_carry(s64 *P)
@@ -198,29 +206,34 @@ __device__ __forceinline__ void fx_pair(const FxGeo &g, const int *r, bool dead,
     const int *m = r + nb;
     if constexpr (S == 0) {
         if (PHI) {
-            fx_mac(m[0], m[1], fx_factor(g.y1, sp), P[0]);                 // q y; the words are q's limbs
+            const s64 t[1] = {mulhi(word_bal(m, 0), bal((s64)g.y1))};      // q y 2^57
+            fx_add<1, S == 2>(t, sp, P);
         }
         if (FIELD) {
-            const I2 q = word_bal(m, PHI ? 2 : 0); // -q 2^61
-            const Fx4 f = fx_factor(g.y3, se);
-            fx_add<3>(mulhi(q, g.x), f, P[e]);     // -q R 2^59
-            fx_add<3>(mulhi(q, g.y), f, P[e + 1]);
-            fx_add<3>(mulhi(q, g.z), f, P[e + 2]);
+            const I2 q = word_bal(m, PHI ? 2 : 0), y = bal((s64)(g.y3 >> 1));      // -q 2^61
+            // -q R 2^59, times y^3 2^57
+            const s64 t[3] = {mulhi(bal_biased(mulhi(q, g.x, kBias)), y), mulhi(bal_biased(mulhi(q, g.y, kBias)), y),
+                              mulhi(bal_biased(mulhi(q, g.z, kBias)), y)};
+            fx_add<3, S == 2>(t, se, P + e);
         }
     } else if constexpr (S == 1) {
         // M.R 2^59
-        const s64 srb = dot3hi(word_bal(m, 0), g.x, word_bal(m, 2), g.y, word_bal(m, 4), g.z, kBias);
-        if (PHI) fx_add<2>(srb - kBias, fx_factor(g.y3, sp), P[0]);        // (M.R) y^3
+        const I2 sr = bal_biased(dot3hi(word_bal(m, 0), g.x, word_bal(m, 2), g.y, word_bal(m, 4), g.z, kBias));
+        const I2 y3 = bal((s64)(g.y3 << 2));
+        if (PHI) {
+            const s64 t[1] = {mulhi(sr, y3)};                              // (M.R) y^3
+            fx_add<1, S == 2>(t, sp, P);
+        }
         if (FIELD) {
-            const I2 v1 = bal_biased(mulhi(bal_biased(srb), bal((s64)g.y2), kBias));   // (M.R) y^2 2^55
+            const I2 v1 = bal_biased(mulhi(sr, bal((s64)g.y2), kBias));    // (M.R) y^2 2^55
             // -3 (M.R) y^2 2^58: the factor -24
-            const s64 vb = madp(v1.l, -24, kBias);
+            const s64 vb = madw(v1.l, -24, kBias);
             const I2 v = {hi32(vb) + v1.h * -24, lo32(vb) ^ (int)0x80000000};
-            const Fx4 f = fx_factor(g.y3, se);
-            // (M - 3 (M.R) y^2 R) 2^56
-            fx_add<0>(mulhi(v, g.x, word64(m, 6)), f, P[e]);
-            fx_add<0>(mulhi(v, g.y, word64(m, 8)), f, P[e + 1]);
-            fx_add<0>(mulhi(v, g.z, word64(m, 10)), f, P[e + 2]);
+            // (M - 3 (M.R) y^2 R) 2^56 (the words of M hold the bias), times y^3 2^60
+            const s64 t[3] = {mulhi(bal_biased(mulhi(v, g.x, word64(m, 6))), y3),
+                              mulhi(bal_biased(mulhi(v, g.y, word64(m, 8))), y3),
+                              mulhi(bal_biased(mulhi(v, g.z, word64(m, 10))), y3)};
+            fx_add<3, S == 2>(t, se, P + e);
         }
     } else {
         // grad q and 2 q(R) of q(R) = sum S_a R^a; the words are 2 S_200, S_110,
@@ -234,15 +247,20 @@ __device__ __forceinline__ void fx_pair(const FxGeo &g, const int *r, bool dead,
                           dot3hi(m2, g.x, m4, g.y, m5, g.z, kBias)};
         const s64 q2 = dot3hi(bal_biased(G[0]), g.x, bal_biased(G[1]), g.y, bal_biased(G[2]), g.z);   // 2 q 2^58
         const s64 p = mulhi_62(bal(q2 << 2), bal((s64)g.y2));              // 2 q y^2 2^58
-        if (PHI) fx_add<3>(p + (p >> 1) - tr, fx_factor(g.y3, sp), P[0]);  // (3 q y^2 - tr) y^3
+        if (PHI) {
+            const s64 t[1] = {mulhi(bal(p + (p >> 1) - tr), bal((s64)(g.y3 << 1)))};       // (3 q y^2 - tr) y^3
+            fx_add<1, S == 2>(t, sp, P);
+        }
         if (FIELD) {
             // 3 y^5 (grad q - (5 q y^2 - tr) R)
             const I2 n = bal(tr - 2 * p - (p >> 1));                       // (tr - 5 q y^2) 2^58
             const u64 y5 = mulhi_u(g.y3 << 2, g.y2);                       // 2^56
-            const Fx4 f = fx_factor(y5 - (y5 >> 2), se);                   // 3 y^5 2^54
-            fx_add<2>(mulhi(n, g.x, (G[0] - kBias) >> 4), f, P[e]);        // 2^56
-            fx_add<2>(mulhi(n, g.y, (G[1] - kBias) >> 4), f, P[e + 1]);
-            fx_add<2>(mulhi(n, g.z, (G[2] - kBias) >> 4), f, P[e + 2]);
+            const I2 y = bal((s64)((y5 - (y5 >> 2)) << 2));                // 3 y^5 2^56
+            constexpr s64 b = kBias - (kBias >> 4);
+            const s64 t[3] = {mulhi(bal_biased(mulhi(n, g.x, (G[0] >> 4) + b)), y),        // 2^56
+                              mulhi(bal_biased(mulhi(n, g.y, (G[1] >> 4) + b)), y),
+                              mulhi(bal_biased(mulhi(n, g.z, (G[2] >> 4) + b)), y)};
+            fx_add<3, S == 2>(t, se, P + e);
         }
     }
 }
@@ -297,17 +315,14 @@ __device__ __forceinline__ void fx_stage_shell(const double *Sj, int base_p, int
     if (FIELD) r[e] = none ? kFar : min(kFar, base_e - em);
     int *m = r + nb;
     if constexpr (S == 0) {
-        if (PHI) {
-            const s64 q = fix64(Sj[0], 57 - em);
-            m[0] = (int)(q >> 28);
-            m[1] = (int)((uint32_t)q & kM28);
-        }
+        if (PHI) put_bal(m, 0, fix64(Sj[0], 59 - em));
         if (FIELD) put_bal(m, PHI ? 2 : 0, -fix64(Sj[0], 61 - em));
     } else if constexpr (S == 1) {
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            put_bal(m, 2 * a, fix64(Sj[a], 61 - em));
-            if (FIELD) put64(m, 6 + 2 * a, fix64(Sj[a], 56 - em));
+            const s64 v = fix64(Sj[a], 61 - em);
+            put_bal(m, 2 * a, v);
+            if (FIELD) put64(m, 6 + 2 * a, ((v + 16) >> 5) + kBias);
         }
     } else {
 #pragma unroll
@@ -374,7 +389,7 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
     s64 *red = (s64 *)stage;                               // [4 NC][nthr], after the last round
     __shared__ int gbeg[kFxGroups], gpre[kFxGroups + 1];
     __shared__ int s_next_q, s_next_j, s_ng, s_key;
-    __shared__ int s_g, s_cnt, s_mx[3];
+    __shared__ int s_g, s_mx[3];
     const int A = leaves[blockIdx.x];
     const int b = begin[A], nt = end[A] - b;
     if (nt == 0) return;
@@ -384,12 +399,12 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
     // the row: range of the separations in half sides of the coarser leaf,
     // sources, largest moment exponent per shell
     if (tid < 3) s_mx[tid] = kNone;
-    if (tid == 3) { s_g = 1; s_cnt = 0; }
+    if (tid == 3) s_g = 1;
     __syncthreads();
     {
         const s64 rA = 1ll << (kLevels - lA);
         const s64 zx = (2ll * cx[A] + 1) * rA, zy = (2ll * cy[A] + 1) * rA, zz = (2ll * cz[A] + 1) * rA;
-        int g = 1, cnt = 0, mx[3] = {kNone, kNone, kNone};
+        int g = 1, mx[3] = {kNone, kNone, kNone};
         for (int q = q0 + warp; q < q1; q += nwarp) {      // a warp per partner leaf
             const int B = src[q], lB = level[B], key = min(lA, lB);
             const s64 rB = 1ll << (kLevels - lB);
@@ -398,7 +413,6 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
             const s64 ext = max(ax, max(ay, az)) + rA + rB;
             g = max(g, (64 - __clzll(ext - 1)) - (kLevels - key));
             const int jb = begin[B], je = end[B];
-            cnt += je - jb;
             const int lu = lside - key - 1;
             for (int j = jb + lane; j < je; j += 32) {
                 const double *Sj = Sm + (int64_t)j * nS;
@@ -417,15 +431,11 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
             const int v = (int)__reduce_max_sync(0xffffffffu, mx[s]);
             if (lane == 0) atomicMax(&s_mx[s], v);
         }
-        if (lane == 0) {
-            atomicMax(&s_g, g);
-            atomicAdd(&s_cnt, cnt);
-        }
+        if (lane == 0) atomicMax(&s_g, g);
     }
     __syncthreads();
     const int g1 = s_g + 1, F = 61 - s_g;
     // bases: the shift of a pair's factor is base - (exponent of its term)
-    const int room = 33 - __clz(max(s_cnt, 1));            // 2^room > 2 x sources
     int be = kNone, bp = kNone;
     bool bad = false;
 #pragma unroll
@@ -437,10 +447,9 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
         bp = max(bp, mx + (s + 1) * (kShMax - g1) - fx_off_p(s));
     }
     if (be == kNone) be = bp = 0;
-    be += room;
     // mx holds em - (s + 2) lu, the potential's terms go with em - (s + 1) lu:
     // at most the row's coarsest unit (its first partner's) more
-    bp += room + lside - 1 - min(lA, q1 > q0 ? level[src[q0]] : lA);
+    bp += lside - 1 - min(lA, q1 > q0 ? level[src[q0]] : lA);
     for (int c = 0; c < NC; ++c) accd[c * nthr + tid] = 0.0;
 
     // tiles: m passes over the sources with k copies each, m / k smallest
