@@ -738,7 +738,7 @@ constexpr double kCloseSpacings = 1.0;    // close: r < this many mean spacings 
 // TT: targets per thread (1 or 2; the autotuner's tile choice): two share each
 // staged source read, one leaves more threads per target and fewer registers.
 template <int S, bool PHI, bool FIELD, int TT>
-__global__ void __launch_bounds__(kP2PThreads, S == 2 ? 4 : 6)
+__global__ void __launch_bounds__(kP2PThreads, S == 2 ? 4 : 8)
 k_p2p32(const int32_t *leaves, const int32_t *begin, const int32_t *end, const int32_t *off,
         const int32_t *src, const int32_t *level, const int32_t *cx, const int32_t *cy,
         const int32_t *cz, const int32_t *sys, const double *sys_box, const double *half,
@@ -747,20 +747,24 @@ k_p2p32(const int32_t *leaves, const int32_t *begin, const int32_t *end, const i
         double *E_out)
 {
     constexpr int nS = S == 2 ? 7 : (S + 1) * (S + 2) / 2;     // + trace for quadrupoles
-    constexpr int nR2 = (nS - 1 + 1) / 2;                       // float4s of moments after the first
-    constexpr int CH = S == 2 ? 448 : (S == 1 ? 512 : 688);   // 6 blocks per SM for S < 2
+    constexpr int nR2 = (nS - 1 + 1) / 2;                       // pairs of moments after the first
+    constexpr int CH = S == 2 ? 448 : (S == 1 ? 512 : 688);
     // a round stages at most CHU sources; the slots up to CH take the padding
     // that gives every thread the same number of steps
     constexpr int CHU = CH - kP2PThreads;
-    // staged sources of a round, every value twice (the f32x2 pairs of the
-    // two-target step): PD = (x, x, y, y), QD = (z, z, S_0, S_0) hi position in
-    // the target leaf's frame and first moment, RD = the other moments two to a
-    // float4, then the positions' low parts; the per-thread totals of the final
-    // reduction reuse the same bytes once the last round is done
-    constexpr int kStageFloats = CH * (8 + 4 * nR2 + 3);
+    // staged sources of a round: PD = (x, y, z, S_0) hi position in the target
+    // leaf's frame and first moment, RD = the other moments in pairs, then the
+    // positions' low parts; the per-thread totals of the final reduction reuse
+    // the same bytes once the last round is done.  A value enters both halves of
+    // the two-target step as it is read; stored twice, as f32x2 pairs, it took
+    // twice the shared-memory bandwidth (a far dipole step 65 instead of 61
+    // clocks) and space (6 blocks an SM, now 8): P2P of 1M dipoles 1.54 -> 1.44 ms,
+    // 4M Plummer 9.90 -> 9.32 ms.  9 blocks spill (10.6 ms).
+    constexpr int kStageFloats = CH * (4 + 2 * nR2 + 3);
     static_assert(kStageFloats >= 2 * 8 * kP2PThreads, "reduction area");
     __shared__ __align__(16) float stage[kStageFloats];
-    float4 *PD = (float4 *)stage, *QD = PD + CH, *RD = QD + CH;
+    float4 *PD = (float4 *)stage;
+    float2 *RD = (float2 *)(PD + CH);
     float *lx = (float *)(RD + nR2 * CH), *ly = lx + CH, *lz = ly + CH;
     df32 (*red)[kP2PThreads] = (df32 (*)[kP2PThreads])stage;
     __shared__ int gbeg[kGroups], gpre[kGroups + 1];
@@ -854,17 +858,17 @@ k_p2p32(const int32_t *leaves, const int32_t *begin, const int32_t *end, const i
                     }
                     const int64_t jsrc = gbeg[lo] + (d - gpre[lo]);
                     float sl[nS], sh[nS];
-                    const float4 pd = PD[d], qd = QD[d];
-                    sh[0] = qd.z;
+                    const float4 pd = PD[d];
+                    sh[0] = pd.w;
 #pragma unroll
                     for (int a2 = 1; a2 < nS; ++a2) {
-                        const float4 r = RD[d * nR2 + (a2 - 1) / 2];
-                        sh[a2] = (a2 - 1) % 2 ? r.z : r.x;
+                        const float2 r = RD[d * nR2 + (a2 - 1) / 2];
+                        sh[a2] = (a2 - 1) % 2 ? r.y : r.x;
                     }
 #pragma unroll
                     for (int a2 = 0; a2 < nS; ++a2) sl[a2] = S32lo[jsrc * nS + a2];
-                    pair_df<S, PHI, FIELD>(sep_df(po.x, pl.x, pd.x, lx[d]), sep_df(po.y, pl.y, pd.z, ly[d]),
-                                           sep_df(po.z, pl.z, qd.x, lz[d]), sh, sl, rf, r0, r1, r2);
+                    pair_df<S, PHI, FIELD>(sep_df(po.x, pl.x, pd.x, lx[d]), sep_df(po.y, pl.y, pd.y, ly[d]),
+                                           sep_df(po.z, pl.z, pd.z, lz[d]), sh, sl, rf, r0, r1, r2);
                 }
                 // my own entries in this batch of 32: positions [s0, s1)
                 const int s0 = max(excl - c0, 0), s1 = min(incl - c0, 32);
@@ -941,10 +945,9 @@ k_p2p32(const int32_t *leaves, const int32_t *begin, const int32_t *end, const i
             for (int d = tid, i = 0; d < steps * k; d += kP2PThreads, ++i) {
                 if (d >= used) {
                     // padding: a far-away source with zero moments adds exactly 0
-                    PD[d] = make_float4(1e18f, 1e18f, 1e18f, 1e18f);
-                    QD[d] = make_float4(1e18f, 1e18f, 0.0f, 0.0f);
+                    PD[d] = make_float4(1e18f, 1e18f, 1e18f, 0.0f);
 #pragma unroll
-                    for (int a = 0; a < nR2; ++a) RD[d * nR2 + a] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int a = 0; a < nR2; ++a) RD[d * nR2 + a] = make_float2(0.f, 0.f);
                     lx[d] = ly[d] = lz[d] = 0.0f;
                     continue;
                 }
@@ -961,13 +964,12 @@ k_p2p32(const int32_t *leaves, const int32_t *begin, const int32_t *end, const i
                 two_sum_lo(v.y, gdy[lo], vl.y, hy, ly[d]);
                 two_sum_lo(v.z, gdz[lo], vl.z, hz, lz[d]);
                 const float s0 = S32[(int64_t)j * nS];
-                PD[d] = make_float4(hx, hx, hy, hy);
-                QD[d] = make_float4(hz, hz, s0, s0);
+                PD[d] = make_float4(hx, hy, hz, s0);
 #pragma unroll
                 for (int a = 0; a < nR2; ++a) {
                     const float u = S32[(int64_t)j * nS + 2 * a + 1];
                     const float v = 2 * a + 2 < nS ? S32[(int64_t)j * nS + 2 * a + 2] : 0.0f;
-                    RD[d * nR2 + a] = make_float4(u, u, v, v);
+                    RD[d * nR2 + a] = make_float2(u, v);
                 }
                 const float bx = fmaxf(fabsf(hx) - hw, 0.0f), by = fmaxf(fabsf(hy) - hw, 0.0f),
                             bz = fmaxf(fabsf(hz) - hw, 0.0f);
@@ -1020,36 +1022,35 @@ k_p2p32(const int32_t *leaves, const int32_t *begin, const int32_t *end, const i
                 constexpr bool NEAR = decltype(near_t)::value;
                 const int jj = order[spx + it2 * k];
                 if constexpr (TT == 1) {
-                    const float4 pd = PD[jj], qd = QD[jj];
+                    const float4 pd = PD[jj];
                     float Sj[nS];
-                    Sj[0] = qd.z;
+                    Sj[0] = pd.w;
 #pragma unroll
                     for (int a = 0; a < nR2; ++a) {
-                        const float4 r = RD[jj * nR2 + a];
+                        const float2 r = RD[jj * nR2 + a];
                         Sj[2 * a + 1] = r.x;
-                        if (2 * a + 2 < nS) Sj[2 * a + 2] = r.z;
+                        if (2 * a + 2 < nS) Sj[2 * a + 2] = r.y;
                     }
-                    const float dx = oi.x - pd.x, dy = oi.y - pd.z, dz = oi.z - qd.x;
+                    const float dx = oi.x - pd.x, dy = oi.y - pd.y, dz = oi.z - pd.z;
                     const float r2a = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
                     pair32<S, PHI, FIELD>(dx, dy, dz, r2a, !NEAR || r2a >= c2a, Sj, f1, e10, e11, e12);
                     if (NEAR && r2a < c2a && r2a > 0.0f) closeq[0][qa++][tid] = (uint16_t)jj;
                     return;
                 }
-                const ulonglong2 pd = reinterpret_cast<const ulonglong2 *>(PD)[jj];
-                const ulonglong2 qd = reinterpret_cast<const ulonglong2 *>(QD)[jj];
+                const float4 pd = PD[jj];
                 f2 Sj[nS];
-                Sj[0] = qd.y;
+                Sj[0] = f2_splat(pd.w);
 #pragma unroll
                 for (int a = 0; a < nR2; ++a) {
-                    const ulonglong2 r = reinterpret_cast<const ulonglong2 *>(RD)[jj * nR2 + a];
-                    Sj[2 * a + 1] = r.x;
-                    if (2 * a + 2 < nS) Sj[2 * a + 2] = r.y;
+                    const float2 r = RD[jj * nR2 + a];
+                    Sj[2 * a + 1] = f2_splat(r.x);
+                    if (2 * a + 2 < nS) Sj[2 * a + 2] = f2_splat(r.y);
                 }
                 // separations from the rounded leaf-frame coordinates: the error is
                 // ~1 ulp of the leaf size, small next to r for every pair this
                 // loop keeps (the closer ones go to the double-float queue, which
                 // takes the low parts too)
-                const f2 dx = f2_sub(OX, pd.x), dy = f2_sub(OY, pd.y), dz = f2_sub(OZ, qd.x);
+                const f2 dx = f2_sub(OX, f2_splat(pd.x)), dy = f2_sub(OY, f2_splat(pd.y)), dz = f2_sub(OZ, f2_splat(pd.z));
                 const f2 r2 = f2_fma(dx, dx, f2_fma(dy, dy, f2_mul(dz, dz)));
                 const float2 r2s = f2_unpack(r2);
                 if constexpr (!NEAR) {
