@@ -136,6 +136,15 @@ void build_tables(OpTables &T, int s, int s_hi, int p, int n_lo, int m2l_threads
         if (!harmonic || I.nz[n] <= 1) T.h_rn.push_back(n);
     T.nLh = (int)T.h_rn.size();
 
+    T.l2l_ix.assign(2 * (size_t)((nK + 3) / 4) * T.nLh, T.nL | T.nL << 16);
+    for (int r = 0; r < T.nLh; ++r) {
+        const int n = T.h_rn[r];
+        for (int q = T.l2l_off[n], t = 0; q < T.l2l_off[n + 1]; ++q, ++t) {      // k = t
+            int &w = T.l2l_ix[2 * ((size_t)(t / 4) * T.nLh + r) + (t % 4) / 2];
+            w = t & 1 ? (w & 0xffff) | T.l2l_q[q] << 16 : (w & ~0xffff) | T.l2l_q[q];
+        }
+    }
+
     // ---- M2L: flat (n, m) term list in n order, cut into equal per-thread
     // chunks; each maximal same-n run inside a chunk owns one partial slot.
     // m is the position r in the kept list h_rm (all m when not harmonic).
@@ -940,6 +949,8 @@ fmm_status upload_tables(fmm_tree *t, int s, int p, int n_lo, DevTables *dt, con
     o_p2m = put(T.p2m_terms); o_m2m_off = put(T.m2m_off); o_m2m_kq = put(T.m2m_kq);
     o_l2l_off = put(T.l2l_off); o_l2l_k = put(T.l2l_k);
     o_l2l_q = put(T.l2l_q); o_grad = put(T.l2p_grad); o_roff = put(T.m2l_red_off);
+    if (buf.size() & 1) buf.push_back(0);                 // read in pairs of words
+    const size_t o_ix = put(T.l2l_ix);
     const size_t o_ord = put(T.l2p_ord);
     size_t o_if;
     {
@@ -981,7 +992,7 @@ fmm_status upload_tables(fmm_tree *t, int s, int p, int n_lo, DevTables *dt, con
     dt->nD = T.nD; dt->m0 = T.m0; dt->nK = ntot(p); dt->nG = ntot(p - 1);
     dt->p2m_terms = B + o_p2m; dt->m2m_off = B + o_m2m_off; dt->m2m_kq = B + o_m2m_kq;
     dt->l2l_off = B + o_l2l_off; dt->l2l_k = B + o_l2l_k;
-    dt->l2l_q = B + o_l2l_q; dt->l2p_grad = B + o_grad; dt->l2p_ord = B + o_ord; dt->inv_fact = B + o_if; dt->m2l_red_off = B + o_roff;
+    dt->l2l_q = B + o_l2l_q; dt->l2p_grad = B + o_grad; dt->l2p_ord = B + o_ord; dt->l2l_ix = B + o_ix; dt->inv_fact = B + o_if; dt->m2l_red_off = B + o_roff;
     dt->m2l_red_src = B + o_rsrc;
     dt->m2l_desc = (const uint32_t *)t->b_tab_u32.ptr;
     dt->m2l_T = T.m2l_T; dt->m2l_slots = T.m2l_slots;
