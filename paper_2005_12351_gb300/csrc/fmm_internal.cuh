@@ -56,10 +56,8 @@ struct OpTables {
     std::vector<int> p2m_terms;          // [nM x nS] mono index or -1
     // M2M (FP32 forms): CSR over outputs n (M storage), terms mono k | M index q << 16
     std::vector<int> m2m_off, m2m_kq;
-    // L2L: CSR over outputs n (L storage), terms (mono k, L index n+k)
-    std::vector<int> l2l_off, l2l_k, l2l_q;
-    // the same for the FP32 forms: per group of four k and stored component r, the
-    // four L indices as two words of 16-bit halves (nL, a zero, past the last)
+    // L2L (FP32 forms): per group of four k and stored component n, the four L
+    // indices n + k as two words of 16-bit halves (nL, a zero, past the last)
     std::vector<int> l2l_ix;
     // L2P gradient: for |k| <= p-1, L index of k + e_d (3 per k)
     std::vector<int> l2p_grad;
@@ -143,7 +141,7 @@ struct DevTables {
     int s, p, n_lo, nS, nM, nL, nD, m0, nK, nG;
     const int *p2m_terms;
     const int *m2m_off, *m2m_kq;
-    const int *l2l_off, *l2l_k, *l2l_q, *l2l_ix;
+    const int *l2l_ix;
     const int *l2p_grad, *l2p_ord;
     const int *inv_fact;                 // 1/k! of every k, a double as two words
     const int *m2l_red_off, *m2l_red_src;

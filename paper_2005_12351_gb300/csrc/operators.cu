@@ -67,16 +67,6 @@ void build_tables(OpTables &T, int s, int s_hi, int p, int n_lo, int m2l_threads
         }
         T.m2m_off.push_back((int)T.m2m_kq.size());
     }
-    T.l2l_off.assign(1, 0); T.l2l_k.clear(); T.l2l_q.clear();
-    for (int n = 0; n < T.nL; ++n) {
-        for (int k = 0; k < nK; ++k) {
-            int qx = I.nx[n] + I.nx[k], qy = I.ny[n] + I.ny[k], qz = I.nz[n] + I.nz[k];
-            if (qx + qy + qz > p) continue;
-            T.l2l_k.push_back(k);
-            T.l2l_q.push_back(I(qx, qy, qz));
-        }
-        T.l2l_off.push_back((int)T.l2l_k.size());
-    }
     const int nG = ntot(p - 1);
     T.l2p_grad.assign((size_t)3 * std::max(nG, 0), 0);
     for (int k = 0; k < nG; ++k) {
@@ -139,9 +129,12 @@ void build_tables(OpTables &T, int s, int s_hi, int p, int n_lo, int m2l_threads
     T.l2l_ix.assign(2 * (size_t)((nK + 3) / 4) * T.nLh, T.nL | T.nL << 16);
     for (int r = 0; r < T.nLh; ++r) {
         const int n = T.h_rn[r];
-        for (int q = T.l2l_off[n], t = 0; q < T.l2l_off[n + 1]; ++q, ++t) {      // k = t
+        for (int k = 0, t = 0; k < nK; ++k) {                 // the k that fit come first
+            const int x = I.nx[n] + I.nx[k], y = I.ny[n] + I.ny[k], z = I.nz[n] + I.nz[k];
+            if (x + y + z > p) continue;
             int &w = T.l2l_ix[2 * ((size_t)(t / 4) * T.nLh + r) + (t % 4) / 2];
-            w = t & 1 ? (w & 0xffff) | T.l2l_q[q] << 16 : (w & ~0xffff) | T.l2l_q[q];
+            w = t & 1 ? (w & 0xffff) | I(x, y, z) << 16 : (w & ~0xffff) | I(x, y, z);
+            ++t;
         }
     }
 
@@ -698,32 +691,45 @@ k_m2l(const int32_t *off, const int32_t *src, const int32_t *didx, const int32_t
 
 // ------------------------------------------------------------------ L2L
 // The local expansion of cell c shifted from its parent's (Eq. (9)-type Taylor
-// shift), added to c's stored components.
+// shift), added to c's stored components; one axis at a time, three stages of at
+// most p + 1 terms in a row in place of (p + 1)(p + 2)(p + 3) / 6: L2L 0.285 ->
+// 0.177 ms at 1M dipoles, p = 6; 0.217 -> 0.102 ms at 262k Plummer, p = 8.
 __device__ __forceinline__ void l2l_cell(int c, int pa, const double *centre, const DevTables &tb,
                                          double *L, double *sm)
 {
-    const int P = tb.p, nK = tb.nK;
-    double *apow = sm;
-    double *mono = apow + 3 * (P + 1);
-    double *Lp = mono + nK;
+    const int p = tb.p, P1 = p + 1, nL = tb.nL;
+    double *pw = sm;                    // [3][P+1]: (z_d - z'_d)^j / j!
+    double *A = pw + 3 * P1;            // [nL]
+    double *B = A + nL;                 // [nL]
     if (threadIdx.x < 3)
-        axis_powers(centre[3 * c + threadIdx.x] - centre[3 * pa + threadIdx.x], P,
-                    apow + threadIdx.x * (P + 1));
-    expand_local_cg(L + (int64_t)pa * tb.nLh, tb, Lp);        // the parent's full expansion
-    for (int k = threadIdx.x; k < nK; k += blockDim.x) {
-        const int v = mi_at(tb.mi, k);
-        mono[k] = apow[mi_nx(v)] * apow[(P + 1) + mi_ny(v)] * apow[2 * (P + 1) + mi_nz(v)];
-    }
-    __syncthreads();
-    // the child's stored components (the shift keeps the expansion harmonic)
-    for (int r = threadIdx.x; r < tb.nLh; r += blockDim.x) {
-        const int n = tb.h_rn[r];
-        const int kn = mi_shell(mi_at(tb.mi, n));
-        if (kn < tb.n_lo) continue;
-        double acc = 0.0;
-        for (int q = tb.l2l_off[n]; q < tb.l2l_off[n + 1]; ++q)
-            acc = fma(mono[tb.l2l_k[q]], Lp[tb.l2l_q[q]], acc);
-        L[(int64_t)c * tb.nLh + r] += acc;
+        axis_powers(centre[3 * c + threadIdx.x] - centre[3 * pa + threadIdx.x], p, pw + threadIdx.x * P1);
+    expand_local_cg(L + (int64_t)pa * tb.nLh, tb, A);         // the parent's full expansion
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        const double *in = ax == 1 ? B : A, *w = pw + ax * P1;
+        // the last stage forms the child's stored components only (the shift keeps
+        // the expansion harmonic)
+        const int outs = ax == 2 ? tb.nLh : nL;
+        for (int t = threadIdx.x; t < outs; t += blockDim.x) {
+            const int n = ax == 2 ? tb.h_rn[t] : t;
+            const int v = mi_at(tb.mi, n);
+            int sh = mi_shell(v), a = mi_ny(v) + mi_nz(v);
+            if (ax == 2 && sh < tb.n_lo) continue;
+            const int js = p - sh;
+            const double *x = in + n;
+            double acc = 0.0;
+            for (int j = 0; j <= js; ++j) {
+                acc = fma(w[j], *x, acc);
+                // n + j e: one shell up, at the same place in it (x), a row up (y),
+                // a row and a place (z)
+                x += (sh + 1) * (sh + 2) / 2 + (ax == 0 ? 0 : (ax == 1 ? a + 1 : a + 2));
+                ++sh;
+                ++a;
+            }
+            if (ax == 2) L[(int64_t)c * tb.nLh + t] += acc;
+            else (ax == 0 ? B : A)[t] = acc;
+        }
+        if (ax < 2) __syncthreads();
     }
 }
 
@@ -906,8 +912,8 @@ k_downward(int64_t nc, const int32_t *parent, const double *centre, DevTables tb
 
 inline unsigned grid(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
-// Table buffer layout (int32): lut | p2m | m2m_off | m2m_kq | l2l_off |
-// l2l_k | l2l_q | l2p_grad | red_off | red_src
+// Table buffer layout (int32): lut | p2m | m2m_off | m2m_kq | l2p_grad | red_off |
+// red_src | l2l_ix | l2p_ord | 1/k! | harmonic maps | packed indices
 fmm_status upload_tables(fmm_tree *t, int s, int p, int n_lo, DevTables *dt, const int32_t **lut)
 {
     static int consts_ready[64] = {0};
@@ -928,7 +934,7 @@ fmm_status upload_tables(fmm_tree *t, int s, int p, int n_lo, DevTables *dt, con
     }
     OpTables &T = t->tab;
     std::vector<int32_t> buf;
-    size_t o_lut, o_p2m, o_m2m_off, o_m2m_kq, o_l2l_off, o_l2l_k, o_l2l_q, o_grad, o_roff, o_rsrc;
+    size_t o_lut, o_p2m, o_m2m_off, o_m2m_kq, o_grad, o_roff, o_rsrc;
     auto put = [&](const std::vector<int> &v) {
         size_t o = buf.size();
         buf.insert(buf.end(), v.begin(), v.end());
@@ -947,8 +953,7 @@ fmm_status upload_tables(fmm_tree *t, int s, int p, int n_lo, DevTables *dt, con
         o_lut = put(lutv);
     }
     o_p2m = put(T.p2m_terms); o_m2m_off = put(T.m2m_off); o_m2m_kq = put(T.m2m_kq);
-    o_l2l_off = put(T.l2l_off); o_l2l_k = put(T.l2l_k);
-    o_l2l_q = put(T.l2l_q); o_grad = put(T.l2p_grad); o_roff = put(T.m2l_red_off);
+    o_grad = put(T.l2p_grad); o_roff = put(T.m2l_red_off);
     if (buf.size() & 1) buf.push_back(0);                 // read in pairs of words
     const size_t o_ix = put(T.l2l_ix);
     const size_t o_ord = put(T.l2p_ord);
@@ -991,8 +996,7 @@ fmm_status upload_tables(fmm_tree *t, int s, int p, int n_lo, DevTables *dt, con
     dt->s = s; dt->p = p; dt->n_lo = n_lo; dt->nS = T.nS; dt->nM = T.nM; dt->nL = T.nL;
     dt->nD = T.nD; dt->m0 = T.m0; dt->nK = ntot(p); dt->nG = ntot(p - 1);
     dt->p2m_terms = B + o_p2m; dt->m2m_off = B + o_m2m_off; dt->m2m_kq = B + o_m2m_kq;
-    dt->l2l_off = B + o_l2l_off; dt->l2l_k = B + o_l2l_k;
-    dt->l2l_q = B + o_l2l_q; dt->l2p_grad = B + o_grad; dt->l2p_ord = B + o_ord; dt->l2l_ix = B + o_ix; dt->inv_fact = B + o_if; dt->m2l_red_off = B + o_roff;
+    dt->l2p_grad = B + o_grad; dt->l2p_ord = B + o_ord; dt->l2l_ix = B + o_ix; dt->inv_fact = B + o_if; dt->m2l_red_off = B + o_roff;
     dt->m2l_red_src = B + o_rsrc;
     dt->m2l_desc = (const uint32_t *)t->b_tab_u32.ptr;
     dt->m2l_T = T.m2l_T; dt->m2l_slots = T.m2l_slots;
@@ -1173,7 +1177,7 @@ fmm_status run_expansions(fmm_tree *t, int p, int want_phi, int want_field)
     if (t->nlevels > 1) {
         unsigned *ctl = (unsigned *)t->b_ud.ptr + nc + 1;
         cudaMemsetAsync(ctl, 0, 4 * (size_t)(nc + 1), st);
-        size_t smem = 8 * (size_t)(3 * P1 + tb.nK + tb.nL);
+        size_t smem = 8 * (size_t)(3 * P1 + 2 * tb.nL);
         k_downward<<<(unsigned)nc, 128, smem, st>>>(nc, (const int32_t *)t->b_parent.ptr, centre, tb, L, ctl);
         ++t->launches;
     }
