@@ -489,6 +489,35 @@ inline int sm_count()
     return sms;
 }
 
+// Programmatic dependent launch: a kernel launched by launch_next may be placed
+// on the SMs as the one before it in the stream drains, and waits at its first
+// statement, pdl_wait, until that one is complete and its writes are visible.
+// It takes the gap between two launches (about 2 us) out of chains of short
+// kernels: 2,000 charges 0.400 -> 0.358 ms a step, 12k quadrupoles FP32 0.803 ->
+// 0.717, 1M dipoles FP32 3.40 -> 3.33, Morton order of 1M points 0.176 -> 0.159.
+// Not for a kernel whose predecessor in the stream is another stream's event, and
+// every kernel launched so calls pdl_wait before anything else.
+__device__ __forceinline__ void pdl_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline void launch_next(cudaStream_t st, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, A &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);      // errors: cudaGetLastError at the chain's end
+}
+
 // Raises a kernel's dynamic shared-memory limit to the most a block can take
 // next to its static shared memory.  The value depends only on the kernel, so
 // handles that launch it concurrently from several threads never lower the

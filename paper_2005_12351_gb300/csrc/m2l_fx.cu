@@ -133,6 +133,7 @@ __device__ __noinline__ void fx_finish(const FxArgs &a, int slot0, s64 *fs)
 template <int NG>
 __global__ void __launch_bounds__(kFxThreads) k_m2l_fx(const __grid_constant__ FxArgs a)
 {
+    pdl_wait();
     extern __shared__ int4 sm4[];
     __shared__ int s_src[kFxRows][32], s_sh[kFxRows][32], s_key[kFxRows], s_act[kFxRows], s_tile, s_last;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -580,7 +581,7 @@ fmm_status run_m2l_fx(fmm_tree *t, const DevTables &tb, double *L)
     const size_t smem = std::max(fx_smem(Ly), 32 * (size_t)Ly.groups * kFxPad);   // the last block's turn
     auto go = [&](auto kern) {
         allow_max_dynamic_smem(kern);
-        kern<<<(unsigned)(4 * t->tc_chunks * a.parts), kFxThreads, smem, st>>>(a);
+        launch_next(st, kern, (unsigned)(4 * t->tc_chunks * a.parts), kFxThreads, smem, a);
     };
     switch (Ly.cap) {
     case 4: go(k_m2l_fx<4>); break;

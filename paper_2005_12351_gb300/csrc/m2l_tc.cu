@@ -513,6 +513,7 @@ __global__ void __launch_bounds__(32 * kReduceWarps)
 k_tc_reduce(int T, const int32_t *tile_tgt, const uint32_t *tile_chunk_off, const float *partial, int Np,
             int ncol, const int32_t *col_n, int nL, int nLh, const int *h_rn, const unsigned *err, float *L)
 {
+    pdl_wait();
     __shared__ float Ls[kReduceWarps][kMaxTot];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int q = blockIdx.x * kReduceWarps + w;
@@ -917,7 +918,7 @@ fmm_status tc_build_plan(fmm_tree *t)
 void launch_tc_reduce(fmm_tree *t, int Np, int ncol, const int32_t *col_n, int nL, const DevTables &tb,
                       const unsigned *err, float *L)
 {
-    k_tc_reduce<<<(unsigned)((t->tc_T + kReduceWarps - 1) / kReduceWarps), 32 * kReduceWarps, 0, t->stream>>>(
+    launch_next(t->stream, k_tc_reduce, (unsigned)((t->tc_T + kReduceWarps - 1) / kReduceWarps), 32 * kReduceWarps, 0, 
         (int)t->tc_T, (const int32_t *)t->b_tc_tgt.ptr, (const uint32_t *)t->b_tc_coff.ptr,
         (const float *)t->b_tc_part.ptr, Np, ncol, col_n, nL, tb.nLh, tb.h_rn, err, L);
     ++t->launches;

@@ -281,6 +281,7 @@ k_upward32(const int32_t *leaves, const int32_t *begin, const int32_t *end, cons
            const double *py, const double *pz, const double *S, int nS_in, int64_t n, float4 *o,
            float *S32, DevTables tb, float *M, unsigned *arrive)
 {
+    pdl_wait();
     extern __shared__ float sf[];
     __shared__ int s_go;
     int c = leaves[blockIdx.x];
@@ -532,6 +533,7 @@ k_l2p32(const int32_t *leaves, const int32_t *begin, const int32_t *end, const d
         const float4 *o, const float *L, DevTables tb, int want_phi, int want_field,
         double *phi, double *E)
 {
+    pdl_wait();
     extern __shared__ float sf[];
     l2p32_leaf<false>(leaves[blockIdx.x], begin, end, half, o, L, tb, want_phi, want_field, phi, E, sf);
 }
@@ -547,6 +549,7 @@ __global__ void __launch_bounds__(128)
 k_downward32(int64_t nint, const int32_t *inner, const int32_t *parent, const int32_t *cx,
              const int32_t *cy, const int32_t *cz, DevTables tb, float *L, unsigned *ctl)
 {
+    pdl_wait();
     extern __shared__ float sf[];
     __shared__ int s_k, s_ok;
     if (threadIdx.x == 0) s_k = (int)atomicAdd(&ctl[0], 1u);
@@ -579,6 +582,7 @@ k_downward32_leaf(const int32_t *leaves, const int32_t *parent, const int32_t *c
                   const int32_t *cz, DevTables tb, float *L, const int32_t *begin, const int32_t *end,
                   const double *half, const float4 *o, int want_phi, int want_field, double *phi, double *E)
 {
+    pdl_wait();
     extern __shared__ float sf[];
     const int c = leaves[blockIdx.x], pa = parent[c];
     if (pa >= 0) {
@@ -777,6 +781,7 @@ k_p2p32(const int32_t *leaves, const int32_t *begin, const int32_t *end, const i
         const double *phi_far, const double *E_far, const int32_t *perm, double *phi_out,
         double *E_out)
 {
+    pdl_wait();
     constexpr int nS = S == 2 ? 7 : (S + 1) * (S + 2) / 2;     // + trace for quadrupoles
     constexpr int nR2 = (nS - 1 + 1) / 2;                       // pairs of moments after the first
     constexpr int CH = S == 2 ? 448 : (S == 1 ? 512 : 688);
@@ -1525,7 +1530,7 @@ template <int S>
 void launch_p2p32(fmm_tree *t, int want_phi, int want_field, double *phi, double *E)
 {
     auto go = [&](auto kern) {
-        kern<<<(unsigned)t->nleaves, kP2PThreads, 0, t->stream>>>(
+        launch_next(t->stream, kern, (unsigned)t->nleaves, kP2PThreads, 0, 
             (const int32_t *)t->b_leaves.ptr, (const int32_t *)t->b_begin.ptr,
             (const int32_t *)t->b_end.ptr, (const int32_t *)t->b_p2p_off.ptr,
             (const int32_t *)t->b_p2p_src.ptr, (const int32_t *)t->b_level.ptr,
@@ -1665,12 +1670,14 @@ fmm_status run_mixed(fmm_tree *t, int p, int want_phi, int want_field, double *p
 
     {
         // prep, P2M and M2M in one launch; the arrival counters start (and end) at zero
-        cudaMemsetAsync(t->b_ud.ptr, 0, 4 * (size_t)nc, st);
+        // and so do the downward pass's flags behind them
+        cudaMemsetAsync(L, 0, 4 * (size_t)nc * tb.nLh, st);
+        cudaMemsetAsync(t->b_ud.ptr, 0, 8 * (size_t)(nc + 1), st);
         size_t smem = 4 * std::max<size_t>((size_t)kCh4 * (3 * P1 + tb.nK + 1 + tb.nS) + 4,
                                            2 * (size_t)tb.nK + 8 * (size_t)tb.nM + 4);
         auto up = [&](auto kern) {
             allow_max_dynamic_smem(kern);
-            kern<<<(unsigned)t->nleaves, 128, smem, st>>>(
+            launch_next(st, kern, (unsigned)t->nleaves, 128, smem, 
                 leaves, begin, end, (const int32_t *)t->b_parent.ptr, (const int32_t *)t->b_child.ptr,
                 (const int32_t *)t->b_nchild.ptr, cx, cy, cz, half, (const double *)t->b_centre.ptr,
                 (const double *)t->b_px.ptr, (const double *)t->b_py.ptr, (const double *)t->b_pz.ptr,
@@ -1682,7 +1689,6 @@ fmm_status run_mixed(fmm_tree *t, int p, int want_phi, int want_field, double *p
     }
     t->launches += 1;
     record(t, 7);
-    cudaMemsetAsync(L, 0, 4 * (size_t)nc * tb.nLh, st);
     // harmonic M2L: the folded multipoles, for either M2L
     const float *Ms = M;
     if (t->n_m2l > 0 && tb.harmonic) {
@@ -1734,18 +1740,17 @@ fmm_status run_mixed(fmm_tree *t, int p, int want_phi, int want_field, double *p
     const size_t smem_l2p = 4 * ((want_field ? 4 * (size_t)tb.nG : 0) + tb.nL + kL2PThreads * 3 * P1 + 4);
     if (t->nlevels > 1) {
         unsigned *ctl = (unsigned *)t->b_ud.ptr + nc + 1;
-        cudaMemsetAsync(ctl, 0, 4 * (size_t)(nc + 1), st);
         const int64_t nint = nc - t->nleaves;        // cells with children: after the leaves in b_leaves
         const int32_t *parent = (const int32_t *)t->b_parent.ptr;
         if (nint > 0) {
             allow_max_dynamic_smem(k_downward32);
-            k_downward32<<<(unsigned)nint, 128, smem_l2l, st>>>(nint, leaves + t->nleaves, parent, cx, cy, cz,
+            launch_next(st, k_downward32, (unsigned)nint, 128, smem_l2l, nint, leaves + t->nleaves, parent, cx, cy, cz,
                                                                tb, L, ctl);
             ++t->launches;
         }
         const size_t smem = std::max(smem_l2l, smem_l2p);
         allow_max_dynamic_smem(k_downward32_leaf);
-        k_downward32_leaf<<<(unsigned)t->nleaves, 128, smem, st>>>(
+        launch_next(st, k_downward32_leaf, (unsigned)t->nleaves, 128, smem, 
             leaves, parent, cx, cy, cz, tb, L, begin, end, half, o, want_phi, want_field, (double *)t->b_phi.ptr,
             (double *)t->b_E.ptr);
         ++t->launches;
@@ -1753,7 +1758,7 @@ fmm_status run_mixed(fmm_tree *t, int p, int want_phi, int want_field, double *p
     } else {
         record(t, 10);
         allow_max_dynamic_smem(k_l2p32);
-        k_l2p32<<<(unsigned)t->nleaves, kL2PThreads, smem_l2p, st>>>(
+        launch_next(st, k_l2p32, (unsigned)t->nleaves, kL2PThreads, smem_l2p, 
             leaves, begin, end, half, o, L, tb, want_phi, want_field, (double *)t->b_phi.ptr,
             (double *)t->b_E.ptr);
         ++t->launches;

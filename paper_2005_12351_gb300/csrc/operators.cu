@@ -553,6 +553,7 @@ k_upward(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
          const int32_t *cz, const double *centre, const double *px, const double *py,
          const double *pz, const double *S, DevTables tb, double *M, unsigned *arrive)
 {
+    pdl_wait();
     extern __shared__ double sm[];
     __shared__ int s_go;
     int c = leaves[blockIdx.x];
@@ -598,6 +599,7 @@ template <typename Tm>
 __global__ void __launch_bounds__(128)
 k_fold_m(const Tm *M, int ldM, int64_t nc, DevTables tb, Tm *Mh, int ldH)
 {
+    pdl_wait();
     extern __shared__ double fsm[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t c = blockIdx.x * 4ll + w;
@@ -623,6 +625,7 @@ k_m2l(const int32_t *off, const int32_t *src, const int32_t *didx, const int32_t
       const int32_t *sys, const int *e_side, const double *M, const double *D, DevTables tb,
       double *L)
 {
+    pdl_wait();
     extern __shared__ double sm[];
     const int c = blockIdx.x;
     const int b = off[c], e = off[c + 1];
@@ -749,6 +752,7 @@ k_l2p(const int32_t *leaves, const int32_t *begin, const int32_t *end, const dou
       const double *px, const double *py, const double *pz, const double *L, DevTables tb,
       double *phi, double *E)
 {
+    pdl_wait();
     extern __shared__ int4 lsm4[];
     constexpr int D0 = FIELD ? 0 : 3, D1 = PHI ? 4 : 3;     // components wanted
     __shared__ int s_re[kL2PThreads / 32];
@@ -881,6 +885,7 @@ __global__ void __launch_bounds__(128)
 k_downward(int64_t nc, const int32_t *parent, const double *centre, DevTables tb, double *L,
            unsigned *ctl)
 {
+    pdl_wait();
     extern __shared__ double sm[];
     __shared__ int s_c, s_ok;
     if (threadIdx.x == 0) s_c = (int)atomicAdd(&ctl[0], 1u);
@@ -1025,14 +1030,14 @@ void launch_fold_m(cudaStream_t st, const double *M, int ldM, int64_t nc, const 
                    double *Mh, int ldH)
 {
     if (nc > 0)
-        k_fold_m<double><<<(unsigned)((nc + 3) / 4), 128, 32 * (size_t)tb.nM, st>>>(M, ldM, nc, tb, Mh, ldH);
+        launch_next(st, k_fold_m<double>, (unsigned)((nc + 3) / 4), 128, 32 * (size_t)tb.nM, M, ldM, nc, tb, Mh, ldH);
 }
 
 void launch_fold_m(cudaStream_t st, const float *M, int ldM, int64_t nc, const DevTables &tb,
                    float *Mh, int ldH)
 {
     if (nc > 0)
-        k_fold_m<float><<<(unsigned)((nc + 3) / 4), 128, 32 * (size_t)tb.nM, st>>>(M, ldM, nc, tb, Mh, ldH);
+        launch_next(st, k_fold_m<float>, (unsigned)((nc + 3) / 4), 128, 32 * (size_t)tb.nM, M, ldM, nc, tb, Mh, ldH);
 }
 
 // derivative tables, one FP64 row per distinct M2L offset key
@@ -1067,13 +1072,13 @@ fmm_status run_upward(fmm_tree *t, const DevTables &tb, bool rec)
     double *M = (double *)t->b_M.ptr;
     const double *centre = (const double *)t->b_centre.ptr;
     // P2M and M2M in one launch; the arrival counters start (and end) at zero
-    cudaMemsetAsync(t->b_ud.ptr, 0, 4 * (size_t)nc, st);
+    cudaMemsetAsync(t->b_ud.ptr, 0, 8 * (size_t)(nc + 1), st);     // with the downward pass's flags behind them
     const size_t smem = 8 * std::max<size_t>(
         (size_t)tb.nK * tb.nS + (size_t)kP2MChunk * 3 * P1 + (size_t)kP2MChunk * tb.nS,
         6 * (size_t)P1 + 12 * (size_t)tb.nM);
     auto go = [&](auto kern) {
         allow_max_dynamic_smem(kern);
-        kern<<<(unsigned)t->nleaves, kP2MThreads, smem, st>>>(
+        launch_next(st, kern, (unsigned)t->nleaves, kP2MThreads, smem, 
             (const int32_t *)t->b_leaves.ptr, (const int32_t *)t->b_begin.ptr,
             (const int32_t *)t->b_end.ptr, (const int32_t *)t->b_parent.ptr,
             (const int32_t *)t->b_child.ptr, (const int32_t *)t->b_nchild.ptr, (const int32_t *)t->b_cx.ptr,
@@ -1119,6 +1124,7 @@ fmm_status run_expansions(fmm_tree *t, int p, int want_phi, int want_field)
         FMM_TRY(side_stream(t));
         FMM_TRY(cuda_check(t, cudaEventRecord(t->ev_lists, st), "event"));
     }
+    cudaMemsetAsync(t->b_L.ptr, 0, 8 * (size_t)nc * tb.nLh, st);   // here, so that the kernels follow one another
     FMM_TRY(run_upward(t, tb, true));
     double *M = (double *)t->b_M.ptr, *L = (double *)t->b_L.ptr;
     const int32_t *leaves = (const int32_t *)t->b_leaves.ptr;
@@ -1126,7 +1132,6 @@ fmm_status run_expansions(fmm_tree *t, int p, int want_phi, int want_field)
     const double *centre = (const double *)t->b_centre.ptr;
     const double *px = (const double *)t->b_px.ptr, *py = (const double *)t->b_py.ptr,
                  *pz = (const double *)t->b_pz.ptr;
-    cudaMemsetAsync(L, 0, 8 * (size_t)nc * tb.nLh, st);
     if (fx) {
         if (side) {
             cudaStreamWaitEvent(t->side_st, t->ev_lists, 0);
@@ -1166,7 +1171,7 @@ fmm_status run_expansions(fmm_tree *t, int p, int want_phi, int want_field)
         size_t fixed = 8 * (size_t)tb.m2l_slots * kM2LThreads + 4 * (size_t)tb.m2l_T * kM2LThreads;
         size_t smem = fixed + 8 * (size_t)kM2LBatch * (ldM + ldD);
         allow_max_dynamic_smem(k_m2l);
-        k_m2l<<<(unsigned)nc, kM2LThreads, smem, st>>>(
+        launch_next(st, k_m2l, (unsigned)nc, kM2LThreads, smem, 
             (const int32_t *)t->b_m2l_off.ptr, (const int32_t *)t->b_m2l_src.ptr,
             (const int32_t *)t->b_m2l_didx.ptr, (const int32_t *)t->b_level.ptr,
             (const int32_t *)t->b_sys.ptr, t->sys_eside_dev(), Ms, (const double *)t->b_D.ptr, tb, L);
@@ -1176,9 +1181,8 @@ fmm_status run_expansions(fmm_tree *t, int p, int want_phi, int want_field)
     // L2L downward, all levels in one launch (flags and claim counter start at zero)
     if (t->nlevels > 1) {
         unsigned *ctl = (unsigned *)t->b_ud.ptr + nc + 1;
-        cudaMemsetAsync(ctl, 0, 4 * (size_t)(nc + 1), st);
         size_t smem = 8 * (size_t)(3 * P1 + 2 * tb.nL);
-        k_downward<<<(unsigned)nc, 128, smem, st>>>(nc, (const int32_t *)t->b_parent.ptr, centre, tb, L, ctl);
+        launch_next(st, k_downward, (unsigned)nc, 128, smem, nc, (const int32_t *)t->b_parent.ptr, centre, tb, L, ctl);
         ++t->launches;
     }
     record(t, 10);
@@ -1186,7 +1190,7 @@ fmm_status run_expansions(fmm_tree *t, int p, int want_phi, int want_field)
     {
         const size_t smem = 32 * (size_t)(want_phi ? tb.nL : tb.nG) + 8 * (size_t)tb.nL;
         auto go = [&](auto kern) {
-            kern<<<(unsigned)t->nleaves, kL2PThreads, smem, st>>>(leaves, begin, end, centre, px, py, pz, L, tb,
+            launch_next(st, kern, (unsigned)t->nleaves, kL2PThreads, smem, leaves, begin, end, centre, px, py, pz, L, tb,
                                                                   (double *)t->b_phi.ptr, (double *)t->b_E.ptr);
         };
         if (want_phi && want_field) go(k_l2p<true, true>);

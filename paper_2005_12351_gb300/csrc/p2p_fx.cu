@@ -376,6 +376,7 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
          const double *Sm, const double *phi_far, const double *E_far, const int32_t *perm, double *phi_out,
          double *E_out)
 {
+    pdl_wait();
     using Rec = FxRec<SLO, SHI, PHI, FIELD>;
     constexpr int nS = Orders<SLO, SHI>::n;
     constexpr int NC = (PHI ? 1 : 0) + (FIELD ? 3 : 0);
@@ -625,7 +626,7 @@ void launch_fx(fmm_tree *t, int want_phi, int want_field, double *phi, double *E
         const size_t smem = 8 * (size_t)nc * nthr +
                             std::max<size_t>(16 * (size_t)nw * ch, 32 * (size_t)nc * nthr);
         allow_max_dynamic_smem(kern);
-        kern<<<(unsigned)t->nleaves, nthr, smem, t->stream>>>(
+        launch_next(t->stream, kern, (unsigned)t->nleaves, nthr, smem, 
             (const int32_t *)t->b_leaves.ptr, (const int32_t *)t->b_begin.ptr, (const int32_t *)t->b_end.ptr,
             (const int32_t *)t->b_p2p_off.ptr, (const int32_t *)t->b_p2p_src.ptr, (const int32_t *)t->b_level.ptr,
             (const int32_t *)t->b_cx.ptr, (const int32_t *)t->b_cy.ptr, (const int32_t *)t->b_cz.ptr,

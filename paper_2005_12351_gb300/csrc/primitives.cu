@@ -111,6 +111,7 @@ __global__ void __launch_bounds__(kSortThreads)
 k_os_hist(const uint64_t *keys, int64_t n, int passes, uint32_t *ghist, uint64_t *status0,
           int64_t ntiles)
 {
+    pdl_wait();
     __shared__ uint32_t h[kRadixMaxPasses][256];
     for (int p = 0; p < passes; ++p) h[p][threadIdx.x] = 0;
     // zero the status words of the first pass (the pass k scatter zeroes those of pass k + 1)
@@ -140,6 +141,7 @@ k_os_scatter(const uint64_t *keys, const uint32_t *vals, uint64_t *okeys, uint32
              int64_t n, int pass, int passes, const uint32_t *ghist, unsigned *tile_ctr,
              uint64_t *status, uint64_t *status_next, int *err, int max_polls)
 {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char os_smem[];
     uint64_t *sk = (uint64_t *)os_smem;                               // [kSortTile]
     uint32_t *sv = (uint32_t *)(sk + kSortTile);                      // [kSortTile]
@@ -325,7 +327,7 @@ static void scatter_passes(uint64_t *&ka, uint32_t *&va, uint64_t *&kb, uint32_t
     int max_polls = kOsWait;
     if (const char *env = getenv("FMM_SORT_POLLS")) max_polls = std::max(0, atoi(env));
     for (int p = p0, q = 0; p < passes; ++p, ++q) {
-        k_os_scatter<<<(unsigned)ntiles, kSortThreads, kOsSmem, st>>>(
+        launch_next(st, k_os_scatter, (unsigned)ntiles, kSortThreads, kOsSmem, 
             ka, va, kb, vb, n, p, passes, ghist, ctr, status[q & 1], status[(q + 1) & 1], err, max_polls);
         ++*launches;
         std::swap(ka, kb);
@@ -352,7 +354,7 @@ void radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys2, uint32_t 
         cudaMemsetAsync(hist, 0, 4 * (size_t)kRadixHead, st);
         const unsigned hgrid = (unsigned)std::min<int64_t>((n + kSortThreads - 1) / kSortThreads,
                                                            4 * (int64_t)sm_count());
-        k_os_hist<<<hgrid, kSortThreads, 0, st>>>(keys, n, passes, hist, (uint64_t *)(hist + kRadixHead), ntiles);
+        launch_next(st, k_os_hist, hgrid, kSortThreads, 0, keys, n, passes, hist, (uint64_t *)(hist + kRadixHead), ntiles);
         ++*launches;
     }
     uint64_t *ka = keys, *kb = keys2;

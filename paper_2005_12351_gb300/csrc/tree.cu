@@ -44,6 +44,7 @@ __global__ void k_sort_init(unsigned long long *box, uint32_t *hist)
 
 __global__ void k_bbox(const double *pos, int64_t n, unsigned long long *box, int *err)
 {
+    pdl_wait();
     unsigned long long mn[3] = {~0ull, ~0ull, ~0ull}, mx[3] = {0ull, 0ull, 0ull};
     bool bad = false;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -137,6 +138,7 @@ __global__ void __launch_bounds__(256)
 k_keys(const double *pos, int64_t n, const unsigned long long *raw_box, double *box_out, uint64_t *keys,
        uint32_t *idx, int p0, uint32_t *ghist, uint64_t *status0, int64_t nstatus)
 {
+    pdl_wait();
     __shared__ uint32_t h[kRadixMaxPasses][256];
     __shared__ double box[4];
     for (int p = p0; p < kRadixMaxPasses; ++p) h[p][threadIdx.x] = 0;
@@ -185,6 +187,7 @@ k_tie_sort(const uint64_t *keys, const uint32_t *idx, int64_t n, int shift, uint
            const double *pos, const double *mom, int nS, double *px, double *py, double *pz, double *S,
            int32_t *perm_out)
 {
+    pdl_wait();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const uint64_t key = keys[i], top = key >> shift;
@@ -346,6 +349,7 @@ __global__ void k_regather_keys(const uint64_t *key_of, const uint32_t *idx, int
 __global__ void k_gather(const double *pos, const double *mom, int nS, const uint32_t *perm,
                          int64_t n, double *px, double *py, double *pz, double *S, int32_t *perm_out)
 {
+    pdl_wait();
     int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= n) return;
     const int64_t o = perm[k];
@@ -363,6 +367,7 @@ struct CellArrays {
 // the traversal's start: counters and row counts zero, one (root, root) pair per system
 __global__ void k_list_init(unsigned *cnt, int ncnt, unsigned *rows, int64_t nrows, int2 *front, int nsys, int nf0)
 {
+    pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     for (int64_t i = i0; i < ncnt; i += stride) cnt[i] = i == nf0 ? (unsigned)nsys : 0u;
     for (int64_t i = i0; i < nrows; i += stride) rows[i] = 0u;
@@ -673,6 +678,7 @@ k_traverse_round(const int4 *__restrict__ tc, int round, double theta2, const in
                  int2 *p2p, uint32_t *slot_p2p, unsigned *rows_p2p, unsigned p2p_cap, int2 *next,
                  unsigned *counters)
 {
+    pdl_wait();
     // the frontier size and the overflow flag, read once per block so that the
     // whole block takes the same way (the loop below has block barriers)
     __shared__ unsigned s_nf, s_stop;
@@ -816,6 +822,7 @@ struct ListArgs {
 };
 __global__ void k_list_scatter(const ListArgs m, const ListArgs p)
 {
+    pdl_wait();
     int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const bool second = k >= m.np;
     const ListArgs &l = second ? p : m;
@@ -933,6 +940,7 @@ k_row_sort(const uint32_t *m2l_off, int32_t *m2l_src, const uint32_t *p2p_off, i
            const int32_t *cbeg, const int32_t *cend, unsigned long long *inter, uint32_t *long_rows,
            unsigned *n_long, int warp_max)
 {
+    pdl_wait();
     __shared__ uint32_t buf[8][kRowWarpMax];
     if (blockIdx.y == 0)
         row_sort<false>(buf, m2l_off, m2l_src, nrows, cbeg, cend, nullptr, long_rows, n_long, warp_max);
@@ -947,6 +955,7 @@ __global__ void __launch_bounds__(1024)
 k_row_sort_long(const uint32_t *m2l_off, int32_t *m2l_src, const uint32_t *p2p_off, int32_t *p2p_src,
                 int64_t nrows, const uint32_t *long_rows, const unsigned *n_long, int *err, int block_max)
 {
+    pdl_wait();
     __shared__ uint32_t v[kRowBlockMax];
     const uint32_t *off = blockIdx.y ? p2p_off : m2l_off;
     int32_t *src = blockIdx.y ? p2p_src : m2l_src;
@@ -1035,6 +1044,7 @@ __global__ void k_offset_keys(CellArrays c, const int32_t *off, const int32_t *s
                               uint64_t *new_key, uint32_t *new_slot, unsigned *n_new, int *err,
                               unsigned *max_gap)
 {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; a < nrows; a += nwarps) {
@@ -1093,6 +1103,7 @@ constexpr unsigned kRankSmall = 4096;
 __global__ void __launch_bounds__(256)
 k_rank_keys(const uint64_t *key, const uint32_t *slot, const unsigned *n_keys, uint64_t *keys_out, uint32_t *rank_of)
 {
+    pdl_wait();
     const unsigned n = *n_keys;
     if (n > kRankSmall) return;
     const unsigned lane = threadIdx.x & 31, nw = gridDim.x * (blockDim.x >> 5);
@@ -1119,6 +1130,7 @@ __global__ void k_rank_sorted(const uint32_t *slot, int64_t n, uint32_t *rank_of
 __global__ void k_slot_to_rank(int32_t *didx, int64_t np, const uint32_t *rank_of, const unsigned *n_keys,
                                unsigned max_keys)
 {
+    pdl_wait();
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (*n_keys <= max_keys && k < np) didx[k] = (int32_t)rank_of[didx[k]];
 }
@@ -1178,9 +1190,9 @@ static void morton_keys(cudaStream_t st, const double *pos, int64_t n, int p0, u
 {
     const unsigned g = (unsigned)std::min<int64_t>(grid(n, 256), 4 * (int64_t)sm_count());
     k_sort_init<<<1, 256, 0, st>>>(box_scratch, hist);
-    k_bbox<<<g, 256, 0, st>>>(pos, n, box_scratch, err);
+    launch_next(st, k_bbox, g, 256, 0, pos, n, box_scratch, err);
     const int64_t ntiles = (n + kRadixTile - 1) / kRadixTile;
-    k_keys<<<g, 256, 0, st>>>(pos, n, box_scratch, box_out, keys, idx, p0, hist, (uint64_t *)(hist + kRadixHead),
+    launch_next(st, k_keys, g, 256, 0, pos, n, box_scratch, box_out, keys, idx, p0, hist, (uint64_t *)(hist + kRadixHead),
                               ntiles * 256);
     *launches += 3;
 }
@@ -1212,7 +1224,7 @@ fmm_status morton_order_raw(cudaStream_t st, const double *pos, int64_t n, uint6
     }
     morton_keys(st, pos, n, p0, ka, va, box_scratch, box_out, err, hist, &launches);
     radix_sort_top(ka, va, kb, vb, n, p0, hist, err, st, &launches);
-    k_tie_sort<false><<<grid(n, 256), 256, 0, st>>>(keys2, idx2, n, 8 * p0, keys, idx, err, nullptr, nullptr, 0,
+    launch_next(st, k_tie_sort<false>, grid(n, 256), 256, 0, keys2, idx2, n, 8 * p0, keys, idx, err, nullptr, nullptr, 0,
                                                      nullptr, nullptr, nullptr, nullptr, nullptr);
     cudaError_t e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -1281,9 +1293,9 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
         record(t, 1);
         radix_sort_top(ka, va, kb, vb, n, p0, hist, err, st, &t->launches);
         if (full)
-            k_gather<<<grid(n, 256), 256, 0, st>>>(pos, mom, t->nS, idx, n, px, py, pz, S, perm);
+            launch_next(st, k_gather, grid(n, 256), 256, 0, pos, mom, t->nS, idx, n, px, py, pz, S, perm);
         else
-            k_tie_sort<true><<<grid(n, 256), 256, 0, st>>>(keys2, idx2, n, 8 * p0, keys, idx, err, pos, mom, t->nS,
+            launch_next(st, k_tie_sort<true>, grid(n, 256), 256, 0, keys2, idx2, n, 8 * p0, keys, idx, err, pos, mom, t->nS,
                                                             px, py, pz, S, perm);
         ++t->launches;
         record(t, 2);
@@ -1315,7 +1327,7 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
         radix_sort_pairs(skeys, idx, (uint64_t *)t->b_keys2.ptr, (uint32_t *)t->b_idx2.ptr, n,
                          sbits, (uint32_t *)t->b_hist.ptr, (int *)t->b_err.ptr, st, &t->launches);
         k_regather_keys<<<grid(n, 256), 256, 0, st>>>(key_of, idx, n, keys);
-        k_gather<<<grid(n, 256), 256, 0, st>>>(pos, mom, t->nS, idx, n, (double *)t->b_px.ptr,
+        launch_next(st, k_gather, grid(n, 256), 256, 0, pos, mom, t->nS, idx, n, (double *)t->b_px.ptr,
                                                (double *)t->b_py.ptr, (double *)t->b_pz.ptr,
                                                (double *)t->b_S.ptr, (int32_t *)t->b_perm.ptr);
         t->launches += 3;
@@ -1422,8 +1434,7 @@ fmm_status build_lists(fmm_tree *t, double theta)
         p2p_cap = t->b_p2p_raw.bytes / 8;
         front_cap = std::min(t->b_front.bytes, t->b_front2.bytes) / 8;
         int2 *fr[2] = {(int2 *)t->b_front.ptr, (int2 *)t->b_front2.ptr};
-        k_list_init<<<(unsigned)std::min<int64_t>(grid(std::max<int64_t>(2 * (nc + 1), nsys), 256), 2 * (int64_t)sm_count()),
-                      256, 0, st>>>(cnt, kTravFront + kTravMaxRounds + 1, rows, 2 * (nc + 1), fr[0], nsys, kTravFront);
+        launch_next(st, k_list_init, (unsigned)std::min<int64_t>(grid(std::max<int64_t>(2 * (nc + 1), nsys), 256), 2 * (int64_t)sm_count()), 256, 0, cnt, kTravFront + kTravMaxRounds + 1, rows, 2 * (nc + 1), fr[0], nsys, kTravFront);
         ++t->launches;
         int r = 0;
         bool retry = false;
@@ -1431,7 +1442,7 @@ fmm_status build_lists(fmm_tree *t, double theta)
         for (;;) {
             const int end = std::min(r + batch, kTravMaxRounds);
             for (; r < end; ++r) {
-                k_traverse_round<<<trav_blocks, 256, 0, st>>>(
+                launch_next(st, k_traverse_round, trav_blocks, 256, 0, 
                     (const int4 *)t->b_tcell.ptr, r, theta2, fr[r & 1], (unsigned)front_cap,
                     (int2 *)t->b_m2l_raw.ptr, (uint32_t *)t->b_m2l_slot.ptr, rows, (unsigned)m2l_cap,
                     (int2 *)t->b_p2p_raw.ptr, (uint32_t *)t->b_p2p_slot.ptr, rows + nc + 1,
@@ -1515,13 +1526,13 @@ fmm_status build_lists(fmm_tree *t, double theta)
                              (const uint32_t *)m2l_off, m2l_src};
         const ListArgs lp = {(const int2 *)t->b_p2p_raw.ptr, (const uint32_t *)t->b_p2p_slot.ptr, np2p,
                              (const uint32_t *)p2p_off, p2p_src};
-        if (nm2l + np2p > 0) k_list_scatter<<<grid(nm2l + np2p, 256), 256, 0, st>>>(lm, lp);
+        if (nm2l + np2p > 0) launch_next(st, k_list_scatter, grid(nm2l + np2p, 256), 256, 0, lm, lp);
         uint32_t *lq = (uint32_t *)t->b_long.ptr;
         const unsigned rgrid = (unsigned)std::min<int64_t>((nc + 7) / 8, 6 * (int64_t)sm_count());
-        k_row_sort<<<dim3(rgrid, 2), 256, 0, st>>>((const uint32_t *)m2l_off, m2l_src, (const uint32_t *)p2p_off,
+        launch_next(st, k_row_sort, dim3(rgrid, 2), 256, 0, (const uint32_t *)m2l_off, m2l_src, (const uint32_t *)p2p_off,
                                                     p2p_src, nc, c.begin, c.end, inter_d, lq, n_long,
                                                     std::min(row_lim, kRowWarpMax));
-        k_row_sort_long<<<dim3((unsigned)sm_count(), 2), 1024, 0, st>>>((const uint32_t *)m2l_off, m2l_src,
+        launch_next(st, k_row_sort_long, dim3((unsigned)sm_count(), 2), 1024, 0, (const uint32_t *)m2l_off, m2l_src,
                                                                          (const uint32_t *)p2p_off, p2p_src, nc, lq,
                                                                          n_long, long_err, row_lim);
         t->launches += 3;
@@ -1575,12 +1586,12 @@ fmm_status build_lists(fmm_tree *t, double theta)
             uint32_t *lslot = (uint32_t *)(lkey + H), *rank_of = (uint32_t *)t->b_scan.ptr;
             cudaMemsetAsync(t->b_hash.ptr, 0xff, 8 * (size_t)H, st);
             if (again) cudaMemsetAsync(cnt + 10, 0, 4 * 4, st);   // errors, gap, count
-            k_offset_keys<<<(unsigned)std::min<int64_t>((nc + 7) / 8, 8 * (int64_t)sm_count()), 256, 0, st>>>(
+            launch_next(st, k_offset_keys, (unsigned)std::min<int64_t>((nc + 7) / 8, 8 * (int64_t)sm_count()), 256, 0, 
                 c, m2l_off, m2l_src, nc, (unsigned long long *)t->b_hash.ptr, H - 1,
                 (uint32_t *)t->b_m2l_didx.ptr, lkey, lslot, cnt + 13, (int *)(cnt + 10), cnt + 12);
-            k_rank_keys<<<(unsigned)sm_count(), 256, 0, st>>>(lkey, lslot, cnt + 13, (uint64_t *)t->b_dkeys.ptr,
+            launch_next(st, k_rank_keys, (unsigned)sm_count(), 256, 0, lkey, lslot, cnt + 13, (uint64_t *)t->b_dkeys.ptr,
                                                               rank_of);
-            k_slot_to_rank<<<grid(nm2l, 256), 256, 0, st>>>((int32_t *)t->b_m2l_didx.ptr, nm2l, rank_of, cnt + 13,
+            launch_next(st, k_slot_to_rank, grid(nm2l, 256), 256, 0, (int32_t *)t->b_m2l_didx.ptr, nm2l, rank_of, cnt + 13,
                                                             kRankSmall);
             t->launches += 3;
             FMM_TRY(read_words());
@@ -1608,7 +1619,7 @@ fmm_status build_lists(fmm_tree *t, double theta)
             radix_sort_pairs(lkey, lslot, (uint64_t *)t->b_lkeys2.ptr, (uint32_t *)t->b_lval2.ptr, ndoff, 57,
                              (uint32_t *)t->b_dsort_h.ptr, sort_err, st, &t->launches);
             k_rank_sorted<<<grid(ndoff, 256), 256, 0, st>>>(lslot, ndoff, rank_of);
-            k_slot_to_rank<<<grid(nm2l, 256), 256, 0, st>>>((int32_t *)t->b_m2l_didx.ptr, nm2l, rank_of, cnt + 13, ~0u);
+            launch_next(st, k_slot_to_rank, grid(nm2l, 256), 256, 0, (int32_t *)t->b_m2l_didx.ptr, nm2l, rank_of, cnt + 13, ~0u);
             t->launches += 2;
             FMM_TRY(cuda_check(t, cudaMemcpyAsync(t->b_dkeys.ptr, lkey, 8 * (size_t)ndoff, cudaMemcpyDeviceToDevice, st),
                                "offset keys"));
