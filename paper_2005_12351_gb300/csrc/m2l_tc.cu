@@ -559,45 +559,6 @@ __global__ void k_tc_tiles(int T, int slots, const uint32_t *vals, int32_t *tile
     if (q < slots) tile_tgt[q] = q < T ? (int32_t)vals[q] : -1;
 }
 
-// The key set of each tile as a bitmap.  One block per tile: the set in
-// shared memory, then written out whole (no memset, no global atomics).
-constexpr int kTcBitsSmemMax = 96 * 1024;
-__global__ void __launch_bounds__(256) k_tc_bits_tile(int T, const int32_t *tile_tgt, const int32_t *m2l_off,
-                                                      const int32_t *didx, int W, uint32_t *bits)
-{
-    extern __shared__ uint32_t sb[];            // [W]
-    const int tile = blockIdx.x;
-    for (int i = threadIdx.x; i < W; i += blockDim.x) sb[i] = 0u;
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    for (int r = threadIdx.x >> 5; r < 128; r += blockDim.x >> 5) {
-        const int w = tile * 128 + r;
-        if (w >= T) break;
-        const int c = tile_tgt[w];
-        for (int e = m2l_off[c] + lane; e < m2l_off[c + 1]; e += 32) {
-            const int d = didx[e];
-            atomicOr(&sb[d >> 5], 1u << (d & 31));
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < W; i += blockDim.x) bits[(size_t)tile * W + i] = sb[i];
-}
-
-// The same with global atomics (one warp per target marks the keys of its
-// list), for key sets too large for shared memory.
-__global__ void k_tc_bits(int T, const int32_t *tile_tgt, const int32_t *m2l_off, const int32_t *didx, int W,
-                          uint32_t *bits)
-{
-    const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (w >= T) return;
-    const int c = tile_tgt[w];
-    uint32_t *tb = bits + (size_t)(w >> 7) * W;
-    for (int e = m2l_off[c] + lane; e < m2l_off[c + 1]; e += 32) {
-        const int d = didx[e];
-        atomicOr(tb + (d >> 5), 1u << (d & 31));
-    }
-}
-
 // block-wide exclusive scan of one value per thread (256 threads); returns the block total
 __device__ __forceinline__ uint32_t block_scan256(uint32_t v, uint32_t &excl)
 {
@@ -619,6 +580,66 @@ __device__ __forceinline__ uint32_t block_scan256(uint32_t v, uint32_t &excl)
     excl = before + x - v;
     __syncthreads();
     return total;
+}
+
+// The targets of each tile and its key set as a bitmap, with the counts that
+// number its rows.  One block per tile: the set in shared memory, then written
+// out whole (no memset, no global atomics).  As three kernels and four clears the
+// plan of a 12k set, which its M2L waits for, took 15 us longer.
+constexpr int kTcBitsSmemMax = 96 * 1024;
+__global__ void __launch_bounds__(256) k_tc_bits_tile(int T, const uint32_t *vals, int32_t *tile_tgt,
+                                                      const int32_t *m2l_off, const int32_t *didx, int W, int G,
+                                                      uint32_t *bits, uint32_t *wpre, uint32_t *tile_rows,
+                                                      uint32_t *tile_chunks)
+{
+    pdl_wait();
+    extern __shared__ uint32_t sb[];            // [W]
+    const int tile = blockIdx.x;
+    for (int i = threadIdx.x; i < W; i += blockDim.x) sb[i] = 0u;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int r = threadIdx.x >> 5; r < 128; r += blockDim.x >> 5) {
+        const int w = tile * 128 + r, c = w < T ? (int)vals[w] : -1;
+        if (lane == 0) tile_tgt[w] = c;
+        if (c < 0) continue;
+        for (int e = m2l_off[c] + lane; e < m2l_off[c + 1]; e += 32) {
+            const int d = didx[e];
+            atomicOr(&sb[d >> 5], 1u << (d & 31));
+        }
+    }
+    __syncthreads();
+    uint32_t carry = 0;
+    for (int base = 0; base < W; base += 256) {
+        const int w = base + threadIdx.x;
+        const uint32_t v = w < W ? sb[w] : 0u;
+        uint32_t ex;
+        const uint32_t tot = block_scan256((uint32_t)__popc(v), ex);
+        if (w < W) {
+            bits[(size_t)tile * W + w] = v;
+            wpre[(size_t)tile * W + w] = carry + ex;
+        }
+        carry += tot;
+    }
+    if (threadIdx.x == 0) {
+        tile_rows[tile] = carry;
+        tile_chunks[tile] = (carry + G - 1) / G;
+        if (tile + 1 == (int)gridDim.x) tile_rows[tile + 1] = tile_chunks[tile + 1] = 0u;     // totals of the scans
+    }
+}
+
+// The same with global atomics (one warp per target marks the keys of its
+// list), for key sets too large for shared memory.
+__global__ void k_tc_bits(int T, const int32_t *tile_tgt, const int32_t *m2l_off, const int32_t *didx, int W,
+                          uint32_t *bits)
+{
+    const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (w >= T) return;
+    const int c = tile_tgt[w];
+    uint32_t *tb = bits + (size_t)(w >> 7) * W;
+    for (int e = m2l_off[c] + lane; e < m2l_off[c + 1]; e += 32) {
+        const int d = didx[e];
+        atomicOr(tb + (d >> 5), 1u << (d & 31));
+    }
 }
 
 // per tile: rows = keys present; prefix of the per-word counts
@@ -644,6 +665,7 @@ __global__ void __launch_bounds__(256) k_tc_rowcount(int W, int G, const uint32_
 __global__ void k_tc_rows(int W, int G, const uint32_t *bits, const uint32_t *wpre, const uint32_t *row_off,
                           const uint32_t *chunk_off, int32_t *row_key, int32_t *chunk_rb, int32_t *chunk_re)
 {
+    pdl_wait();
     const int tile = blockIdx.x;
     const uint32_t rb = row_off[tile], re = row_off[tile + 1];
     for (int w = threadIdx.x; w < W; w += blockDim.x) {
@@ -668,6 +690,7 @@ __global__ void k_tc_slots(int T, const int32_t *tile_tgt, const int32_t *m2l_of
                            const int32_t *didx, int W, const uint32_t *bits, const uint32_t *wpre,
                            const uint32_t *row_off, int32_t *slot)
 {
+    pdl_wait();
     const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (w >= T) return;
     const int c = tile_tgt[w], tile = w >> 7;
@@ -853,35 +876,37 @@ fmm_status build_plan(fmm_tree *t)
     const int64_t tiles = t->tc_tiles, W = (t->n_doff + 31) / 32;
     t->tc_W = W;
     FMM_TRY(ensure(t, t->b_tc_tgt, 4 * (size_t)tiles * 128));
-    k_tc_tiles<<<gridn(tiles * 128, 256), 256, 0, st>>>((int)T, (int)(tiles * 128),
-                                                         (const uint32_t *)t->b_tc_vals.ptr,
-                                                         (int32_t *)t->b_tc_tgt.ptr);
     FMM_TRY(ensure(t, t->b_tc_bits, 4 * (size_t)tiles * W));
     FMM_TRY(ensure(t, t->b_tc_wpre, 4 * (size_t)tiles * W));
+    for (DevBuf *b : {&t->b_tc_rcnt, &t->b_tc_ccnt, &t->b_tc_roff, &t->b_tc_coff})
+        FMM_TRY(ensure(t, *b, 4 * (size_t)(tiles + 1)));
+    uint32_t *rcnt = (uint32_t *)t->b_tc_rcnt.ptr, *ccnt = (uint32_t *)t->b_tc_ccnt.ptr;
     if (4 * W <= kTcBitsSmemMax) {
         allow_max_dynamic_smem(k_tc_bits_tile);
-        k_tc_bits_tile<<<(unsigned)tiles, 256, 4 * (size_t)W, st>>>(
-            (int)T, (const int32_t *)t->b_tc_tgt.ptr, (const int32_t *)t->b_m2l_off.ptr,
-            (const int32_t *)t->b_m2l_didx.ptr, (int)W, (uint32_t *)t->b_tc_bits.ptr);
+        launch_next(st, k_tc_bits_tile, (unsigned)tiles, 256, 4 * (size_t)W, (int)T,
+                    (const uint32_t *)t->b_tc_vals.ptr, (int32_t *)t->b_tc_tgt.ptr, (const int32_t *)t->b_m2l_off.ptr,
+                    (const int32_t *)t->b_m2l_didx.ptr, (int)W, G, (uint32_t *)t->b_tc_bits.ptr,
+                    (uint32_t *)t->b_tc_wpre.ptr, rcnt, ccnt);
     } else {
+        k_tc_tiles<<<gridn(tiles * 128, 256), 256, 0, st>>>((int)T, (int)(tiles * 128),
+                                                             (const uint32_t *)t->b_tc_vals.ptr,
+                                                             (int32_t *)t->b_tc_tgt.ptr);
         cudaMemsetAsync(t->b_tc_bits.ptr, 0, 4 * (size_t)tiles * W, st);
         k_tc_bits<<<gridn((int64_t)T * 32, 256), 256, 0, st>>>((int)T, (const int32_t *)t->b_tc_tgt.ptr,
                                                                 (const int32_t *)t->b_m2l_off.ptr,
                                                                 (const int32_t *)t->b_m2l_didx.ptr, (int)W,
                                                                 (uint32_t *)t->b_tc_bits.ptr);
+        cudaMemsetAsync(rcnt + tiles, 0, 4, st);
+        cudaMemsetAsync(ccnt + tiles, 0, 4, st);
+        k_tc_rowcount<<<(unsigned)tiles, 256, 0, st>>>((int)W, G, (const uint32_t *)t->b_tc_bits.ptr,
+                                                       (uint32_t *)t->b_tc_wpre.ptr, rcnt, ccnt);
+        t->launches += 2;
     }
-    for (DevBuf *b : {&t->b_tc_rcnt, &t->b_tc_ccnt, &t->b_tc_roff, &t->b_tc_coff}) {
-        FMM_TRY(ensure(t, *b, 4 * (size_t)(tiles + 1)));
-        cudaMemsetAsync(b->ptr, 0, 4 * (size_t)(tiles + 1), st);
-    }
-    k_tc_rowcount<<<(unsigned)tiles, 256, 0, st>>>((int)W, G, (const uint32_t *)t->b_tc_bits.ptr,
-                                                   (uint32_t *)t->b_tc_wpre.ptr, (uint32_t *)t->b_tc_rcnt.ptr,
-                                                   (uint32_t *)t->b_tc_ccnt.ptr);
     exclusive_scan_u32((const uint32_t *)t->b_tc_rcnt.ptr, (uint32_t *)t->b_tc_roff.ptr, tiles + 1,
                        (uint32_t *)t->b_tc_scan.ptr, st, &t->launches);
     exclusive_scan_u32((const uint32_t *)t->b_tc_ccnt.ptr, (uint32_t *)t->b_tc_coff.ptr, tiles + 1,
                        (uint32_t *)t->b_tc_scan.ptr, st, &t->launches);
-    t->launches += 4;
+    t->launches += 1;
     uint32_t R = 0, C = 0;
     FMM_TRY(cuda_check(t, cudaMemcpyAsync(&R, (const uint32_t *)t->b_tc_roff.ptr + tiles, 4,
                                           cudaMemcpyDeviceToHost, st), "copy"));
@@ -891,14 +916,14 @@ fmm_status build_plan(fmm_tree *t)
     FMM_TRY(ensure(t, t->b_tc_rowkey, 4 * (size_t)R));
     FMM_TRY(ensure(t, t->b_tc_crb, 4 * (size_t)C));
     FMM_TRY(ensure(t, t->b_tc_cre, 4 * (size_t)C));
+    FMM_TRY(ensure(t, t->b_tc_slot, 4 * (size_t)R * 128));
+    cudaMemsetAsync(t->b_tc_slot.ptr, 0xff, 4 * (size_t)R * 128, st);
     k_tc_rows<<<(unsigned)tiles, 256, 0, st>>>((int)W, G, (const uint32_t *)t->b_tc_bits.ptr,
                                                (const uint32_t *)t->b_tc_wpre.ptr,
                                                (const uint32_t *)t->b_tc_roff.ptr,
                                                (const uint32_t *)t->b_tc_coff.ptr, (int32_t *)t->b_tc_rowkey.ptr,
                                                (int32_t *)t->b_tc_crb.ptr, (int32_t *)t->b_tc_cre.ptr);
-    FMM_TRY(ensure(t, t->b_tc_slot, 4 * (size_t)R * 128));
-    cudaMemsetAsync(t->b_tc_slot.ptr, 0xff, 4 * (size_t)R * 128, st);
-    k_tc_slots<<<gridn((int64_t)T * 32, 256), 256, 0, st>>>(
+    launch_next(st, k_tc_slots, gridn((int64_t)T * 32, 256), 256, 0,
         (int)T, (const int32_t *)t->b_tc_tgt.ptr, (const int32_t *)t->b_m2l_off.ptr,
         (const int32_t *)t->b_m2l_src.ptr, (const int32_t *)t->b_m2l_didx.ptr, (int)W,
         (const uint32_t *)t->b_tc_bits.ptr, (const uint32_t *)t->b_tc_wpre.ptr, (const uint32_t *)t->b_tc_roff.ptr,
@@ -918,7 +943,7 @@ fmm_status tc_build_plan(fmm_tree *t)
 void launch_tc_reduce(fmm_tree *t, int Np, int ncol, const int32_t *col_n, int nL, const DevTables &tb,
                       const unsigned *err, float *L)
 {
-    launch_next(t->stream, k_tc_reduce, (unsigned)((t->tc_T + kReduceWarps - 1) / kReduceWarps), 32 * kReduceWarps, 0, 
+    launch_next(t->stream, k_tc_reduce, (unsigned)((t->tc_T + kReduceWarps - 1) / kReduceWarps), 32 * kReduceWarps, 0,
         (int)t->tc_T, (const int32_t *)t->b_tc_tgt.ptr, (const uint32_t *)t->b_tc_coff.ptr,
         (const float *)t->b_tc_part.ptr, Np, ncol, col_n, nL, tb.nLh, tb.h_rn, err, L);
     ++t->launches;

@@ -1530,7 +1530,7 @@ template <int S>
 void launch_p2p32(fmm_tree *t, int want_phi, int want_field, double *phi, double *E)
 {
     auto go = [&](auto kern) {
-        launch_next(t->stream, kern, (unsigned)t->nleaves, kP2PThreads, 0, 
+        launch_next(t->stream, kern, (unsigned)t->nleaves, kP2PThreads, 0,
             (const int32_t *)t->b_leaves.ptr, (const int32_t *)t->b_begin.ptr,
             (const int32_t *)t->b_end.ptr, (const int32_t *)t->b_p2p_off.ptr,
             (const int32_t *)t->b_p2p_src.ptr, (const int32_t *)t->b_level.ptr,
@@ -1677,7 +1677,7 @@ fmm_status run_mixed(fmm_tree *t, int p, int want_phi, int want_field, double *p
                                            2 * (size_t)tb.nK + 8 * (size_t)tb.nM + 4);
         auto up = [&](auto kern) {
             allow_max_dynamic_smem(kern);
-            launch_next(st, kern, (unsigned)t->nleaves, 128, smem, 
+            launch_next(st, kern, (unsigned)t->nleaves, 128, smem,
                 leaves, begin, end, (const int32_t *)t->b_parent.ptr, (const int32_t *)t->b_child.ptr,
                 (const int32_t *)t->b_nchild.ptr, cx, cy, cz, half, (const double *)t->b_centre.ptr,
                 (const double *)t->b_px.ptr, (const double *)t->b_py.ptr, (const double *)t->b_pz.ptr,
@@ -1750,7 +1750,7 @@ fmm_status run_mixed(fmm_tree *t, int p, int want_phi, int want_field, double *p
         }
         const size_t smem = std::max(smem_l2l, smem_l2p);
         allow_max_dynamic_smem(k_downward32_leaf);
-        launch_next(st, k_downward32_leaf, (unsigned)t->nleaves, 128, smem, 
+        launch_next(st, k_downward32_leaf, (unsigned)t->nleaves, 128, smem,
             leaves, parent, cx, cy, cz, tb, L, begin, end, half, o, want_phi, want_field, (double *)t->b_phi.ptr,
             (double *)t->b_E.ptr);
         ++t->launches;
@@ -1758,7 +1758,7 @@ fmm_status run_mixed(fmm_tree *t, int p, int want_phi, int want_field, double *p
     } else {
         record(t, 10);
         allow_max_dynamic_smem(k_l2p32);
-        launch_next(st, k_l2p32, (unsigned)t->nleaves, kL2PThreads, smem_l2p, 
+        launch_next(st, k_l2p32, (unsigned)t->nleaves, kL2PThreads, smem_l2p,
             leaves, begin, end, half, o, L, tb, want_phi, want_field, (double *)t->b_phi.ptr,
             (double *)t->b_E.ptr);
         ++t->launches;

@@ -1078,7 +1078,7 @@ fmm_status run_upward(fmm_tree *t, const DevTables &tb, bool rec)
         6 * (size_t)P1 + 12 * (size_t)tb.nM);
     auto go = [&](auto kern) {
         allow_max_dynamic_smem(kern);
-        launch_next(st, kern, (unsigned)t->nleaves, kP2MThreads, smem, 
+        launch_next(st, kern, (unsigned)t->nleaves, kP2MThreads, smem,
             (const int32_t *)t->b_leaves.ptr, (const int32_t *)t->b_begin.ptr,
             (const int32_t *)t->b_end.ptr, (const int32_t *)t->b_parent.ptr,
             (const int32_t *)t->b_child.ptr, (const int32_t *)t->b_nchild.ptr, (const int32_t *)t->b_cx.ptr,
@@ -1171,7 +1171,7 @@ fmm_status run_expansions(fmm_tree *t, int p, int want_phi, int want_field)
         size_t fixed = 8 * (size_t)tb.m2l_slots * kM2LThreads + 4 * (size_t)tb.m2l_T * kM2LThreads;
         size_t smem = fixed + 8 * (size_t)kM2LBatch * (ldM + ldD);
         allow_max_dynamic_smem(k_m2l);
-        launch_next(st, k_m2l, (unsigned)nc, kM2LThreads, smem, 
+        launch_next(st, k_m2l, (unsigned)nc, kM2LThreads, smem,
             (const int32_t *)t->b_m2l_off.ptr, (const int32_t *)t->b_m2l_src.ptr,
             (const int32_t *)t->b_m2l_didx.ptr, (const int32_t *)t->b_level.ptr,
             (const int32_t *)t->b_sys.ptr, t->sys_eside_dev(), Ms, (const double *)t->b_D.ptr, tb, L);

@@ -626,7 +626,7 @@ void launch_fx(fmm_tree *t, int want_phi, int want_field, double *phi, double *E
         const size_t smem = 8 * (size_t)nc * nthr +
                             std::max<size_t>(16 * (size_t)nw * ch, 32 * (size_t)nc * nthr);
         allow_max_dynamic_smem(kern);
-        launch_next(t->stream, kern, (unsigned)t->nleaves, nthr, smem, 
+        launch_next(t->stream, kern, (unsigned)t->nleaves, nthr, smem,
             (const int32_t *)t->b_leaves.ptr, (const int32_t *)t->b_begin.ptr, (const int32_t *)t->b_end.ptr,
             (const int32_t *)t->b_p2p_off.ptr, (const int32_t *)t->b_p2p_src.ptr, (const int32_t *)t->b_level.ptr,
             (const int32_t *)t->b_cx.ptr, (const int32_t *)t->b_cy.ptr, (const int32_t *)t->b_cz.ptr,

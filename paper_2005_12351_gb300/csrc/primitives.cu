@@ -327,7 +327,7 @@ static void scatter_passes(uint64_t *&ka, uint32_t *&va, uint64_t *&kb, uint32_t
     int max_polls = kOsWait;
     if (const char *env = getenv("FMM_SORT_POLLS")) max_polls = std::max(0, atoi(env));
     for (int p = p0, q = 0; p < passes; ++p, ++q) {
-        launch_next(st, k_os_scatter, (unsigned)ntiles, kSortThreads, kOsSmem, 
+        launch_next(st, k_os_scatter, (unsigned)ntiles, kSortThreads, kOsSmem,
             ka, va, kb, vb, n, p, passes, ghist, ctr, status[q & 1], status[(q + 1) & 1], err, max_polls);
         ++*launches;
         std::swap(ka, kb);

@@ -1442,7 +1442,7 @@ fmm_status build_lists(fmm_tree *t, double theta)
         for (;;) {
             const int end = std::min(r + batch, kTravMaxRounds);
             for (; r < end; ++r) {
-                launch_next(st, k_traverse_round, trav_blocks, 256, 0, 
+                launch_next(st, k_traverse_round, trav_blocks, 256, 0,
                     (const int4 *)t->b_tcell.ptr, r, theta2, fr[r & 1], (unsigned)front_cap,
                     (int2 *)t->b_m2l_raw.ptr, (uint32_t *)t->b_m2l_slot.ptr, rows, (unsigned)m2l_cap,
                     (int2 *)t->b_p2p_raw.ptr, (uint32_t *)t->b_p2p_slot.ptr, rows + nc + 1,
@@ -1586,7 +1586,7 @@ fmm_status build_lists(fmm_tree *t, double theta)
             uint32_t *lslot = (uint32_t *)(lkey + H), *rank_of = (uint32_t *)t->b_scan.ptr;
             cudaMemsetAsync(t->b_hash.ptr, 0xff, 8 * (size_t)H, st);
             if (again) cudaMemsetAsync(cnt + 10, 0, 4 * 4, st);   // errors, gap, count
-            launch_next(st, k_offset_keys, (unsigned)std::min<int64_t>((nc + 7) / 8, 8 * (int64_t)sm_count()), 256, 0, 
+            launch_next(st, k_offset_keys, (unsigned)std::min<int64_t>((nc + 7) / 8, 8 * (int64_t)sm_count()), 256, 0,
                 c, m2l_off, m2l_src, nc, (unsigned long long *)t->b_hash.ptr, H - 1,
                 (uint32_t *)t->b_m2l_didx.ptr, lkey, lslot, cnt + 13, (int *)(cnt + 10), cnt + 12);
             launch_next(st, k_rank_keys, (unsigned)sm_count(), 256, 0, lkey, lslot, cnt + 13, (uint64_t *)t->b_dkeys.ptr,
