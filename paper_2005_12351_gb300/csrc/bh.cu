@@ -247,7 +247,8 @@ k_bh(BHArgs a)
              f, e0, e1, e2);
     };
     // FP32 copies for the MAC: most cells pass or fail it by far more than the
-    // rounding of the copies, which spares them the ten FP64 operations
+    // rounding of the copies, which spares them the ten FP64 operations (squares
+    // near FP32's smallest, whose rounding is not relative, take the FP64 test)
     const float xf = (float)x, yf = (float)y, zf = (float)z, t2f = (float)a.theta2;
     const float af = fmaxf(fabsf(xf), fmaxf(fabsf(yf), fabsf(zf)));
     unsigned long long n_m2p = 0, n_p2p = 0;
@@ -284,7 +285,7 @@ k_bh(BHArgs a)
             const float fx = xf - (float)cx, fy = yf - (float)cy, fz = zf - (float)cz, hf = (float)h;
             const float dd = fmaf(fx, fx, fmaf(fy, fy, fz * fz)), d1 = fabsf(fx) + fabsf(fy) + fabsf(fz);
             const float m = fmaf(4.8e-7f * (af + d1), d1 + af * 2.4e-7f, 2e-6f * dd), hh = hf * hf;
-            if (dd > 1e-30f && dd < 1e30f && hh < 1e30f && hh * 1.000002f < t2f * (dd - m) * 0.999998f) {
+            if (dd > 1e-30f && dd < 1e30f && hh > 1e-30f && hh < 1e30f && hh * 1.000002f < t2f * (dd - m) * 0.999998f) {
                 acc = true;
             } else if (!(dd > 1e-30f && dd < 1e30f && hh > 1e-30f && hh * 0.999998f > t2f * (dd + m) * 1.000002f)) {
                 const double dx = __dsub_rn(x, cx), dy = __dsub_rn(y, cy), dz = __dsub_rn(z, cz);
