@@ -521,8 +521,9 @@ fmm_status fmm_check_umma(const float *A, const float *B, float *D, int nkb, int
  *   stream capture and outside any allocator callback, so that later calls
  *   allocate nothing.
  *   Sharing: all calls on a device use the same array, and each call leaves
- *   its contents behind.  Calls that overlap on the GPU (different streams
- *   or threads without ordering between them) race on it: serialise them.
+ *   its contents behind.  Calls of several threads take turns: a call holds
+ *   the array until its work on the GPU has ended.  fmm_morton_order uses it
+ *   too when no other call does.
  *   Synchronises cuda_stream before returning; allocates nothing.
  */
 #define FMM_NOALLOC_MAX_POINTS (1 << 20)
