@@ -31,11 +31,11 @@ METRIC = "FMM particles/sec at p=6 & rel err vs FP64 direct sum; served p50/p99 
 UNIT = "particles/s"
 L2_FLUSH_BYTES = 256 << 20          # > 129 MB L2
 
-# DRAM bytes (read + write) per particle of the dominant kernels, from full ncu captures of
-# the 125k-dipole case (same leaf occupancy; the kernels' traffic grows with the particles):
-# k_p2p_sym 7.546 MB + 0.183 MB, k_p2p32 11.210 MB + 0 MB per launch
+# DRAM bytes (read + write) per particle of the dominant kernels, from ncu captures of the
+# 125k-dipole case (same leaf occupancy; the kernels' traffic grows with the particles):
+# k_p2p_fx 7.859 GB/s over 1.297 ms, k_p2p32 11.210 MB + 0 MB per launch
 # (profiles/fp64_pass_kernels_dipole_125k_p6.md, profiles/k_p2p32_k_m2l32_tile2_fp32_dipole_125k_p6.md)
-TRAFFIC_PER_PARTICLE = {("fp64", 1): 7.7291e6 / 125_000, ("fp32", 1): 11.2097e6 / 125_000,
+TRAFFIC_PER_PARTICLE = {("fp64", 1): 10.193e6 / 125_000, ("fp32", 1): 11.2097e6 / 125_000,
                         ("3xtf32", 1): 11.2097e6 / 125_000}
 
 
@@ -382,6 +382,9 @@ def measure_form(args, w, precision, dev, world, rank, pos_h, S_h, pos_d, S_d, f
                 "traffic_source": ("ncu dram bytes of the 125k-dipole capture, scaled by particles"
                                    if tpp is not None else None),
                 "algorithmic_flops": cand[dom], "peak_source": src}
+    if precision == "fp64":
+        # the pair terms run in 64-bit fixed point: the FP64 peak is not their bound
+        roofline["pipes"] = "integer multiply-add and ALU (64-bit fixed point); the peak is the FP64 pipe's"
     if precision == "3xtf32" and info["tc_rows"] > 0:
         # the M2L on the tensor cores: 3 TF32 products per FP32 multiply-add of the method
         tpk, tsrc = tf32_peak()
@@ -515,7 +518,7 @@ def measure_mixed_orders(args, w, dev, world, flush):
     """Mixed source orders on the headline geometry: every particle carries a charge and
     a dipole (orders 0..1; the expansion starts at order 0, so multipoles run to p).  A
     step = tree build + evaluate, as the main line; FP64, the handle's default P2P (the
-    symmetric kernel, each shell's reverse term with its own parity)."""
+    fixed-point kernel, both shells in one pair)."""
     import torch
     from paper_2005_12351_gb300 import fmm
     n, p, theta = w["n"], w["p"], w["theta"]
@@ -559,7 +562,7 @@ def measure_mixed_orders(args, w, dev, world, flush):
     tree.destroy()
     return {"sources": "charge + dipole per particle (orders 0..1)", "p": p, "theta": theta,
             "value": n * world / (ms / 1e3), "unit": UNIT, "ms_per_step": ms, "field_rel_rms": err,
-            "targets": int(len(tg)), "phase_ms": ph, "p2p_kernel": "symmetric",
+            "targets": int(len(tg)), "phase_ms": ph, "p2p_kernel": "fixed-point",
             "roofline": {"bound": "alu", "kernel": "p2p", "achieved": achieved,
                          "peak": args.fp64_peak_tflops, "unit": "TFLOP/s",
                          "frac": achieved / args.fp64_peak_tflops, "traffic": None,
