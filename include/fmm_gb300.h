@@ -399,7 +399,8 @@ fmm_status fmm_server_destroy(fmm_server *s);
  * then captures the evaluate into a CUDA graph; later calls with the same
  * parameters replay it with one graph launch (every phase of the path, all
  * systems of a batch).  Any other parameter set recaptures.  fmm_set_sources,
- * fmm_set_sources_batch and fmm_autotune drop the graph.  Profiling phase
+ * fmm_set_sources_batch, fmm_autotune, fmm_set_tuning, fmm_evaluate_bh and an
+ * fmm_evaluate of another p, theta or choice of outputs drop the graph.  Profiling phase
  * times are not updated by replays.  Errors as fmm_evaluate; FMM_ECUDA if
  * the capture fails.
  */

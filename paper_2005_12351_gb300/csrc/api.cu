@@ -373,6 +373,11 @@ fmm_status fmm_evaluate(fmm_tree *t, int p, double theta, int want_potential, in
     if ((want_potential && !potential) || (want_field && !field))
         return fail(t, FMM_EINVAL, "NULL output for a requested quantity");
     DeviceGuard g(t->device);
+    // A captured evaluate of other parameters holds the tables, lists, plan and
+    // buffers by address; this one rewrites or regrows them.  One of the same
+    // parameters finds all of them as they are.
+    if (t->graph_exec && (t->g_p != p || t->g_theta != theta || t->g_phi != want_potential || t->g_field != want_field))
+        drop_graph(t);
     record(t, 4);
     if (!t->have_lists || t->theta != theta) FMM_TRY(build_lists(t, theta));
     record(t, 5);
