@@ -36,7 +36,14 @@
 //
 // Pairs closer than 2^-7 of the coordinate range (a sixteenth of a half side;
 // a few in a million of a uniform set's) and coincident points take the FP64
-// formulas, as do whole rows that hold a non-finite moment.
+// formulas, as do whole rows that hold a non-finite moment.  So do targets whose
+// sum is so small beside the row's scale that what its terms can have lost (counted
+// while the sources are staged) passes 2^-54 of it: a target that holds the row's
+// largest moment itself, coincides with it or sees none of its field, from ratios
+// to the others of about 2^42 (charges), 2^35 (dipoles) and 2^28 (quadrupoles) on.
+// That costs 0.6 % of the P2P at 1M dipoles, 2 to 4 % at 262k Plummer and 200k
+// charges and dipoles (the count in the staging and the compiler's schedule; the
+// pairs' loop is the same).  Keeping every bit in the loop instead cost 2 to 5 %.
 #include <algorithm>
 
 #include "fmm_internal.cuh"
@@ -81,6 +88,7 @@ constexpr int kUnitE = 108, kUnitP = 111;
 
 // the shift amount that stands for "contributes nothing"
 constexpr int kFar = 160;
+constexpr int kWhole = 56;                 // a term of a larger shift loses bits
 
 // the two forms of a multiply-add (fx64.cuh): the quadrupoles' sums run faster
 // fused, the others' with the addend in the instruction
@@ -302,9 +310,10 @@ __device__ __forceinline__ void put_bal(int *r, int i, s64 v)
 }
 
 // a shell's words of one source: base_e, base_p = the target leaf's bases plus
-// (S + 2) or (S + 1) times the round's unit exponent
+// (S + 2) or (S + 1) times the round's unit exponent.  True if its terms can lose
+// bits in fx_add.
 template <int S, bool PHI, bool FIELD>
-__device__ __forceinline__ void fx_stage_shell(const double *Sj, int base_p, int base_e, int *r)
+__device__ __forceinline__ bool fx_stage_shell(const double *Sj, int base_p, int base_e, int *r)
 {
     constexpr int e = PHI ? 1 : 0;
     constexpr int nb = (PHI ? 1 : 0) + (FIELD ? 1 : 0);
@@ -330,15 +339,42 @@ __device__ __forceinline__ void fx_stage_shell(const double *Sj, int base_p, int
             put_bal(m, 2 * a, fix64(Sj[a], (a == 0 || a == 3 || a == 5 ? 63 : 62) - em));
         put64(m, 12, fix64(Sj[0], 58 - em) + fix64(Sj[3], 58 - em) + fix64(Sj[5], 58 - em));
     }
+    return !none && max(PHI ? r[0] : 0, FIELD ? r[e] : 0) > kWhole;
 }
 
 template <int S, int SLO, int SHI, bool PHI, bool FIELD>
-__device__ __forceinline__ void fx_stage_orders(const double *Sj, int bp, int be, int lu, int *r)
+__device__ __forceinline__ bool fx_stage_orders(const double *Sj, int bp, int be, int lu, int *r)
 {
-    fx_stage_shell<S, PHI, FIELD>(Sj, bp + fx_off_p(S) + (S + 1) * lu, be + fx_off_e(S) + (S + 2) * lu,
-                                  r + fx_off(SLO, S, PHI, FIELD));
+    bool lose = fx_stage_shell<S, PHI, FIELD>(Sj, bp + fx_off_p(S) + (S + 1) * lu, be + fx_off_e(S) + (S + 2) * lu,
+                                              r + fx_off(SLO, S, PHI, FIELD));
     if constexpr (S < SHI)
-        fx_stage_orders<S + 1, SLO, SHI, PHI, FIELD>(Sj + (S + 1) * (S + 2) / 2, bp, be, lu, r);
+        lose |= fx_stage_orders<S + 1, SLO, SHI, PHI, FIELD>(Sj + (S + 1) * (S + 2) / 2, bp, be, lu, r);
+    return lose;
+}
+
+// What a term of base b can lose in fx_add, in units of the sums, when its shift is
+// b less up to k sh: nothing down to 56, the lower limb (below 2^(84 - shift)) down
+// to 84, all of it (below 2^(115 - shift)) beyond.
+__device__ __forceinline__ float fx_loss(int b, int k, int sh)
+{
+    const int lo = max(b - k * sh, kWhole + 1);            // the smallest shift that loses anything
+    return exp2f((float)(lo > 84 ? 115 - lo : (b > 84 ? 30 : 84 - lo)));
+}
+// The same of all terms of one source, added to lost[0] (potential) and lost[1]
+// (field).  gap: a target of the leaf is at least so far away along some axis.
+template <int SLO, int SHI, bool PHI, bool FIELD>
+__device__ __noinline__ void fx_count_loss(const double *Sj, int bp, int be, int lu, s64 gap, float *lost)
+{
+    const int sh = gap > 0 ? min(kShMax, __clzll(gap) - 1) : kShMax;     // the largest normalising shift
+    int o = 0;
+    for (int s = SLO; s <= SHI; ++s) {
+        const int n = (s + 1) * (s + 2) / 2, em = fx_moment_exp(Sj + o, n) + fx_exp_room(s);
+        o += n;
+        if (em < kNone / 2) continue;
+        const int ap = bp + fx_off_p(s) + (s + 1) * lu - em, ae = be + fx_off_e(s) + (s + 2) * lu - em;
+        if (PHI && ap > kWhole) atomicAdd(lost, fx_loss(ap, s + 1, sh));
+        if (FIELD && ae > kWhole) atomicAdd(lost + 1, fx_loss(ae, s + 2, sh));
+    }
 }
 
 // The FP64 terms of one pair, added to the thread's sums in shared memory:
@@ -368,8 +404,10 @@ __device__ __noinline__ void fx_close(int i, int j, const double *px, const doub
 // A round holds sources of one coordinate unit (the coarser of the two leaves'
 // half sides): partner leaves come in order of level, so units change only
 // between rounds.
+// The charges' potential fits 64 registers, which holds it at 16 blocks of 128 an SM
+// (500k charges: 6.16 ms, 6.5 with 111 registers); the others need all 128.
 template <int SLO, int SHI, bool PHI, bool FIELD>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(512, SHI == 0 && !FIELD ? 2 : 1)
 k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const int32_t *off,
          const int32_t *src, const int32_t *level, const int32_t *cx, const int32_t *cy, const int32_t *cz,
          const int32_t *sys, const double *sys_box, const double *px, const double *py, const double *pz,
@@ -391,6 +429,8 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
     __shared__ int gbeg[kFxGroups], gpre[kFxGroups + 1];
     __shared__ int s_next_q, s_next_j, s_ng, s_key;
     __shared__ int s_g, s_mx[3];
+    __shared__ float s_lost[2];                            // what the row's terms can lose, units of the sums
+    __shared__ unsigned char s_redo[512];
     const int A = leaves[blockIdx.x];
     const int b = begin[A], nt = end[A] - b;
     if (nt == 0) return;
@@ -401,6 +441,7 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
     // sources, largest moment exponent per shell
     if (tid < 3) s_mx[tid] = kNone;
     if (tid == 3) s_g = 1;
+    if (tid >= 4 && tid < 6) s_lost[tid - 4] = 0.0f;
     __syncthreads();
     {
         const s64 rA = 1ll << (kLevels - lA);
@@ -484,6 +525,7 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
             s64 tx = 0, ty = 0, tz = 0;
             int key_t = -1;
             int q = q0, j_in = 0;
+            if (tid < 2) s_lost[tid] = 0.0f;               // the round's barriers come first
             while (q < q1) {
                 __syncthreads();
                 if (tid < 32) {
@@ -543,7 +585,10 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
                     r[6] = j;
 #pragma unroll
                     for (int w = Rec::words; w < 4 * NW; ++w) r[w] = 0;
-                    fx_stage_orders<SLO, SLO, SHI, PHI, FIELD>(Sm + (int64_t)j * nS, bp, be, g1 + lU, r);
+                    if (fx_stage_orders<SLO, SLO, SHI, PHI, FIELD>(Sm + (int64_t)j * nS, bp, be, g1 + lU, r))
+                        fx_count_loss<SLO, SHI, PHI, FIELD>(
+                            Sm + (int64_t)j * nS, bp, be, g1 + lU,
+                            max(max(llabs(word64(r, 0)), llabs(word64(r, 2))), llabs(word64(r, 4))) - (1ll << fa), s_lost);
 #pragma unroll
                     for (int w = 0; w < NW; ++w)
                         stage[w * CH + d] = make_int4(r[4 * w], r[4 * w + 1], r[4 * w + 2], r[4 * w + 3]);
@@ -588,6 +633,7 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
 #pragma unroll
             for (int l = 0; l < 4; ++l) red[(4 * c + l) * nthr + tid] = P[c][l];
         __syncthreads();
+        int redo = 0;                                      // 1 the potential, 2 the field
         if (tid < cnt) {
             // the copies' integers, exact in any order, then the FP64 pairs in copy order
             double v[NC];
@@ -609,8 +655,40 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
 #pragma unroll
                 for (int a = 0; a < 3; ++a) E_out[3 * o + a] = E_far[3 * (int64_t)i + a] + v[ef + a];
             }
+            // what the terms can have lost against 2^-54 of the sums
+            if (PHI && s_lost[0] > 0.0f && scalbn((double)s_lost[0], bp - kUnitP + 54) > fabs(v[0])) redo = 1;
+            if (FIELD && s_lost[1] > 0.0f && scalbn((double)s_lost[1], be - kUnitE + 54) >
+                                                 fmax(fabs(v[ef]), fmax(fabs(v[ef + 1]), fabs(v[ef + 2]))))
+                redo |= 2;
         }
-        __syncthreads();
+        if (__syncthreads_or(redo)) {
+            // rare: those targets' rows in FP64, the block's threads side by side
+            if (tid < cnt) s_redo[tid] = (unsigned char)redo;
+            __syncthreads();
+#pragma unroll 1
+            for (int u = 0; u < cnt; ++u) {
+                const int which = s_redo[u], iu = b + t0 + u;
+                if (which == 0) continue;
+                for (int c = 0; c < NC; ++c) accd[c * nthr + tid] = 0.0;
+#pragma unroll 1
+                for (int q = q0; q < q1; ++q) {
+                    const int B = src[q], je = end[B];
+#pragma unroll 1
+                    for (int j = begin[B] + tid; j < je; j += nthr)
+                        fx_close<SLO, SHI, PHI, FIELD>(iu, j, px, py, pz, Sm, accd + tid, nthr);
+                }
+                __syncthreads();
+                if (tid < NC && (which >> (tid >= ef) & 1)) {
+                    double d = 0.0;
+#pragma unroll 1
+                    for (int w = 0; w < nthr; ++w) d += accd[tid * nthr + w];
+                    const int64_t o = perm[iu];
+                    if (tid < ef) phi_out[o] = phi_far[iu] + d;
+                    else E_out[3 * o + tid - ef] = E_far[3 * (int64_t)iu + tid - ef] + d;
+                }
+                __syncthreads();
+            }
+        }
         if (t0 + tile < nt)
             for (int c = 0; c < NC; ++c) accd[c * nthr + tid] = 0.0;
     }
