@@ -265,7 +265,7 @@ __device__ __forceinline__ void axis_powers(double d, int P, double *out)
 // ------------------------------------------------------------------ P2M
 constexpr int kP2MThreads = 128;
 constexpr int kP2MChunk = 32;             // particles staged at a time
-constexpr int kP2MPer = 4;                // up to 4 * 128 = 512 M components
+constexpr int kP2MRun = 16 * kP2MChunk;   // particles whose sums share 64 bits
 // source terms of one particle: the kernel is instantiated for 3, 6 and 10 (one
 // order up to a dipole, a quadrupole, mixed orders) and takes the smallest that fits
 
@@ -275,8 +275,10 @@ constexpr int kP2MPer = 4;                // up to 4 * 128 = 512 M components
 //   displacement d = u 2^re, |u| <= 1 + 2^-10: u and the monomials u^k at 2^60
 //   monomials in the sums at 2^56 (error below 2^-56), as limbs h 2^26 + l
 //   moments at 2^53 of a power of two above the largest, so that the sum over a
-//   chunk of 32 particles stays below 2^63; the chunks' sums are shifted right by
-//   the bits their number needs
+//   chunk of 32 particles stays below 2^63; the chunks' sums are shifted right,
+//   rounded, by the bits their number needs: at most four, as after 16 chunks they
+//   go to the FP64 row and start again (leaves of any size: deep ones of coincident
+//   points, or a large max_leaf)
 //   L_n rho^k / k! at 2^56 of a power of two above the sum of their magnitudes,
 //   so that the sum over them stays below 2^61
 using fx::I2;
@@ -371,6 +373,32 @@ __device__ __forceinline__ double inv_factorial(const DevTables &tb, int k)
     return __hiloint2double(__ldg(tb.inv_fact + 2 * k + 1), __ldg(tb.inv_fact + 2 * k));
 }
 
+// The sums of a run that is not its leaf's last, as doubles into the leaf's row, and cleared
+__device__ __noinline__ void p2m_run_end(s64 *G, int nK, int nS, const int *s_es, int re, int room, const int *mis,
+                                         const int *inv_fact, const int *terms, int nM, bool first, double *M)
+{
+    double *Gd = (double *)G;
+    for (int k = threadIdx.x; k < nK; k += kP2MThreads) {
+        const int ek = mi_shell(mi_at(mis, k)) * re;
+        const double f = __hiloint2double(__ldg(inv_fact + 2 * k + 1), __ldg(inv_fact + 2 * k));
+        for (int a = 0; a < nS; ++a) {
+            const s64 g = G[k * nS + a];
+            Gd[k * nS + a] = g ? scale2((double)g * f, s_es[a] + ek + room - 57) : 0.0;
+        }
+    }
+    __syncthreads();
+    for (int m = threadIdx.x; m < nM; m += kP2MThreads) {
+        double acc = first ? 0.0 : M[m];
+        for (int a = 0; a < nS; ++a) {
+            const int k = terms[m * nS + a];
+            if (k >= 0) acc += Gd[k * nS + a];
+        }
+        M[m] = acc;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < nK * nS; k += kP2MThreads) G[k] = 0;      // the staging's barrier comes next
+}
+
 // One block per leaf.  A thread owns monomials k and sums u^k S_a over the
 // particles for every source term a (a moment's limbs read by all lanes at
 // once); the multipole m is then the sum over a of the terms m - a.  Per
@@ -414,7 +442,8 @@ __device__ __forceinline__ void p2m_leaf(int c, const int32_t *begin, const int3
     for (int k = threadIdx.x; k < nK * nS; k += kP2MThreads) G[k] = 0;
     __syncthreads();
     re = max(max(s_re[0], s_re[1]), max(s_re[2], s_re[3]));
-    const int room = 32 - __clz((n - 1) / kP2MChunk);   // 2^room > chunks - 1
+    const int room = 32 - __clz((min(n, kP2MRun) - 1) / kP2MChunk);      // 2^room > chunks of a run - 1
+    const int half = (1 << room) >> 1;
     for (int j0 = b; j0 < e; j0 += kP2MChunk) {
         const int nj = min(kP2MChunk, e - j0);
         for (int t = threadIdx.x; t < 3 * nj; t += kP2MThreads)
@@ -430,7 +459,7 @@ __device__ __forceinline__ void p2m_leaf(int c, const int32_t *begin, const int3
             s64 a1[kMaxSrc], a0[kMaxSrc];
 #pragma unroll
             for (int a = 0; a < kMaxSrc; ++a) {
-                a1[a] = 0;
+                a1[a] = half;
                 a0[a] = 1ll << 25;
             }
             for (int j = 0; j < nj; ++j) {
@@ -450,6 +479,9 @@ __device__ __forceinline__ void p2m_leaf(int c, const int32_t *begin, const int3
                 if (a < nS) G[k * nS + a] += (a1[a] + (a0[a] >> 26)) >> room;
         }
         __syncthreads();
+        if ((j0 - b) % kP2MRun == kP2MRun - kP2MChunk && j0 + kP2MChunk < e)
+            p2m_run_end(G, nK, nS, s_es, re, room, tb.mi, tb.inv_fact, tb.p2m_terms, tb.nM, j0 - b < kP2MRun,
+                        M + (int64_t)c * tb.nM);
     }
     // the sums as doubles: u^k S_a 2^(57 - room) -> (z - x)^k / k! S_a
     double *Gd = (double *)G;
@@ -465,7 +497,7 @@ __device__ __forceinline__ void p2m_leaf(int c, const int32_t *begin, const int3
     }
     __syncthreads();
     for (int mi = threadIdx.x; mi < tb.nM; mi += kP2MThreads) {
-        double acc = 0.0;
+        double acc = n > kP2MRun ? M[(int64_t)c * tb.nM + mi] : 0.0;     // the runs before, by the same thread
         for (int a = 0; a < nS; ++a) {
             const int k = tb.p2m_terms[mi * nS + a];
             if (k >= 0) acc += Gd[k * nS + a];
