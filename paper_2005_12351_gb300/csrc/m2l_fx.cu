@@ -230,66 +230,81 @@ __global__ void __launch_bounds__(kFxThreads) k_m2l_fx(const __grid_constant__ F
     if (s_last) fx_finish(a, slot0, (s64 *)sm4);
 }
 
-// The cells' multipoles as limbs, then the exponents of the plan's targets, in
-// one cooperative launch (every block is resident, so the barrier between the
-// two ends; it is bounded all the same).  One warp per cell: the row folded as
-// in k_fold_m, its exponent, the limbs.  One warp per target: e_t from its list.
+// The cells' multipoles as limbs, then the exponents of the plan's targets.  One
+// warp per cell: the row folded as in k_fold_m, its exponent, the limbs.  One warp
+// per target: e_t from its list.  Blocks claim their work in order, the cells
+// first, so that every cell is with a running block when the first targets' block
+// waits for them: the wait ends whatever else holds the rest of the chip (as
+// blocks of a cooperative launch that met at a grid barrier, it could run into its
+// bound).  ctl: [0] claimed, [1] blocks of cells done, from 0.
+constexpr int kExpPer = 16;                          // cells or targets of a block
 __global__ void __launch_bounds__(128)
 k_fx_exps(const double *M, int64_t nc, DevTables tb, const int32_t *am, const int32_t *level, const int32_t *sys,
           const int *e_side, int nq, int bits, int2 *Mx, int *eM, int slots, const int32_t *tile_tgt,
-          const int32_t *off, const int32_t *src, const int32_t *didx, const int *ekey, int *etgt, unsigned *bar)
+          const int32_t *off, const int32_t *src, const int32_t *didx, const int *ekey, int *etgt, unsigned *ctl)
 {
     extern __shared__ double fsm[];
+    __shared__ unsigned s_id;
     __shared__ int s_ok;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double *v = fsm + w * tb.nM;
-    for (int64_t c = blockIdx.x * 4ll + w; c < nc; c += gridDim.x * 4ll) {
-        for (int m = lane; m < tb.nM; m += 32) v[m] = M[c * tb.nM + m];
-        __syncwarp();
-        for (int l = 0; l < tb.h_fold_lev; ++l) {
-            for (int q = tb.h_fold_off[l] + lane; q < tb.h_fold_off[l + 1]; q += 32) {
-                const int i = tb.h_fold[3 * q], a = tb.h_fold[3 * q + 1], b = tb.h_fold[3 * q + 2];
-                double x = v[i];
-                if (a >= 0) x -= v[a];
-                if (b >= 0) x -= v[b];
-                v[i] = x;
+    const unsigned ncb = (unsigned)((nc + kExpPer - 1) / kExpPer);
+    if (threadIdx.x == 0) s_id = atomicAdd(ctl, 1u);
+    __syncthreads();
+    if (s_id < ncb) {
+        double *v = fsm + w * tb.nM;
+        const int64_t c0 = (int64_t)s_id * kExpPer, c1 = min(nc, c0 + kExpPer);
+        for (int64_t c = c0 + w; c < c1; c += 4) {
+            for (int m = lane; m < tb.nM; m += 32) v[m] = M[c * tb.nM + m];
+            __syncwarp();
+            for (int l = 0; l < tb.h_fold_lev; ++l) {
+                for (int q = tb.h_fold_off[l] + lane; q < tb.h_fold_off[l + 1]; q += 32) {
+                    const int i = tb.h_fold[3 * q], a = tb.h_fold[3 * q + 1], b = tb.h_fold[3 * q + 2];
+                    double x = v[i];
+                    if (a >= 0) x -= v[a];
+                    if (b >= 0) x -= v[b];
+                    v[i] = x;
+                }
+                __syncwarp();
+            }
+            const int hl = e_side[sys[c]] - level[c] - 1;        // log2 of the half side
+            int e = kZeroExp;
+            for (int r = lane; r < tb.nMh; r += 32) {
+                const int k = am[r], wr = (k >> 8) - (k & 255) * hl;
+                const u64 b = (u64)__double_as_longlong(v[tb.h_rm[r]]) & 0x7fffffffffffffffull;
+                if (b >= 0x7ff0000000000000ull) e = kBadExp;
+                // a value within 2^-29 of the next power of two would round to it: Mh < 2^31
+                else if (b) e = max(e, (int)((b + (1ull << 23)) >> 52) - 1022 + wr);
+            }
+            e = __reduce_max_sync(0xffffffffu, e);
+            if (lane == 0) eM[c] = e;
+            for (int r = lane; r < 2 * nq; r += 32) {
+                s64 x = 0;
+                if (r < tb.nMh && e != kBadExp) {
+                    const int k = am[r], wr = (k >> 8) - (k & 255) * hl;
+                    x = fix64(v[tb.h_rm[r]], wr + bits - e);
+                }
+                const int h = (int)((x + (1ll << 25)) >> 26);
+                Mx[c * 2 * nq + r] = make_int2(h, (int)(x - ((s64)h << 26)));
             }
             __syncwarp();
         }
-        const int hl = e_side[sys[c]] - level[c] - 1;        // log2 of the half side
-        int e = kZeroExp;
-        for (int r = lane; r < tb.nMh; r += 32) {
-            const int k = am[r], wr = (k >> 8) - (k & 255) * hl;
-            const u64 b = (u64)__double_as_longlong(v[tb.h_rm[r]]) & 0x7fffffffffffffffull;
-            if (b >= 0x7ff0000000000000ull) e = kBadExp;
-            // a value within 2^-29 of the next power of two would round to it: Mh < 2^31
-            else if (b) e = max(e, (int)((b + (1ull << 23)) >> 52) - 1022 + wr);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            atomicAdd(ctl + 1, 1u);
         }
-        e = __reduce_max_sync(0xffffffffu, e);
-        if (lane == 0) eM[c] = e;
-        for (int r = lane; r < 2 * nq; r += 32) {
-            s64 x = 0;
-            if (r < tb.nMh && e != kBadExp) {
-                const int k = am[r], wr = (k >> 8) - (k & 255) * hl;
-                x = fix64(v[tb.h_rm[r]], wr + bits - e);
-            }
-            const int h = (int)((x + (1ll << 25)) >> 26);
-            Mx[c * 2 * nq + r] = make_int2(h, (int)(x - ((s64)h << 26)));
-        }
-        __syncwarp();
+        return;
     }
-    __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(bar, 1u);
-        const volatile unsigned *b = bar;
+        const volatile unsigned *done = ctl + 1;
         const long long t0 = clock64();
-        while (*b < gridDim.x && clock64() - t0 < (1ll << 31)) __nanosleep(32);
-        s_ok = *b >= gridDim.x;
+        while (*done < ncb && clock64() - t0 < (1ll << 31)) __nanosleep(32);
+        s_ok = *done >= ncb;
         __threadfence();
     }
     __syncthreads();
-    for (int q = blockIdx.x * 4 + w; q < slots; q += gridDim.x * 4) {
+    const int q0 = (int)(s_id - ncb) * kExpPer, q1 = min(slots, q0 + kExpPer);
+    for (int q = q0 + w; q < q1; q += 4) {
         const int c = tile_tgt[q];
         int e = kZeroExp;
         if (c >= 0 && s_ok) {
@@ -495,7 +510,7 @@ fmm_status fx_prepare(fmm_tree *t, int p)
     }
     FMM_TRY(ensure(t, t->b_fx_em, 4 * (size_t)t->ncells));
     FMM_TRY(ensure(t, t->b_fx_et, 4 * slots));
-    // the sums, the blocks done per 32 targets, the barrier
+    // the sums, the blocks done per 32 targets, k_fx_exps' counters
     FMM_TRY(ensure(t, t->b_fx_acc, 32 * slots * Ly.groups + slots / 8 + 16));
     // the limbs take the place of the folded multipoles
     return ensure(t, t->b_Mh, 16 * (size_t)t->ncells * Ly.nq);
@@ -510,29 +525,17 @@ fmm_status run_fx_exps(fmm_tree *t, const double *M, const DevTables &tb)
         return FMM_EINVAL;                   // not reachable: both follow the handle's flag
     }
     if (t->tc_chunks == 0) return FMM_OK;
-    int slots = (int)t->tc_tiles * 128, per_sm = 0;
-    const size_t acc = 32 * (size_t)slots * Ly.groups, smem = 32 * (size_t)tb.nM;
+    const int slots = (int)t->tc_tiles * 128;
+    const size_t acc = 32 * (size_t)slots * Ly.groups;
     FMM_TRY(cuda_check(t, cudaMemsetAsync(t->b_fx_acc.ptr, 0, acc + slots / 8 + 16, st), "memset"));
-    FMM_TRY(cuda_check(t, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fx_exps, 128, smem), "occupancy"));
-    const int64_t grid = std::min<int64_t>((std::max<int64_t>(t->ncells, slots) + 3) / 4,
-                                           (int64_t)std::max(per_sm, 1) * sm_count());
-    int64_t nc = t->ncells;
-    DevTables tv = tb;
     const int32_t *am = (const int32_t *)t->b_fx_el.ptr + Ly.E + Ly.first.size();
-    const int32_t *level = (const int32_t *)t->b_level.ptr, *sys = (const int32_t *)t->b_sys.ptr;
-    const int *es = t->sys_eside_dev();
-    int nq = Ly.nq, bits = Ly.bits;
-    int2 *Mx = (int2 *)t->b_Mh.ptr;
-    int *eM = (int *)t->b_fx_em.ptr, *et = (int *)t->b_fx_et.ptr;
-    const int32_t *tgt = (const int32_t *)t->b_tc_tgt.ptr, *off = (const int32_t *)t->b_m2l_off.ptr,
-                  *src = (const int32_t *)t->b_m2l_src.ptr, *didx = (const int32_t *)t->b_m2l_didx.ptr;
-    const int *ekey = (const int *)t->b_fx_ekey.ptr;
-    unsigned *bar = (unsigned *)((char *)t->b_fx_acc.ptr + acc + slots / 8);
-    void *args[] = {&M, &nc, &tv, &am, &level, &sys, &es, &nq, &bits, &Mx, &eM, &slots, &tgt, &off, &src, &didx,
-                    &ekey, &et, &bar};
+    k_fx_exps<<<gridn(t->ncells, kExpPer) + gridn(slots, kExpPer), 128, 32 * (size_t)tb.nM, st>>>(
+        M, t->ncells, tb, am, (const int32_t *)t->b_level.ptr, (const int32_t *)t->b_sys.ptr, t->sys_eside_dev(), Ly.nq,
+        Ly.bits, (int2 *)t->b_Mh.ptr, (int *)t->b_fx_em.ptr, slots, (const int32_t *)t->b_tc_tgt.ptr,
+        (const int32_t *)t->b_m2l_off.ptr, (const int32_t *)t->b_m2l_src.ptr, (const int32_t *)t->b_m2l_didx.ptr,
+        (const int *)t->b_fx_ekey.ptr, (int *)t->b_fx_et.ptr, (unsigned *)((char *)t->b_fx_acc.ptr + acc + slots / 8));
     ++t->launches;
-    return cuda_check(t, cudaLaunchCooperativeKernel((const void *)k_fx_exps, dim3((unsigned)grid), dim3(128), args,
-                                                     smem, st), "fixed-point multipoles");
+    return cuda_check(t, cudaGetLastError(), "fixed-point multipoles");
 }
 
 fmm_status run_m2l_fx(fmm_tree *t, const DevTables &tb, double *L)
