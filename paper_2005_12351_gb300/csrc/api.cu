@@ -117,11 +117,16 @@ fmm_status ensure(fmm_tree *t, DevBuf &b, size_t bytes)
 void release(fmm_tree *t, DevBuf &b)
 {
     if (b.ptr) {
-        // work already queued on the handle's stream may still read this buffer
-        // (a grow copy, an earlier kernel): once freed, another handle's
+        // work already queued on the handle's streams may still read this buffer
+        // (a grow copy, an earlier kernel, the upward pass beside a plan that is
+        // being built on the side stream): once freed, another handle's
         // allocation on another stream may receive the same memory
-        if (t->stream) cudaStreamSynchronize(t->stream);
-        else cudaDeviceSynchronize();
+        if (t->home) {
+            cudaStreamSynchronize(t->home);
+            if (t->stream != t->home) cudaStreamSynchronize(t->stream);
+        } else {
+            cudaDeviceSynchronize();
+        }
         cudaFree(b.ptr);
         t->held -= b.bytes;
     }
@@ -222,7 +227,7 @@ fmm_status fmm_create_tree(fmm_tree **out, int device, void *cuda_stream, int ma
     fmm_tree *t = new (std::nothrow) fmm_tree();
     if (!t) { g_create_err = "host allocation failed"; return FMM_ENOMEM; }
     t->device = device;
-    t->stream = (cudaStream_t)cuda_stream;
+    t->stream = t->home = (cudaStream_t)cuda_stream;
     t->max_leaf = max_leaf;
     t->prec = prec;
     // one way in every form: the FP64 form's fixed-point pairs and the FP32 forms'

@@ -216,7 +216,8 @@ struct DevBuf {
 
 struct fmm_tree {
     int device = 0;
-    cudaStream_t stream = nullptr;
+    cudaStream_t stream = nullptr;         // work goes here; the handle's own but for plans and captures
+    cudaStream_t home = nullptr;           // the handle's own, as given at creation
     int max_leaf = 64;
     fmm_precision prec = FMM_FP64;
     size_t budget = 0;
