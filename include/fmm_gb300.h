@@ -93,6 +93,9 @@ typedef enum {
  * Testing hook: when the environment variable FMM_FAIL_ALLOC holds k >= 1 as
  * the handle is created, the handle's k-th device allocation (counted from
  * this call, which makes two) fails as cudaMalloc would, once.
+ * FMM_FAIL_SOFT_ALLOC = k does the same, from the k-th on, to the allocations
+ * an evaluate can do without: those of the FP64 form's M2L plan.  It then
+ * takes the M2L that needs none, for these lists and orders from there on.
  */
 fmm_status fmm_create_tree(fmm_tree **out, int device, void *cuda_stream, int max_leaf,
                            fmm_precision prec, size_t mem_budget_bytes);

@@ -61,6 +61,7 @@ static void forget_state(fmm_tree *t)
     t->tc_img_p = -1;
     t->m32_img_p = -1;
     t->fx_img_p = -1;
+    t->fx_off = false;
     t->sym_plan = false;
     t->bh_ran = false;
     t->bh_key_s = -1;
@@ -99,9 +100,10 @@ fmm_status ensure(fmm_tree *t, DevBuf &b, size_t bytes)
     release(t, b);
     void *p = nullptr;
     const bool injected = t->fail_alloc_at > 0 && ++t->alloc_count == t->fail_alloc_at;
-    cudaError_t e = injected ? cudaErrorMemoryAllocation : cudaMalloc(&p, bytes);
+    const bool soft = t->soft_alloc && t->fail_soft_at > 0 && ++t->soft_count >= t->fail_soft_at;
+    cudaError_t e = injected || soft ? cudaErrorMemoryAllocation : cudaMalloc(&p, bytes);
     if (e != cudaSuccess) {
-        if (!injected) cudaGetLastError();
+        if (!injected && !soft) cudaGetLastError();
         t->err = "cudaMalloc of " + std::to_string(bytes) + " bytes failed: " + cudaGetErrorString(e) +
                  (injected ? " (injected by FMM_FAIL_ALLOC)" : "");
         if (t->soft_alloc && !injected) return FMM_EBUDGET;
@@ -235,6 +237,7 @@ fmm_status fmm_create_tree(fmm_tree **out, int device, void *cuda_stream, int ma
     t->p2p_variant = 1;
     t->budget = mem_budget_bytes;
     if (const char *env = getenv("FMM_FAIL_ALLOC")) t->fail_alloc_at = std::max(0ll, atoll(env));
+    if (const char *env = getenv("FMM_FAIL_SOFT_ALLOC")) t->fail_soft_at = std::max(0ll, atoll(env));
     std::memset(t->phase_ms, 0, sizeof(t->phase_ms));
     fmm_status st = ensure(t, t->b_err, 16);
     if (st == FMM_OK) st = ensure(t, t->b_box, 256);

@@ -227,6 +227,9 @@ struct fmm_tree {
     // allocation-failure injection (FMM_FAIL_ALLOC at create): the fail_alloc_at-th
     // device allocation of the handle fails once; 0 = off
     int64_t alloc_count = 0, fail_alloc_at = 0;
+    // the same for the allocations a call can do without (soft_alloc below): from
+    // the fail_soft_at-th on they fail (FMM_FAIL_SOFT_ALLOC at create)
+    int64_t soft_count = 0, fail_soft_at = 0;
 
     // system
     int64_t n = 0;
@@ -309,6 +312,7 @@ struct fmm_tree {
     fmm::FxLayout fx_lay;
     int fx_img_p = -1;
     DevBuf b_fx_el, b_fx_img, b_fx_ekey, b_fx_em, b_fx_et, b_fx_acc;
+    bool fx_off = false;                   // no memory for it on these lists and orders: the per-cell M2L
     bool soft_alloc = false;               // a failing allocation is FMM_EBUDGET, the handle keeps its state
 
     // symmetric FP64 P2P (p2p_variant 2), derived from the lists: per list
@@ -415,7 +419,7 @@ fmm_status run_bh(fmm_tree *t, int p, double theta, int want_phi, int want_field
                   double *E_out);
 // M' of the harmonic M2L for every cell: Mh[c][r] = fold(M[c])[h_rm[r]]
 void launch_fold_m(cudaStream_t st, const double *M, int ldM, int64_t nc, const DevTables &tb,
-                   double *Mh, int ldH);
+                   double *Mh, int ldH, bool dependent);
 void launch_fold_m(cudaStream_t st, const float *M, int ldM, int64_t nc, const DevTables &tb,
                    float *Mh, int ldH);
 // mixed.cu (FMM_FP32): scaled FP32 expansions, FP32 pair arithmetic, FP64 outputs
@@ -496,15 +500,17 @@ inline int sm_count()
 // It takes the gap between two launches (about 2 us) out of chains of short
 // kernels: 2,000 charges 0.400 -> 0.358 ms a step, 12k quadrupoles FP32 0.803 ->
 // 0.717, 1M dipoles FP32 3.40 -> 3.33, Morton order of 1M points 0.176 -> 0.159.
-// Not for a kernel whose predecessor in the stream is another stream's event, and
-// every kernel launched so calls pdl_wait before anything else.
+// Not for a kernel whose predecessor in the stream is another stream's event
+// (launch_next_if without `dependent`: an ordinary launch), and every kernel
+// launched so calls pdl_wait before anything else.
 __device__ __forceinline__ void pdl_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 template <typename... P, typename... A>
-inline void launch_next(cudaStream_t st, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, A &&...args)
+inline void launch_next_if(bool dependent, cudaStream_t st, void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
+                           A &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -515,8 +521,13 @@ inline void launch_next(cudaStream_t st, void (*kern)(P...), dim3 grid, dim3 blo
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = dependent ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);      // errors: cudaGetLastError at the chain's end
+}
+template <typename... P, typename... A>
+inline void launch_next(cudaStream_t st, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, A &&...args)
+{
+    launch_next_if(true, st, kern, grid, block, smem, static_cast<A &&>(args)...);
 }
 
 // Raises a kernel's dynamic shared-memory limit to the most a block can take

@@ -251,6 +251,7 @@ fmm_status fmm_set_tuning(fmm_tree *t, const fmm_tuning *tuning)
     if (c.p2p_targets > 2) return fail(t, FMM_EINVAL, "p2p_targets must be 1 or 2");
     if (c.m2l_tiled > 1) return fail(t, FMM_EINVAL, "m2l_tiled must be 0 or 1");
     drop_graph(t);
+    t->fx_off = false;
     if (c.p2p_variant >= 0) t->p2p_variant = c.p2p_variant;
     if (c.m2l_tensor >= 0) t->m2l_simt = c.m2l_tensor == 0;
     if (c.m2l_harmonic >= 0) t->m2l_harmonic = c.m2l_harmonic == 1;

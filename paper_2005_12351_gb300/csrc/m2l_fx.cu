@@ -473,7 +473,9 @@ bool fx_usable(fmm_tree *t, int s, int p, int harmonic, int n_lo)
     if (Ly.s != s || Ly.p != p || Ly.h != h || Ly.n_lo != n_lo) {
         build_layout_fx(Ly, s, p, h, n_lo);
         t->fx_img_p = -1;                     // images and maps of the old layout
+        t->fx_off = false;
     }
+    if (t->fx_off) return false;
     const double nsys = (double)std::max<int64_t>(1, (int64_t)t->sys_off.size() - 1);
     return (double)t->n_m2l * Ly.products >= kFxMinWork * nsys && Ly.cap > 0 && Ly.nM <= kFxMaxNM &&
            fx_smem(Ly) <= (size_t)kFxSmemMax;

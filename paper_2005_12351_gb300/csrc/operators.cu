@@ -1059,10 +1059,10 @@ void record(fmm_tree *t, int i)
 }  // namespace
 
 void launch_fold_m(cudaStream_t st, const double *M, int ldM, int64_t nc, const DevTables &tb,
-                   double *Mh, int ldH)
+                   double *Mh, int ldH, bool dependent)
 {
     if (nc > 0)
-        launch_next(st, k_fold_m<double>, (unsigned)((nc + 3) / 4), 128, 32 * (size_t)tb.nM, M, ldM, nc, tb, Mh, ldH);
+        launch_next_if(dependent, st, k_fold_m<double>, (unsigned)((nc + 3) / 4), 128, 32 * (size_t)tb.nM, M, ldM, nc, tb, Mh, ldH);
 }
 
 void launch_fold_m(cudaStream_t st, const float *M, int ldM, int64_t nc, const DevTables &tb,
@@ -1146,12 +1146,15 @@ fmm_status run_expansions(fmm_tree *t, int p, int want_phi, int want_field)
     // lists are long enough, else one block per target cell.  A plan that has to
     // be built (new lists or p: two host syncs) is built on the handle's side
     // stream while the upward pass runs; not while the stream is being captured
-    // (the graph's evaluate follows an ordinary one, which built it).
+    // (the graph's evaluate follows an ordinary one, which built it).  Where the
+    // device has no memory for it, the per-cell kernel serves these lists and
+    // orders from then on (fx_off), in later evaluates and captures too.
     bool fx = t->n_m2l > 0 && fx_usable(t, s, p, tb.harmonic, tb.n_lo);
     const bool stale = fx && (!t->tc_plan || t->fx_img_p != p);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (stale) FMM_TRY(cuda_check(t, cudaStreamIsCapturing(st, &cap), "capture status"));
     const bool side = stale && cap == cudaStreamCaptureStatusNone;
+    if (stale && !side) fx = false;           // nothing may be allocated or waited for in a capture
     if (side) {
         FMM_TRY(side_stream(t));
         FMM_TRY(cuda_check(t, cudaEventRecord(t->ev_lists, st), "event"));
@@ -1181,6 +1184,7 @@ fmm_status run_expansions(fmm_tree *t, int p, int want_phi, int want_field)
             tc_release(t);
             t->err.clear();
             fx = false;
+            t->fx_off = true;
         } else {
             FMM_TRY(ps);
         }
@@ -1191,7 +1195,7 @@ fmm_status run_expansions(fmm_tree *t, int p, int want_phi, int want_field)
         FMM_TRY(run_fx_exps(t, M, tb));
     } else if (t->n_m2l > 0 && tb.harmonic) {
         FMM_TRY(ensure(t, t->b_Mh, 8 * (size_t)nc * tb.nMh));
-        launch_fold_m(st, M, tb.nM, nc, tb, (double *)t->b_Mh.ptr, tb.nMh);
+        launch_fold_m(st, M, tb.nM, nc, tb, (double *)t->b_Mh.ptr, tb.nMh, !side);
         ++t->launches;
         Ms = (const double *)t->b_Mh.ptr;
     }
@@ -1203,7 +1207,7 @@ fmm_status run_expansions(fmm_tree *t, int p, int want_phi, int want_field)
         size_t fixed = 8 * (size_t)tb.m2l_slots * kM2LThreads + 4 * (size_t)tb.m2l_T * kM2LThreads;
         size_t smem = fixed + 8 * (size_t)kM2LBatch * (ldM + ldD);
         allow_max_dynamic_smem(k_m2l);
-        launch_next(st, k_m2l, (unsigned)nc, kM2LThreads, smem,
+        launch_next_if(!side || Ms != M, st, k_m2l, (unsigned)nc, kM2LThreads, smem,
             (const int32_t *)t->b_m2l_off.ptr, (const int32_t *)t->b_m2l_src.ptr,
             (const int32_t *)t->b_m2l_didx.ptr, (const int32_t *)t->b_level.ptr,
             (const int32_t *)t->b_sys.ptr, t->sys_eside_dev(), Ms, (const double *)t->b_D.ptr, tb, L);
