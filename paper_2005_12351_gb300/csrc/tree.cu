@@ -384,16 +384,26 @@ __device__ __forceinline__ int digit_at(uint64_t key, int level)
 // small launches a level, or one cluster barrier and a few block barriers.  A
 // cluster of eight blocks is co-scheduled, so its barriers need no host and no
 // bounded waits; eight SMs are enough for the work (a binary search per cell
-// and octant), which is a chain of memory latencies whatever the width.
+// and octant) of a level that is a chain of memory latencies whatever the width.
 // Cells phase, before (26 launches, two host syncs) and now: 0.165 -> 0.054 ms at 2,000 points,
 // 0.22 -> 0.12 ms at 1M, 0.43 -> 0.34 ms at 4M.
+// A level of more than kWideLevel cells ends it: from there on two launches a
+// level over the whole chip (k_wide_count, k_wide_write).  Such trees took longer
+// in the cluster than in three launches a level, now less than either: 4M points,
+// leaves of 4 (2.5M cells) 1.13 and 2.37, now 0.59 ms; leaves of 16 (1.0M) 0.54 and
+// 0.89, now 0.44; 1M points, leaves of 8 (318k) 0.30, 0.32, 0.31.
 //
 // ctl: [0] overflow (more cells than cap), [1 + l] first cell of level l, then
 // the leaf count, the error word, the tie flag (a run the tie sort left: no
-// cells, the host sorts again), and the first system's box as four doubles.
-constexpr int kCtlOverflow = 0, kCtlLevel = 1, kCtlLeaves = 26, kCtlErr = 27, kCtlTie = 28, kCtlBox = 32,
-              kCtlHost = 40, kCtlTot = 40, kCtlWords = 40 + 4 * 16;   // words [0, kCtlHost) go to the host
+// cells, the host sorts again), one more than the level where the whole chip
+// takes over (0: none), and the first system's box as four doubles; behind the
+// words that go to the host the blocks' totals, and per level the leaves and the
+// cells with children before it.
+constexpr int kCtlOverflow = 0, kCtlLevel = 1, kCtlLeaves = 26, kCtlErr = 27, kCtlTie = 28, kCtlWide = 29,
+              kCtlBox = 32, kCtlHost = 40, kCtlTot = 40, kCtlBefore = 40 + 4 * 16,
+              kCtlWords = kCtlBefore + 2 * (kLevels + 2);             // words [0, kCtlHost) go to the host
 constexpr int kCellBlocks = 8, kCellThreads = 1024;
+constexpr int kWideLevel = 1 << 16;
 
 __device__ __forceinline__ void cluster_sync_all()
 {
@@ -480,7 +490,7 @@ k_cells(CellArrays c, const int64_t *off, int nsys, const double *box, const int
     unsigned leaves = 0, inner = 0;            // before this level
     bool over = (int64_t)le > cap;
     int level = 0;
-    for (; level <= kLevels && le > lb && !over; ++level) {
+    for (; level <= kLevels && le > lb && le - lb <= kWideLevel && !over; ++level) {
         const int ncl = le - lb;
         const int chunk = (ncl + kCellBlocks - 1) / kCellBlocks;
         const int i0 = min(ncl, blk * chunk), i1 = min(ncl, i0 + chunk);
@@ -586,15 +596,188 @@ k_cells(CellArrays c, const int64_t *off, int nsys, const double *box, const int
         le += (int)ca;
         cluster_sync_all();
     }
+    const bool wide_next = level <= kLevels && le > lb && !over;       // levels are left
     if (blk == 0) {
-        for (int l = level + tid; l <= kLevels + 2; l += kCellThreads) ctl[kCtlLevel + l] = (unsigned)lb;
+        for (int l = level + tid; l <= kLevels + 2; l += kCellThreads)
+            ctl[kCtlLevel + l] = (unsigned)(wide_next && l > level ? le : lb);
         if (tid == 0) {
+            ctl[kCtlWide] = wide_next ? (unsigned)level + 1u : 0u;
+            if (wide_next) {
+                ctl[kCtlBefore + 2 * level] = leaves;
+                ctl[kCtlBefore + 2 * level + 1] = inner;
+            }
             ctl[kCtlOverflow] = over;
             ctl[kCtlLeaves] = leaves;
             ctl[kCtlErr] = e;
             ctl[kCtlTie] = tie;
         }
         if (tid < 4) ((double *)(ctl + kCtlBox))[tid] = box[tid];
+    }
+}
+
+// ---- the cells of one wide level, part of it per block (the same part in both kernels).
+constexpr int kWideThreads = 256, kWideBlocksPerSM = 8;
+struct WidePart {
+    int lb, ncl, i0, i1;                     // the level's first cell and cells; the block's part
+};
+__device__ __forceinline__ WidePart wide_part(const unsigned *ctl, int level)
+{
+    WidePart w;
+    w.lb = (int)ctl[kCtlLevel + level];
+    w.ncl = (int)ctl[kCtlLevel + level + 1] - w.lb;
+    const int chunk = (w.ncl + (int)gridDim.x - 1) / (int)gridDim.x;
+    w.i0 = min(w.ncl, (int)blockIdx.x * chunk);
+    w.i1 = min(w.ncl, w.i0 + chunk);
+    return w;
+}
+
+// Children of every cell of the level (0 for a leaf) into c.nchild, the
+// octants' particle ranges of cell lb + i at cb, ce [8 i + o], and the block's
+// children and split cells into tot.  Eight lanes a cell.
+__global__ void __launch_bounds__(kWideThreads)
+k_wide_count(CellArrays c, int level, int ncrit, const uint64_t *keys, int32_t *cb, int32_t *ce, uint32_t *tot,
+             const unsigned *ctl)
+{
+    pdl_wait();
+    __shared__ unsigned s_ch[kWideThreads / 32], s_sp[kWideThreads / 32];
+    const WidePart p = wide_part(ctl, level);
+    if (p.ncl == 0) return;
+    const int tid = threadIdx.x, lane = tid & 31, o = lane & 7;
+    const unsigned gm = 0xffu << (lane & ~7);
+    unsigned nch = 0, nsp = 0;
+    for (int i = p.i0 + (tid >> 3); i < p.i1; i += kWideThreads / 8) {
+        const int cell = p.lb + i, b = c.begin[cell], en = c.end[cell];
+        if (level >= kLevels || en - b <= ncrit) {
+            if (o == 0) c.nchild[cell] = 0;
+            continue;
+        }
+        const int lo = o ? first_digit_ge(keys, b, en, level + 1, o) : b;
+        int hi = __shfl_down_sync(gm, lo, 1, 8);
+        if (o == 7) hi = en;
+        const int m = __popc((__ballot_sync(gm, hi > lo) >> (lane & ~7)) & 0xffu);
+        cb[8 * (int64_t)i + o] = lo;
+        ce[8 * (int64_t)i + o] = hi;
+        if (o == 0) {
+            c.nchild[cell] = m;
+            nch += (unsigned)m;
+            ++nsp;
+        }
+    }
+    nch = __reduce_add_sync(0xffffffffu, nch);
+    nsp = __reduce_add_sync(0xffffffffu, nsp);
+    if (lane == 0) {
+        s_ch[tid >> 5] = nch;
+        s_sp[tid >> 5] = nsp;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 1; w < kWideThreads / 32; ++w) {
+            nch += s_ch[w];
+            nsp += s_sp[w];
+        }
+        tot[2 * blockIdx.x] = nch;
+        tot[2 * blockIdx.x + 1] = nsp;
+    }
+}
+
+// The children of the level's cells and each cell's rank, after the totals of
+// the blocks before this one; the first block leaves the next level's bounds
+// (an empty level where the cells would pass the capacity, so that the launches behind do nothing).
+__global__ void __launch_bounds__(kWideThreads)
+k_wide_write(CellArrays c, int level, int64_t cap, const int32_t *cb, const int32_t *ce, const uint32_t *tot,
+             uint32_t *rank, unsigned *ctl)
+{
+    pdl_wait();
+    constexpr int kW = kWideThreads / 32;
+    __shared__ unsigned s_t[4], s_w[kW];
+    __shared__ int s_ch0[kWideThreads];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const WidePart p = wide_part(ctl, level);
+    if (p.ncl == 0) {
+        if (blockIdx.x == 0 && tid == 0) ctl[kCtlLevel + level + 2] = ctl[kCtlLevel + level + 1];
+        return;
+    }
+    const unsigned leaves = ctl[kCtlBefore + 2 * level], inner = ctl[kCtlBefore + 2 * level + 1];
+    if (tid < 4) s_t[tid] = 0;
+    __syncthreads();
+    {
+        unsigned v[4] = {0, 0, 0, 0};        // children and split cells: of the blocks before, of all
+        for (unsigned k = tid; k < gridDim.x; k += kWideThreads) {
+            const unsigned x = tot[2 * k], y = tot[2 * k + 1];
+            if (k < blockIdx.x) {
+                v[0] += x;
+                v[1] += y;
+            }
+            v[2] += x;
+            v[3] += y;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            v[q] = __reduce_add_sync(0xffffffffu, v[q]);
+            if (lane == 0 && v[q]) atomicAdd(&s_t[q], v[q]);
+        }
+    }
+    __syncthreads();
+    const int le = p.lb + p.ncl;
+    unsigned ch = s_t[0], sp = s_t[1];       // children and split cells before the next one
+    const bool over = (int64_t)le + s_t[2] > cap;
+    if (blockIdx.x == 0 && tid == 0) {
+        ctl[kCtlLevel + level + 2] = (unsigned)le + (over ? 0u : s_t[2]);
+        ctl[kCtlBefore + 2 * level + 2] = leaves + (unsigned)p.ncl - s_t[3];
+        ctl[kCtlBefore + 2 * level + 3] = inner + s_t[3];
+        ctl[kCtlLeaves] = leaves + (unsigned)p.ncl - s_t[3];
+        if (over) ctl[kCtlOverflow] = 1u;
+    }
+    if (over) return;
+    for (int base = p.i0; base < p.i1; base += kWideThreads) {
+        const int i = base + tid, cell = p.lb + i;
+        const unsigned n = i < p.i1 ? (unsigned)c.nchild[cell] : 0u;
+        // children and split cells in one scan: up to 2,048 and 256
+        unsigned x = n | (n ? 1u << 16 : 0u);
+        const unsigned v = x;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, d);
+            if (lane >= d) x += y;
+        }
+        if (lane == 31) s_w[warp] = x;
+        __syncthreads();
+        unsigned before = x - v, all = 0;
+#pragma unroll
+        for (int w = 0; w < kW; ++w) {
+            if (w < warp) before += s_w[w];
+            all += s_w[w];
+        }
+        const int ch0 = le + (int)(ch + (before & 0xffffu));
+        const unsigned k = sp + (before >> 16);
+        s_ch0[tid] = n ? ch0 : -1;
+        if (i < p.i1) {
+            c.child[cell] = n ? ch0 : -1;
+            rank[cell] = n ? inner + k : leaves + (unsigned)i - k;
+        }
+        __syncthreads();
+        for (int t = tid; t < 8 * kWideThreads; t += kWideThreads) {         // eight lanes per cell
+            const int q = t >> 3, o = t & 7, first = s_ch0[q];
+            if (first < 0) continue;
+            const int64_t at = 8 * (int64_t)(base + q) + o;
+            const int beg = cb[at], en = ce[at], pa = p.lb + base + q;
+            const unsigned gm = 0xffu << (lane & ~7);
+            const unsigned m = (__ballot_sync(gm, en > beg) >> (lane & ~7)) & 0xffu;
+            if (en > beg) {
+                const int to = first + __popc(m & ((1u << o) - 1u));
+                c.level[to] = level + 1;
+                c.parent[to] = pa;
+                c.begin[to] = beg;
+                c.end[to] = en;
+                c.cx[to] = 2 * c.cx[pa] + ((o >> 2) & 1);
+                c.cy[to] = 2 * c.cy[pa] + ((o >> 1) & 1);
+                c.cz[to] = 2 * c.cz[pa] + (o & 1);
+                c.sys[to] = c.sys[pa];
+            }
+        }
+        ch += all & 0xffffu;
+        sp += all >> 16;
+        __syncthreads();                     // s_w and s_ch0 are free again
     }
 }
 
@@ -1364,6 +1547,22 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
             cudaMemsetAsync(t->b_err.ptr, 0, sizeof(int), st);
             sort_one(full);
             continue;
+        }
+        // wide levels: four at a time, then a look whether any are left
+        const unsigned wide = hc[kCtlWide];
+        for (int l = (int)wide - 1; wide && !hc[kCtlOverflow] && l <= kLevels &&
+                                    hc[kCtlLevel + l + 1] > hc[kCtlLevel + l];) {
+            const unsigned g = (unsigned)(kWideBlocksPerSM * std::max(1, sm_count()));   // totals: 2 g <= cap words
+            for (const int to = std::min(l + 4, kLevels + 1); l < to; ++l) {
+                launch_next(st, k_wide_count, g, kWideThreads, 0, cells_of(t), l, t->max_leaf, keys, cbeg, cend,
+                            (uint32_t *)t->b_scan.ptr, ctl);
+                launch_next(st, k_wide_write, g, kWideThreads, 0, cells_of(t), l, cap, cbeg, cend,
+                            (const uint32_t *)t->b_scan.ptr, (uint32_t *)t->b_flags.ptr, ctl);
+                t->launches += 2;
+            }
+            FMM_TRY(cuda_check(t, cudaGetLastError(), "wide levels"));
+            FMM_TRY(cuda_check(t, cudaMemcpyAsync(hc, ctl, sizeof(hc), cudaMemcpyDeviceToHost, st), "level counts"));
+            FMM_TRY(cuda_check(t, cudaStreamSynchronize(st), "sync"));
         }
         if (!hc[kCtlOverflow]) break;
         cap *= 2;
