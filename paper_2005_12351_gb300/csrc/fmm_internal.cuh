@@ -237,6 +237,7 @@ struct fmm_tree {
     int s = -1, s_hi = -1, nS = 0;
     bool have_sources = false;
     int64_t ncells = 0, nleaves = 0;
+    int long_leaf = 0;                     // particles of the longest leaf past max_leaf (the deepest level), 0: none
     int nlevels = 0;
     std::vector<int> level_begin;          // host copy, nlevels + 1
     double lo[3] = {0, 0, 0}, side = 1.0;  // root box of system 0

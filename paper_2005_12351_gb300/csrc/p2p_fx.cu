@@ -396,9 +396,12 @@ __device__ __noinline__ void fx_close(int i, int j, const double *px, const doub
     }
 }
 
-// One block per target leaf.  The leaf's targets are cut into m tiles of t
-// (the cut that leaves the fewest threads without work), each covered k =
-// floor(threads / t) times; copy c takes the staged sources c, c + k, ...
+// One block per target leaf, several (blockIdx.y) where a leaf of the deepest level
+// holds more than max_leaf: one block took its tiles in turn (3,000 coincident
+// dipoles among 50,000 others 200 -> 35 ms, most of it the FP64 sums of those
+// targets; 3,000 within 1e-9 of each other 86 -> 15.5 ms).  The leaf's targets are
+// cut into m tiles of t (the cut that leaves the fewest threads without work), each
+// covered k = floor(threads / t) times; copy c takes the staged sources c, c + k, ...
 // Sources are staged already in fixed point and in the target leaf's frame: a
 // thread converts one source, about 3 % of the work of the pairs it serves.
 // A round holds sources of one coordinate unit (the coarser of the two leaves'
@@ -433,7 +436,8 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
     __shared__ unsigned char s_redo[512];
     const int A = leaves[blockIdx.x];
     const int b = begin[A], nt = end[A] - b;
-    if (nt == 0) return;
+    const int parts = nt > 2 * nthr ? (int)gridDim.y : 1;  // blocks that share the leaf
+    if (nt == 0 || (int)blockIdx.y >= parts) return;
     const int q0 = off[A], q1 = off[A + 1];
     const int lA = level[A], sy = sys[A];
     const int lside = ilogb(sys_box[4 * sy + 3]);
@@ -503,7 +507,8 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
             if (cost < best) { best = cost; tile = t; }
         }
     }
-    for (int t0 = 0; t0 < nt; t0 += tile) {
+    const int stride = parts * tile;
+    for (int t0 = (int)blockIdx.y * tile; t0 < nt; t0 += stride) {
         const int cnt = min(tile, nt - t0), k = nthr / cnt;
         const int ti = tid % cnt, sp = tid / cnt;
         const bool act = sp < k;
@@ -689,7 +694,7 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
                 __syncthreads();
             }
         }
-        if (t0 + tile < nt)
+        if (t0 + stride < nt)
             for (int c = 0; c < NC; ++c) accd[c * nthr + tid] = 0.0;
     }
 }
@@ -704,7 +709,10 @@ void launch_fx(fmm_tree *t, int want_phi, int want_field, double *phi, double *E
         const size_t smem = 8 * (size_t)nc * nthr +
                             std::max<size_t>(16 * (size_t)nw * ch, 32 * (size_t)nc * nthr);
         allow_max_dynamic_smem(kern);
-        launch_next(t->stream, kern, (unsigned)t->nleaves, nthr, smem,
+        // blocks a leaf: two tiles or so each, and not many millions of blocks with nothing to do
+        const int64_t want = t->long_leaf ? (t->long_leaf + 2 * nthr - 1) / (2 * nthr) : 1;
+        const unsigned parts = (unsigned)std::min<int64_t>({want, 256, std::max<int64_t>(8, (1 << 20) / t->nleaves)});
+        launch_next(t->stream, kern, dim3((unsigned)t->nleaves, parts), nthr, smem,
             (const int32_t *)t->b_leaves.ptr, (const int32_t *)t->b_begin.ptr, (const int32_t *)t->b_end.ptr,
             (const int32_t *)t->b_p2p_off.ptr, (const int32_t *)t->b_p2p_src.ptr, (const int32_t *)t->b_level.ptr,
             (const int32_t *)t->b_cx.ptr, (const int32_t *)t->b_cy.ptr, (const int32_t *)t->b_cz.ptr,

@@ -396,11 +396,12 @@ __device__ __forceinline__ int digit_at(uint64_t key, int level)
 // ctl: [0] overflow (more cells than cap), [1 + l] first cell of level l, then
 // the leaf count, the error word, the tie flag (a run the tie sort left: no
 // cells, the host sorts again), one more than the level where the whole chip
-// takes over (0: none), and the first system's box as four doubles; behind the
-// words that go to the host the blocks' totals, and per level the leaves and the
-// cells with children before it.
+// takes over (0: none), the particles of the longest leaf past n_crit (deepest
+// level), and the first system's box as four doubles; behind the words that go to
+// the host the blocks' totals, and per level the leaves and the cells with children
+// before it.
 constexpr int kCtlOverflow = 0, kCtlLevel = 1, kCtlLeaves = 26, kCtlErr = 27, kCtlTie = 28, kCtlWide = 29,
-              kCtlBox = 32, kCtlHost = 40, kCtlTot = 40, kCtlBefore = 40 + 4 * 16,
+              kCtlLong = 30, kCtlBox = 32, kCtlHost = 40, kCtlTot = 40, kCtlBefore = 40 + 4 * 16,
               kCtlWords = kCtlBefore + 2 * (kLevels + 2);             // words [0, kCtlHost) go to the host
 constexpr int kCellBlocks = 8, kCellThreads = 1024;
 constexpr int kWideLevel = 1 << 16;
@@ -485,6 +486,7 @@ k_cells(CellArrays c, const int64_t *off, int nsys, const double *box, const int
         c.cx[s] = c.cy[s] = c.cz[s] = 0;
         c.sys[s] = s;
     }
+    if (blk == 0 && tid == 0) ctl[kCtlLong] = 0u;
     cluster_sync_all();
     int lb = 0, le = tie ? 0 : nsys;
     unsigned leaves = 0, inner = 0;            // before this level
@@ -582,8 +584,11 @@ k_cells(CellArrays c, const int64_t *off, int nsys, const double *box, const int
                 }
             }
             for (int i = i0 + tid; i < i1; i += kCellThreads) {
-                const int cell = lb + i;
-                if (level < kLevels && __ldcg(c.end + cell) - __ldcg(c.begin + cell) > ncrit) continue;
+                const int cell = lb + i, held = __ldcg(c.end + cell) - __ldcg(c.begin + cell);
+                if (held > ncrit) {
+                    if (level < kLevels) continue;
+                    atomicMax(ctl + kCtlLong, (unsigned)held);
+                }
                 c.nchild[cell] = 0;
                 c.child[cell] = -1;
                 rank[cell] = leaves + (unsigned)i - (p0 + rank[cell]);
@@ -636,7 +641,7 @@ __device__ __forceinline__ WidePart wide_part(const unsigned *ctl, int level)
 // children and split cells into tot.  Eight lanes a cell.
 __global__ void __launch_bounds__(kWideThreads)
 k_wide_count(CellArrays c, int level, int ncrit, const uint64_t *keys, int32_t *cb, int32_t *ce, uint32_t *tot,
-             const unsigned *ctl)
+             unsigned *ctl)
 {
     pdl_wait();
     __shared__ unsigned s_ch[kWideThreads / 32], s_sp[kWideThreads / 32];
@@ -648,7 +653,10 @@ k_wide_count(CellArrays c, int level, int ncrit, const uint64_t *keys, int32_t *
     for (int i = p.i0 + (tid >> 3); i < p.i1; i += kWideThreads / 8) {
         const int cell = p.lb + i, b = c.begin[cell], en = c.end[cell];
         if (level >= kLevels || en - b <= ncrit) {
-            if (o == 0) c.nchild[cell] = 0;
+            if (o == 0) {
+                c.nchild[cell] = 0;
+                if (en - b > ncrit) atomicMax(ctl + kCtlLong, (unsigned)(en - b));
+            }
             continue;
         }
         const int lo = o ? first_digit_ge(keys, b, en, level + 1, o) : b;
@@ -1432,6 +1440,7 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
     cudaStream_t st = t->stream;
     t->have_lists = false;
     t->ncells = t->nleaves = 0;
+    t->long_leaf = 0;
     t->nlevels = 0;
     t->level_begin.clear();
     if (n == 0) return FMM_OK;
@@ -1577,6 +1586,7 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
     t->ncells = t->level_begin.back();
     t->nlevels = nlev;
     t->nleaves = hc[kCtlLeaves];
+    t->long_leaf = (int)hc[kCtlLong];
     t->lo[0] = t->sys_box[0]; t->lo[1] = t->sys_box[1]; t->lo[2] = t->sys_box[2];
     t->side = t->sys_box[3];
     const int64_t nc = t->ncells;
