@@ -1787,13 +1787,15 @@ fmm_status build_lists(fmm_tree *t, double theta)
     int64_t ndoff = 0;
     if (nm2l > 0) {
         uint32_t H = 1u << 16;
+        size_t dcap = 0;
         for (bool again = false;; again = true) {
             FMM_TRY(ensure(t, t->b_hash, 8 * (size_t)H));
-            FMM_TRY(ensure(t, t->b_dsort, 12 * (size_t)H));       // the list: keys, then slots
+            dcap = (size_t)std::min<int64_t>(H, nm2l);            // distinct keys, at most
+            FMM_TRY(ensure(t, t->b_dsort, 12 * dcap));            // the list: keys, then slots
             FMM_TRY(ensure(t, t->b_scan, 4 * (size_t)H));         // slot -> rank
             FMM_TRY(ensure(t, t->b_dkeys, 8 * (size_t)kRankSmall));
             uint64_t *lkey = (uint64_t *)t->b_dsort.ptr;
-            uint32_t *lslot = (uint32_t *)(lkey + H), *rank_of = (uint32_t *)t->b_scan.ptr;
+            uint32_t *lslot = (uint32_t *)(lkey + dcap), *rank_of = (uint32_t *)t->b_scan.ptr;
             cudaMemsetAsync(t->b_hash.ptr, 0xff, 8 * (size_t)H, st);
             if (again) cudaMemsetAsync(cnt + 10, 0, 4 * 4, st);   // errors, gap, count
             launch_next(st, k_offset_keys, (unsigned)std::min<int64_t>((nc + 7) / 8, 8 * (int64_t)sm_count()), 256, 0,
@@ -1821,7 +1823,7 @@ fmm_status build_lists(fmm_tree *t, double theta)
         ndoff = hw.nd;
         if (ndoff > (int64_t)kRankSmall) {
             uint64_t *lkey = (uint64_t *)t->b_dsort.ptr;
-            uint32_t *lslot = (uint32_t *)(lkey + H), *rank_of = (uint32_t *)t->b_scan.ptr;
+            uint32_t *lslot = (uint32_t *)(lkey + dcap), *rank_of = (uint32_t *)t->b_scan.ptr;
             FMM_TRY(ensure(t, t->b_dkeys, 8 * (size_t)ndoff));
             FMM_TRY(ensure(t, t->b_lkeys2, 8 * (size_t)ndoff));
             FMM_TRY(ensure(t, t->b_lval2, 4 * (size_t)ndoff));
