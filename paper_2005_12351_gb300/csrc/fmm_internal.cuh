@@ -33,6 +33,7 @@ constexpr int kErrTcTimeout = 8;       // a tensor-core M2L wait gave up (word 1
 constexpr int kErrSortWait = 16;       // a look-back wait of the radix sort gave up
 constexpr int kErrLongRow = 32;        // a row of an interaction list too long for the row sort
 constexpr int kErrTieRun = 64;         // a run of equal leading key bits too long for the tie sort
+constexpr int kErrLongTies = 128;      // the same seen after a sort by all bits (no error)
 
 inline int ntot(int p) { return p < 0 ? 0 : (p + 1) * (p + 2) * (p + 3) / 6; }
 inline int nshell(int k) { return (k + 1) * (k + 2) / 2; }
@@ -249,7 +250,7 @@ struct fmm_tree {
     bool have_lists = false;
     int64_t n_m2l = 0, n_p2p = 0, n_p2p_inter = 0, n_doff = 0;
     size_t m2l_cap_hint = 0;
-    bool sort_full = false;                // an earlier set had a long run of equal leading key bits
+    bool sort_full = false;                // the last set had a long run of equal leading key bits
     int max_gap = 0;                       // largest level gap of an M2L pair
     // D tables / operator tables
     int d_p = -1;                          // p the D table was built for

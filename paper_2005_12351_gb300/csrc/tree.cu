@@ -181,6 +181,36 @@ inline int first_pass(int64_t n) { return n <= (1 << 14) ? 5 : (n <= (1 << 22) ?
 // arrays in the new order too.
 constexpr int kTieRun = 256;
 
+// The elements of the run of `top` next to element i on one side, at most
+// kTieRun: one by one up to kTieNear, then by doubling and halving steps (the run
+// is contiguous).  move: of the first kTieNear, those out of order with `key`.
+constexpr int kTieNear = 8;
+template <int DIR>
+__device__ __forceinline__ int run_reach(const uint64_t *keys, int64_t i, int64_t n, int shift, uint64_t key, int &move)
+{
+    auto at = [&](int q, uint64_t &o) {
+        const int64_t j = i + DIR * q;
+        if (DIR < 0 ? j < 0 : j >= n) return false;
+        o = keys[j];
+        return o >> shift == key >> shift;
+    };
+    uint64_t o;
+    int lo = 0;
+    for (; lo < kTieNear && at(lo + 1, o); ++lo) move += DIR < 0 ? -(int)(o > key) : (int)(o < key);
+    if (lo < kTieNear) return lo;
+    int hi = 2 * kTieNear;                  // lo is in the run
+    while (hi <= kTieRun && at(hi, o)) {
+        lo = hi;
+        hi *= 2;
+    }
+    hi = min(hi, kTieRun + 1);              // hi is not, or does not matter
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (at(mid, o)) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
 template <bool GATHER>
 __global__ void __launch_bounds__(256)
 k_tie_sort(const uint64_t *keys, const uint32_t *idx, int64_t n, int shift, uint64_t *okeys, uint32_t *oidx, int *err,
@@ -190,22 +220,18 @@ k_tie_sort(const uint64_t *keys, const uint32_t *idx, int64_t n, int shift, uint
     pdl_wait();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const uint64_t key = keys[i], top = key >> shift;
+    const uint64_t key = keys[i];
     const uint32_t id = idx[i];
-    int left = 0, right = 0, move = 0;
-    for (; left < kTieRun && i - left - 1 >= 0; ++left) {
-        const uint64_t o = keys[i - left - 1];
-        if (o >> shift != top) break;
-        move -= o > key;
-    }
-    for (; right < kTieRun && i + right + 1 < n; ++right) {
-        const uint64_t o = keys[i + right + 1];
-        if (o >> shift != top) break;
-        move += o < key;
-    }
+    int move = 0;
+    const int left = run_reach<-1>(keys, i, n, shift, key, move), right = run_reach<1>(keys, i, n, shift, key, move);
     if (left + right + 1 > kTieRun) {
         move = 0;
         if ((*(volatile int *)err & kErrTieRun) == 0) atomicOr(err, kErrTieRun);
+    } else {
+#pragma unroll 4
+        for (int q = kTieNear + 1; q <= left; ++q) move -= keys[i - q] > key;
+#pragma unroll 4
+        for (int q = kTieNear + 1; q <= right; ++q) move += keys[i + q] < key;
     }
     const int64_t k = i + move;
     okeys[k] = key;
@@ -346,12 +372,17 @@ __global__ void k_regather_keys(const uint64_t *key_of, const uint32_t *idx, int
     if (k < n) keys[k] = key_of[idx[k]];
 }
 
+// keys (or NULL): sorted; a run of more than kTieRun equal ones from bit `shift` up sets kErrLongTies
 __global__ void k_gather(const double *pos, const double *mom, int nS, const uint32_t *perm,
-                         int64_t n, double *px, double *py, double *pz, double *S, int32_t *perm_out)
+                         int64_t n, double *px, double *py, double *pz, double *S, int32_t *perm_out,
+                         const uint64_t *keys, int shift, int *err)
 {
     pdl_wait();
     int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= n) return;
+    if (keys && k + kTieRun < n && keys[k] >> shift == keys[k + kTieRun] >> shift &&
+        (*(volatile int *)err & kErrLongTies) == 0)
+        atomicOr(err, kErrLongTies);
     const int64_t o = perm[k];
     px[k] = pos[3 * o];
     py[k] = pos[3 * o + 1];
@@ -1468,8 +1499,8 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
     cudaMemsetAsync(t->b_err.ptr, 0, sizeof(int), st);
     FMM_TRY(cuda_check(t, cudaMemcpyAsync(off, t->sys_off.data(), 8 * (size_t)(nsys + 1),
                                           cudaMemcpyHostToDevice, st), "system offsets"));
-    // one system: by the leading key bits and the tie sort, by all bits where an
-    // earlier set of this handle (or, below, this one) had a long run of ties
+    // one system: by the leading key bits and the tie sort, by all bits where the
+    // last set of this handle (or, below, this one) had a long run of ties
     auto sort_one = [&](bool full) {
         uint64_t *keys2 = (uint64_t *)t->b_keys2.ptr;
         uint32_t *idx2 = (uint32_t *)t->b_idx2.ptr, *hist = (uint32_t *)t->b_hist.ptr;
@@ -1485,7 +1516,8 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
         record(t, 1);
         radix_sort_top(ka, va, kb, vb, n, p0, hist, err, st, &t->launches);
         if (full)
-            launch_next(st, k_gather, grid(n, 256), 256, 0, pos, mom, t->nS, idx, n, px, py, pz, S, perm);
+            launch_next(st, k_gather, grid(n, 256), 256, 0, pos, mom, t->nS, idx, n, px, py, pz, S, perm, keys,
+                        8 * first_pass(n), err);
         else
             launch_next(st, k_tie_sort<true>, grid(n, 256), 256, 0, keys2, idx2, n, 8 * p0, keys, idx, err, pos, mom, t->nS,
                                                             px, py, pz, S, perm);
@@ -1521,7 +1553,7 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
         k_regather_keys<<<grid(n, 256), 256, 0, st>>>(key_of, idx, n, keys);
         launch_next(st, k_gather, grid(n, 256), 256, 0, pos, mom, t->nS, idx, n, (double *)t->b_px.ptr,
                                                (double *)t->b_py.ptr, (double *)t->b_pz.ptr,
-                                               (double *)t->b_S.ptr, (int32_t *)t->b_perm.ptr);
+                                               (double *)t->b_S.ptr, (int32_t *)t->b_perm.ptr, nullptr, 0, nullptr);
         t->launches += 3;
         record(t, 2);
     }
@@ -1577,7 +1609,7 @@ fmm_status build_tree(fmm_tree *t, const double *pos, const double *mom)
         cap *= 2;
     }
     FMM_TRY(check_err(t, (int)hc[kCtlErr]));
-    t->sort_full = nsys == 1 && full;
+    t->sort_full = nsys == 1 && full && (hc[kCtlErr] & kErrLongTies);
     if (nsys == 1) std::memcpy(t->sys_box.data(), hc + kCtlBox, 32);
     // levels 0 .. nlev - 1 hold cells
     int nlev = 1;
