@@ -949,6 +949,25 @@ k_downward(int64_t nc, const int32_t *parent, const double *centre, DevTables tb
 
 inline unsigned grid(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
+// 1/(k_x! k_y! k_z!) of every index, a double as two words; the same for all
+// handles and orders, formed once (every evaluate assembles the tables)
+static const std::vector<int> &inv_factorial_words()
+{
+    static const std::vector<int> words = [] {
+        const MultiIndex &I = multi_index();
+        std::vector<int> v(2 * (size_t)kMaxTot);
+        for (int i = 0; i < kMaxTot; ++i) {
+            double f = 1.0;                      // exact: at most 12!
+            for (int q : {I.nx[i], I.ny[i], I.nz[i]})
+                for (int j = 2; j <= q; ++j) f *= j;
+            f = 1.0 / f;
+            std::memcpy(&v[2 * i], &f, 8);
+        }
+        return v;
+    }();
+    return words;
+}
+
 // Table buffer layout (int32): lut | p2m | m2m_off | m2m_kq | l2p_grad | red_off |
 // red_src | l2l_ix | l2p_ord | 1/k! | harmonic maps | packed indices
 fmm_status upload_tables(fmm_tree *t, int s, int p, int n_lo, DevTables *dt, const int32_t **lut)
@@ -994,19 +1013,7 @@ fmm_status upload_tables(fmm_tree *t, int s, int p, int n_lo, DevTables *dt, con
     if (buf.size() & 1) buf.push_back(0);                 // read in pairs of words
     const size_t o_ix = put(T.l2l_ix);
     const size_t o_ord = put(T.l2p_ord);
-    size_t o_if;
-    {
-        const MultiIndex &I = multi_index();
-        std::vector<int> v(2 * (size_t)kMaxTot);
-        for (int i = 0; i < kMaxTot; ++i) {
-            double f = 1.0;                      // exact: at most 12!
-            for (int q : {I.nx[i], I.ny[i], I.nz[i]})
-                for (int j = 2; j <= q; ++j) f *= j;
-            f = 1.0 / f;
-            std::memcpy(&v[2 * i], &f, 8);
-        }
-        o_if = put(v);
-    }
+    const size_t o_if = put(inv_factorial_words());
     o_rsrc = put(T.m2l_red_src);
     const size_t o_hrm = put(T.h_rm), o_hf = put(T.h_fold), o_hfo = put(T.h_fold_off);
     const size_t o_hu = put(T.h_unfold), o_huo = put(T.h_unfold_off), o_hrn = put(T.h_rn);
