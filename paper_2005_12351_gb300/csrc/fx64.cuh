@@ -30,10 +30,9 @@ __device__ __forceinline__ s64 madw(int a, int b, s64 c)
     asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
     return d;
 }
-// The same as a product and an addition, which the compiler fuses: a chain of
-// them into one sum costs 4.6 clocks each where madw, whose sum it moves first,
-// costs 5.4.  Where several results meet in later additions it reorders those
-// and the form with the addend can be the faster one (the sums of p2p_fx.cu).
+// The same written as a product and an addition: measured, a chain of them into
+// one sum takes 4.6 clocks each, of madw 5.4.  Where several results meet in later
+// additions the form with the addend can be the faster one (the sums of p2p_fx.cu).
 __device__ __forceinline__ s64 madp(int a, int b, s64 c)
 {
     s64 d;
@@ -47,23 +46,11 @@ __device__ __forceinline__ u64 madu(uint32_t a, uint32_t b, u64 c)
     return d + c;
 }
 
-// shifts whose amount may pass the width (the result is then 0)
-__device__ __forceinline__ uint32_t shr32(uint32_t a, uint32_t n)
-{
-    uint32_t d;
-    asm("shr.u32 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(n));
-    return d;
-}
+// a shift whose amount may pass the width (the result is then 0)
 __device__ __forceinline__ uint32_t shl32(uint32_t a, uint32_t n)
 {
     uint32_t d;
     asm("shl.b32 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(n));
-    return d;
-}
-__device__ __forceinline__ u64 shr64(u64 a, uint32_t n)
-{
-    u64 d;
-    asm("shr.u64 %0, %1, %2;" : "=l"(d) : "l"(a), "r"(n));
     return d;
 }
 

@@ -354,16 +354,18 @@ __device__ __forceinline__ bool fx_stage_orders(const double *Sj, int bp, int be
 
 // What a term of base b can lose in fx_add, in units of the sums, when its shift is
 // b less up to k sh: nothing down to 56, the lower limb (below 2^(84 - shift)) down
-// to 84, all of it (below 2^(115 - shift)) beyond.
-__device__ __forceinline__ float fx_loss(int b, int k, int sh)
+// to 84, all of it (below 2^(115 - shift)) beyond.  At least one unit, a whole
+// number, so that the count does not depend on the order of its atomics (as a float
+// it did in its last bits, and with it which sums a set at the line forms again).
+__device__ __forceinline__ u64 fx_loss(int b, int k, int sh)
 {
     const int lo = max(b - k * sh, kWhole + 1);            // the smallest shift that loses anything
-    return exp2f((float)(lo > 84 ? 115 - lo : (b > 84 ? 30 : 84 - lo)));
+    return 1ull << (lo > 84 ? max(115 - lo, 0) : (b > 84 ? 30 : 84 - lo));
 }
 // The same of all terms of one source, added to lost[0] (potential) and lost[1]
 // (field).  gap: a target of the leaf is at least so far away along some axis.
 template <int SLO, int SHI, bool PHI, bool FIELD>
-__device__ __noinline__ void fx_count_loss(const double *Sj, int bp, int be, int lu, s64 gap, float *lost)
+__device__ __noinline__ void fx_count_loss(const double *Sj, int bp, int be, int lu, s64 gap, u64 *lost)
 {
     const int sh = gap > 0 ? min(kShMax, __clzll(gap) - 1) : kShMax;     // the largest normalising shift
     int o = 0;
@@ -432,7 +434,7 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
     __shared__ int gbeg[kFxGroups], gpre[kFxGroups + 1];
     __shared__ int s_next_q, s_next_j, s_ng, s_key;
     __shared__ int s_g, s_mx[3];
-    __shared__ float s_lost[2];                            // what the row's terms can lose, units of the sums
+    __shared__ u64 s_lost[2];                              // what the row's terms can lose, units of the sums
     __shared__ unsigned char s_redo[512];
     const int A = leaves[blockIdx.x];
     const int b = begin[A], nt = end[A] - b;
@@ -445,7 +447,7 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
     // sources, largest moment exponent per shell
     if (tid < 3) s_mx[tid] = kNone;
     if (tid == 3) s_g = 1;
-    if (tid >= 4 && tid < 6) s_lost[tid - 4] = 0.0f;
+    if (tid >= 4 && tid < 6) s_lost[tid - 4] = 0;
     __syncthreads();
     {
         const s64 rA = 1ll << (kLevels - lA);
@@ -530,7 +532,7 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
             s64 tx = 0, ty = 0, tz = 0;
             int key_t = -1;
             int q = q0, j_in = 0;
-            if (tid < 2) s_lost[tid] = 0.0f;               // the round's barriers come first
+            if (tid < 2) s_lost[tid] = 0;                  // the round's barriers come first
             while (q < q1) {
                 __syncthreads();
                 if (tid < 32) {
@@ -661,8 +663,8 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
                 for (int a = 0; a < 3; ++a) E_out[3 * o + a] = E_far[3 * (int64_t)i + a] + v[ef + a];
             }
             // what the terms can have lost against 2^-54 of the sums
-            if (PHI && s_lost[0] > 0.0f && scalbn((double)s_lost[0], bp - kUnitP + 54) > fabs(v[0])) redo = 1;
-            if (FIELD && s_lost[1] > 0.0f && scalbn((double)s_lost[1], be - kUnitE + 54) >
+            if (PHI && s_lost[0] && scalbn((double)s_lost[0], bp - kUnitP + 54) > fabs(v[0])) redo = 1;
+            if (FIELD && s_lost[1] && scalbn((double)s_lost[1], be - kUnitE + 54) >
                                                  fmax(fabs(v[ef]), fmax(fabs(v[ef + 1]), fabs(v[ef + 2]))))
                 redo |= 2;
         }
