@@ -456,14 +456,26 @@ inline unsigned gridn(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs);
 }  // namespace
 
 // The line between this form and the per-cell k_m2l: the list's products a
-// system.  The plan costs 40 to 100 us on new lists, and small or strongly
-// graded sets fill the 32 lanes badly.  Evaluates with new lists, per cell ->
-// here: 1 6 (source order, p) uniform, 419k pairs (3.4e8 products) 2.00 -> 1.60
-// ms; 1 6 Plummer, 174k pairs (1.4e8) 1.82 -> 1.84; 2 8 Plummer, 78k pairs
-// (2.0e8) 2.22 -> 2.33 and 172k pairs (4.3e8) 3.10 -> 2.86; 0 3 uniform, 419k
-// pairs (0.4e8) no difference.  Handles with a memory budget keep the per-cell
-// kernel, so that a served request's bits do not depend on its slot's memory.
+// system, and its pairs per distinct offset, on which depends how full the plan's
+// rows are (a row holds a tile's pairs of one offset; an adaptive tree has six times
+// the offsets of a uniform one).  Evaluates with new lists, per cell -> here, ms:
+//   uniform          1 6 (source order, p) 419k pairs, 3.4e8 products   1.76 -> 1.30
+//                    0 3 419k pairs, 0.4e8 products                     no difference
+//                    1 11 38k pairs, 2.0e8 (110 pairs an offset)        2.09 -> 1.44
+//   Plummer          2 8 91k pairs, 2.3e8 (44)                          2.09 -> 2.18
+//                    2 8 143k, 3.6e8 (60)                               2.51 -> 2.48
+//                    1 10 61k, 2.4e8 (29)                               2.09 -> 2.40
+//                    1 10 129k, 5.1e8 (55)                              2.92 -> 2.94
+//                    1 6 272k, 2.2e8 (126)                              1.94 -> 1.88
+//   theta 0.4        1 7 286k, 3.7e8 (37)                               3.36 -> 3.65
+// Past p + s = 11 of charges and dipoles the per-cell kernel falls off and the line
+// lies lower: Plummer 1 11 49k pairs (25) 2.65 -> 2.71, 68k (33) 3.24 -> 2.94; 0 12 the same.
+// Lists that stay (loops) gain 0.1 to 0.3 ms more than these, the plan's time.
+// Handles with a memory budget keep the per-cell kernel, so that a served request's
+// bits do not depend on its slot's memory.
 constexpr double kFxMinWork = 2.0e8;
+constexpr int64_t kFxMinFill = 56, kFxMinFillHigh = 30;    // pairs an offset
+constexpr int kFxHighProducts = 5000;
 
 bool fx_usable(fmm_tree *t, int s, int p, int harmonic, int n_lo)
 {
@@ -477,8 +489,9 @@ bool fx_usable(fmm_tree *t, int s, int p, int harmonic, int n_lo)
     }
     if (t->fx_off) return false;
     const double nsys = (double)std::max<int64_t>(1, (int64_t)t->sys_off.size() - 1);
-    return (double)t->n_m2l * Ly.products >= kFxMinWork * nsys && Ly.cap > 0 && Ly.nM <= kFxMaxNM &&
-           fx_smem(Ly) <= (size_t)kFxSmemMax;
+    const double fill = (double)(Ly.products > kFxHighProducts ? kFxMinFillHigh : kFxMinFill) * t->n_doff;
+    return (double)t->n_m2l * Ly.products >= kFxMinWork * nsys && (double)t->n_m2l >= fill * nsys && Ly.cap > 0 &&
+           Ly.nM <= kFxMaxNM && fx_smem(Ly) <= (size_t)kFxSmemMax;
 }
 
 fmm_status fx_prepare(fmm_tree *t, int p)
