@@ -41,10 +41,11 @@
 // while the sources are staged) passes 2^-54 of it: a target that holds the row's
 // largest moment itself, coincides with it or sees none of its field, from ratios
 // to the others of about 2^42 (charges), 2^35 (dipoles) and 2^28 (quadrupoles) on.
-// That costs 0.6 % of the P2P at 1M dipoles, 2 to 4 % at 262k Plummer and 200k
-// charges and dipoles (the count in the staging and the compiler's schedule; the
-// pairs' loop is the same).  Keeping every bit in the loop instead cost 2 to 5 %.
+// That costs about 0.6 % of the P2P at 1M dipoles, 1 % at 262k Plummer and 200k
+// charges and dipoles (the count in the staging; the pairs' loop is the same).
+// Keeping every bit in the loop instead cost 2 to 5 %.
 #include <algorithm>
+#include <type_traits>
 
 #include "fmm_internal.cuh"
 #include "fx64.cuh"
@@ -398,12 +399,56 @@ __device__ __noinline__ void fx_close(int i, int j, const double *px, const doub
     }
 }
 
+// What the terms of a row can have lost against 2^-54 of a target's sums: 1 the
+// potential, 2 the field.  Out of line, like the next one: rare, and written into
+// k_p2p_fx the two took 1.5 % of its time (200k Plummer charges 3.33 instead of 3.28
+// ms an evaluate).
+template <bool PHI, bool FIELD>
+__device__ __noinline__ int fx_lost(const u64 *lost, int bp, int be, double f, double e0, double e1, double e2)
+{
+    int redo = 0;
+    if (PHI && lost[0] && scalbn((double)lost[0], bp - kUnitP + 54) > fabs(f)) redo = 1;
+    if (FIELD && lost[1] && scalbn((double)lost[1], be - kUnitE + 54) > fmax(fabs(e0), fmax(fabs(e1), fabs(e2)))) redo |= 2;
+    return redo;
+}
+// The marked targets' rows in FP64, the block's threads side by side
+template <int SLO, int SHI, bool PHI, bool FIELD>
+__device__ __noinline__ void fx_redo(const unsigned char *redo, int cnt, int i0, int q0, int q1, const int32_t *src,
+                                     const int32_t *begin, const int32_t *end, const double *px, const double *py,
+                                     const double *pz, const double *Sm, double *accd, const double *phi_far,
+                                     const double *E_far, const int32_t *perm, double *phi_out, double *E_out)
+{
+    constexpr int NC = (PHI ? 1 : 0) + (FIELD ? 3 : 0), ef = PHI ? 1 : 0;
+    const int nthr = blockDim.x, tid = threadIdx.x;
+    for (int u = 0; u < cnt; ++u) {
+        const int which = redo[u], iu = i0 + u;
+        if (which == 0) continue;
+        for (int c = 0; c < NC; ++c) accd[c * nthr + tid] = 0.0;
+        for (int q = q0; q < q1; ++q) {
+            const int B = src[q], je = end[B];
+            for (int j = begin[B] + tid; j < je; j += nthr)
+                fx_close<SLO, SHI, PHI, FIELD>(iu, j, px, py, pz, Sm, accd + tid, nthr);
+        }
+        __syncthreads();
+        if (tid < NC && (which >> (tid >= ef) & 1)) {
+            double d = 0.0;
+            for (int w = 0; w < nthr; ++w) d += accd[tid * nthr + w];
+            const int64_t o = perm[iu];
+            if (tid < ef) phi_out[o] = phi_far[iu] + d;
+            else E_out[3 * o + tid - ef] = E_far[3 * (int64_t)iu + tid - ef] + d;
+        }
+        __syncthreads();
+    }
+}
+
 // One block per target leaf, several (blockIdx.y) where a leaf of the deepest level
 // holds more than max_leaf: one block took its tiles in turn (3,000 coincident
 // dipoles among 50,000 others 200 -> 35 ms, most of it the FP64 sums of those
-// targets; 3,000 within 1e-9 of each other 86 -> 15.5 ms).  The leaf's targets are
-// cut into m tiles of t (the cut that leaves the fewest threads without work), each
-// covered k = floor(threads / t) times; copy c takes the staged sources c, c + k, ...
+// targets; 3,000 within 1e-9 of each other 86 -> 15.5 ms).  That is the LONG form: the
+// kernel without it is faster (262k Plummer dipoles 8.43 instead of 8.58 ms an
+// evaluate).  The leaf's targets are cut into m tiles of t (the cut that leaves the
+// fewest threads without work), each covered k = floor(threads / t) times; copy c
+// takes the staged sources c, c + k, ...
 // Sources are staged already in fixed point and in the target leaf's frame: a
 // thread converts one source, about 3 % of the work of the pairs it serves.
 // A round holds sources of one coordinate unit (the coarser of the two leaves'
@@ -411,7 +456,7 @@ __device__ __noinline__ void fx_close(int i, int j, const double *px, const doub
 // between rounds.
 // The charges' potential fits 64 registers, which holds it at 16 blocks of 128 an SM
 // (500k charges: 6.16 ms, 6.5 with 111 registers); the others need all 128.
-template <int SLO, int SHI, bool PHI, bool FIELD>
+template <int SLO, int SHI, bool PHI, bool FIELD, bool LONG>
 __global__ void __launch_bounds__(512, SHI == 0 && !FIELD ? 2 : 1)
 k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const int32_t *off,
          const int32_t *src, const int32_t *level, const int32_t *cx, const int32_t *cy, const int32_t *cz,
@@ -438,8 +483,8 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
     __shared__ unsigned char s_redo[512];
     const int A = leaves[blockIdx.x];
     const int b = begin[A], nt = end[A] - b;
-    const int parts = nt > 2 * nthr ? (int)gridDim.y : 1;  // blocks that share the leaf
-    if (nt == 0 || (int)blockIdx.y >= parts) return;
+    const int parts = LONG && nt > 2 * nthr ? (int)gridDim.y : 1;     // blocks that share the leaf
+    if (nt == 0 || (LONG && (int)blockIdx.y >= parts)) return;
     const int q0 = off[A], q1 = off[A + 1];
     const int lA = level[A], sy = sys[A];
     const int lside = ilogb(sys_box[4 * sy + 3]);
@@ -510,7 +555,7 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
         }
     }
     const int stride = parts * tile;
-    for (int t0 = (int)blockIdx.y * tile; t0 < nt; t0 += stride) {
+    for (int t0 = LONG ? (int)blockIdx.y * tile : 0; t0 < nt; t0 += stride) {
         const int cnt = min(tile, nt - t0), k = nthr / cnt;
         const int ti = tid % cnt, sp = tid / cnt;
         const bool act = sp < k;
@@ -662,39 +707,14 @@ k_p2p_fx(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
 #pragma unroll
                 for (int a = 0; a < 3; ++a) E_out[3 * o + a] = E_far[3 * (int64_t)i + a] + v[ef + a];
             }
-            // what the terms can have lost against 2^-54 of the sums
-            if (PHI && s_lost[0] && scalbn((double)s_lost[0], bp - kUnitP + 54) > fabs(v[0])) redo = 1;
-            if (FIELD && s_lost[1] && scalbn((double)s_lost[1], be - kUnitE + 54) >
-                                                 fmax(fabs(v[ef]), fmax(fabs(v[ef + 1]), fabs(v[ef + 2]))))
-                redo |= 2;
+            if (s_lost[0] | s_lost[1])
+                redo = fx_lost<PHI, FIELD>(s_lost, bp, be, v[0], v[FIELD ? ef : 0], v[FIELD ? ef + 1 : 0], v[FIELD ? ef + 2 : 0]);
         }
         if (__syncthreads_or(redo)) {
-            // rare: those targets' rows in FP64, the block's threads side by side
             if (tid < cnt) s_redo[tid] = (unsigned char)redo;
             __syncthreads();
-#pragma unroll 1
-            for (int u = 0; u < cnt; ++u) {
-                const int which = s_redo[u], iu = b + t0 + u;
-                if (which == 0) continue;
-                for (int c = 0; c < NC; ++c) accd[c * nthr + tid] = 0.0;
-#pragma unroll 1
-                for (int q = q0; q < q1; ++q) {
-                    const int B = src[q], je = end[B];
-#pragma unroll 1
-                    for (int j = begin[B] + tid; j < je; j += nthr)
-                        fx_close<SLO, SHI, PHI, FIELD>(iu, j, px, py, pz, Sm, accd + tid, nthr);
-                }
-                __syncthreads();
-                if (tid < NC && (which >> (tid >= ef) & 1)) {
-                    double d = 0.0;
-#pragma unroll 1
-                    for (int w = 0; w < nthr; ++w) d += accd[tid * nthr + w];
-                    const int64_t o = perm[iu];
-                    if (tid < ef) phi_out[o] = phi_far[iu] + d;
-                    else E_out[3 * o + tid - ef] = E_far[3 * (int64_t)iu + tid - ef] + d;
-                }
-                __syncthreads();
-            }
+            fx_redo<SLO, SHI, PHI, FIELD>(s_redo, cnt, b + t0, q0, q1, src, begin, end, px, py, pz, Sm, accd, phi_far, E_far,
+                                          perm, phi_out, E_out);
         }
         if (t0 + stride < nt)
             for (int c = 0; c < NC; ++c) accd[c * nthr + tid] = 0.0;
@@ -707,13 +727,13 @@ void launch_fx(fmm_tree *t, int want_phi, int want_field, double *phi, double *E
     // 128 threads a leaf; where the leaves would leave the chip idle, more copies of each
     const int64_t sms = std::max(1, sm_count());
     const int nthr = t->nleaves >= 4 * sms ? 128 : (t->nleaves >= 2 * sms ? 256 : 512);
+    // blocks a leaf: two tiles or so each, and not many millions of blocks with nothing to do
+    const int64_t want = t->long_leaf ? (t->long_leaf + 2 * nthr - 1) / (2 * nthr) : 1;
+    const unsigned parts = (unsigned)std::min<int64_t>({want, 256, std::max<int64_t>(8, (1 << 20) / t->nleaves)});
     auto go = [&](auto kern, int nw, int ch, int nc) {
         const size_t smem = 8 * (size_t)nc * nthr +
                             std::max<size_t>(16 * (size_t)nw * ch, 32 * (size_t)nc * nthr);
         allow_max_dynamic_smem(kern);
-        // blocks a leaf: two tiles or so each, and not many millions of blocks with nothing to do
-        const int64_t want = t->long_leaf ? (t->long_leaf + 2 * nthr - 1) / (2 * nthr) : 1;
-        const unsigned parts = (unsigned)std::min<int64_t>({want, 256, std::max<int64_t>(8, (1 << 20) / t->nleaves)});
         launch_next(t->stream, kern, dim3((unsigned)t->nleaves, parts), nthr, smem,
             (const int32_t *)t->b_leaves.ptr, (const int32_t *)t->b_begin.ptr, (const int32_t *)t->b_end.ptr,
             (const int32_t *)t->b_p2p_off.ptr, (const int32_t *)t->b_p2p_src.ptr, (const int32_t *)t->b_level.ptr,
@@ -722,12 +742,16 @@ void launch_fx(fmm_tree *t, int want_phi, int want_field, double *phi, double *E
             (const double *)t->b_py.ptr, (const double *)t->b_pz.ptr, (const double *)t->b_S.ptr,
             (const double *)t->b_phi.ptr, (const double *)t->b_E.ptr, (const int32_t *)t->b_perm.ptr, phi, E);
     };
-    if (want_phi && want_field)
-        go(k_p2p_fx<SLO, SHI, true, true>, FxRec<SLO, SHI, true, true>::nw, FxRec<SLO, SHI, true, true>::ch, 4);
-    else if (want_phi)
-        go(k_p2p_fx<SLO, SHI, true, false>, FxRec<SLO, SHI, true, false>::nw, FxRec<SLO, SHI, true, false>::ch, 1);
-    else
-        go(k_p2p_fx<SLO, SHI, false, true>, FxRec<SLO, SHI, false, true>::nw, FxRec<SLO, SHI, false, true>::ch, 3);
+    auto pick = [&](auto phi_t, auto field_t) {
+        constexpr bool PHI = decltype(phi_t)::value, FIELD = decltype(field_t)::value;
+        using Rec = FxRec<SLO, SHI, PHI, FIELD>;
+        constexpr int nc = (PHI ? 1 : 0) + (FIELD ? 3 : 0);
+        if (parts > 1) go(k_p2p_fx<SLO, SHI, PHI, FIELD, true>, Rec::nw, Rec::ch, nc);
+        else go(k_p2p_fx<SLO, SHI, PHI, FIELD, false>, Rec::nw, Rec::ch, nc);
+    };
+    if (want_phi && want_field) pick(std::true_type(), std::true_type());
+    else if (want_phi) pick(std::true_type(), std::false_type());
+    else pick(std::false_type(), std::true_type());
 }
 
 }  // namespace
