@@ -236,23 +236,26 @@ __global__ void __launch_bounds__(kFxThreads) k_m2l_fx(const __grid_constant__ F
 // first, so that every cell is with a running block when the first targets' block
 // waits for them: the wait ends whatever else holds the rest of the chip (as
 // blocks of a cooperative launch that met at a grid barrier, it could run into its
-// bound).  ctl: [0] claimed, [1] blocks of cells done, from 0.
-constexpr int kExpPer = 16;                          // cells or targets of a block
+// bound).  per: cells or targets of a block; four where all blocks fit the chip at
+// once or nearly (one for each warp), eight beyond, as each claim is an atomic on one
+// word (125k and 1M dipoles, us: 4 30, 102; 8 34, 87; 16 43, 90; as blocks that met at
+// a barrier 29, 80).  ctl: [0] claimed, [1] blocks of cells done, from 0.
+constexpr int kExpSmall = 1 << 15;                   // cells and targets up to which a block takes four
 __global__ void __launch_bounds__(128)
 k_fx_exps(const double *M, int64_t nc, DevTables tb, const int32_t *am, const int32_t *level, const int32_t *sys,
           const int *e_side, int nq, int bits, int2 *Mx, int *eM, int slots, const int32_t *tile_tgt,
-          const int32_t *off, const int32_t *src, const int32_t *didx, const int *ekey, int *etgt, unsigned *ctl)
+          const int32_t *off, const int32_t *src, const int32_t *didx, const int *ekey, int *etgt, unsigned *ctl, int per)
 {
     extern __shared__ double fsm[];
     __shared__ unsigned s_id;
     __shared__ int s_ok;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned ncb = (unsigned)((nc + kExpPer - 1) / kExpPer);
+    const unsigned ncb = (unsigned)((nc + per - 1) / per);
     if (threadIdx.x == 0) s_id = atomicAdd(ctl, 1u);
     __syncthreads();
     if (s_id < ncb) {
         double *v = fsm + w * tb.nM;
-        const int64_t c0 = (int64_t)s_id * kExpPer, c1 = min(nc, c0 + kExpPer);
+        const int64_t c0 = (int64_t)s_id * per, c1 = min(nc, c0 + per);
         for (int64_t c = c0 + w; c < c1; c += 4) {
             for (int m = lane; m < tb.nM; m += 32) v[m] = M[c * tb.nM + m];
             __syncwarp();
@@ -303,7 +306,7 @@ k_fx_exps(const double *M, int64_t nc, DevTables tb, const int32_t *am, const in
         __threadfence();
     }
     __syncthreads();
-    const int q0 = (int)(s_id - ncb) * kExpPer, q1 = min(slots, q0 + kExpPer);
+    const int q0 = (int)(s_id - ncb) * per, q1 = min(slots, q0 + per);
     for (int q = q0 + w; q < q1; q += 4) {
         const int c = tile_tgt[q];
         int e = kZeroExp;
@@ -544,11 +547,12 @@ fmm_status run_fx_exps(fmm_tree *t, const double *M, const DevTables &tb)
     const size_t acc = 32 * (size_t)slots * Ly.groups;
     FMM_TRY(cuda_check(t, cudaMemsetAsync(t->b_fx_acc.ptr, 0, acc + slots / 8 + 16, st), "memset"));
     const int32_t *am = (const int32_t *)t->b_fx_el.ptr + Ly.E + Ly.first.size();
-    k_fx_exps<<<gridn(t->ncells, kExpPer) + gridn(slots, kExpPer), 128, 32 * (size_t)tb.nM, st>>>(
+    const int per = t->ncells + slots <= kExpSmall ? 4 : 8;
+    k_fx_exps<<<gridn(t->ncells, per) + gridn(slots, per), 128, 32 * (size_t)tb.nM, st>>>(
         M, t->ncells, tb, am, (const int32_t *)t->b_level.ptr, (const int32_t *)t->b_sys.ptr, t->sys_eside_dev(), Ly.nq,
         Ly.bits, (int2 *)t->b_Mh.ptr, (int *)t->b_fx_em.ptr, slots, (const int32_t *)t->b_tc_tgt.ptr,
         (const int32_t *)t->b_m2l_off.ptr, (const int32_t *)t->b_m2l_src.ptr, (const int32_t *)t->b_m2l_didx.ptr,
-        (const int *)t->b_fx_ekey.ptr, (int *)t->b_fx_et.ptr, (unsigned *)((char *)t->b_fx_acc.ptr + acc + slots / 8));
+        (const int *)t->b_fx_ekey.ptr, (int *)t->b_fx_et.ptr, (unsigned *)((char *)t->b_fx_acc.ptr + acc + slots / 8), per);
     ++t->launches;
     return cuda_check(t, cudaGetLastError(), "fixed-point multipoles");
 }
