@@ -10,7 +10,7 @@
 // per factor: a pair term's error is at or below an FP64 evaluation's (about
 // ten roundings of 2^-53), and the sums over pairs are exact integers.
 // Measured, one million dipoles, field, 946 M interactions: 36.3 ms with the
-// symmetric FP64 kernel -> 10.3 ms; error against long double at or below the
+// symmetric FP64 kernel -> 10.4 ms; error against long double at or below the
 // FP64 kernels' (a set of 700: 1e-16 to 4e-16 against 2e-16 to 1e-15).
 // Bound: the integer multiply pipe and the ALU together; 16 or 32 warps per SM
 // run alike.  Measured and not better: cross products by IMAD.HI, sums by
