@@ -813,7 +813,9 @@ k_l2p(const int32_t *leaves, const int32_t *begin, const int32_t *end, const dou
     if (lane == 0) s_re[w] = re;
     expand_local_cg(L + (int64_t)c * tb.nLh, tb, Lsm);      // ends with a barrier
     re = max(max(s_re[0], s_re[1]), max(s_re[2], s_re[3]));
-    if (re == kNoExp) re = 0;                               // every particle at the centre
+    // every particle at the centre: a radius below FP64's range leaves the coefficients
+    // of k = 0 their scale (at a radius of 1 the others set it, and those lost their bits)
+    if (re == kNoExp) re = -2200;
     int top[4] = {kNoExp, kNoExp, kNoExp, kNoExp};
     for (int i = threadIdx.x; i < nst; i += kL2PThreads) {
         const int k = ord[i], up = mi_shell(mi_at(tb.mi, k)) * re;
