@@ -185,6 +185,7 @@ namespace {
 
 constexpr int kM2LThreads = 128;
 constexpr int kM2LBatch = 16;
+constexpr size_t kM2LSmemMax = 226 * 1024;   // next to the kernel's static shared memory
 
 __constant__ int8_t c_nx[kMaxTot], c_ny[kMaxTot], c_nz[kMaxTot];
 
@@ -612,7 +613,8 @@ k_upward(const int32_t *leaves, const int32_t *begin, const int32_t *end, const 
 }
 
 // ------------------------------------------------------------------ M2L
-// One block per target cell.  Sources are taken kM2LBatch at a time: their
+// One block per target cell.  Sources are taken `batch` at a time (16; 8 where the full
+// Cartesian sums of p + s = 12 leave no shared memory for more): their
 // multipoles and derivative-table rows are staged in shared memory, then
 // each thread walks its fixed chunk of (n, m) terms, accumulating
 // D_{n+m} M_m over the staged sources, and flushes each finished n-run to its
@@ -655,7 +657,7 @@ k_fold_m(const Tm *M, int ldM, int64_t nc, DevTables tb, Tm *Mh, int ldH)
 __global__ void __launch_bounds__(kM2LThreads)
 k_m2l(const int32_t *off, const int32_t *src, const int32_t *didx, const int32_t *level,
       const int32_t *sys, const int *e_side, const double *M, const double *D, DevTables tb,
-      double *L)
+      double *L, int batch)
 {
     pdl_wait();
     extern __shared__ double sm[];
@@ -666,16 +668,16 @@ k_m2l(const int32_t *off, const int32_t *src, const int32_t *didx, const int32_t
     const int nM = tb.nMh, nD = tb.nD, T = tb.m2l_T, Tn = kM2LThreads;
     const int ldM = nM | 1, ldD = nD | 1;              // odd strides spread banks
     double *Msm = sm;                                  // [batch][ldM]
-    double *Dsm = Msm + kM2LBatch * ldM;               // [batch][ldD]
-    double *part = Dsm + kM2LBatch * ldD;              // [slots][Tn]
+    double *Dsm = Msm + batch * ldM;                   // [batch][ldD]
+    double *part = Dsm + batch * ldD;                  // [slots][Tn]
     uint32_t *desc = (uint32_t *)(part + tb.m2l_slots * Tn);   // [T][Tn]
     const int tid = threadIdx.x;
     const int lt = level[c], es = e_side[sys[c]];
     __shared__ int bsrc[kM2LBatch], bdidx[kM2LBatch], beu[kM2LBatch];
     for (int i = tid; i < T * Tn; i += Tn) desc[i] = tb.m2l_desc[i];
     for (int i = tid; i < tb.m2l_slots * Tn; i += Tn) part[i] = 0.0;
-    for (int k0 = b; k0 < e; k0 += kM2LBatch) {
-        const int kb = min(kM2LBatch, e - k0);
+    for (int k0 = b; k0 < e; k0 += batch) {
+        const int kb = min(batch, e - k0);
         __syncthreads();
         if (tid < kb) {                    // batch metadata, loaded in parallel
             const int s = src[k0 + tid];
@@ -1214,12 +1216,14 @@ fmm_status run_expansions(fmm_tree *t, int p, int want_phi, int want_field)
     } else if (t->n_m2l > 0) {
         const int ldM = tb.nMh | 1, ldD = tb.nD | 1;
         size_t fixed = 8 * (size_t)tb.m2l_slots * kM2LThreads + 4 * (size_t)tb.m2l_T * kM2LThreads;
-        size_t smem = fixed + 8 * (size_t)kM2LBatch * (ldM + ldD);
+        const size_t row = 8 * (size_t)(ldM + ldD);
+        const int batch = fixed + kM2LBatch * row <= kM2LSmemMax ? kM2LBatch : kM2LBatch / 2;
+        const size_t smem = fixed + batch * row;
         allow_max_dynamic_smem(k_m2l);
         launch_next_if(!side || Ms != M, st, k_m2l, (unsigned)nc, kM2LThreads, smem,
             (const int32_t *)t->b_m2l_off.ptr, (const int32_t *)t->b_m2l_src.ptr,
             (const int32_t *)t->b_m2l_didx.ptr, (const int32_t *)t->b_level.ptr,
-            (const int32_t *)t->b_sys.ptr, t->sys_eside_dev(), Ms, (const double *)t->b_D.ptr, tb, L);
+            (const int32_t *)t->b_sys.ptr, t->sys_eside_dev(), Ms, (const double *)t->b_D.ptr, tb, L, batch);
         ++t->launches;
     }
     record(t, 9);
