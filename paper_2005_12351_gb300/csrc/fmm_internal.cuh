@@ -132,6 +132,8 @@ struct FxLayout {
     int s = -1, p = -1, h = -1, n_lo = -1, nM = 0, nq = 0, ncol = 0, groups = 0, E = 0, cap = 0;
     int bits = 0, products = 0;   // fraction bits of a multipole, terms (n, m) of a pair
     std::vector<int> el, first, am, col, owner;
+    int K = 0;                    // classes of rows with exponents of their own
+    std::vector<int> cls;         // a group's class: its lowest order, at least 1 (n = 0 alone is class 0)
 };
 
 // threads of the M2L blocks (the per-thread term lists are built for it)

@@ -22,6 +22,13 @@
 //   per cell  e_s:  |M'| < 2^e_s;  M' = (Mh 2^26 + Ml) 2^(e_s - B), B = 57 (56 for nM > 126)
 //   per key   e_k:  sum_m |T'_nm| < 2^e_k for every n; T' likewise at 2^(e_k - 57)
 //   per target e_t: sum over its list of 2^(e_s + e_k) <= 2^e_t
+// both for every class of n: n = 0 alone, then the groups of four columns by their
+// lowest order.  The row sums grow with the order where cells are close (theta 0.7,
+// p = 9: a hundred times those of n = 0) and fall by 2^-g an order where the source is g
+// levels coarser: in one unit for all n the field was off by 9e-15 of the magnitudes of
+// its terms there, 5e-13 at p = 12, 4e-12 on small sets of 22 levels; FP64 1e-16.
+// With their own units it is within 4e-16 up to p = 10 at theta 0.6 and p = 9 at 0.7;
+// beyond (1e-15 to 1e-14: the multipoles share one unit a cell) the per-cell kernel stays.
 // A row's sum A1 + A0 / 2^26, A1 = sum Th Mh, A0 = sum (Th Ml + Tl Mh), stays
 // below 2^(B + 5) (the row sums of T' bound it) and A0 below 2^63 (nM 2^(B - 1)
 // and 2^56); it is shifted right by e_t - e_s - e_k into a 64-bit sum that
@@ -48,6 +55,7 @@ constexpr int kFxThreads = 128;
 // rows of a block: a part of a chunk (1M dipoles, p = 6: 1.84 ms with 8 rows,
 // 1.86 with 16, 1.91 with 32; 200k: 0.25, 0.275, 0.33: the last blocks' wait)
 constexpr int kFxRows = 8;
+constexpr int kFxMaxK = 13;          // classes: orders up to 12
 constexpr int kFxMaxNM = 253;        // A0 stays below 2^63
 constexpr int kFxSmemMax = 216 * 1024;
 constexpr int kFxPad = 33;           // 16-byte pieces per line of 32 targets: staging by rows without conflicts
@@ -56,7 +64,7 @@ constexpr int kBadExp = 1 << 24;     // a row that holds an infinity or a NaN
 
 // What turns a target's sums into its row of L
 struct FxOut {
-    const int32_t *tile_tgt, *col, *level, *sys, *rn;    // rn: full index of each stored component
+    const int32_t *tile_tgt, *col, *cls, *level, *sys, *rn;      // rn: full index of each stored component
     const int *e_side;
     double *L;
     int s, ncol, nL, nLh, unit;
@@ -66,16 +74,18 @@ struct FxArgs {
     const int32_t *chunk_rb, *chunk_re, *row_key, *slot;
     const uint32_t *tile_chunk;          // [tiles + 1] first chunk of each tile
     const int4 *M;                       // [cells][nq]: two limb pairs (h, l, h, l) each
-    const int *eM, *ekey, *etgt;
+    const int *eM;
+    const int *ekey, *etgt;              // [key][K], [target][K] exponents of the classes
     const int2 *img;                     // [keys][E] limb pairs
     u64 *acc;                            // [tile][4][ncolp][32]
     unsigned *arrive;                    // [tile][4] blocks done, from 0
     FxOut out;
+    int K, with0;                        // classes; column 0 is n = 0
     int parts, tiles, nq, E, ncolp;      // parts: blocks of kFxRows rows a chunk can take
     // the column groups (4 columns each) dealt to the four warps: image offset
     // (elements), pairs of multipoles, first column
     int ng[4];
-    int g_off[4][kFxMaxGroups], g_mq[4][kFxMaxGroups], g_col[4][kFxMaxGroups];
+    int g_off[4][kFxMaxGroups], g_mq[4][kFxMaxGroups], g_col[4][kFxMaxGroups], g_cls[4][kFxMaxGroups];
 };
 
 struct Sum {
@@ -106,14 +116,15 @@ __device__ __noinline__ void fx_finish(const FxArgs &a, int slot0, s64 *fs)
     for (int t = w; t < 32; t += 4) {
         const int c = o.tile_tgt[slot0 + t];
         if (c < 0) continue;
-        const int et = a.etgt[slot0 + t], hl = o.e_side[o.sys[c]] - o.level[c] - 1;
+        const int *et = a.etgt + (size_t)(slot0 + t) * a.K;
+        const int hl = o.e_side[o.sys[c]] - o.level[c] - 1;
         for (int r = lane; r < o.nLh; r += 32) {
             const int k = s_pos[o.rn[r]];
             double v = 0.0;
             if (k >= 0) {
-                const int cv = o.col[k], nn = (cv >> 9) & 15, bn = cv >> 13;
-                v = ldexp((double)fs[k * kFxPad + t], et - o.unit + bn - (nn + 1 + o.s) * hl);
-                if (et >= kBadExp / 2) v = __longlong_as_double(0x7ff8000000000000ll);
+                const int cv = o.col[k], nn = (cv >> 9) & 15, bn = cv >> 13, e = et[nn ? o.cls[k >> 2] : 0];
+                v = ldexp((double)fs[k * kFxPad + t], e - o.unit + bn - (nn + 1 + o.s) * hl);
+                if (e >= kBadExp / 2) v = __longlong_as_double(0x7ff8000000000000ll);
             }
             o.L[(size_t)c * o.nLh + r] = v;
         }
@@ -131,24 +142,28 @@ __device__ __noinline__ void fx_finish(const FxArgs &a, int slot0, s64 *fs)
 // row's copies in flight halve the blocks an SM holds: 1M dipoles, p = 6, 1.96
 // instead of 1.86 ms; 262k Plummer, p = 8, 1.99 instead of 1.67.)
 template <int NG>
-__global__ void __launch_bounds__(kFxThreads) k_m2l_fx(const __grid_constant__ FxArgs a)
+__global__ void __launch_bounds__(kFxThreads, NG <= 4 ? 5 : (NG <= 8 ? 4 : 2)) k_m2l_fx(const __grid_constant__ FxArgs a)
 {
     pdl_wait();
     extern __shared__ int4 sm4[];
-    __shared__ int s_src[kFxRows][32], s_sh[kFxRows][32], s_key[kFxRows], s_act[kFxRows], s_tile, s_last;
+    __shared__ int s_src[kFxRows][32], s_es[kFxRows][32], s_ek[kFxRows][kFxMaxK], s_key[kFxRows],
+        s_act[kFxRows], s_tile, s_last;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int qt = blockIdx.x & 3, chunk = (blockIdx.x >> 2) / a.parts, part = (blockIdx.x >> 2) - chunk * a.parts;
     const int rb = a.chunk_rb[chunk] + part * kFxRows, n = min(a.chunk_re[chunk] - rb, kFxRows);
     for (int i = tid; i < a.tiles; i += kFxThreads)
         if ((int)a.tile_chunk[i] <= chunk && chunk < (int)a.tile_chunk[i + 1]) s_tile = i;
     __syncthreads();
-    const int slot0 = s_tile * 128 + 32 * qt, et = a.etgt[slot0 + lane];
+    const int slot0 = s_tile * 128 + 32 * qt;
+    int4 *Ts = sm4 + a.nq * kFxPad;
+    int *Es = (int *)(Ts + (a.E >> 1));              // [K][32] exponents of the targets
+    for (int k = w; k < a.K; k += 4) Es[32 * k + lane] = a.etgt[(size_t)(slot0 + lane) * a.K + k];
     int any = 0;
     for (int r = w; r < n; r += 4) {
         const int src = a.slot[(size_t)(rb + r) * 128 + 32 * qt + lane], key = a.row_key[rb + r];
         s_src[r][lane] = src;
-        // 0..62: a pair 2^62 below its target's unit adds nothing
-        s_sh[r][lane] = src >= 0 ? min(max(et - a.eM[src] - a.ekey[key], 0), 62) : 0;
+        s_es[r][lane] = src >= 0 ? a.eM[src] : 0;
+        if (lane < a.K) s_ek[r][lane] = a.ekey[(size_t)key * a.K + lane];
         const int act = __any_sync(0xffffffffu, src >= 0);
         any |= act;
         if (lane == 0) {
@@ -157,7 +172,6 @@ __global__ void __launch_bounds__(kFxThreads) k_m2l_fx(const __grid_constant__ F
         }
     }
     any = __syncthreads_or(any);
-    int4 *Ts = sm4 + a.nq * kFxPad;
     auto stage = [&](int r) {
         for (int k = tid, t = tid / a.nq, q = tid - t * a.nq; k < 32 * a.nq; k += kFxThreads) {
             const int src = s_src[r][t];
@@ -184,16 +198,19 @@ __global__ void __launch_bounds__(kFxThreads) k_m2l_fx(const __grid_constant__ F
         cp_async_wait<0>();
         __syncthreads();
         const int4 *Ms = sm4 + lane;
-        const int sh = s_sh[r][lane];
-        const s64 half = (1ll << sh) >> 1;
+        const int es = s_es[r][lane];
+        // 0..62: a pair 2^62 below its target's unit adds nothing
+        auto shift = [&](int k) { return min(max(Es[32 * k + lane] - es - s_ek[r][k], 0), 62); };
 #pragma unroll
         for (int g = 0; g < NG; ++g) {
             if (g < ng) {
                 const int4 *T4 = Ts + (a.g_off[w][g] >> 1);
-                const int mq = a.g_mq[w][g];
+                const int mq = a.g_mq[w][g], sh = shift(a.g_cls[w][g]);
+                const int sh0 = g == 0 && w == 0 && a.with0 ? shift(0) : sh;
+                const s64 half = (1ll << sh) >> 1, half0 = (1ll << sh0) >> 1;
                 Sum s[4];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) s[c] = {half, 1ll << 25};    // both shifts round
+                for (int c = 0; c < 4; ++c) s[c] = {g + c ? half : half0, 1ll << 25};    // both shifts round
 #pragma unroll 4
                 for (int q = 0; q < mq; ++q) {
                     const int4 m = Ms[q * kFxPad];
@@ -208,7 +225,7 @@ __global__ void __launch_bounds__(kFxThreads) k_m2l_fx(const __grid_constant__ F
                     mac(s[3], t3.z, t3.w, m.z, m.w);
                 }
 #pragma unroll
-                for (int c = 0; c < 4; ++c) P[g][c] += (s[c].a1 + (s[c].a0 >> 26)) >> sh;
+                for (int c = 0; c < 4; ++c) P[g][c] += (s[c].a1 + (s[c].a0 >> 26)) >> (g + c ? sh : sh0);
             }
         }
         __syncthreads();                             // before the next row is staged
@@ -244,7 +261,8 @@ constexpr int kExpSmall = 1 << 15;                   // cells and targets up to 
 __global__ void __launch_bounds__(128)
 k_fx_exps(const double *M, int64_t nc, DevTables tb, const int32_t *am, const int32_t *level, const int32_t *sys,
           const int *e_side, int nq, int bits, int2 *Mx, int *eM, int slots, const int32_t *tile_tgt,
-          const int32_t *off, const int32_t *src, const int32_t *didx, const int *ekey, int *etgt, unsigned *ctl, int per)
+          const int32_t *off, const int32_t *src, const int32_t *didx, int k0, int K, const int *ekey, int *etgt, unsigned *ctl,
+          int per)
 {
     extern __shared__ double fsm[];
     __shared__ unsigned s_id;
@@ -309,18 +327,41 @@ k_fx_exps(const double *M, int64_t nc, DevTables tb, const int32_t *am, const in
     const int q0 = (int)(s_id - ncb) * per, q1 = min(slots, q0 + per);
     for (int q = q0 + w; q < q1; q += 4) {
         const int c = tile_tgt[q];
-        int e = kZeroExp;
+        constexpr int kK = kFxMaxK;
+        int e[kK];
+#pragma unroll
+        for (int k = 0; k < kK; ++k) e[k] = kZeroExp;
         if (c >= 0 && s_ok) {
             const int b = off[c], en = off[c + 1];
-            for (int k = b + lane; k < en; k += 32) e = max(e, __ldcg(eM + src[k]) + ekey[didx[k]]);
-            e = __reduce_max_sync(0xffffffffu, e);
-            float f = 0.0f;
-            for (int k = b + lane; k < en; k += 32)
-                f += exp2f((float)max(__ldcg(eM + src[k]) + ekey[didx[k]] - e, -100));
-            for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-            e += ilogbf(f * 1.01f) + 1;
+            float f[kK];
+            for (int q2 = b + lane; q2 < en; q2 += 32) {
+                const int es = __ldcg(eM + src[q2]), *ek = ekey + (size_t)didx[q2] * K;
+#pragma unroll
+                for (int k = 0; k < kK; ++k)
+                    if (k >= k0 && k < K) e[k] = max(e[k], es + ek[k]);
+            }
+#pragma unroll
+            for (int k = 0; k < kK; ++k) {
+                f[k] = 0.0f;
+                if (k >= k0 && k < K) e[k] = __reduce_max_sync(0xffffffffu, e[k]);
+            }
+            for (int q2 = b + lane; q2 < en; q2 += 32) {
+                const int es = __ldcg(eM + src[q2]), *ek = ekey + (size_t)didx[q2] * K;
+#pragma unroll
+                for (int k = 0; k < kK; ++k)
+                    if (k >= k0 && k < K) f[k] += __int_as_float((127 + max(es + ek[k] - e[k], -100)) << 23);   // 2 to that
+            }
+#pragma unroll
+            for (int k = 0; k < kK; ++k)
+                if (k >= k0 && k < K) {
+                    for (int o = 16; o > 0; o >>= 1) f[k] += __shfl_xor_sync(0xffffffffu, f[k], o);
+                    e[k] += ilogbf(f[k] * 1.01f) + 1;
+                }
         }
-        if (lane == 0) etgt[q] = s_ok ? e : kBadExp;          // a wait that gave up shows as NaN
+        if (lane == 0)
+#pragma unroll
+            for (int k = 0; k < kK; ++k)
+                if (k < K) etgt[(size_t)q * K + k] = s_ok ? e[k] : kBadExp;      // a wait that gave up shows as NaN
     }
 }
 
@@ -335,37 +376,41 @@ __device__ __forceinline__ double fx_element(int el, const double *D, int esc, i
 
 __global__ void __launch_bounds__(128)
 k_fx_images(const uint64_t *dkeys, const double *D, int nD, int E, int ngroups, const int32_t *g_first,
-            const int32_t *el, int2 *img, int *ekey)
+            const int32_t *g_cls, const int32_t *el, int with0, int K, int2 *img, int *ekey)
 {
-    __shared__ double s_max[4];
+    __shared__ u64 s_big[kFxMaxK];             // largest row sum of each class, its bits
+    __shared__ int s_ek[kFxMaxK];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t r = blockIdx.x;
     const uint64_t key = dkeys[r];
     const int gap = (int)((key >> 52) & 31), tfiner = (int)((key >> 51) & 1);
     const int esc = tfiner ? 0 : gap, dl = tfiner ? gap : -gap;
     const double *Dr = D + r * nD;
-    double big = 0.0;
+    if (threadIdx.x < K) s_big[threadIdx.x] = 0;
+    __syncthreads();
     for (int g = w; g < ngroups; g += 4) {
         double v = 0.0;                              // lanes of equal (lane & 3) share a column
         for (int e = g_first[g] + lane; e < g_first[g + 1]; e += 32) v += fabs(fx_element(el[e], Dr, esc, dl));
         v += __shfl_xor_sync(0xffffffffu, v, 4);
         v += __shfl_xor_sync(0xffffffffu, v, 8);
         v += __shfl_xor_sync(0xffffffffu, v, 16);
-        big = fmax(big, v);
+        if (lane < 4) atomicMax(&s_big[with0 && g + lane == 0 ? 0 : g_cls[g]], (u64)__double_as_longlong(v));
     }
-    big = fmax(big, __shfl_xor_sync(0xffffffffu, big, 1));
-    big = fmax(big, __shfl_xor_sync(0xffffffffu, big, 2));
-    if (lane == 0) s_max[w] = big;
     __syncthreads();
-    big = fmax(fmax(s_max[0], s_max[1]), fmax(s_max[2], s_max[3]));
     // row sums below 2^ek less a margin for their own rounding: Th < 2^31
-    const int ek = big > 0.0 ? ilogb(big * 1.004) + 1 : 0;
-    if (threadIdx.x == 0) ekey[r] = ek;
-    for (int e = threadIdx.x; e < E; e += blockDim.x) {
-        const s64 x = __double2ll_rn(ldexp(fx_element(el[e], Dr, esc, dl), 57 - ek));
-        const int h = (int)((x + (1ll << 25)) >> 26);
-        img[r * E + e] = make_int2(h, (int)(x - ((s64)h << 26)));
+    if (threadIdx.x < K) {
+        const double big = __longlong_as_double((long long)s_big[threadIdx.x]);
+        s_ek[threadIdx.x] = big > 0.0 ? ilogb(big * 1.004) + 1 : 0;
+        ekey[r * K + threadIdx.x] = s_ek[threadIdx.x];
     }
+    __syncthreads();
+    for (int g = w; g < ngroups; g += 4)
+        for (int e = g_first[g] + lane; e < g_first[g + 1]; e += 32) {
+            const int ek = s_ek[with0 && g + (lane & 3) == 0 ? 0 : g_cls[g]];
+            const s64 x = __double2ll_rn(ldexp(fx_element(el[e], Dr, esc, dl), 57 - ek));
+            const int h = (int)((x + (1ll << 25)) >> 26);
+            img[r * E + e] = make_int2(h, (int)(x - ((s64)h << 26)));
+        }
 }
 
 int log2_factorial(const MultiIndex &I, int k)
@@ -399,6 +444,8 @@ void build_layout_fx(FxLayout &Ly, int s, int p, int h, int n_lo)
     for (int gm : ms) Ly.am.push_back(a_of(gm) * 256 + (shell(gm) - s));
     Ly.col.clear();
     for (int n : ns) Ly.col.push_back(n | shell(n) << 9 | log2_factorial(I, n) << 13);
+    Ly.cls.clear();
+    Ly.K = std::max(p, 1) + 1;
     Ly.first.assign(1, 0);
     Ly.el.clear();
     Ly.products = 0;
@@ -425,6 +472,7 @@ void build_layout_fx(FxLayout &Ly, int s, int p, int h, int n_lo)
                 Ly.el.push_back(v);
             }
         Ly.first.push_back((int)Ly.el.size());
+        Ly.cls.push_back(std::max(shell(ns[4 * g]), 1));
     }
     Ly.E = (int)Ly.el.size();
     // columns to warps: the longest group to the least loaded warp, at most cap
@@ -452,7 +500,10 @@ void build_layout_fx(FxLayout &Ly, int s, int p, int h, int n_lo)
     }
 }
 
-inline size_t fx_smem(const FxLayout &Ly) { return 16 * (size_t)Ly.nq * kFxPad + 8 * (size_t)Ly.E; }
+inline size_t fx_smem(const FxLayout &Ly)
+{
+    return 16 * (size_t)Ly.nq * kFxPad + 8 * (size_t)Ly.E + 128 * (size_t)Ly.K;
+}
 
 inline unsigned gridn(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
@@ -490,7 +541,7 @@ bool fx_usable(fmm_tree *t, int s, int p, int harmonic, int n_lo)
         t->fx_img_p = -1;                     // images and maps of the old layout
         t->fx_off = false;
     }
-    if (t->fx_off) return false;
+    if (t->fx_off || (p >= 11 && t->theta > 0.5) || (p >= 10 && t->theta > 0.6)) return false;
     const double nsys = (double)std::max<int64_t>(1, (int64_t)t->sys_off.size() - 1);
     const double fill = (double)(Ly.products > kFxHighProducts ? kFxMinFillHigh : kFxMinFill) * t->n_doff;
     return (double)t->n_m2l * Ly.products >= kFxMinWork * nsys && (double)t->n_m2l >= fill * nsys && Ly.cap > 0 &&
@@ -505,8 +556,9 @@ fmm_status fx_prepare(fmm_tree *t, int p)
     if (t->tc_chunks == 0) return FMM_OK;
     const size_t slots = (size_t)t->tc_tiles * 128;
     if (t->fx_img_p != p) {
-        const size_t n1 = (size_t)Ly.E, n2 = Ly.first.size(), n3 = Ly.am.size(), n4 = Ly.col.size();
-        FMM_TRY(ensure(t, t->b_fx_el, 4 * (n1 + n2 + n3 + n4)));
+        const size_t n1 = (size_t)Ly.E, n2 = Ly.first.size(), n3 = Ly.am.size(), n4 = Ly.col.size(),
+                     n5 = Ly.cls.size();
+        FMM_TRY(ensure(t, t->b_fx_el, 4 * (n1 + n2 + n3 + n4 + n5)));
         int32_t *d = (int32_t *)t->b_fx_el.ptr;
         auto up = [&](const std::vector<int> &v) {
             const cudaError_t e = cudaMemcpyAsync(d, v.data(), 4 * v.size(), cudaMemcpyHostToDevice, st);
@@ -517,17 +569,18 @@ fmm_status fx_prepare(fmm_tree *t, int p)
         FMM_TRY(up(Ly.first));
         FMM_TRY(up(Ly.am));
         FMM_TRY(up(Ly.col));
+        FMM_TRY(up(Ly.cls));
         FMM_TRY(ensure(t, t->b_fx_img, 8 * (size_t)t->n_doff * Ly.E));
-        FMM_TRY(ensure(t, t->b_fx_ekey, 4 * (size_t)t->n_doff));
+        FMM_TRY(ensure(t, t->b_fx_ekey, 4 * (size_t)t->n_doff * Ly.K));
         d = (int32_t *)t->b_fx_el.ptr;
         k_fx_images<<<(unsigned)t->n_doff, 128, 0, st>>>(
-            (const uint64_t *)t->b_dkeys.ptr, (const double *)t->b_D.ptr, ntot(p + t->s), Ly.E, Ly.groups, d + n1, d,
-            (int2 *)t->b_fx_img.ptr, (int *)t->b_fx_ekey.ptr);
+            (const uint64_t *)t->b_dkeys.ptr, (const double *)t->b_D.ptr, ntot(p + t->s), Ly.E, Ly.groups, d + n1,
+            d + n1 + n2 + n3 + n4, d, Ly.n_lo == 0, Ly.K, (int2 *)t->b_fx_img.ptr, (int *)t->b_fx_ekey.ptr);
         ++t->launches;
         t->fx_img_p = p;
     }
     FMM_TRY(ensure(t, t->b_fx_em, 4 * (size_t)t->ncells));
-    FMM_TRY(ensure(t, t->b_fx_et, 4 * slots));
+    FMM_TRY(ensure(t, t->b_fx_et, 4 * slots * Ly.K));
     // the sums, the blocks done per 32 targets, k_fx_exps' counters
     FMM_TRY(ensure(t, t->b_fx_acc, 32 * slots * Ly.groups + slots / 8 + 16));
     // the limbs take the place of the folded multipoles
@@ -552,7 +605,8 @@ fmm_status run_fx_exps(fmm_tree *t, const double *M, const DevTables &tb)
         M, t->ncells, tb, am, (const int32_t *)t->b_level.ptr, (const int32_t *)t->b_sys.ptr, t->sys_eside_dev(), Ly.nq,
         Ly.bits, (int2 *)t->b_Mh.ptr, (int *)t->b_fx_em.ptr, slots, (const int32_t *)t->b_tc_tgt.ptr,
         (const int32_t *)t->b_m2l_off.ptr, (const int32_t *)t->b_m2l_src.ptr, (const int32_t *)t->b_m2l_didx.ptr,
-        (const int *)t->b_fx_ekey.ptr, (int *)t->b_fx_et.ptr, (unsigned *)((char *)t->b_fx_acc.ptr + acc + slots / 8), per);
+        Ly.n_lo, Ly.K, (const int *)t->b_fx_ekey.ptr, (int *)t->b_fx_et.ptr,
+        (unsigned *)((char *)t->b_fx_acc.ptr + acc + slots / 8), per);
     ++t->launches;
     return cuda_check(t, cudaGetLastError(), "fixed-point multipoles");
 }
@@ -579,6 +633,7 @@ fmm_status run_m2l_fx(fmm_tree *t, const DevTables &tb, double *L)
     a.arrive = (unsigned *)(a.acc + (size_t)slots * ncolp);
     a.out.tile_tgt = (const int32_t *)t->b_tc_tgt.ptr;
     a.out.col = (const int32_t *)t->b_fx_el.ptr + Ly.E + Ly.first.size() + Ly.am.size();
+    a.out.cls = a.out.col + Ly.col.size();
     a.out.level = (const int32_t *)t->b_level.ptr;
     a.out.sys = (const int32_t *)t->b_sys.ptr;
     a.out.rn = tb.h_rn;
@@ -591,6 +646,8 @@ fmm_status run_m2l_fx(fmm_tree *t, const DevTables &tb, double *L)
     a.out.unit = Ly.bits + 5;
     a.tiles = (int)t->tc_tiles;
     a.parts = (t->tc_G + kFxRows - 1) / kFxRows;
+    a.K = Ly.K;
+    a.with0 = Ly.n_lo == 0;
     a.nq = Ly.nq;
     a.E = Ly.E;
     a.ncolp = ncolp;
@@ -599,6 +656,7 @@ fmm_status run_m2l_fx(fmm_tree *t, const DevTables &tb, double *L)
         a.g_off[w][k] = Ly.first[g];
         a.g_mq[w][k] = (Ly.first[g + 1] - Ly.first[g]) / 8;
         a.g_col[w][k] = 4 * g;
+        a.g_cls[w][k] = Ly.cls[g];
     }
     const size_t smem = std::max(fx_smem(Ly), 32 * (size_t)Ly.groups * kFxPad);   // the last block's turn
     auto go = [&](auto kern) {
