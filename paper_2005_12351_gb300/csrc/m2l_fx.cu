@@ -15,10 +15,10 @@
 //   T'_nm = D_{n+m} (level factors) 2^(-a_m - b_n),   b_n = round(log2 n!),
 //   L_n = h_t^(-|n|-1-s) 2^(b_n) sum_pairs sum_m T'_nm M'_m.
 // a_m and b_n level the magnitudes over the orders: for particles spread over
-// a cell, or bunched in its corner, 1 <= p <= 12, max |M'| times the largest
-// row sum of |T'| is 1.2 to 7 times the sum of the absolute values of the
+// a cell, or bunched in its corner, at theta 0.5, 1 <= p <= 12, max |M'| times the
+// largest row sum of |T'| is 1.2 to 7 times the sum of the absolute values of the
 // terms of a first-order component, so that 57 bits of the product of those
-// bounds are more than the 53 of each FP64 rounding.
+// bounds are more than the 53 of each FP64 rounding (wider angles: below).
 //   per cell  e_s:  |M'| < 2^e_s;  M' = (Mh 2^26 + Ml) 2^(e_s - B), B = 57 (56 for nM > 126)
 //   per key   e_k:  sum_m |T'_nm| < 2^e_k for every n; T' likewise at 2^(e_k - 57)
 //   per target e_t: sum over its list of 2^(e_s + e_k) <= 2^e_t
@@ -136,7 +136,7 @@ __device__ __noinline__ void fx_finish(const FxArgs &a, int slot0, s64 *fs)
 // memory: [nq][33] 16-byte multipole pieces and E limb pairs of the operator of
 // one row; the other blocks of the SM compute while one waits for its row.  Bound
 // by the integer pipes, 3 multiply-adds a product: M2L phase (this kernel; the
-// per-cell k_m2l before) 5.59 -> 1.69 ms at 1M dipoles, p = 6 (32 targets 87 %
+// per-cell k_m2l before) 5.59 -> 1.73 ms at 1M dipoles, p = 6 (32 targets 87 %
 // full); 3.30 -> 1.54 ms at 262k Plummer, p = 8 (47 % full); 0.57 -> 0.23 ms at
 // 200k charges and dipoles, p = 6; 125k dipoles, p = 6: 0.68 -> 0.28 ms.  (Two stages with the next
 // row's copies in flight halve the blocks an SM holds: 1M dipoles, p = 6, 1.96
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kFxThreads, NG <= 4 ? 5 : (NG <= 8 ? 4 : 2)) k
 // bound).  per: cells or targets of a block; four where all blocks fit the chip at
 // once or nearly (one for each warp), eight beyond, as each claim is an atomic on one
 // word (125k and 1M dipoles, us: 4 30, 102; 8 34, 87; 16 43, 90; as blocks that met at
-// a barrier 29, 80).  ctl: [0] claimed, [1] blocks of cells done, from 0.
+// a barrier 29, 80; with an exponent for every order since, 125k 25, 1M 120).  ctl: [0] claimed, [1] blocks of cells done, from 0.
 constexpr int kExpSmall = 1 << 15;                   // cells and targets up to which a block takes four
 __global__ void __launch_bounds__(128)
 k_fx_exps(const double *M, int64_t nc, DevTables tb, const int32_t *am, const int32_t *level, const int32_t *sys,
