@@ -217,8 +217,9 @@ class FMMTree:
     def evaluate_graph(self, p: int, theta: float, want_potential=True, want_field=True,
                        potential=None, field=None):
         """fmm_evaluate replayed as one CUDA graph launch while (p, theta, flags, outputs)
-        stay the same.  Output tensors are allocated once per parameter set and reused."""
-        key = (int(p), float(theta), bool(want_potential), bool(want_field))
+        stay the same.  Output tensors are allocated once per parameter set and number of
+        particles, and reused."""
+        key = (self.n, int(p), float(theta), bool(want_potential), bool(want_field))
         cache = getattr(self, "_graph_out", None)
         if potential is None and field is None and cache and cache[0] == key:
             potential, field = cache[1], cache[2]
